@@ -709,20 +709,26 @@ WorkMap Engine::make_map(const std::vector<int>& counts) {
 
 // Maps of the GEMMs whose CTA counts follow the tile knobs.
 void Engine::build_gemm_maps() {
-  std::vector<int> ww, bw, dw, tc, nntc;
+  std::vector<int> ww, bw, dw, tc, nntc, red[3][2];
   for (auto* c : ctx_) {
     const Prob& d = c->d;
-    const int nsplit = div_up(d.npw, tn_kc_);
-    const int tw = div_up(d.nb, TN_TILE), ta = div_up(d.nproj, TN_TILE), td = div_up(3 * d.nproj, TN_TILE);
+    const int nsplit = div_up(d.npw, tn_kc_ > 0 ? tn_kc_ : tn_kc_f64(d.npw));
+    const int tw = tn_blocks(d.nb), ta = tn_blocks(d.nproj), td = tn_blocks(3 * d.nproj);
     ww.push_back(tw * tw * nsplit);
     bw.push_back(ta * tw * nsplit);
     dw.push_back(td * tw * nsplit);
     tc.push_back(div_up(d.npw, tc_kc_));
     nntc.push_back(div_up(div_up(d.npw, 128), nn_tpc_));
+    const int nin[3] = {d.nb, d.nproj, 3 * d.nproj};
+    for (int k = 0; k < 3; ++k)
+      for (int t = 0; t < 2; ++t)
+        red[k][t].push_back(div_up(nin[k] * d.nb, 256 / tn_reduce_lanes(t ? tc.back() : nsplit)));
   }
-  m_tn_ww_ = make_map(ww);
-  m_tn_bw_ = make_map(bw);
-  m_tn_dw_ = make_map(dw);
+  m_tn_[OPK_WB] = make_map(ww);
+  m_tn_[OPK_B] = make_map(bw);
+  m_tn_[OPK_DB] = make_map(dw);
+  for (int k = 0; k < 3; ++k)
+    for (int t = 0; t < 2; ++t) m_red_[k][t] = make_map(red[k][t]);
   m_tc_ = make_map(tc);
   m_nntc_ = make_map(nntc);
 }
@@ -790,6 +796,7 @@ Engine::Engine(const std::vector<sgo_ctx*>& ctxs, cudaStream_t stream) : ctx_(ct
   n_ = (int)ctxs.size();
   if (n_ == 0) return;
   precision_ = ctxs[0]->precision;
+  if (!precision_) tn_kc_ = 0;
   for (auto* c : ctxs) {
     if (c->precision != precision_) {
       set_error("all members of a batch must use the same precision");
@@ -801,8 +808,7 @@ Engine::Engine(const std::vector<sgo_ctx*>& ctxs, cudaStream_t stream) : ctx_(ct
     }
   }
   std::vector<Prob> host(n_);
-  std::vector<int> c_zcol, c_plane, c_dens, c_gz, c_gp, c_gew, c_gch, c_bands, c_tnww, c_tnbw, c_tndw, c_rww, c_rbw,
-      c_rdw, c_nn, c_atoms, c_projs, c_atomch, c_ewsg, c_prob, c_tc, c_nntc, c_preg[2], c_dreg[2], c_zreg[2], c_ppair,
+  std::vector<int> c_zcol, c_plane, c_dens, c_gz, c_gp, c_gew, c_gch, c_bands, c_rww, c_nn, c_atoms, c_projs, c_atomch, c_ewsg, c_prob, c_tc, c_nntc, c_preg[2], c_dreg[2], c_zreg[2], c_ppair,
       c_dpair, c_zpair, c_gx, c_gy, c_bigy, c_bigx, c_bigdy, c_bigd;
   size_t part = 0;
   int max_nproj = 0;
@@ -816,7 +822,8 @@ Engine::Engine(const std::vector<sgo_ctx*>& ctxs, cudaStream_t stream) : ctx_(ct
     max_nb_ = std::max(max_nb_, d.nb);
     const int nch = div_up(d.ngrid, GRID_CHUNK);
     maxchunk_ = std::max(maxchunk_, nch);
-    const int nsplit = div_up(d.npw, 128);  // the smallest CUDA-core K chunk the autotuner tries
+    // the smallest CUDA-core K chunk the autotuner tries, or the FP64 path's
+    const int nsplit = div_up(d.npw, precision_ ? 128 : tn_kc_f64(d.npw));
     // z-column passes: register FFTs on the mixed path where n3 has one (single thread or
     // lane pair per line), the shared-memory engine otherwise
     const bool zreg = precision_ == 1 && zreg_ok(d.n3);
@@ -866,9 +873,8 @@ Engine::Engine(const std::vector<sgo_ctx*>& ctxs, cudaStream_t stream) : ctx_(ct
     c_gch.push_back(nch);
     c_bands.push_back(d.nb);
     c_rww.push_back(div_up(d.nb * d.nb, 256));
-    c_rbw.push_back(div_up(d.nproj * d.nb, 256));
-    c_rdw.push_back(div_up(3 * d.nproj * d.nb, 256));
-    c_nn.push_back(div_up(d.npw, 64 * NN_RT) * div_up(d.nb, 64));
+    c_nn.push_back(precision_ ? div_up(d.npw, 64 * NN_RT) * div_up(d.nb, 64)
+                              : div_up(d.npw, nn_rows_f64(d.nb, d.npw)) * tn_blocks(d.nb));
     c_atoms.push_back(d.natom);
     c_projs.push_back(d.nproj);
     c_atomch.push_back(div_up(d.natom, LF_GROUP) * nch);
@@ -899,9 +905,7 @@ Engine::Engine(const std::vector<sgo_ctx*>& ctxs, cudaStream_t stream) : ctx_(ct
   m_gew_ = make_map(c_gew);
   m_gch_ = make_map(c_gch);
   m_bands_ = make_map(c_bands);
-  m_red_ww_ = make_map(c_rww);
-  m_red_bw_ = make_map(c_rbw);
-  m_red_dw_ = make_map(c_rdw);
+  m_asm_ = make_map(c_rww);
   m_nn_ = make_map(c_nn);
   m_atoms_ = make_map(c_atoms);
   m_projs_ = make_map(c_projs);
@@ -1159,18 +1163,15 @@ void Engine::grid_fft_raw(int which, int sign) {
 // feed F and the forces directly, where 3xTF32 noise would exceed the SCF tolerance.
 template <typename T>
 void Engine::tn(int akind, int arole, int bkind, int brole, int dst, bool allow_tc) {
-  const WorkMap* m = &m_tn_ww_;
-  const WorkMap* r = &m_red_ww_;
-  if (akind == OPK_B) { m = &m_tn_bw_; r = &m_red_bw_; }
-  if (akind == OPK_DB) { m = &m_tn_dw_; r = &m_red_dw_; }
   const int kind = akind == OPK_WB ? TK_GEMM_TN : TK_GEMM_SMALL;
   tbeg(kind);
   if (sizeof(T) == 4 && allow_tc && tc_ok_[akind]) {
     launch_gemm_tn_tc(L(m_tc_), d_tmaps_, akind, arole, bkind, brole, d_part_, part_stride_, tc_kc_);
-    launch_gemm_tn_reduce(L(*r), akind, bkind, dst, d_part_, part_stride_, tc_kc_);
+    launch_gemm_tn_reduce(L(m_red_[akind][1]), akind, bkind, dst, d_part_, part_stride_, tc_kc_);
   } else {
-    launch_gemm_tn<T>(L(*m), akind, arole, bkind, brole, d_part_, part_stride_, tn_kc_);
-    launch_gemm_tn_reduce(L(*r), akind, bkind, dst, d_part_, part_stride_, tn_kc_, akind == bkind && arole == brole);
+    launch_gemm_tn<T>(L(m_tn_[akind]), akind, arole, bkind, brole, d_part_, part_stride_, tn_kc_);
+    launch_gemm_tn_reduce(L(m_red_[akind][0]), akind, bkind, dst, d_part_, part_stride_, tn_kc_,
+                          akind == bkind && arole == brole);
   }
   tend(kind);
 }
@@ -1315,10 +1316,10 @@ void Engine::davidson_step() {
   tn<T>(OPK_WB, WB_X, OPK_WB, WB_HX, DD_HS);
   tn<T>(OPK_WB, WB_X, OPK_WB, WB_P, DD_TM, false);
   tn<T>(OPK_WB, WB_X, OPK_WB, WB_HP, DD_CM);
-  launch_rr2_assemble(L(m_red_ww_), 0);
+  launch_rr2_assemble(L(m_asm_), 0);
   tn<T>(OPK_WB, WB_P, OPK_WB, WB_P, DD_S, false);
   tn<T>(OPK_WB, WB_P, OPK_WB, WB_HP, DD_HS);
-  launch_rr2_assemble(L(m_red_ww_), 1);
+  launch_rr2_assemble(L(m_asm_), 1);
   rr_solve(2);
   // the Ritz vectors and their H images into the dead W, W2, which then take the roles of
   // X and HX

@@ -75,12 +75,18 @@ constexpr float RR_DROPPED = -2.f;  // pivot deviation recorded for a left-out d
 constexpr int RR_SPARSE = 256;
 
 // ---------------------------------------------------------------------------
-// C = A^T B, split-K partials.  CTA = (problem, tile_i, tile_j, split).  Thread (ti, tj)
-// owns rows 4 ti .. 4 ti + 3 and columns 4 tj .. 4 tj + 3 of the 64 x 64 tile, so every
-// K step reads its A and B values as one 16-byte shared load each (two for FP64).  A K
-// chunk of 32 is staged from 16-byte global loads along K (zero beyond the split's end:
-// splits end on multiples of 32 or at npw, whose tail up to ld is zero).  A^T A (same
-// operand twice) computes the tiles with tile_i <= tile_j only; the reduction mirrors them.
+// C = A^T B, split-K partials.  CTA = (problem, tile block, split).  The outputs are dealt in
+// 4 x 4 tiles: na / 4 x nb / 4 of them (rounded up), in blocks of at most 16 x 16 tiles of
+// about equal size, and a block's tiles go to the CTA's threads one by one, several K slices
+// of each when the block has fewer than 129 tiles (thread t: tile t mod nt, slice t / nt; the
+// slices are added in order at the end).  A product with itself (same operand twice) takes
+// only the tiles on and above the diagonal; the reduction mirrors them.
+// Why: the FP64 path is bound by its 2 FP64 lanes per SM (a warp's DFMA holds them 16
+// cycles), so every idle lane and every padded output costs time.  With whole 64 x 64 tiles
+// (16 of 4 x 4 per side for every block) the 8-atom crystal (24 bands) spent 264 us on a
+// product of 1.9 MFLOP, the 24-atom layer (70 bands) 437 us; see the figures at tn_kc_f64.
+// K chunks of 32 are staged from 16-byte global loads along K (zero beyond the split's end:
+// splits end on multiples of 32 or at npw, whose tail up to ld is zero).
 // ---------------------------------------------------------------------------
 template <typename T>
 __device__ __forceinline__ void lds4(const T* p, T (&o)[4]) {
@@ -99,80 +105,135 @@ struct alignas(16) KPack {
   T e[W];
 };
 
+constexpr int TN_K = 32;                   // K values staged at a time
+constexpr int TN_LS = 4 * TN_BLOCK + 4;    // row stride of a staged operand (16-byte aligned rows)
+
+// Tile of thread tile index t in a block of ca x cb tiles; tri: the ca (ca + 1) / 2 tiles with
+// ti <= tj of a diagonal block, row by row.
+__device__ __forceinline__ void tn_tile(int t, int ca, int cb, bool tri, int* ti, int* tj) {
+  if (!tri) {
+    *ti = t / cb;
+    *tj = t - *ti * cb;
+    return;
+  }
+  int r = 0;
+  while (t >= ca - r) t -= ca - r++;
+  *ti = r;
+  *tj = r + t;
+}
+
 template <typename T>
 __global__ void __launch_bounds__(256) k_gemm_tn(KArgs ka, int akind, int arole, int bkind, int brole, double* part_base,
-                                                size_t part_stride, int kc) {
-  constexpr int W = KPack<T>::W;                 // K values per 16-byte load
-  constexpr int NLD = 32 * TN_TILE / W / 256;    // loads per thread per operand per chunk
-  constexpr int LS = TN_TILE + 4;                // row stride (16-byte aligned rows)
-  __shared__ __align__(16) T As[32][LS];
-  __shared__ __align__(16) T Bs[32][LS];
+                                                size_t part_stride, int kc_arg) {
+  constexpr int W = KPack<T>::W;                      // K values per 16-byte load
+  constexpr int V = 4 * TN_BLOCK;                     // rows staged per operand
+  constexpr int NLD = TN_K * V / W / 256;             // loads per thread per operand per chunk
+  constexpr int SB = 2 * TN_K * TN_LS * (int)sizeof(T);
+  constexpr int RB = 256 * 16 * (int)sizeof(T);
+  __shared__ __align__(16) unsigned char stage[SB > RB ? SB : RB];
+  T(*As)[TN_LS] = reinterpret_cast<T(*)[TN_LS]>(stage);
   const int p = locate(ka.start, ka.nprob, blockIdx.x);
   if (!ka.active[p]) return;
   const Prob& P = ka.probs[p];
   int local = blockIdx.x - ka.start[p];
+  const int kc = kc_arg > 0 ? kc_arg : tn_kc_f64(P.npw);
   const int na = opnd_count(P, akind), nbv = opnd_count(P, bkind);
-  const int ta = (na + TN_TILE - 1) / TN_TILE, tb = (nbv + TN_TILE - 1) / TN_TILE;
-  const int split = local / (ta * tb);
-  local -= split * ta * tb;
-  const int ti0 = (local / tb) * TN_TILE, tj0 = (local % tb) * TN_TILE;
-  if (akind == bkind && arole == brole && ti0 > tj0) return;  // mirrored by the reduction
+  const int ga = (na + 3) / 4, gb = (nbv + 3) / 4, pa = tn_block_groups(na), pb = tn_block_groups(nbv);
+  const int ba = tn_blocks(na), bb = tn_blocks(nbv);
+  const int split = local / (ba * bb);
+  local -= split * ba * bb;
+  const int bi = local / bb, bj = local - bi * bb;
+  const bool same = akind == bkind && arole == brole;
+  if (same && bi > bj) return;  // mirrored by the reduction
+  const bool tri = same && bi == bj;
+  T(*Bs)[TN_LS] = tri ? As : As + TN_K;
   const T* A = opnd<T>(P, akind, arole);
   const T* Bm = opnd<T>(P, bkind, brole);
   const int ld = P.ld;
+  const int ti0 = 4 * bi * pa, tj0 = 4 * bj * pb;
+  const int ca = min(pa, ga - bi * pa), cb = min(pb, gb - bj * pb);  // tiles of this block
+  const int nt = tri ? ca * (ca + 1) / 2 : ca * cb;
+  const int ks = 256 / nt;
   const int k0 = split * kc, k1 = min(P.npw, k0 + kc);
   const int t = threadIdx.x;
-  const int ti = t & 15, tj = t >> 4;
+  const int tile = t % nt, slice = t / nt;
+  const bool work = slice < ks;
+  int ti, tj;
+  tn_tile(tile, ca, cb, tri, &ti, &tj);
   T acc[4][4];
 #pragma unroll
   for (int a = 0; a < 4; ++a)
 #pragma unroll
     for (int b = 0; b < 4; ++b) acc[a][b] = T(0);
-  // load f = t + 256 q: vector f % 64, K offset (f / 64) W within the chunk
+  // load f = t + 256 q: vector f % V, K offset (f / V) W within the chunk
   KPack<T> ra[NLD], rb[NLD];
   auto fetch = [&](int kb) {
 #pragma unroll
     for (int q = 0; q < NLD; ++q) {
       const int f = t + 256 * q;
-      const int v = f & (TN_TILE - 1), k = kb + (f / TN_TILE) * W;
+      const int v = f & (V - 1), k = kb + (f / V) * W;
       KPack<T> za, zb;
 #pragma unroll
       for (int c = 0; c < W; ++c) za.e[c] = zb.e[c] = T(0);
       if (k < k1) {
-        if (ti0 + v < na) za = *reinterpret_cast<const KPack<T>*>(A + (size_t)(ti0 + v) * ld + k);
-        if (tj0 + v < nbv) zb = *reinterpret_cast<const KPack<T>*>(Bm + (size_t)(tj0 + v) * ld + k);
+        if (v < 4 * ca && ti0 + v < na) za = *reinterpret_cast<const KPack<T>*>(A + (size_t)(ti0 + v) * ld + k);
+        if (!tri && v < 4 * cb && tj0 + v < nbv) zb = *reinterpret_cast<const KPack<T>*>(Bm + (size_t)(tj0 + v) * ld + k);
       }
       ra[q] = za;
       rb[q] = zb;
     }
   };
   fetch(k0);
-  for (int kb = k0; kb < k1; kb += 32) {
+  int kk0 = slice;  // first K of this slice in the chunk at hand (K = slice mod ks over the split)
+  for (int kb = k0; kb < k1; kb += TN_K) {
 #pragma unroll
     for (int q = 0; q < NLD; ++q) {
       const int f = t + 256 * q;
-      const int v = f & (TN_TILE - 1), kq = (f / TN_TILE) * W;
+      const int v = f & (V - 1), kq = (f / V) * W;
 #pragma unroll
       for (int c = 0; c < W; ++c) {
         As[kq + c][v] = ra[q].e[c];
-        Bs[kq + c][v] = rb[q].e[c];
+        if (!tri) Bs[kq + c][v] = rb[q].e[c];
       }
     }
     __syncthreads();
-    if (kb + 32 < k1) fetch(kb + 32);
-#pragma unroll 8
-    for (int kk = 0; kk < 32; ++kk) {
-      T a[4], b[4];
-      lds4(&As[kk][4 * ti], a);
-      lds4(&Bs[kk][4 * tj], b);
+    if (kb + TN_K < k1) fetch(kb + TN_K);
+    const int kn = min(TN_K, k1 - kb);
+    if (work) {
+      int kk = kk0;
+#pragma unroll 4
+      for (; kk < kn; kk += ks) {
+        T a[4], b[4];
+        lds4(&As[kk][4 * ti], a);
+        lds4(&Bs[kk][4 * tj], b);
 #pragma unroll
-      for (int i = 0; i < 4; ++i)
+        for (int i = 0; i < 4; ++i)
 #pragma unroll
-        for (int j2 = 0; j2 < 4; ++j2) acc[i][j2] += a[i] * b[j2];
+          for (int j2 = 0; j2 < 4; ++j2) acc[i][j2] += a[i] * b[j2];
+      }
+      kk0 = kk - TN_K;
     }
     __syncthreads();
   }
   double* part = part_base + (size_t)p * part_stride + (size_t)split * na * nbv;
+  if (ks > 1) {  // add the slices of each tile in order
+    T* red = reinterpret_cast<T*>(stage);  // [16][256]
+    if (work)
+#pragma unroll
+      for (int e = 0; e < 16; ++e) red[e * 256 + t] = acc[e >> 2][e & 3];
+    __syncthreads();
+    for (int o = t; o < 16 * nt; o += 256) {
+      const int e = o / nt, q = o - e * nt;
+      T s = T(0);
+      for (int k = 0; k < ks; ++k) s += red[e * 256 + k * nt + q];
+      int qi, qj;
+      tn_tile(q, ca, cb, tri, &qi, &qj);
+      const int i = ti0 + 4 * qi + (e >> 2), j = tj0 + 4 * qj + (e & 3);
+      if (i < na && j < nbv) part[(size_t)i * nbv + j] = (double)s;
+    }
+    return;
+  }
+  if (!work) return;
 #pragma unroll
   for (int a = 0; a < 4; ++a)
 #pragma unroll
@@ -182,26 +243,42 @@ __global__ void __launch_bounds__(256) k_gemm_tn(KArgs ka, int akind, int arole,
     }
 }
 
-// Sum the partials in split order.  CTA = (problem, chunk of 256 outputs).  sym: A^T A
-// from k_gemm_tn, whose tiles below the diagonal were not computed (read mirrored).
+// Sum the partials of every output: CTA = (problem, chunk of 256 / L outputs), L =
+// tn_reduce_lanes(nsplit) threads per output taking every L-th partial, added in order.
+// sym: A^T A from k_gemm_tn, whose tiles below the diagonal were not computed (read mirrored).
+// L keeps the serial chain of loads at about eight: with one thread per output the 83
+// partials of the 24-atom layer's FP64 products would be one chain of 83 (11.9 -> 7 us there
+// on the mixed path's 42).
 __global__ void k_gemm_tn_reduce(KArgs ka, int akind, int bkind, int dst, const double* part_base, size_t part_stride,
-                                 int kc, int sym) {
+                                 int kc_arg, int sym) {
+  __shared__ double red[256];
   const int p = locate(ka.start, ka.nprob, blockIdx.x);
   if (!ka.active[p]) return;
   const Prob& P = ka.probs[p];
   const int na = opnd_count(P, akind), nbv = opnd_count(P, bkind);
-  const int o = (blockIdx.x - ka.start[p]) * 256 + threadIdx.x;
-  if (o >= na * nbv) return;
-  const int nsplit = (P.npw + kc - 1) / kc;
+  const int kc = kc_arg > 0 ? kc_arg : tn_kc_f64(P.npw);
+  const int nsplit = (P.npw + kc - 1) / kc, L = tn_reduce_lanes(nsplit), no = 256 / L;
+  const int lo = threadIdx.x % no, sl = threadIdx.x / no;
+  const int o = (blockIdx.x - ka.start[p]) * no + lo;
+  const bool in = o < na * nbv;
   const double* part = part_base + (size_t)p * part_stride;
-  int src = o;
-  if (sym) {
-    const int i = o / nbv, j = o - i * nbv;
-    if (i / TN_TILE > j / TN_TILE) src = j * nbv + i;
-  }
   double s = 0.0;
-  for (int k = 0; k < nsplit; ++k) s += part[(size_t)k * na * nbv + src];
-  dense_ptr(P, dst)[o] = s;
+  if (in) {
+    int src = o;
+    if (sym) {
+      const int i = o / nbv, j = o - i * nbv;
+      if (i / 4 > j / 4) src = j * nbv + i;
+    }
+#pragma unroll 4
+    for (int k = sl; k < nsplit; k += L) s += part[(size_t)k * na * nbv + src];
+  }
+  if (L > 1) {
+    red[threadIdx.x] = s;
+    __syncthreads();
+    if (sl == 0)
+      for (int k = 1; k < L; ++k) s += red[k * no + lo];
+  }
+  if (in && sl == 0) dense_ptr(P, dst)[o] = s;
 }
 
 // ---------------------------------------------------------------------------
@@ -303,6 +380,106 @@ __global__ void __launch_bounds__(256) k_gemm_nn(KArgs ka, int akind, RolePairs 
       }
     }
   }
+}
+
+// ---------------------------------------------------------------------------
+// The same product on the FP64 path.  Bound by the FP64 lanes (2 per SM), so the outputs are
+// dealt to the threads in 4 x 4 tiles without padding the bands to 64: a CTA takes
+// nn_rows_f64(nb, npw) rows and a block of at most 16 column groups of 4 (blocks of about
+// equal size), one tile per thread, and several slices of the inner index per tile when that
+// leaves threads over (added in order at the end).  Before, with 64 x 64 outputs per pass and
+// 256 rows per CTA: 95 us for the 8-atom crystal (24 bands, 10 CTAs), 460 us for the 24-atom
+// layer (70 bands padded to 128); the figures after are at nn_rows_f64.
+// ---------------------------------------------------------------------------
+constexpr int NN64_K = 16;  // inner values staged at a time
+__global__ void __launch_bounds__(256) k_gemm_nn_f64(KArgs ka, int akind, RolePairs rp, int msel, double alpha,
+                                                    double beta) {
+  __shared__ __align__(16) double stage[NN64_K * (NN64_MAXROWS + 4 * TN_BLOCK)];
+  const int arole = rp.a[blockIdx.y], yrole = rp.y[blockIdx.y];
+  const int p = locate(ka.start, ka.nprob, blockIdx.x);
+  if (!ka.active[p]) return;
+  const Prob& P = ka.probs[p];
+  const int nb = P.nb, ld = P.ld, npw = P.npw, inner = opnd_count(P, akind);
+  const int bb = tn_blocks(nb), pb = tn_block_groups(nb), rows = nn_rows_f64(nb, npw);
+  const int local = blockIdx.x - ka.start[p];
+  const int rt = local / bb, bj = local - rt * bb;
+  const int r0 = rt * rows, c0 = 4 * bj * pb;
+  const int cg = min(pb, (nb + 3) / 4 - bj * pb), rg = rows / 4;
+  const int nt = rg * cg, ks = 256 / nt;
+  const double* A = opnd<double>(P, akind, arole);
+  const double* M = dense_ptr(P, msel);
+  double* Y = wbuf<double>(P, yrole);
+  double* As = stage;                  // [NN64_K][rows]
+  double* Ms = stage + NN64_K * rows;  // [NN64_K][4 pb]
+  const int t = threadIdx.x, tile = t % nt, slice = t / nt;
+  const bool work = slice < ks;
+  const int tr = tile % rg, tc = tile / rg;
+  double acc[4][4];
+#pragma unroll
+  for (int i = 0; i < 4; ++i)
+#pragma unroll
+    for (int j = 0; j < 4; ++j) acc[i][j] = 0.0;
+  int kk0 = slice;
+  for (int kb = 0; kb < inner; kb += NN64_K) {
+    const int kn = min(NN64_K, inner - kb);
+    const int np = rows / 2;  // 16-byte packs of a staged row (ld is even; rows up to npw + 1 are zero)
+    for (int e = t; e < kn * np; e += 256) {
+      const int kk = e / np, r = 2 * (e - kk * np);
+      double2 v = make_double2(0.0, 0.0);
+      if (r0 + r < ld) v = *reinterpret_cast<const double2*>(A + (size_t)(kb + kk) * ld + r0 + r);
+      *reinterpret_cast<double2*>(As + kk * rows + r) = v;
+    }
+    for (int e = t; e < kn * 4 * cg; e += 256) {
+      const int kk = e / (4 * cg), c = e - kk * 4 * cg, k = kb + kk;
+      double mv = 0.0;
+      if (c0 + c < nb) {
+        mv = M[(size_t)k * nb + c0 + c];
+        if (msel == DD_PROJ_D) mv *= P.pj_d[k];
+      }
+      Ms[kk * 4 * pb + c] = mv;
+    }
+    __syncthreads();
+    if (work) {
+      int kk = kk0;
+      for (; kk < kn; kk += ks) {
+        double a[4], m[4];
+        lds4(As + kk * rows + 4 * tr, a);
+        lds4(Ms + kk * 4 * pb + 4 * tc, m);
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+#pragma unroll
+          for (int j = 0; j < 4; ++j) acc[i][j] += a[i] * m[j];
+      }
+      kk0 = kk - NN64_K;
+    }
+    __syncthreads();
+  }
+  auto store = [&](int r, int c, double v) {
+    if (r >= npw || c >= nb) return;
+    double* y = Y + (size_t)c * ld + r;
+    v *= alpha;
+    if (beta != 0.0) v += beta * (*y);
+    *y = v;
+  };
+  if (ks > 1) {
+    double* red = stage;  // [16][256]
+    if (work)
+#pragma unroll
+      for (int e = 0; e < 16; ++e) red[e * 256 + t] = acc[e & 3][e >> 2];
+    __syncthreads();
+    for (int o = t; o < 16 * nt; o += 256) {
+      const int e = o / nt, q = o - e * nt;
+      double s = 0.0;
+      for (int k = 0; k < ks; ++k) s += red[e * 256 + k * nt + q];
+      store(r0 + 4 * (q % rg) + (e & 3), c0 + 4 * (q / rg) + (e >> 2), s);
+    }
+    return;
+  }
+  if (!work) return;
+#pragma unroll
+  for (int j = 0; j < 4; ++j)
+#pragma unroll
+    for (int i = 0; i < 4; ++i) store(r0 + 4 * tr + i, c0 + 4 * tc + j, acc[i][j]);
 }
 
 // ---------------------------------------------------------------------------
@@ -1703,8 +1880,9 @@ void launch_gemm_tn_reduce(const Launch& L, int akind, int bkind, int dst, const
 template <typename T>
 void launch_gemm_nn(const Launch& L, int akind, const RolePairs& rp, int msel, double alpha, double beta) {
   if (!L.map.total || rp.n < 1) return;
-  k_gemm_nn<T><<<dim3(L.map.total, rp.n), 256, (size_t)NN_KP * 64 * sizeof(T), L.stream>>>(L.ka, akind, rp, msel, alpha,
-                                                                               beta);
+  const dim3 grid(L.map.total, rp.n);
+  if constexpr (sizeof(T) == 8) k_gemm_nn_f64<<<grid, 256, 0, L.stream>>>(L.ka, akind, rp, msel, alpha, beta);
+  else k_gemm_nn<T><<<grid, 256, (size_t)NN_KP * 64 * sizeof(T), L.stream>>>(L.ka, akind, rp, msel, alpha, beta);
 }
 template <typename T>
 void launch_band_kinetic(const Launch& L, int xrole) {
@@ -1788,9 +1966,8 @@ void linalg_set_smem_limits(size_t bytes) {
   // (k_rr_f32 keeps its matrices in shared memory up to 216 KB; its static arrays take the
   // rest of the 227 KB)
   cudaFuncSetAttribute(k_rr_f32, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)std::min(bytes, (size_t)216 * 1024));
-  // the NN kernel also has 8-16 KB of static shared memory: request only what it uses
+  // the NN kernel also has 8 KB of static shared memory: request only what it uses
   cudaFuncSetAttribute(k_gemm_nn<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, NN_KP * 64 * (int)sizeof(float));
-  cudaFuncSetAttribute(k_gemm_nn<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, NN_KP * 64 * (int)sizeof(double));
 }
 
 #define INST(T)                                                                                  \

@@ -19,11 +19,33 @@ constexpr int PAIR_REG_MAXN = 128;      // longest line a lane pair transforms
 constexpr int ZREG_CP = 64;             // column pairs per register z-column CTA
 constexpr int ZREG_THREADS = 2 * ZREG_CP;
 // GEMM geometry
-constexpr int TN_TILE = 64;
+constexpr int TN_BLOCK = 16;           // 4 x 4 output tiles per side of a CUDA-core GEMM block, at most
 constexpr int TN_KC = 256;             // K chunk of one split-K partial (CUDA-core GEMM)
 constexpr int TC_KC = 512;             // K chunk of one split-K partial (tensor-core GEMM)
 constexpr int NN_RT = 4;              // row tiles of 64 per NN CTA
 constexpr int NN_KP = 128;             // rows of the small matrix staged per pass
+constexpr int NN64_MAXROWS = 256;      // rows of an FP64 NN CTA, at most
+// n vectors in groups of 4, dealt to blocks of at most TN_BLOCK groups of about equal size
+__host__ __device__ inline int tn_blocks(int n) { return ((n + 3) / 4 + TN_BLOCK - 1) / TN_BLOCK; }
+__host__ __device__ inline int tn_block_groups(int n) { return ((n + 3) / 4 + tn_blocks(n) - 1) / tn_blocks(n); }
+// K chunk of the FP64 split-K products.  A function of the member's own size, so that its sums
+// do not depend on the batch it is in.  One structure alone has to fill 152 SMs: chunks of 32
+// up to 4096 plane waves (the 8-atom crystal: 51 CTAs), 64 up to 8192, 128 beyond (the 24-atom
+// layer: 83 splits x 3 or 4 blocks).  With the 4 x 4 tiles of k_gemm_tn, mean per product: the
+// crystal 264 -> 10.7 us, the layer 437 -> 106 us, six uneven members 555 -> 204 us (chunks of
+// 256 and whole 64 x 64 tiles before).
+__host__ __device__ inline int tn_kc_f64(int npw) { return npw < 4096 ? 32 : npw < 8192 ? 64 : 128; }
+// Threads that share one output of the split-K reduction (a power of two up to 8, about eight
+// partials each)
+__host__ __device__ inline int tn_reduce_lanes(int nsplit) { return nsplit < 16 ? 1 : nsplit < 32 ? 2 : nsplit < 64 ? 4 : 8; }
+// Rows of an FP64 NN CTA: as many groups of 4 as give each of 256 threads a 4 x 4 tile, at most
+// 8 groups while a structure has few plane waves (so that it fills the GPU).  Mean per launch
+// (1 to 4 products): the 8-atom crystal 95 -> 15 us, the 24-atom layer 460 -> 189 us (1.1
+// TFLOP/s in the four-product launches, the FP64 lanes' rate), six uneven members 719 -> 436 us.
+__host__ __device__ inline int nn_rows_f64(int nb, int npw) {
+  const int cg = tn_block_groups(nb), cap = npw < 4096 ? 8 : NN64_MAXROWS / 4;
+  return 4 * (256 / cg < cap ? 256 / cg : cap);
+}
 constexpr int BAND_THREADS = 256;
 constexpr int GRID_CHUNK = 4096;       // grid points per reduction CTA
 constexpr int RR_THREADS = 1024;
@@ -142,6 +164,7 @@ void launch_plane_density_reg(const Launch& L, int cls, size_t smem, const doubl
 template <typename T>
 void launch_gemm_tn(const Launch& L, int akind, int arole, int bkind, int brole, double* part, size_t stride,
                     int kc = TN_KC);
+// (kc 0 here and below: tn_kc_f64 of each member)
 // sym: the partials are k_gemm_tn's A^T A (same operand twice; tiles below the diagonal mirrored)
 void launch_gemm_tn_reduce(const Launch& L, int akind, int bkind, int dst, const double* part, size_t stride,
                            int kc = TN_KC, bool sym = false);
