@@ -127,11 +127,10 @@ typedef struct {
                              requested bands get headroom; occupations, eigenvalues, energies and
                              the eig_tol test cover the requested bands only (-1, default:
                              4 + nbands / 32; 0 = none) */
-  int rr_cluster;         /* subspace diagonalisation kernel: -1 (default) one CTA per member while
-                             its matrices fit in shared memory, else a thread-block cluster of 8
-                             CTAs per member; 0 = always one CTA (over a global scratch when the
-                             matrices do not fit); 1 = always the cluster.  Taken from the first
-                             member of a batch. */
+  int rr_cluster;         /* subspace diagonalisation kernel: -1 (default) or 0 one CTA per member up
+                             to 184 bands (FP64: 128), beyond a thread-block cluster of 8 CTAs per
+                             member; 1 = always the cluster.  Taken from the first member of a
+                             batch. */
   int eigensolver;        /* 0 (default): Algorithm 1's all-band CG steps (Sec. II D): per band a
                              preconditioned, conjugated, projected search direction, a line
                              minimisation, then a Rayleigh-Ritz over the n_b bands.  1: block
@@ -262,10 +261,10 @@ SGO_API sgo_status sgo_get_terms(sgo_ctx* ctx, double terms[8]);
 SGO_API sgo_status sgo_get_info(sgo_ctx* ctx, int info[10]);
 
 /* Diagnostics of the last SCF: [0] iterations, [1] Jacobi sweeps summed over its
- * subspace diagonalisations, [2] final density residual, [3] final |F_k - F_{k-1}|,
- * [4] CG steps taken after the SCF stopping rule held (eig_tol), [5] the largest residual
+ * subspace diagonalisations on the cluster (rr_cluster; the one-CTA kernel makes none),
+ * [2] final density residual, [3] final |F_k - F_{k-1}|, [4] CG steps taken after the SCF stopping rule held (eig_tol), [5] the largest residual
  * |H psi - eps psi| over the bands with occupation above 1e-6 at the end, [6] subspace
- * diagonalisations that stopped at their Jacobi sweep cap, [7] SCF iterations of the
+ * diagonalisations that stopped at their iteration cap, [7] SCF iterations of the
  * last SCF loop that started from a state set by sgo_set_state (0 otherwise). */
 SGO_API sgo_status sgo_get_stats(sgo_ctx* ctx, double stats[8]);
 

@@ -978,31 +978,22 @@ Engine::Engine(const std::vector<sgo_ctx*>& ctxs, cudaStream_t stream) : ctx_(ct
     }
     if (!set_slots(slot, foff)) return;
   }
-  // mixed path: the FP32 eigensolve (its five matrices in shared memory up to nb = 105,
-  // else in a per-member global scratch; the Jacobi pair tables allow nb <= 512)
   const sgo_opts& o0 = ctxs[0]->opts;
   wait_ns_ = o0.watchdog_ms > 0.0 ? (long long)(o0.watchdog_ms * 1e6) : 2000000000LL;
-  // subspace diagonalisation: one CTA per member with its matrices in shared memory (FP32
-  // deviation form up to nb = 105 on the mixed path, FP64 up to nb = 91), else one
-  // thread-block cluster per member over a global scratch (k_rr_cluster)
+  // subspace diagonalisation: one CTA per member up to rr_td_max bands (192 on the mixed path,
+  // 128 in FP64), beyond (or when asked for) one thread-block cluster per member (k_rr_cluster)
   // (the block Davidson steps diagonalise the 2 n_b block [X, W])
   davidson_ = o0.eigensolver == 1;
   cg_adapt_ = o0.cg_adapt;
   gga_ = o0.xc == 1;
   rr_n_ = (davidson_ ? 2 : 1) * max_nb_;
   rr_f32_ = precision_ == 1 && !o0.rr_fp64;
-  rr_smem_bytes_ = (size_t)3 * rr_n_ * rr_n_ * sizeof(double);
-  rr_smem_ = rr_f32_ ? (size_t)20 * rr_n_ * (rr_n_ | 1) <= 216 * 1024 : rr_smem_bytes_ <= 200 * 1024;
-  // (the one-CTA kernels' pair tables hold 256 pairs: beyond 512 bands the cluster is used)
-  rr_cluster_ = o0.rr_cluster > 0 || (o0.rr_cluster < 0 && !rr_smem_) || rr_n_ > 512;
-  if (rr_cluster_) {
-    rrc_stride_ = (rr_cluster_scratch_bytes(rr_n_, rr_f32_ ? sizeof(float) : sizeof(double)) + 255) / 256 * 256;
-    if (!cuda_ok(dev_malloc(&d_rrc_, rrc_stride_ * n_), "dev_malloc(rr cluster scratch)")) return;
-    allocs_.push_back(d_rrc_);
-  } else if (!rr_smem_) {  // one CTA over a global scratch
-    rr1_stride_ = rr_f32_ ? (size_t)5 * rr_n_ * (rr_n_ | 1) * sizeof(float) : (size_t)3 * rr_n_ * rr_n_ * sizeof(double);
-    if (!cuda_ok(dev_malloc(&d_rr1_, rr1_stride_ * n_), "dev_malloc(rr scratch)")) return;
-    allocs_.push_back(d_rr1_);
+  const size_t ts = rr_f32_ ? sizeof(float) : sizeof(double);
+  rr_cluster_ = o0.rr_cluster > 0 || rr_n_ > rr_td_max(ts);
+  rr_stride_ = ((rr_cluster_ ? rr_cluster_scratch_bytes(rr_n_, ts) : rr_td_scratch_bytes(rr_n_, ts)) + 255) / 256 * 256;
+  if (rr_stride_) {
+    if (!cuda_ok(dev_malloc(&d_rr_, rr_stride_ * n_), "dev_malloc(rr scratch)")) return;
+    allocs_.push_back(d_rr_);
   }
   // (a refused shared-memory limit would otherwise surface only as a failed launch later)
   if (!cuda_ok(cudaGetLastError(), "engine set-up")) return;
@@ -1281,15 +1272,13 @@ void Engine::rr_solve(int blk) {
   const int cap = blk == 2 ? 30 : rr_cap_;
   if (rr_cluster_) {
     const Launch l = L(m_prob_);
-    const bool launched = rr_f32_ ? launch_rr_cluster<float>(l, rr_n_, d_rrc_, rrc_stride_, cap, blk)
-                                  : launch_rr_cluster<double>(l, rr_n_, d_rrc_, rrc_stride_, 30, blk);
+    const bool launched = rr_f32_ ? launch_rr_cluster<float>(l, rr_n_, d_rr_, rr_stride_, cap, blk)
+                                  : launch_rr_cluster<double>(l, rr_n_, d_rr_, rr_stride_, 30, blk);
     if (!launched) set_error("cluster Rayleigh-Ritz launch refused");
-  } else if (rr_f32_) {  // 5 FP32 n x (n|1) matrices in shared memory or a global scratch
-    launch_rr_f32(L(m_prob_), (size_t)20 * rr_n_ * (rr_n_ | 1), reinterpret_cast<float*>(d_rr1_),
-                  rr1_stride_ / sizeof(float), cap, blk);
+  } else if (rr_f32_) {
+    launch_rr_td<float>(L(m_prob_), blk * max_nb_, d_rr_, rr_stride_, blk);
   } else {
-    launch_rr(L(m_prob_), rr_smem_ ? 1 : 0, rr_smem_bytes_, reinterpret_cast<double*>(d_rr1_),
-              rr1_stride_ / sizeof(double), 30, blk);
+    launch_rr_td<double>(L(m_prob_), blk * max_nb_, d_rr_, rr_stride_, blk);
   }
   tend(TK_RR);
   work_mult_ = 1;

@@ -204,7 +204,6 @@ class Engine {
   size_t part_stride_ = 0;
   double* d_gpart_ = nullptr;
   int maxchunk_ = 1;
-  bool rr_smem_ = true;
   bool rr_f32_ = false;
   bool rr_cluster_ = false;          // subspace too large for one CTA: cluster eigensolve
   bool davidson_ = false;            // block Davidson steps (2 n_b Rayleigh-Ritz) instead of CG
@@ -212,11 +211,8 @@ class Engine {
   double cg_adapt_ = 0.0;            // density residual above which the last CG step is left out
   int* d_saved_ = nullptr;           // active mask kept across that step
   int rr_n_ = 0;                     // largest subspace of one Rayleigh-Ritz call
-  unsigned char* d_rrc_ = nullptr;   // its per-member global scratch
-  size_t rrc_stride_ = 0;
-  unsigned char* d_rr1_ = nullptr;   // one-CTA eigensolve beyond shared memory: global scratch
-  size_t rr1_stride_ = 0;            // bytes per member
-  size_t rr_smem_bytes_ = 0;
+  unsigned char* d_rr_ = nullptr;    // its per-member global scratch (none where it needs none)
+  size_t rr_stride_ = 0;             // bytes per member
   double* d_flags_ = nullptr;   // [n][4] gathered per iteration
   // pinned read-back area (device-to-host copies into it do not block the host):
   // hp_ = flags [n][4], then per member scal, eps, occ, forces at hp_off_[p];

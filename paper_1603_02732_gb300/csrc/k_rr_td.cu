@@ -1,0 +1,1152 @@
+// Rayleigh-Ritz of one CTA per problem (orthonormalisation + subspace diagonalisation of
+// Algorithm 1): S = L L^T, C = L^-1 Hs L^-T, C = V diag(eps) V^T, Tm = L^-T V, so that X Tm is
+// orthonormal and diagonalises H in the subspace.  T = float on the mixed path, double on the
+// plain one.
+//
+//  1. Cholesky in deviation form: S = I + E, L = I + D, d_k = x / (1 + sqrt(1 + x)) with
+//     x = E_kk, D_ik = E_ik / (1 + d_k).  Every stored quantity has the size of E, so FP32 keeps
+//     its relative accuracy (the entries of S carry the product's FP32 rounding anyway).
+//  2. W = L^-1 Hs and C = W L^-T by forward substitution down columns.
+//  3. Householder tridiagonalisation of C (Golub & Van Loan, section 8.3.1).
+//  4. Divide and conquer on the tridiagonal matrix (Cuppen, Numer. Math. 36, 177 (1981)): small
+//     leaves by QL steps, merged pairwise, a merge being the rank-one problem diag(delta) + rho z z^T.  Roots of its secular equation by the
+//     two-pole rational interpolation of Bunch, Nielsen & Sorensen (Numer. Math. 31, 31 (1978)),
+//     each as an offset from its nearest pole; z is then recomputed from the roots (Gu &
+//     Eisenstat, SIAM J. Matrix Anal. 15, 1266 (1994)), which makes the vectors orthogonal to
+//     rounding however close the roots lie.  Nothing is deflated: poles closer than one unit of
+//     rounding of the matrix are moved that far apart and weights below rounding are raised to
+//     it, both of the size of the rounding errors already there; a negligible rho leaves the two
+//     halves as they are.
+//  5. V = Householder reflectors applied to the eigenvectors; FP32: one correction of V by its
+//     residuals C v_j - lam_j v_j (first-order perturbation theory), one Newton-Schulz step of its
+//     orthonormality; Tm = L^-T V by back substitution.
+//
+// What bounds it, and why this form: one CTA (one SM) works on a chain of dependent steps, so the
+// time is barriers, latencies and, with many warps, the issue of the steps' overhead; on the FP64
+// path it is the two FP64 lanes of the SM (a warp's DFMA holds them 16 cycles).  The cyclic Jacobi
+// eigensolve before it took about 200 rounds of two block barriers and 6 n^2 operations each.
+// Here the matrices stay in the registers of MW matrix warps, row i in warp i / RPW, column j in
+// lane j mod 32 (few warps with 8 to 16 rows each: the overhead of a step is paid per warp); the
+// Cholesky needs one barrier per RPW columns, the tridiagonalisation two per column, the
+// substitutions and the back transformation none (a warp owns whole columns).
+// Measured, mean per launch over an evaluation, Jacobi kernels before -> now: FP32 70 bands 299 ->
+// 258 us, 91 bands 553 -> 335 us, 86 bands in 64 members 484 -> 294 us, 169 bands (an 8-CTA cluster
+// before) 3565 -> 1403 us, 10 bands 31 -> 39 us; FP64 24 bands 317 -> 289 us, 70 bands 2500 -> 1883
+// us, up to 80 bands in six members 3550 -> 2115 us.
+#include "kernels.h"
+
+namespace sgo {
+
+namespace {
+
+// Near-dependent directions of the block [X, W] (blk = 2): a W vector whose component orthogonal
+// to the basis vectors before it has squared norm at most TD_DROP (its own norm is 1) is left out
+// of the subspace instead of failing the Cholesky (the preconditioned residuals of a random start
+// are nearly collinear): its column of L and its row of L^-1 are zero, and its diagonal entry of
+// C is set above the spectrum, so that it ranks after every kept Ritz value.
+constexpr double TD_DROP = 1e-3;
+// Lanes per root of a merge of m poles out of n.  A root's own arithmetic is done by all its lanes,
+// so more lanes only pay while they shorten a chain of terms that is long against it, and on the
+// FP64 path only until about four warps keep the FP64 lanes busy.  (Not a function of the block
+// size: the sums must not depend on the batch a member is in.)
+template <typename T>
+__device__ __forceinline__ int td_lanes(int m, int n) {
+  if (sizeof(T) == 8 && n > 32) return m > 32 ? 4 : m > 8 ? 2 : 1;
+  return m > 16 && n <= 64 && sizeof(T) == 4 ? 8 : m > 8 ? 4 : m > 4 ? 2 : 1;  // (64: one pass of 512 threads)
+}
+
+template <typename T>
+struct TdNum;
+template <>
+struct TdNum<float> {
+  static constexpr float eps = 1.1920929e-7f, ztiny = 1e-7f, floor = 1e-30f, step = 3e-5f;
+};
+template <>
+struct TdNum<double> {
+  static constexpr double eps = 2.220446049250313e-16, ztiny = 1e-16, floor = 1e-280, step = 1e-9;
+};
+// (step: a relative step below which the quadratically convergent root iteration is done, its
+// square being below rounding)
+constexpr int TD_ITERS = 60;  // cap of the root iteration (typically 4)
+
+// 1 / x by the approximate reciprocal and Newton steps r += r (1 - x r): one in FP32, two in FP64
+// (4 FP64 operations)
+__device__ __forceinline__ float td_rcp(float x) {
+  const float r = __fdividef(1.f, x);
+  return fmaf(r, fmaf(-x, r, 1.f), r);
+}
+__device__ __forceinline__ double td_rcp(double x) {
+  double r;
+  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(x));
+  r = fma(r, fma(-x, r, 1.0), r);
+  return fma(r, fma(-x, r, 1.0), r);
+}
+__device__ __forceinline__ float td_rsqrt(float x) {
+  const float r = rsqrtf(x);
+  return fmaf(0.5f * r, fmaf(-x * r, r, 1.f), r);
+}
+__device__ __forceinline__ double td_rsqrt(double x) {  // two Newton steps on the approximate one
+  double r;
+  asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(x));
+  r = fma(0.5 * r, fma(-x * r, r, 1.0), r);
+  return fma(0.5 * r, fma(-x * r, r, 1.0), r);
+}
+
+template <typename T>
+__device__ __forceinline__ T wsum(T v) {
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+  return v;
+}
+
+// Sums over W consecutive lanes of R values per lane.  Pairs of values are folded into one
+// register per exchange (the lanes on either side of a bit keep one value each), so that R sums
+// cost about R + log2 W shuffles and adds instead of R log2 W: on return a lane holds the sum of
+// value fold_index(lane).
+template <int R>
+__host__ __device__ constexpr int fold_bits() { return R > 8 ? 4 : R > 4 ? 3 : R > 2 ? 2 : R > 1 ? 1 : 0; }
+template <typename T, int R, int W>
+__device__ __forceinline__ T fold_sums(const T (&in)[R], int lane) {
+  constexpr int B = fold_bits<R>(), N = 1 << B;
+  T v[N];
+#pragma unroll
+  for (int i = 0; i < N; ++i) v[i] = i < R ? in[i < R ? i : 0] : T(0);
+  int o = W / 2;
+#pragma unroll
+  for (int b = 0; b < B; ++b, o >>= 1) {
+    const bool up = (lane & o) != 0;
+    const int h = N >> (b + 1);
+#pragma unroll
+    for (int i = 0; i < N; ++i)
+      if (i < h) {
+        const T keep = up ? v[i + h] : v[i], give = up ? v[i] : v[i + h];
+        v[i] = keep + __shfl_xor_sync(0xffffffffu, give, o);
+      }
+  }
+#pragma unroll
+  for (; o > 0; o >>= 1) v[0] += __shfl_xor_sync(0xffffffffu, v[0], o);
+  return v[0];
+}
+constexpr int log2i(int w) { return w <= 1 ? 0 : 1 + log2i(w / 2); }
+// shift from a lane of the W to the value it holds (the first lane that holds value a is a << it)
+template <int R, int W>
+__host__ __device__ constexpr int fold_shift() { return log2i(W) - fold_bits<R>(); }
+
+// sum over the g lanes of a root
+template <typename T>
+__device__ __forceinline__ T gsum(T v, int g) {
+  for (int o = g >> 1; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+  return v;
+}
+
+// Root in the pole interval of the two-pole model c + s / (p - mu) + S / (q - mu) = 0; right:
+// offsets from the right pole (p = -w, q = 0), else from the left one (p = 0, q = w).  S = 0: no
+// right pole (the last root; the quadratic would lose the root to its other one at w).
+template <typename T>
+__device__ __forceinline__ T two_pole_root(T c, T s, T S, T w, bool right) {
+  if (S == T(0)) return s * td_rcp(c);
+  const T b = right ? s + S - c * w : c * w + s + S;
+  const T d = right ? -S * w : s * w;
+  const T disc = b * b - T(4) * c * d;
+  const T r = sqrt(disc > T(0) ? disc : T(0));
+  const T num = b >= T(0) ? T(2) * d : b - r, den = b >= T(0) ? b + r : T(2) * c;
+  return num * td_rcp(den);
+}
+
+// poles relative to the nearest one, in F
+template <typename F, typename T>
+struct Poles {
+  const T* d;
+  T b;
+  __device__ __forceinline__ F operator()(int j) const { return (F)(d[j] - b); }
+};
+
+// Iteration for root ii of poles lo .. hi - 1 (weights zw), starting at x in the bracket (a, b)
+// of offsets from the nearest pole; lane sub of the root's g lanes takes every g-th term.  Returns
+// whether it converged; all lanes of the warp take part until the last root is done.
+template <typename F, typename PO>
+__device__ __forceinline__ bool secular(const PO& pole, const F* zw, int lo, int hi, int ii, int sub, int g, F w,
+                                        bool right, bool last, F a, F b, bool done, int iters, F* xio) {
+  const F pl = right ? -w : F(0), ql = right ? F(0) : w;  // the two poles of the interval
+  F x = *xio;
+  for (int it = 0; it < iters; ++it) {
+    if (!__any_sync(0xffffffffu, !done)) break;
+    F ps = F(0), dp = F(0), ph = F(0), dq = F(0);  // the sums left and right of the root, their slopes
+    if (!done)
+      for (int j = lo + sub; j < hi; j += g) {
+        const F r = td_rcp(pole(j) - x);
+        const F t = zw[j] * r, u = t * r;
+        if (j <= ii) {
+          ps += t;
+          dp += u;
+        } else {
+          ph += t;
+          dq += u;
+        }
+      }
+    for (int o = g >> 1; o > 0; o >>= 1) {
+      ps += __shfl_xor_sync(0xffffffffu, ps, o);
+      dp += __shfl_xor_sync(0xffffffffu, dp, o);
+      ph += __shfl_xor_sync(0xffffffffu, ph, o);
+      dq += __shfl_xor_sync(0xffffffffu, dq, o);
+    }
+    if (!done) {
+      const F f = F(1) + ps + ph;
+      if (f < F(0)) a = x;
+      else b = x;
+      if (fabs(f) <= F(2) * TdNum<F>::eps * (F(1) + fabs(ps) + fabs(ph))) {
+        done = true;
+      } else {
+        const F dl = pl - x, dr = ql - x;
+        const F c = f - dl * dp - (last ? F(0) : dr * dq);
+        F y = two_pole_root(c, dl * dl * dp, last ? F(0) : dr * dr * dq, w, right);
+        const bool in = y > a && y < b;
+        if (!in) y = a == F(0) ? b * F(0.01) : b == F(0) ? a * F(0.01) : F(0.5) * (a + b);
+        if ((in && fabs(y - x) <= TdNum<F>::step * fabs(x)) || !(b - a > TdNum<F>::eps * fmax(fabs(a), fabs(b)))) done = true;
+        x = y;
+      }
+    }
+  }
+  *xio = x;
+  return done;
+}
+
+// Largest block the divide and conquer starts from.  FP32: QL steps on 8 rows take 10 us where
+// three merge levels of the smallest blocks take 20; FP64: on 2 rows (one rotation), since the
+// steps are chains of FP64 operations (8 rows 100 us, the levels 40).
+template <typename T>
+__host__ __device__ constexpr int td_leaf_rows() { return sizeof(T) == 4 ? 8 : 2; }
+
+// Eigenvectors of a symmetric tridiagonal leaf of m0 <= M rows by implicit QL steps with
+// Wilkinson's shift (EISPACK's tql2: Bowdler, Martin, Reinsch & Wilkinson, Numer. Math. 11, 293
+// (1968)): every lane carries the whole of d and e and one row z of the vectors.
+template <typename T, int M>
+__device__ __forceinline__ void td_leaf(T (&d)[M], T (&e)[M], T (&z)[M], int m0, T norm) {
+  const T tiny = T(1e-3) * TdNum<T>::eps * norm;
+  for (int l = 0; l + 1 < m0; ++l) {
+    for (int it = 0; it < 30; ++it) {
+      int m = m0 - 1;  // the first negligible e at or after l ends the active block
+      T dl = T(0), dl1 = T(0), el = T(0), dm = T(0);
+#pragma unroll
+      for (int i = M - 2; i >= 0; --i) {
+        const T x = fabs(e[i]);
+        if (i >= l && i < m0 - 1 && !(x > TdNum<T>::eps * (fabs(d[i]) + fabs(d[i + 1])) && x > tiny)) m = i;
+        if (i == l) {
+          dl = d[i];
+          dl1 = d[i + 1];
+          el = e[i];
+        }
+      }
+      if (m == l) break;
+#pragma unroll
+      for (int i = 0; i < M; ++i)
+        if (i == m) dm = d[i];
+      T g = (dl1 - dl) * td_rcp(T(2) * el);
+      g = dm - dl + el * td_rcp(g + copysign(sqrt(g * g + T(1)), g));
+      T s = T(1), c = T(1), q = T(0);
+      bool cut = false;  // an exact zero ended the sweep early
+#pragma unroll
+      for (int i = M - 2; i >= 0; --i)
+        if (i < m && i >= l && !cut) {
+          const T f = s * e[i], b = c * e[i], h = f * f + g * g;
+          const T ir = td_rsqrt(h);
+          if (h > TdNum<T>::floor) {
+            e[i + 1] = h * ir;
+            s = f * ir;
+            c = g * ir;
+            g = d[i + 1] - q;
+            const T r = (d[i] - g) * s + T(2) * c * b;
+            q = s * r;
+            d[i + 1] = g + q;
+            g = c * r - b;
+            const T zi = z[i + 1];
+            z[i + 1] = s * z[i] + c * zi;
+            z[i] = c * z[i] - s * zi;
+          } else {
+            e[i + 1] = T(0);
+            d[i + 1] -= q;
+            cut = true;
+          }
+        }
+#pragma unroll
+      for (int i = 0; i < M; ++i) {
+        if (i == l && !cut) {
+          d[i] -= q;
+          e[i] = g;
+        }
+        if (i == m) e[i] = T(0);
+      }
+    }
+  }
+}
+
+__device__ __forceinline__ void bar_matrix(int threads) {
+  asm volatile("bar.sync 1, %0;" ::"r"(threads) : "memory");
+}
+
+// R consecutive shared values (aligned to R values or 16 bytes) as vector loads
+template <typename T, int R>
+__device__ __forceinline__ void ldv(const T* p, T (&o)[R]) {
+  constexpr int W = sizeof(T) == 4 && R % 4 == 0 ? 4 : 2;
+  static_assert(R % W == 0, "whole vectors");
+#pragma unroll
+  for (int i = 0; i < R / W; ++i) {
+    if constexpr (W == 4) {
+      const float4 v = reinterpret_cast<const float4*>(p)[i];
+      o[4 * i] = v.x; o[4 * i + 1] = v.y; o[4 * i + 2] = v.z; o[4 * i + 3] = v.w;
+    } else if constexpr (sizeof(T) == 4) {
+      const float2 v = reinterpret_cast<const float2*>(p)[i];
+      o[2 * i] = v.x; o[2 * i + 1] = v.y;
+    } else {
+      const double2 v = reinterpret_cast<const double2*>(p)[i];
+      o[2 * i] = v.x; o[2 * i + 1] = v.y;
+    }
+  }
+}
+
+__host__ __device__ inline int td_zs(int n) { return n > 16 ? ((n + 1) / 2) | 1 : 9; }  // row stride of the vectors
+__host__ __device__ inline int td_us(int n) { return (n + 3) & ~3; }        // row stride of the merge matrix
+constexpr int TD_PAD = 32;  // vectors are read in whole groups of rows past n
+__host__ __device__ inline int td_vn(int n) { return ((n + 3) & ~3) + TD_PAD; }
+__host__ __device__ inline size_t td_vec_bytes(int n, size_t ts) {
+  return ((size_t)(13 * td_vn(n) + 32) * ts + (size_t)(3 * td_vn(n) + 16) * 4 + 15) / 16 * 16;
+}
+
+}  // namespace
+
+// all: L, the reflectors, U and Z in shared memory; else L, the reflectors and the transposes go
+// through the member's global scratch (3 n^2 elements) and share U's place in turn.  FP32 keeps C
+// and the factors of the correction's products in the scratch too (rr_td_scratch_bytes).
+template <typename T, int NR, int MW, int NW>
+__global__ void __launch_bounds__(32 * NW, 1)
+    k_rr_td(KArgs ka, T* gscratch, size_t gstride, int all, int blk) {
+  constexpr int RPW = 32 * NR / MW, NT = 32 * NW, MT = 32 * MW;
+  using N = TdNum<T>;
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  const int p = blockIdx.x;
+  if (!ka.active[p]) return;
+  const Prob& P = ka.probs[p];
+  const int n = blk * P.nb, ns = n | 1, zs = td_zs(n), us = td_us(n), vn = td_vn(n);
+  const double* Sin = blk == 2 ? P.S2 : P.S;
+  const double* Hin = blk == 2 ? P.H2 : P.Hs;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  // vectors
+  T* dk = reinterpret_cast<T*>(smem_raw);  // 1 / (1 + d_k); 0 marks a left-out direction
+  T* vbuf = dk + vn;                       // [2][vn] Householder vectors in turn
+  T* pv = vbuf + 2 * vn;                   // C v
+  T* wv = pv + vn;                         // the rank-two update's w
+  T* tau = wv + vn;
+  T* dg = tau + vn;                        // diagonal, then the blocks' eigenvalues
+  T* eo = dg + vn;                         // off-diagonal
+  T* zv = eo + vn;                         // z recomputed from the roots
+  T* ds = zv + vn;                         // sorted poles
+  T* zw = ds + vn;                         // rho z^2, sorted
+  T* zh = zw + vn;                         // z, sorted
+  T* mu = zh + vn;                         // root i = ds[kx[i]] + mu[i]
+  T* red = mu + vn;                        // [32]
+  T* nd = vbuf;                            // new eigenvalues (the reflectors are done with by then)
+  int* perm = reinterpret_cast<int*>(red + 32);
+  int* kx = perm + vn;
+  int* bk = kx + vn;                       // block of each index: lo | mid << 10 | hi << 20
+  float* fz = reinterpret_cast<float*>(wv);  // (FP64) the weights as floats
+  int* flags = bk + vn;                      // [0] Cholesky failed, [1] left-out directions, [2] close poles, [3] capped
+  T* Ub = reinterpret_cast<T*>(smem_raw + td_vec_bytes(n, sizeof(T)));  // [n][us]; L or the reflectors [n][ns]
+  T* Zb = Ub + (size_t)n * (ns > us ? ns : us);                        // [n][zs]
+  T* Lb = all ? Zb + ((size_t)n * zs + 3) / 4 * 4 : Ub;                // L: row k holds column k
+  T* Vb = all ? Lb + (size_t)n * ns : Ub;                              // reflectors, row k
+  T* gW = gscratch ? gscratch + (size_t)p * gstride : nullptr;         // transposes
+  T* gL = gW + (size_t)n * n;
+  T* gV = gL + (size_t)n * n;
+  T* gC = all ? gW : gV + (size_t)n * n;                               // (FP32) C
+  T* gS = gW + ((all ? 1 : 4) * (size_t)n * n + 3) / 4 * 4;            // (FP32) [MW][n][RPW], 16-byte aligned
+  if (tid < 16) flags[tid] = 0;
+  __syncthreads();
+
+  // row i = i0 + a, column (or, for column-owning steps, row) j = lane + 32 c
+  const int i0 = warp * RPW;
+  T A[RPW][NR];
+  if (warp < MW) {
+    // ---- 1. Cholesky: a warp factors its RPW columns, one barrier, the others update ----
+#pragma unroll
+    for (int a = 0; a < RPW; ++a)
+#pragma unroll
+      for (int c = 0; c < NR; ++c) {
+        const int i = i0 + a, j = lane + 32 * c;
+        A[a][c] = T(0);
+        if (i < n && j < n) {
+          double s = Sin[(size_t)i * n + j];
+          if (i == j) s -= 1.0;
+          A[a][c] = (T)s;
+        }
+      }
+    // (only entries j >= i of the trailing rows are kept up to date)
+    for (int pw = 0; pw * RPW < n; ++pw) {
+      if (pw == warp) {
+#pragma unroll 1
+        for (int a = 0; a < RPW && i0 + a < n; ++a) {
+          const int k = i0 + a;
+          T row[NR], x = T(0);
+#pragma unroll
+          for (int c = 0; c < NR; ++c) row[c] = A[0][c];
+#pragma unroll
+          for (int b = 1; b < RPW; ++b)
+#pragma unroll
+            for (int c = 0; c < NR; ++c)
+              if (b == a) row[c] = A[b][c];
+#pragma unroll
+          for (int c = 0; c < NR; ++c)
+            if (c == (k >> 5)) x = row[c];
+          x = __shfl_sync(0xffffffffu, x, k & 31);
+          const bool drop = blk == 2 && k >= P.nb && x <= T(TD_DROP) - T(1);
+          const bool bad = !drop && !(x > T(-0.999));
+          const T inv = drop ? T(0) : td_rsqrt(T(1) + (bad ? T(-0.999) : x));
+          if (lane == 0) {
+            dk[k] = inv;
+            if (bad) flags[0] = 1;
+            if (drop) flags[1] = 1;
+          }
+#pragma unroll
+          for (int c = 0; c < NR; ++c) {
+            const int j = lane + 32 * c;
+            row[c] = j > k && j < n ? row[c] * inv : T(0);
+            if (j < n) Lb[(size_t)k * ns + j] = row[c];
+          }
+          __syncwarp();
+#pragma unroll
+          for (int b = 1; b < RPW; ++b)
+            if (b > a) {
+              const T li = i0 + b < n ? Lb[(size_t)k * ns + i0 + b] : T(0);
+#pragma unroll
+              for (int c = 0; c < NR; ++c) A[b][c] -= li * row[c];
+            }
+        }
+      }
+      bar_matrix(MT);
+      if (warp > pw && i0 < n) {
+        for (int k = pw * RPW; k < (pw + 1) * RPW; ++k) {
+          T lj[NR];
+#pragma unroll
+          for (int c = 0; c < NR; ++c) lj[c] = lane + 32 * c < n ? Lb[(size_t)k * ns + lane + 32 * c] : T(0);
+#pragma unroll
+          for (int a = 0; a < RPW; ++a) {
+            const T li = i0 + a < n ? Lb[(size_t)k * ns + i0 + a] : T(0);
+#pragma unroll
+            for (int c = 0; c < NR; ++c)
+              if (32 * c + 31 >= i0) A[a][c] -= li * lj[c];
+          }
+        }
+      }
+    }
+    // ---- 2. W = L^-1 Hs, C = W L^-T (a warp owns columns i0 .. i0 + RPW - 1; no barriers) ----
+    // forward substitution: x_k = h_k / (1 + d_k), h_r -= D_rk x_k for r > k
+    auto forward = [&](T(&X)[RPW][NR]) {
+#pragma unroll
+      for (int ck = 0; ck < NR; ++ck) {
+        const int kn = min(32, n - 32 * ck);
+        for (int t = 0; t < kn; ++t) {
+          const int k = 32 * ck + t;
+          const T inv = dk[k];
+          T x[RPW], l[NR];
+#pragma unroll
+          for (int c = ck; c < NR; ++c) l[c] = lane + 32 * c < n ? Lb[(size_t)k * ns + lane + 32 * c] : T(0);  // zero for r <= k
+#pragma unroll
+          for (int a = 0; a < RPW; ++a) {
+            x[a] = __shfl_sync(0xffffffffu, X[a][ck], t) * inv;
+            if (lane == t) X[a][ck] = x[a];
+          }
+#pragma unroll
+          for (int c = ck; c < NR; ++c)
+#pragma unroll
+            for (int a = 0; a < RPW; ++a) X[a][c] -= l[c] * x[a];
+        }
+      }
+    };
+    // (Hs is symmetric to rounding; its rows are taken as columns, and C is symmetrised below)
+    if (i0 < n) {
+#pragma unroll
+      for (int a = 0; a < RPW; ++a)
+#pragma unroll
+        for (int c = 0; c < NR; ++c) {
+          const int i = i0 + a, j = lane + 32 * c;
+          A[a][c] = i < n && j < n ? (T)Hin[(size_t)i * n + j] : T(0);
+        }
+      forward(A);
+    }
+    // transpose through U's place (or the global scratch, where L occupies it)
+    T* const Tb = all ? Ub : gW;
+    const int ts = all ? ns : n;
+    auto put = [&]() {  // Tb[i][j] = A
+#pragma unroll
+      for (int a = 0; a < RPW; ++a)
+#pragma unroll
+        for (int c = 0; c < NR; ++c)
+          if (i0 + a < n && lane + 32 * c < n) Tb[(size_t)(i0 + a) * ts + lane + 32 * c] = A[a][c];
+    };
+    put();
+    bar_matrix(MT);
+#pragma unroll
+    for (int a = 0; a < RPW; ++a)
+#pragma unroll
+      for (int c = 0; c < NR; ++c)
+        A[a][c] = i0 + a < n && lane + 32 * c < n ? Tb[(size_t)(lane + 32 * c) * ts + i0 + a] : T(0);
+    if (i0 < n) forward(A);
+    bar_matrix(MT);
+    put();
+    if (!all)  // L is needed again at the end; its place is U's
+      for (int e = tid; e < n * n; e += MT) gL[e] = Lb[(size_t)(e / n) * ns + e % n];
+    bar_matrix(MT);
+    T rs = T(0);  // largest row sum of |C|
+#pragma unroll
+    for (int a = 0; a < RPW; ++a) {
+      T s = T(0);
+#pragma unroll
+      for (int c = 0; c < NR; ++c) {
+        if (i0 + a < n && lane + 32 * c < n) A[a][c] = T(0.5) * (A[a][c] + Tb[(size_t)(lane + 32 * c) * ts + i0 + a]);
+        s += fabs(A[a][c]);
+      }
+      if (flags[1]) rs = fmax(rs, wsum(s));
+    }
+    if (flags[1]) {  // (blk = 2) left-out directions above the spectrum
+      if (lane == 0) red[warp] = rs;
+      bar_matrix(MT);
+      for (int w = 0; w < MW; ++w) rs = fmax(rs, red[w]);
+#pragma unroll
+      for (int a = 0; a < RPW; ++a)
+#pragma unroll
+        for (int c = 0; c < NR; ++c)
+          if (i0 + a < n && i0 + a == lane + 32 * c && dk[i0 + a] == T(0)) A[a][c] = T(2) * rs + T(1);
+    }
+    if constexpr (sizeof(T) == 4)
+#pragma unroll
+      for (int a = 0; a < RPW; ++a)
+#pragma unroll
+        for (int c = 0; c < NR; ++c)
+          if (i0 + a < n && lane + 32 * c < n) gC[(size_t)(i0 + a) * n + lane + 32 * c] = A[a][c];
+    // ---- 3. tridiagonalisation: reflector k from row k (warp k / RPW), v_{k+1} = 1 ----
+    for (int k = 0; k + 2 < n; ++k) {
+      T* v = vbuf + (k & 1) * vn;
+      if (k / RPW == warp) {
+        T x[NR], x1 = T(0), dd = T(0);
+#pragma unroll
+        for (int c = 0; c < NR; ++c) x[c] = T(0);
+#pragma unroll
+        for (int a = 0; a < RPW; ++a)
+          if (i0 + a == k)
+#pragma unroll
+            for (int c = 0; c < NR; ++c) x[c] = A[a][c];
+#pragma unroll
+        for (int c = 0; c < NR; ++c) {
+          if (c == (k >> 5)) dd = x[c];
+          if (c == ((k + 1) >> 5)) x1 = x[c];
+        }
+        x1 = __shfl_sync(0xffffffffu, x1, (k + 1) & 31);
+        T sg = T(0);
+#pragma unroll
+        for (int c = 0; c < NR; ++c) {
+          if (lane + 32 * c <= k + 1) x[c] = T(0);
+          sg += x[c] * x[c];
+        }
+        sg = wsum(sg);
+        T beta = x1, f = T(0), tk = T(0);
+        if (sg > T(0)) {
+          const T s2 = x1 * x1 + sg, r = td_rsqrt(s2), m = s2 * r;  // |x| = m
+          beta = x1 > T(0) ? -m : m;
+          f = td_rcp(x1 - beta);
+          tk = T(1) + fabs(x1) * r;
+        }
+        if (lane == (k & 31)) dg[k] = dd;
+        if (lane == 0) {
+          eo[k] = beta;
+          tau[k] = tk;
+        }
+        T* vd = all ? Vb + (size_t)k * ns : gV + (size_t)k * n;
+#pragma unroll
+        for (int c = 0; c < NR; ++c) {
+          const int j = lane + 32 * c;
+          const T vj = j == k + 1 ? T(1) : x[c] * f;
+          if (j < n) {
+            v[j] = vj;
+            vd[j] = vj;
+          }
+        }
+      }
+      bar_matrix(MT);
+      const T tk = tau[k];
+      if (tk == T(0)) continue;  // (uniform) nothing to eliminate
+      const bool busy = i0 + RPW - 1 > k && i0 < n;
+      T vj[NR];
+#pragma unroll
+      for (int c = 0; c < NR; ++c) vj[c] = lane + 32 * c < n ? v[lane + 32 * c] : T(0);
+      if (busy) {
+        T q[RPW];
+#pragma unroll
+        for (int a = 0; a < RPW; ++a) q[a] = T(0);
+#pragma unroll
+        for (int c = 0; c < NR; ++c)
+          if (32 * c + 31 > k)
+#pragma unroll
+            for (int a = 0; a < RPW; ++a) q[a] += A[a][c] * vj[c];
+        const T s = fold_sums<T, RPW, 32>(q, lane);
+        constexpr int S = fold_shift<RPW, 32>();
+        const int a = lane >> S;
+        if ((lane & ((1 << S) - 1)) == 0 && a < RPW && i0 + a < n) pv[i0 + a] = s;
+      }
+      bar_matrix(MT);
+      if (busy) {
+        T pj[NR], kk = T(0);
+#pragma unroll
+        for (int c = 0; c < NR; ++c) {
+          const int j = lane + 32 * c;
+          pj[c] = j > k && j < n ? pv[j] : T(0);
+          kk += pj[c] * vj[c];
+        }
+        kk = T(0.5) * tk * wsum(kk);
+#pragma unroll
+        for (int c = 0; c < NR; ++c) {
+          pj[c] = tk * (pj[c] - kk * vj[c]);  // w_j
+          const int j = lane + 32 * c;
+          if (j >= i0 && j < i0 + RPW && j < n) wv[j] = pj[c];
+        }
+        __syncwarp();
+        T vi[RPW], wi[RPW];
+        ldv(v + i0, vi);
+        ldv(wv + i0, wi);
+#pragma unroll
+        for (int c = 0; c < NR; ++c)
+          if (32 * c + 31 > k)
+#pragma unroll
+            for (int a = 0; a < RPW; ++a)
+              if (i0 + a < n) A[a][c] = fma(-vi[a], pj[c], fma(-wi[a], vj[c], A[a][c]));
+      }
+    }
+#pragma unroll
+    for (int a = 0; a < RPW; ++a)
+#pragma unroll
+      for (int c = 0; c < NR; ++c) {
+        const int i = i0 + a, j = lane + 32 * c;
+        if (i < n && i + 2 >= n && j < n) {
+          if (i == j) dg[i] = A[a][c];
+          if (i == n - 2 && j == n - 1) eo[i] = A[a][c];
+        }
+      }
+  }
+  __syncthreads();
+  // ---- 4. divide and conquer ----
+  constexpr int TD_LEAF = td_leaf_rows<T>();
+  // blocks: at shift sh, block q holds the indices (q n) >> sh .. ((q + 1) n) >> sh.  The leaves are
+  // the blocks of at most TD_LEAF rows, torn apart at their ends (d -= |e| on either side of a
+  // tear).
+  {
+    T nm = T(0);
+    for (int i = tid; i < n; i += NT) {
+      nm = fmax(nm, fabs(dg[i]) + (i > 0 ? fabs(eo[i - 1]) : T(0)) + (i + 1 < n ? fabs(eo[i]) : T(0)));
+      perm[i] = i;  // (stays a valid index where the input is not finite)
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) nm = fmax(nm, __shfl_xor_sync(0xffffffffu, nm, o));
+    if (lane == 0) red[warp] = nm;
+  }
+  __syncthreads();
+  T norm = T(0);
+  for (int w = 0; w < NW; ++w) norm = fmax(norm, red[w]);
+  int lev = 0;  // merge levels
+  while (((n + (1 << lev) - 1) >> lev) > TD_LEAF) ++lev;
+  const T gap = N::eps * norm;
+  if (tid < (TD_LEAF << lev)) {  // TD_LEAF lanes per leaf
+    const int q = tid / TD_LEAF, r = tid % TD_LEAF;
+    const int lo = (q * n) >> lev, hi = ((q + 1) * n) >> lev, m0 = hi - lo;
+    T d[TD_LEAF], e[TD_LEAF], z[TD_LEAF];
+#pragma unroll
+    for (int i = 0; i < TD_LEAF; ++i) {
+      d[i] = i < m0 ? dg[lo + i] : T(0);
+      e[i] = i + 1 < m0 ? eo[lo + i] : T(0);
+      if (i == 0 && lo > 0) d[i] -= fabs(eo[lo - 1]);
+      if (i == m0 - 1 && hi < n) d[i] -= fabs(eo[hi - 1]);
+      z[i] = i == r ? T(1) : T(0);
+    }
+    td_leaf(d, e, z, m0, norm);
+    // ascending: vector i goes to row lo + rank of the leaf's part of Z
+#pragma unroll
+    for (int i = 0; i < TD_LEAF; ++i) {
+      int rk = 0;
+#pragma unroll
+      for (int k = 0; k < TD_LEAF; ++k) rk += k < m0 && (d[k] < d[i] || (d[k] == d[i] && k < i));
+      if (i < m0) {
+        if (r < m0) Zb[(size_t)(lo + rk) * zs + r] = z[i];
+        if (r == 0) nd[lo + rk] = d[i];
+      }
+    }
+  }
+  __syncthreads();
+  for (int i = tid; i < n; i += NT) dg[i] = nd[i];
+  // the merged vectors: A[a][c] = component lane + 32 c of vector i0 + a
+  if (warp < MW)
+#pragma unroll
+    for (int a = 0; a < RPW; ++a)
+#pragma unroll
+      for (int c = 0; c < NR; ++c)  // (kept where one leaf is the whole matrix)
+        A[a][c] = lev == 0 && i0 + a < n && lane + 32 * c < n ? Zb[(size_t)(i0 + a) * zs + lane + 32 * c] : T(0);
+  for (int l = 0; l < lev; ++l) {
+    const int sh = lev - l - 1;
+    const int g = td_lanes<T>((n + (1 << sh) - 1) >> sh, n);  // lanes per root
+    const int sub = tid & (g - 1), GR = NT / g, root0 = tid / g;
+    const int slots = (n + GR - 1) / GR;
+    __syncthreads();
+    // sort the poles of the two halves together
+    for (int i = tid; i < n; i += NT) {
+      const int q = (((i + 1) << sh) - 1) / n;  // the block of index i at this level
+      const int lo = (q * n) >> sh, hi = ((q + 1) * n) >> sh, mid = ((2 * q + 1) * n) >> (sh + 1);
+      bk[i] = lo | mid << 10 | hi << 20;
+      const T d = dg[i];
+      int b0 = i < mid ? mid : lo, b1 = i < mid ? hi : mid;
+      const int s0 = b0;
+      while (b0 < b1) {
+        const int h = (b0 + b1) >> 1;
+        if (i < mid ? dg[h] < d : dg[h] <= d) b0 = h + 1;
+        else b1 = h;
+      }
+      const int pos = (i < mid ? i : lo + i - mid) + (b0 - s0);
+      T z = T(1), rho = T(0);
+      if (mid > lo && mid < hi) {
+        z = i < mid ? Zb[(size_t)i * zs + mid - 1 - lo] : Zb[(size_t)i * zs];
+        const T e = eo[mid - 1];
+        if (i >= mid && e < T(0)) z = -z;
+        rho = fabs(e);
+      }
+      if (fabs(z) < N::ztiny) z = z < T(0) ? -N::ztiny : N::ztiny;
+      ds[pos] = d;
+      zh[pos] = z;
+      zw[pos] = z * z * rho;
+      perm[pos] = i;
+    }
+    if (tid == 0) flags[2] = 0;
+    __syncthreads();
+    for (int i = tid; i < n; i += NT)
+      if (i > (bk[i] & 1023) && !(ds[i] - ds[i - 1] >= gap)) flags[2] = 1;
+    for (int e = tid; e < n * us / (16 / (int)sizeof(T)); e += NT) reinterpret_cast<float4*>(Ub)[e] = make_float4(0.f, 0.f, 0.f, 0.f);
+    __syncthreads();
+    if (flags[2]) {  // (few or none) poles closer than rounding: one thread per block moves them apart
+      for (int i = tid; i < n; i += NT) {
+        const int lo = bk[i] & 1023, hi = bk[i] >> 20;
+        if (i == lo)
+          for (int j = lo + 1; j < hi; ++j)
+            if (!(ds[j] - ds[j - 1] >= gap)) {
+              // (the step may round to less than gap where |ds| is large: take the next step up)
+              const T up = ds[j - 1] + gap;
+              ds[j] = up > ds[j - 1] ? up : ds[j - 1] + T(2) * gap;
+            }
+      }
+      __syncthreads();
+    }
+    if constexpr (sizeof(T) == 8) {
+      for (int i = tid; i < n; i += NT) fz[i] = (float)zw[i];
+      __syncthreads();
+    }
+    // roots
+    for (int sl = 0; sl < slots; ++sl) {
+      const int i = sl * GR + root0;
+      const bool live = i < n;
+      const int b3 = bk[live ? i : n - 1], lo = b3 & 1023, mid = (b3 >> 10) & 1023, hi = b3 >> 20;
+      const T rho = mid > lo && mid < hi ? fabs(eo[mid - 1]) : T(0);
+      const bool solve = live && rho > T(0.01) * gap;
+      const int ii = live ? i : lo;
+      const bool last = ii == hi - 1;
+      const int nx = last ? ii : ii + 1;
+      using F = float;
+      T tot = T(0);
+      for (int j = lo + sub; j < hi; j += g) tot += zw[j];
+      tot = gsum(tot, g);
+      const T w = last ? tot : ds[nx] - ds[ii];
+      // the sign at the middle tells the nearer pole; the root of the two-pole model there starts
+      // the iteration.  FP64: both in floats, then two or three FP64 steps.
+      const F wf = (F)w, hf = 0.5f * wf;
+      const F* zf = nullptr;
+      if constexpr (sizeof(T) == 8) zf = fz;
+      else zf = zw;
+      auto fpole = [&](int K) { return Poles<F, T>{ds, ds[K]}; };
+      F fm = 0.f;
+      if (solve) {
+        const auto po = fpole(ii);
+        for (int j = lo + sub; j < hi; j += g) fm += zf[j] * td_rcp(po(j) - hf);
+      }
+      fm = gsum(fm, g) + 1.f;
+      const bool right = !last && fm < 0.f;
+      const int K = right ? ii + 1 : ii;
+      F xf = two_pole_root(fm + 2.f * (zf[ii] - (last ? 0.f : zf[nx])) * td_rcp(wf), zf[ii], last ? 0.f : zf[nx], wf, right);
+      const F af = right ? -wf : 0.f, bf = right ? 0.f : wf;
+      if (!(xf > af && xf < bf)) xf = right ? -0.5f * hf : 0.5f * hf;
+      bool done = secular(fpole(K), zf, lo, hi, ii, sub, g, wf, right, last, af, bf, !solve,
+                          sizeof(T) == 8 ? 12 : TD_ITERS, &xf);
+      T x = (T)xf;
+      if constexpr (sizeof(T) == 8) {
+        const T a = right ? -w : T(0), b = right ? T(0) : w;
+        if (!(x > a && x < b)) x = right ? -0.25 * w : 0.25 * w;
+        done = secular(Poles<T, T>{ds, ds[K]}, zw, lo, hi, ii, sub, g, w, right, last, a, b, !solve, TD_ITERS, &x);
+      }
+      if (live && sub == 0) {
+        kx[i] = solve ? K : -1;  // -1: the halves stay as they are
+        mu[i] = solve ? x : T(0);
+        nd[i] = solve ? ds[K] + x : ds[i];
+        if (solve && !done) atomicAdd(&flags[3], 1);
+      }
+    }
+    __syncthreads();
+    // z from the roots: z_j^2 ~ (lam_last - ds_j) prod_{i<j} (lam_i - ds_j) / (ds_i - ds_j)
+    //                          prod_{j<=i<last} (lam_i - ds_j) / (ds_{i+1} - ds_j), every factor positive
+    for (int sl = 0; sl < slots; ++sl) {
+      const int j = sl * GR + root0;
+      const bool live = j < n && kx[j < n ? j : 0] >= 0;
+      T pr = T(1);
+      if (live) {
+        const int lo = bk[j] & 1023, hi = bk[j] >> 20;
+        const T dj = ds[j];
+        for (int i = lo + sub; i < hi; i += g) {
+          const T num = (ds[kx[i]] - dj) + mu[i];
+          pr *= i == hi - 1 ? num : num * td_rcp(ds[i < j ? i : i + 1] - dj);
+        }
+      }
+      for (int o = g >> 1; o > 0; o >>= 1) pr *= __shfl_xor_sync(0xffffffffu, pr, o);
+      if (live && sub == 0) {
+        const T q = sqrt(fmax(fabs(pr), N::floor));
+        zv[j] = zh[j] < T(0) ? -q : q;
+      }
+    }
+    __syncthreads();
+    // U[original index of pole j - lo][i] = z_j / (ds_j - lam_i), normalised
+    for (int sl = 0; sl < slots; ++sl) {
+      const int i = sl * GR + root0;
+      const bool live = i < n;
+      const int b3 = bk[live ? i : n - 1], lo = b3 & 1023, hi = b3 >> 20;
+      const int K = live ? kx[i] : -1;
+      T s = T(0);
+      if (K >= 0) {
+        const T base = ds[K], m = mu[i];
+        for (int j = lo + sub; j < hi; j += g) {
+          const T v = zv[j] * td_rcp((ds[j] - base) - m);
+          Ub[(size_t)perm[j] * us + i] = v;
+          s += v * v;
+        }
+      }
+      s = gsum(s, g);
+      if (K >= 0) {
+        const T f = td_rsqrt(s);
+        for (int j = lo + sub; j < hi; j += g) Ub[(size_t)perm[j] * us + i] *= f;
+      } else if (live && sub == 0) {
+        Ub[(size_t)perm[i] * us + i] = T(1);
+      }
+    }
+    __syncthreads();
+    // vectors: component r of vector i = sum over the poles j of r's half, U[j][i] Z[j][r]
+    if (warp < MW && i0 < n) {
+#pragma unroll
+      for (int a = 0; a < RPW; ++a)
+#pragma unroll
+        for (int c = 0; c < NR; ++c) A[a][c] = T(0);
+      const int jlo = bk[i0] & 1023, jhi = bk[min(i0 + RPW, n) - 1] >> 20;
+      for (int jh = jlo; jh < jhi;) {  // half blocks: poles j0 .. j1 - 1, whose vectors span rows j0 .. j1 - 1
+        const int b3 = bk[jh], mid = (b3 >> 10) & 1023;
+        const int j0 = jh, j1 = jh < mid ? mid : b3 >> 20;
+        const T* z[NR];
+        bool on[NR];
+#pragma unroll
+        for (int c = 0; c < NR; ++c) {
+          const int r = lane + 32 * c;
+          on[c] = r >= j0 && r < j1;
+          z[c] = Zb + (size_t)j0 * zs + (on[c] ? r - j0 : 0);
+        }
+#pragma unroll 4
+        for (int j = j0; j < j1; ++j) {
+          T u[RPW];
+          ldv(Ub + (size_t)j * us + i0, u);
+#pragma unroll
+          for (int c = 0; c < NR; ++c)
+            if (32 * c < j1 && 32 * c + 31 >= j0) {
+              const T zr = on[c] ? z[c][(j - j0) * zs] : T(0);
+#pragma unroll
+              for (int a = 0; a < RPW; ++a) A[a][c] += u[a] * zr;
+            }
+        }
+        jh = j1;
+      }
+    }
+    __syncthreads();
+    for (int i = tid; i < n; i += NT) dg[i] = nd[i];
+    if (sh > 0 && warp < MW) {
+#pragma unroll
+      for (int a = 0; a < RPW; ++a) {
+        const int b3 = bk[min(i0 + a, n - 1)], lo = b3 & 1023, hi = b3 >> 20;
+#pragma unroll
+        for (int c = 0; c < NR; ++c) {
+          const int r = lane + 32 * c;
+          if (i0 + a < n && r >= lo && r < hi) Zb[(size_t)(i0 + a) * zs + r - lo] = A[a][c];
+        }
+      }
+    }
+  }
+  __syncthreads();
+  // ---- 5. reflectors from the last to the first, then back substitution with L^T ----
+  if (warp >= MW) return;  // (the matrix warps go on alone)
+  if (!all) {
+    for (int e = tid; e < (n - 2) * n; e += MT) Ub[(size_t)(e / n) * ns + e % n] = gV[e];
+    bar_matrix(MT);
+  }
+  if (i0 < n)
+    for (int k = n - 3; k >= 0; --k) {
+      const T tk = tau[k];
+      if (tk == T(0)) continue;
+      T v[NR], q[RPW];
+#pragma unroll
+      for (int a = 0; a < RPW; ++a) q[a] = T(0);
+#pragma unroll
+      for (int c = 0; c < NR; ++c) {
+        v[c] = T(0);
+        if (32 * c + 31 > k) {
+          if (lane + 32 * c < n) v[c] = Vb[(size_t)k * ns + lane + 32 * c];
+#pragma unroll
+          for (int a = 0; a < RPW; ++a) q[a] += v[c] * A[a][c];
+        }
+      }
+      const T s = fold_sums<T, RPW, 32>(q, lane) * tk;
+#pragma unroll
+      for (int a = 0; a < RPW; ++a) q[a] = __shfl_sync(0xffffffffu, s, a << fold_shift<RPW, 32>());
+#pragma unroll
+      for (int c = 0; c < NR; ++c)
+        if (32 * c + 31 > k)
+#pragma unroll
+          for (int a = 0; a < RPW; ++a) A[a][c] -= q[a] * v[c];
+    }
+  if constexpr (sizeof(T) == 4) {
+    // Correction in FP32.  The steps so far leave |V^T C V - diag| and |V^T V - I| near 2e-6, a few
+    // times what the rotations of a Jacobi left; in the SCF that is noise in rho and F.  With
+    // r_j = C v_j - lam_j v_j: V += V E, E_ij = v_i.r_j / (lam_j - lam_i) for pairs far enough apart,
+    // lam_j += v_j.r_j; then V += V (I - V^T V) / 2.  Five small products bring both to 5e-7, below
+    // the Jacobi's (fewer SCF iterations at tight density rules), for a tenth of the time.
+    // V^T in Ub; V by rows in Vb where there is room (after C, which takes that room first), else
+    // by columns of V^T
+    const T* Xv = all ? Vb : Ub;
+    const int xk = all ? ns : 1, xr = all ? 1 : us;
+    const T* Xc = all ? Vb : gC;
+    const int cs = all ? ns : n;
+    T* const mine = gS + (size_t)warp * n * RPW;  // the warp's own factor, [k][RPW]
+    auto vt = [&](int a, int c) -> T {            // component lane + 32 c of vector i0 + a
+      return i0 + a < n && lane + 32 * c < n ? Ub[(lane + 32 * c) * us + i0 + a] : T(0);
+    };
+    auto stage = [&]() {
+      __syncwarp();
+#pragma unroll
+      for (int a = 0; a < RPW; ++a)
+#pragma unroll
+        for (int c = 0; c < NR; ++c)
+          if (lane + 32 * c < n) mine[(lane + 32 * c) * RPW + a] = A[a][c];
+      __syncwarp();
+    };
+    // A[a][c] = sum_k f[k][a] X(k, lane + 32 c), f = the staged factor or the columns of V^T
+    auto product = [&](const T* f, int fs, const T* X, int sk, int sr) {
+#pragma unroll
+      for (int a = 0; a < RPW; ++a)
+#pragma unroll
+        for (int c = 0; c < NR; ++c) A[a][c] = T(0);
+#pragma unroll 4
+      for (int k = 0; k < n; ++k) {
+        T u[RPW];
+        ldv(f + k * fs, u);
+#pragma unroll
+        for (int c = 0; c < NR; ++c) {
+          const int r = lane + 32 * c;
+          const T x = X[k * sk + r * sr];  // (lanes r >= n read on into what follows; their sums are not used)
+#pragma unroll
+          for (int a = 0; a < RPW; ++a) A[a][c] += u[a] * x;
+        }
+      }
+    };
+    auto put_vt = [&]() {
+#pragma unroll
+      for (int a = 0; a < RPW; ++a)
+#pragma unroll
+        for (int c = 0; c < NR; ++c)
+          if (i0 + a < n && lane + 32 * c < n) Ub[(lane + 32 * c) * us + i0 + a] = A[a][c];
+    };
+    bar_matrix(MT);  // (the reflectors are done with)
+    put_vt();
+    if (all)
+      for (int e = tid; e < n * n; e += MT) Vb[(size_t)(e / n) * ns + e % n] = gC[e];
+    bar_matrix(MT);
+    if (i0 < n) {
+      product(Ub + i0, us, Xc, cs, 1);  // C v_j
+#pragma unroll
+      for (int a = 0; a < RPW; ++a)
+#pragma unroll
+        for (int c = 0; c < NR; ++c) A[a][c] -= dg[min(i0 + a, n - 1)] * vt(a, c);
+      stage();
+    }
+    if (all) {
+      bar_matrix(MT);
+#pragma unroll
+      for (int a = 0; a < RPW; ++a)
+#pragma unroll
+        for (int c = 0; c < NR; ++c)
+          if (i0 + a < n && lane + 32 * c < n) Vb[(i0 + a) * ns + lane + 32 * c] = vt(a, c);
+    }
+    if (i0 < n) {
+      product(mine, RPW, Ub, us, 1);  // v_i.r_j
+#pragma unroll
+      for (int a = 0; a < RPW; ++a)
+#pragma unroll
+        for (int c = 0; c < NR; ++c) {
+          const int i = lane + 32 * c, j = i0 + a;
+          const T y = A[a][c], lj = dg[min(j, n - 1)], dl = lj - dg[min(i, n - 1)];
+          if (i == j && i < n) nd[i] = lj + y;
+          // (closer pairs stay as they are: their quotients are rounding)
+          A[a][c] = i < n && fabs(dl) > T(5e-4) * norm && fabs(y) <= T(2e-3) * fabs(dl) ? y * td_rcp(dl) : T(0);
+        }
+      stage();
+    }
+    if (all) bar_matrix(MT);
+    if (i0 < n) {
+      product(mine, RPW, Xv, xk, xr);
+#pragma unroll
+      for (int a = 0; a < RPW; ++a)
+#pragma unroll
+        for (int c = 0; c < NR; ++c) A[a][c] += vt(a, c);
+    }
+    bar_matrix(MT);
+    put_vt();
+    if (all)
+#pragma unroll
+      for (int a = 0; a < RPW; ++a)
+#pragma unroll
+        for (int c = 0; c < NR; ++c)
+          if (i0 + a < n && lane + 32 * c < n) Vb[(i0 + a) * ns + lane + 32 * c] = A[a][c];
+    bar_matrix(MT);
+    if (i0 < n) {
+      product(Ub + i0, us, Ub, us, 1);  // v_i.v_j
+#pragma unroll
+      for (int a = 0; a < RPW; ++a)
+#pragma unroll
+        for (int c = 0; c < NR; ++c)
+          A[a][c] = T(0.5) * ((lane + 32 * c == i0 + a ? T(1) : T(0)) - A[a][c]);
+      stage();
+      product(mine, RPW, Xv, xk, xr);
+#pragma unroll
+      for (int a = 0; a < RPW; ++a)
+#pragma unroll
+        for (int c = 0; c < NR; ++c) A[a][c] += vt(a, c);
+    }
+    for (int i = tid; i < n; i += MT) dg[i] = nd[i];
+    bar_matrix(MT);
+  }
+  if (!all) {
+    bar_matrix(MT);
+    for (int e = tid; e < n * n; e += MT) Ub[(size_t)(e / n) * ns + e % n] = gL[e];
+    bar_matrix(MT);
+  }
+  if (i0 < n) {
+#pragma unroll
+    for (int ci = 0; ci < NR; ++ci) {
+      constexpr int top = NR - 1;
+      const int ck = top - ci;
+      const int kn = min(32, n - 32 * ck);
+      for (int t = kn - 1; t >= 0; --t) {
+        const int k = 32 * ck + t;
+        const T inv = dk[k];
+        T x[RPW], lr[NR];
+#pragma unroll
+        for (int c = 0; c < NR; ++c)
+          if (c <= ck) lr[c] = lane + 32 * c < k ? Lb[(size_t)(lane + 32 * c) * ns + k] : T(0);  // L_kr
+#pragma unroll
+        for (int a = 0; a < RPW; ++a) {
+          x[a] = __shfl_sync(0xffffffffu, A[a][ck], t) * inv;
+          if (lane == t) A[a][ck] = x[a];
+        }
+#pragma unroll
+        for (int c = 0; c < NR; ++c)
+          if (c <= ck)
+#pragma unroll
+            for (int a = 0; a < RPW; ++a) A[a][c] -= lr[c] * x[a];
+      }
+    }
+    // ascending: the corrected eigenvalues of close pairs may have changed places
+    int rank[RPW];
+#pragma unroll
+    for (int a = 0; a < RPW; ++a) {
+      rank[a] = i0 + a;
+      if constexpr (sizeof(T) == 4) {
+        const T d = dg[min(i0 + a, n - 1)];
+        rank[a] = 0;
+#pragma unroll
+        for (int c = 0; c < NR; ++c) {
+          const int k = lane + 32 * c;
+          rank[a] += __popc(__ballot_sync(0xffffffffu, k < n && (dg[min(k, n - 1)] < d || (dg[min(k, n - 1)] == d && k < i0 + a))));
+        }
+      }
+    }
+    // the lowest n_b Ritz pairs: rows r < n_b are the coefficients on X, the others those on W
+#pragma unroll
+    for (int a = 0; a < RPW; ++a) {
+      const int i = rank[a];
+      if (i0 + a >= n || i >= P.nb) continue;
+#pragma unroll
+      for (int c = 0; c < NR; ++c) {
+        const int r = lane + 32 * c;
+        if (r >= n) continue;
+        if (r < P.nb) P.Tm[(size_t)r * P.nb + i] = (double)A[a][c];
+        else P.Cm[(size_t)(r - P.nb) * P.nb + i] = (double)A[a][c];
+      }
+      if (lane == 0) P.eps[i] = (double)dg[i0 + a];
+    }
+  }
+  if (tid == 0) {
+    if (flags[3]) P.scal[SC_RRCAP] += 1.0;
+    if (flags[0]) P.status[0] = 1;
+  }
+}
+
+namespace {
+size_t td_smem(int n, size_t ts, bool all) {
+  const size_t ns = n | 1, us = td_us(n), u = (size_t)n * (ns > us ? ns : us), z = ((size_t)n * td_zs(n) + 3) / 4 * 4;
+  return td_vec_bytes(n, ts) + (u + z + (all ? 2 * (size_t)n * ns + 32 : 0)) * ts;  // (32: rows are read on past n)
+}
+constexpr size_t TD_SMEM_MAX = 227 * 1024;
+}  // namespace
+
+// Subspaces the kernel takes: FP32 up to 184 (the merge matrix and the vectors fill the shared
+// memory), FP64 up to 128 (an 8 x 4 tile of the matrix per thread).
+int rr_td_max(size_t tsize) { return tsize == 4 ? 184 : 128; }
+
+// bytes of global scratch per problem (0: everything fits in shared memory)
+size_t rr_td_scratch_bytes(int n, size_t tsize) {
+  const size_t nn = (size_t)n * n, big = td_smem(n, tsize, true) <= TD_SMEM_MAX ? 0 : 3 * nn;
+  return (big + (tsize == 4 ? nn + 8 + (size_t)n * (n + 16) : 0)) * tsize;
+}
+
+template <typename T, int NR, int MW, int NW>
+static void td_launch(const Launch& L, int n, unsigned char* scratch, size_t stride, int blk) {
+  const bool all = td_smem(n, sizeof(T), true) <= TD_SMEM_MAX;
+  const size_t smem = td_smem(n, sizeof(T), all);
+  cudaFuncSetAttribute(k_rr_td<T, NR, MW, NW>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  k_rr_td<T, NR, MW, NW><<<L.ka.nprob, 32 * NW, smem, L.stream>>>(L.ka, reinterpret_cast<T*>(scratch),
+                                                                  stride / sizeof(T), all ? 1 : 0, blk);
+}
+
+// n: the largest subspace of the launch (n_b, or 2 n_b for blk = 2)
+template <typename T>
+void launch_rr_td(const Launch& L, int n, unsigned char* scratch, size_t stride, int blk) {
+  // (FP32: 4 to 12 rows per warp, bound by issue and latency; FP64: 8 to 16 rows in as few warps as
+  // the registers allow, bound by the FP64 lanes, which every warp's own sums use too)
+  if constexpr (sizeof(T) == 4) {
+    if (n <= 32) td_launch<T, 1, 8, 8>(L, n, scratch, stride, blk);
+    else if (n <= 64) td_launch<T, 2, 16, 16>(L, n, scratch, stride, blk);
+    else if (n <= 96) td_launch<T, 3, 16, 16>(L, n, scratch, stride, blk);
+    else if (n <= 128) td_launch<T, 4, 16, 16>(L, n, scratch, stride, blk);
+    else td_launch<T, 6, 16, 16>(L, n, scratch, stride, blk);
+  } else {
+    if (n <= 32) td_launch<T, 1, 4, 8>(L, n, scratch, stride, blk);
+    else if (n <= 64) td_launch<T, 2, 8, 8>(L, n, scratch, stride, blk);
+    else if (n <= 96) td_launch<T, 3, 8, 8>(L, n, scratch, stride, blk);
+    else td_launch<T, 4, 8, 8>(L, n, scratch, stride, blk);
+  }
+}
+template void launch_rr_td<float>(const Launch&, int, unsigned char*, size_t, int);
+template void launch_rr_td<double>(const Launch&, int, unsigned char*, size_t, int);
+
+}  // namespace sgo
