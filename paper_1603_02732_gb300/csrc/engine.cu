@@ -283,7 +283,7 @@ PlanePaths plane_paths(const Prob& d, int precision) {
   const size_t cap = 220 * 1024;
   PlanePaths q;
   q.preg = precision == 1 && plane_reg_ok(d.n1, d.n2) && plane_reg_smem(d.n1, d.n2, d.m1max) <= cap;
-  q.dreg = q.preg && plane_density_reg_smem(d.n1, d.n2, d.m1max) <= cap;
+  q.dreg = q.preg && plane_density_ms_smem(d.n1, d.n2, d.n3) <= cap;
   q.ppair = precision == 1 && !q.preg && pair_plane_ok(d.n1, d.n2) && pair_plane_smem(d.n1, d.n2, d.m1max) <= cap;
   q.dpair = q.ppair && pair_density_smem(d.n1, d.n2, d.m1max) <= cap;
   q.psmem = (size_t)(2 * d.n1 * d.n2 + d.n1 + d.n2) * 16 <= cap && d.n1 * d.n2 <= 8192;
@@ -679,15 +679,16 @@ const char* const kTimerNames[TK_COUNT] = {"plane_vpsi", "wave_to_cols", "cols_t
 // ---------------------------------------------------------------------------
 // Engine
 // ---------------------------------------------------------------------------
-WorkMap Engine::make_map(const std::vector<int>& counts) {
+// totals and largest dimensions of a map, its start indices appended to *start
+WorkMap Engine::map_of(const std::vector<int>& counts, std::vector<int>* start) const {
   WorkMap m;
-  std::vector<int> st(counts.size() + 1, 0);
-  int mx = 0;
-  for (size_t i = 0; i < counts.size(); ++i) {
-    st[i + 1] = st[i] + counts[i];
-    mx = std::max(mx, counts[i]);
+  int sum = 0, mx = 0;
+  start->push_back(0);
+  for (int c : counts) {
+    start->push_back(sum += c);
+    mx = std::max(mx, c);
   }
-  m.total = st.back();
+  m.total = sum;
   m.maxper = mx;
   m.max_n1 = m.max_n2 = m.max_n3 = m.max_n12 = m.max_nb = 0;
   for (size_t i = 0; i < counts.size() && i < ctx_.size(); ++i) {
@@ -699,6 +700,12 @@ WorkMap Engine::make_map(const std::vector<int>& counts) {
     m.max_n12 = std::max(m.max_n12, d.n1 * d.n2);
     m.max_nb = std::max(m.max_nb, d.nb);
   }
+  return m;
+}
+
+WorkMap Engine::make_map(const std::vector<int>& counts) {
+  std::vector<int> st;
+  WorkMap m = map_of(counts, &st);
   int* d = nullptr;
   if (!cuda_ok(dev_malloc(&d, st.size() * sizeof(int)), "dev_malloc(map)")) return m;
   cudaMemcpy(d, st.data(), st.size() * sizeof(int), cudaMemcpyHostToDevice);
@@ -724,13 +731,22 @@ void Engine::build_gemm_maps() {
       for (int t = 0; t < 2; ++t)
         red[k][t].push_back(div_up(nin[k] * d.nb, 256 / tn_reduce_lanes(t ? tc.back() : nsplit)));
   }
-  m_tn_[OPK_WB] = make_map(ww);
-  m_tn_[OPK_B] = make_map(bw);
-  m_tn_[OPK_DB] = make_map(dw);
+  // one buffer and one copy for all of them (the autotuner rebuilds them for every candidate)
+  std::vector<std::pair<WorkMap*, const std::vector<int>*>> maps = {
+      {&m_tn_[OPK_WB], &ww}, {&m_tn_[OPK_B], &bw}, {&m_tn_[OPK_DB], &dw}, {&m_tc_, &tc}, {&m_nntc_, &nntc}};
   for (int k = 0; k < 3; ++k)
-    for (int t = 0; t < 2; ++t) m_red_[k][t] = make_map(red[k][t]);
-  m_tc_ = make_map(tc);
-  m_nntc_ = make_map(nntc);
+    for (int t = 0; t < 2; ++t) maps.push_back({&m_red_[k][t], &red[k][t]});
+  const size_t len = ctx_.size() + 1;
+  if (!d_gmaps_) {
+    if (!cuda_ok(dev_malloc(&d_gmaps_, maps.size() * len * sizeof(int)), "dev_malloc(gemm maps)")) return;
+    allocs_.push_back(d_gmaps_);
+  }
+  std::vector<int> st;
+  for (size_t i = 0; i < maps.size(); ++i) {
+    *maps[i].first = map_of(*maps[i].second, &st);
+    maps[i].first->start = d_gmaps_ + i * len;
+  }
+  cudaMemcpy(d_gmaps_, st.data(), st.size() * sizeof(int), cudaMemcpyHostToDevice);
 }
 
 // Autotuner of the GEMM tile knobs (mixed path): for each knob, every candidate runs its
@@ -861,12 +877,12 @@ Engine::Engine(const std::vector<sgo_ctx*>& ctxs, cudaStream_t stream) : ctx_(ct
       c_preg[k].push_back(pcls != k ? 0
                           : kPlaneMultiPass ? plane_ms_ctas(d.n1, d.n2, d.n3, d.npair)
                                             : plane_reg_ctas(d.n2, d.n3, d.npair));
-      c_dreg[k].push_back(dreg && pcls == k ? plane_density_reg_ctas(d.n2, d.n3) : 0);
+      c_dreg[k].push_back(dreg && pcls == k ? plane_density_ms_ctas(d.n1, d.n2, d.n3) : 0);
     }
     if (preg)
       preg_smem_[pcls] = std::max(preg_smem_[pcls], kPlaneMultiPass ? plane_ms_smem(d.n1, d.n2, d.n3)
                                                                     : plane_reg_smem(d.n1, d.n2, d.m1max));
-    if (dreg) dreg_smem_[pcls] = std::max(dreg_smem_[pcls], plane_density_reg_smem(d.n1, d.n2, d.m1max));
+    if (dreg) dreg_smem_[pcls] = std::max(dreg_smem_[pcls], plane_density_ms_smem(d.n1, d.n2, d.n3));
     c_gz.push_back(div_up(d.n1 * d.n2, QZ));
     c_gp.push_back(gbig ? 0 : d.n3);
     c_gew.push_back(div_up(d.ngrid, GRID_EW_POINTS));
@@ -1415,7 +1431,7 @@ void Engine::density_energy(int mode) {
   wave_to_cols<T>(WB_X);
   tbeg(TK_PLANE_DENSITY);
   launch_plane_density<T>(L(m_dens_), nullptr);
-  for (int k = 0; k < 2; ++k) launch_plane_density_reg(L(m_dreg_[k]), k, dreg_smem_[k], nullptr);
+  for (int k = 0; k < 2; ++k) launch_plane_density_ms(L(m_dreg_[k]), dreg_smem_[k], nullptr);
   launch_plane_density_pair(L(m_dpair_), dpair_smem_, nullptr);
   launch_big_y<T>(L(m_bigdy_), 1, 1, nullptr);
   launch_big_density<T>(L(m_bigd_), nullptr);
@@ -1834,7 +1850,7 @@ sgo_status Engine::density(int nvec, const double* psi, const double* occ, doubl
     launch_copy_in<float>(L(m_bands_), WB_W, dpsi, nvec);
     wave_to_cols<float>(WB_W);
     launch_plane_density<float>(L(m_dens_), docc);
-    for (int k = 0; k < 2; ++k) launch_plane_density_reg(L(m_dreg_[k]), k, dreg_smem_[k], docc);
+    for (int k = 0; k < 2; ++k) launch_plane_density_ms(L(m_dreg_[k]), dreg_smem_[k], docc);
     launch_plane_density_pair(L(m_dpair_), dpair_smem_, docc);
     launch_big_y<float>(L(m_bigdy_), 1, 1, docc);
     launch_big_density<float>(L(m_bigd_), docc);

@@ -173,6 +173,7 @@ class Engine {
   void swap_roles(int a, int b);
   Launch L(const WorkMap& m) const;
   WorkMap make_map(const std::vector<int>& counts);
+  WorkMap map_of(const std::vector<int>& counts, std::vector<int>* start) const;
 
   std::vector<sgo_ctx*> ctx_;
   int n_ = 0;
@@ -234,6 +235,7 @@ class Engine {
   // the CUDA-core TN; the maps that depend on them
   int tc_kc_ = TC_KC, nn_tpc_ = NN_TPC, tn_kc_ = TN_KC;  // (tn_kc_ 0 on the FP64 path: tn_kc_f64)
   void build_gemm_maps();
+  int* d_gmaps_ = nullptr;      // their start indices
   cudaGraphExec_t g_nonscf_ = nullptr, g_scf_ = nullptr;
   // the residual-controlled CG steps after the SCF stopping rule (a WHILE node whose body
   // is one step) and the density and energy of the refined bands

@@ -121,6 +121,10 @@ constexpr bool kPlaneMultiPass = true;
 int plane_ms_ctas(int n1, int n2, int n3, int npair);
 size_t plane_ms_smem(int n1, int n2, int n3);
 void launch_plane_vpsi_ms(const Launch& L, size_t smem);
+// the density of the same lengths (multi-pass too, clusters of CTAs over the band pairs)
+int plane_density_ms_ctas(int n1, int n2, int n3);
+size_t plane_density_ms_smem(int n1, int n2, int n3);
+void launch_plane_density_ms(const Launch& L, size_t smem, const double* occ_override);
 bool plane_ms_init();
 void plane_ms_set_smem_limits(size_t bytes);
 int plane_reg_class(int n1, int n2);          // 0: both <= 40, 1: up to PLANE_REG_MAXN
@@ -128,9 +132,7 @@ int plane_reg_ctas(int n2, int n3, int npair);
 size_t plane_reg_smem(int n1, int n2, int m1max);
 bool fft_reg_init();                          // twiddle tables on the current device
 bool plane_vpsi_reg_init();
-bool plane_density_reg_init();
 void plane_vpsi_reg_set_smem_limits(size_t bytes);
-void plane_density_reg_set_smem_limits(size_t bytes);
 // register-FFT z-column passes (mixed path), k_cols_reg.cu
 int zreg_class(int n3);
 bool zreg_ok(int n3);
@@ -156,9 +158,6 @@ void launch_cols_to_wave_pair(const Launch& L, size_t smem, int src, int dst);
 bool pair_reg_init();
 void pair_reg_set_smem_limits(size_t bytes);
 void launch_plane_vpsi_reg(const Launch& L, int cls, size_t smem);
-size_t plane_density_reg_smem(int n1, int n2, int m1max);
-int plane_density_reg_ctas(int n2, int n3);
-void launch_plane_density_reg(const Launch& L, int cls, size_t smem, const double* occ_override);
 
 // k_linalg.cu
 template <typename T>

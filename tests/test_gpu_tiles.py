@@ -70,3 +70,31 @@ def test_subspace_eigensolve_sizes(sgo, carried, precision):
     occ = res[0][2] > 1e-6
     assert abs(res[0][0] - res[1][0]) < (1e-9 if precision == "fp64" else 4e-6)
     assert np.abs(res[0][1] - res[1][1])[occ].max() < (1e-7 if precision == "fp64" else 1e-4)
+
+
+# plane lengths: smallest, one plane and several per CTA, odd, the largest; fewer z-planes than a
+# block; band counts below, at and above the cluster's CTAs
+@pytest.mark.parametrize("grid,bands,ecut", [((10, 10, 10), 5, 0.5), ((12, 16, 10), 3, 0.6), ((25, 27, 12), 16, 1.0),
+                                             ((45, 25, 16), 17, 1.0), ((72, 72, 10), 18, 0.6), ((64, 10, 15), 31, 0.9)])
+def test_density_sizes_mixed(sgo, grid, bands, ecut):
+    """rho(r) = (1/Omega) sum_n occ_n |psi_n(r)|^2 from NumPy's FP64 transform, for FP32 bands with
+    some occupations zero: 2e-6 of the largest value (the FP32 line transforms' 1e-7 a value, log N
+    stages, squared)."""
+    st = dataclasses.replace(workloads.tiny(nat=1, ecut=ecut, kT=0.0, nbands=bands), fft=grid)
+    st = dataclasses.replace(st, cell=np.diag([10.0, 11.0, 12.0]), pos=np.array([[1.0, 2.0, 3.0]]))
+    ctx = sgo.Context(st, precision="mixed", extra_bands=0)
+    rng = np.random.default_rng(4)
+    psi = rng.normal(size=(bands, ctx.npw)).astype(np.float32).astype(np.float64)
+    occ = np.where(np.arange(bands) % 5 == 3, 0.0, rng.uniform(0.0, 2.0, size=bands))
+    m = ctx.basis()[1:]
+    rho = np.zeros(grid)
+    for n in range(bands):
+        box = np.zeros(grid, complex)
+        c = (psi[n, 1::2] + 1j * psi[n, 2::2]) / np.sqrt(2.0)
+        box[tuple(m.T % np.array(grid)[:, None])] = c
+        box[tuple(-m.T % np.array(grid)[:, None])] = c.conj()
+        box[0, 0, 0] = psi[n, 0]
+        rho += occ[n] * np.abs(np.fft.ifftn(box) * box.size) ** 2
+    rho /= abs(np.linalg.det(st.cell))
+    got = ctx.density_of(psi, occ)
+    assert np.abs(got - rho).max() < 2e-6 * rho.max()
