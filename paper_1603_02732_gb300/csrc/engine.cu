@@ -825,7 +825,7 @@ Engine::Engine(const std::vector<sgo_ctx*>& ctxs, cudaStream_t stream) : ctx_(ct
   }
   std::vector<Prob> host(n_);
   std::vector<int> c_zcol, c_plane, c_dens, c_gz, c_gp, c_gew, c_gch, c_bands, c_rww, c_nn, c_atoms, c_projs, c_atomch, c_ewsg, c_prob, c_tc, c_nntc, c_preg[2], c_dreg[2], c_zreg[2], c_ppair,
-      c_dpair, c_zpair, c_gx, c_gy, c_bigy, c_bigx, c_bigdy, c_bigd;
+      c_dpair, c_zpair, c_gx, c_gy, c_gaxis[3], c_gold, c_bigy, c_bigx, c_bigdy, c_bigd;
   size_t part = 0;
   int max_nproj = 0;
   for (int p = 0; p < n_; ++p) {
@@ -851,9 +851,15 @@ Engine::Engine(const std::vector<sgo_ctx*>& ctxs, cudaStream_t stream) : ctx_(ct
     if (zpair) zpair_smem_ = std::max(zpair_smem_, zpair_smem(d.n3));
     // FP64 grid transforms: a whole plane per CTA when two planes fit in shared memory,
     // otherwise line blocks along x and y
-    const bool gbig = (size_t)(2 * d.n1 * d.n2 + d.n1 + d.n2) * 16 > 220 * 1024;
+    // (all of it only for grids with a length that has no such transform, see k_grid_axis)
+    int fa, fb, fc;
+    const bool gaxis = grid_factors(d.n1, &fa, &fb, &fc) && grid_factors(d.n2, &fa, &fb, &fc) &&
+                       grid_factors(d.n3, &fa, &fb, &fc);
+    const bool gbig = !gaxis && (size_t)(2 * d.n1 * d.n2 + d.n1 + d.n2) * 16 > 220 * 1024;
+    for (int k = 0; k < 3; ++k) c_gaxis[k].push_back(gaxis ? grid_axis_ctas(d.n1, d.n2, d.n3, k) : 0);
     c_gx.push_back(gbig ? div_up(d.n3 * d.n2, QZ) : 0);
     c_gy.push_back(gbig ? div_up(d.n3 * d.n1, QZ) : 0);
+    c_gold.push_back(gaxis ? 0 : div_up(d.ngrid, GRID_EW_POINTS));
     // plane passes: register FFTs on the mixed path where both plane lengths have one
     // and the kernels' shared memory fits; the shared-memory engine otherwise
     const PlanePaths pp = plane_paths(d, precision_);
@@ -883,8 +889,8 @@ Engine::Engine(const std::vector<sgo_ctx*>& ctxs, cudaStream_t stream) : ctx_(ct
       preg_smem_[pcls] = std::max(preg_smem_[pcls], kPlaneMultiPass ? plane_ms_smem(d.n1, d.n2, d.n3)
                                                                     : plane_reg_smem(d.n1, d.n2, d.m1max));
     if (dreg) dreg_smem_[pcls] = std::max(dreg_smem_[pcls], plane_density_ms_smem(d.n1, d.n2, d.n3));
-    c_gz.push_back(div_up(d.n1 * d.n2, QZ));
-    c_gp.push_back(gbig ? 0 : d.n3);
+    c_gz.push_back(gaxis ? 0 : div_up(d.n1 * d.n2, QZ));
+    c_gp.push_back(gaxis || gbig ? 0 : d.n3);
     c_gew.push_back(div_up(d.ngrid, GRID_EW_POINTS));
     c_gch.push_back(nch);
     c_bands.push_back(d.nb);
@@ -909,6 +915,8 @@ Engine::Engine(const std::vector<sgo_ctx*>& ctxs, cudaStream_t stream) : ctx_(ct
   m_ppair_ = make_map(c_ppair);
   m_dpair_ = make_map(c_dpair);
   m_zpair_ = make_map(c_zpair);
+  for (int k = 0; k < 3; ++k) m_gaxis_[k] = make_map(c_gaxis[k]);
+  m_gold_ = make_map(c_gold);
   m_gx_ = make_map(c_gx);
   m_gy_ = make_map(c_gy);
   m_bigy_ = make_map(c_bigy);
@@ -1138,20 +1146,26 @@ void Engine::set_scal(int idx, double v, bool only_active) {
   k_set_scal<<<n_, 32, 0, stream_>>>(L(m_prob_).ka, idx, v, only_active ? 1 : 0);
 }
 
-void Engine::grid_fft(int which, int sign, bool fp32) {
+// real_src 1: the forward transform of rho_out (else of the grid's contents).
+void Engine::grid_fft(int which, int sign, int real_src) {
+  if (real_src) launch_real_to_grid(L(m_gold_), 1, which);
   tbeg(TK_GRID_FFT);
   // the mixed path's FP64 grids are transformed in float-float arithmetic (FP64 runs at
   // about 1/64 of the FP32 rate on this GPU); the plain path stays FP64 throughout
-  if (fp32) grid_fft_raw<float>(which, sign);
-  else if (precision_) grid_fft_raw<ff>(which, sign);
-  else grid_fft_raw<double>(which, sign);
+  if (precision_) grid_fft_raw<ff>(which, sign, real_src);
+  else grid_fft_raw<double>(which, sign, real_src);
   tend(TK_GRID_FFT);
 }
 
 template <typename T>
-void Engine::grid_fft_raw(int which, int sign) {
-  // forward: planes (y, x), then z; inverse: z, then planes.  Large planes go by line
-  // blocks along y and x.
+void Engine::grid_fft_raw(int which, int sign, int real_src) {
+  // forward: y, x, z; inverse: z, x, y
+  for (int k = 0; k < 3; ++k) {
+    const int axis = sign < 0 ? (k == 0 ? 1 : k == 1 ? 0 : 2) : (k == 0 ? 2 : k == 1 ? 0 : 1);
+    launch_grid_axis<T>(L(m_gaxis_[axis]), which, sign, axis, k, real_src != 0);
+  }
+  // grids with a length that has no such transform: planes (y, x), large ones by line
+  // blocks, and z lines
   auto planes = [&](int sg) {
     launch_grid_plane_fft<T>(L(m_gp_), which, sg);
     launch_grid_line_fft<T>(L(m_gy_), which, sg, 1);
@@ -1439,10 +1453,7 @@ void Engine::density_energy(int mode) {
   // energy at (Psi, rho_out) and the convergence test
   launch_band_kinetic<T>(L(m_bands_), WB_X);
   tn<T>(OPK_B, 0, OPK_WB, WB_X, DD_PROJ, false);
-  tbeg(TK_GRID_OTHER);
-  launch_real_to_grid(L(m_gew_), 1, 1);
-  tend(TK_GRID_OTHER);
-  grid_fft(1, -1);
+  grid_fft(1, -1, 1);
   if (gga_) {  // PBE energy: grad rho_out
     tbeg(TK_GRID_OTHER);
     launch_gga_grad(L(m_gew_), 1);
@@ -1681,8 +1692,7 @@ sgo_status Engine::launch_t(bool want_forces) {
     launch_build_projectors<T>(L(m_projs_), 1);
     tn<T>(OPK_DB, 0, OPK_WB, WB_X, DD_DPROJ, false);
     tn<T>(OPK_B, 0, OPK_WB, WB_X, DD_PROJ, false);
-    launch_real_to_grid(L(m_gew_), 1, 0);
-    grid_fft(0, -1);
+    grid_fft(0, -1, 1);
     launch_local_forces(L(m_atomch_), maxchunk_);
     launch_force_total(L(m_prob_), maxchunk_);
   }

@@ -153,8 +153,8 @@ class Engine {
   void nn_pairs(int akind, const RolePairs& rp, int msel, double alpha, double beta, bool image_ready);
   template <typename T> void rotate_pairs(const RolePairs& rp, const RolePairs& swap);
   int work_mult_ = 1;  // operand pairs of the NN launch being timed
-  void grid_fft(int which, int sign, bool fp32 = false);
-  template <typename T> void grid_fft_raw(int which, int sign);
+  void grid_fft(int which, int sign, int real_src = 0);
+  template <typename T> void grid_fft_raw(int which, int sign, int real_src);
   void potential();
   void energies_at_rho_out(bool count_iter);
   void pulay();
@@ -191,7 +191,8 @@ class Engine {
   size_t preg_smem_[2] = {0, 0}, dreg_smem_[2] = {0, 0}, zreg_smem_[2] = {0, 0};
   WorkMap m_ppair_, m_dpair_, m_zpair_;         // lane-pair register FFT kernels (lengths 96-128)
   size_t ppair_smem_ = 0, dpair_smem_ = 0, zpair_smem_ = 0;
-  WorkMap m_gx_, m_gy_;                         // FP64 grid transforms of planes too large for one CTA
+  WorkMap m_gaxis_[3];                          // grid transforms along x, y, z
+  WorkMap m_gold_, m_gx_, m_gy_;                // grids with a length outside those; planes too large for one CTA
   WorkMap m_bigy_, m_bigx_, m_bigdy_, m_bigd_;  // plane passes by line blocks (big planes)
   template <typename T> void wave_to_cols(int src);
   template <typename T> void cols_to_wave(int src, int dst);

@@ -344,6 +344,149 @@ __global__ void __launch_bounds__(ZCOL_THREADS) k_grid_z_fft(KArgs ka, int which
   }
 }
 
+// ---------------------------------------------------------------------------
+// Grid transform along one axis, lengths N = A B C with short DFTs (grid_factors; B = 1 where two
+// are enough).  With M = B C, W_n = exp(s 2 pi i / n):
+//   step 1, group g < M:      Y[M k1 + g] = W_N^(g k1) sum_{n1 < A} x[M n1 + g] W_A^(n1 k1)
+//   step 2, (k1 < A, h < C):  Z[M k1 + C k2 + h] = W_M^(h k2) sum_{n2 < B} Y[M k1 + C n2 + h] W_B^(n2 k2)
+//   step 3, (k1 < A, k2 < B): X[k1 + A (k2 + B k3)] = sum_{h < C} Z[M k1 + C k2 + h] W_C^(h k3)
+// CTA = (problem, GA_LINES lines): step 1 reads global memory, step 3 writes it, the lines stay in
+// shared memory in between.  Between the axes of a float-float transform the grid holds the float
+// pairs themselves: converting FP64 takes four FP64-rate instructions a value (MODE, a template
+// parameter so that no conversion is executed and then not used).
+// Bound by latency and instruction fetch (about 250 FP32 instructions a point and axis in
+// float-float, straight-line code per DFT), so short DFTs, whose code stays in the instruction
+// cache, few registers and many small CTAs: 648 for one axis of a 72^3 grid.  A whole transform,
+// against the kernels below (one CTA a plane, then blocks of z lines, general radix loops):
+// 72^3 123 -> 69 us, a 24-atom layer 87 -> 49, 8 atoms 51 -> 31, 64 structures in a batch
+// 537 -> 427 (FP64: the layer 85 -> 50, 8 atoms 43 -> 27).  Two steps with DFTs up to 16 took
+// 118 us and 760 us for the first and the batch, 13 % of the issue slots used; 16 lines a CTA
+// 74 and 354; 64 threads 76 and 403; 64 registers 69 and 411.
+// ---------------------------------------------------------------------------
+constexpr int GA_LINES = 8;      // lines per CTA
+constexpr int GA_THREADS = 128;
+enum { GA_FIRST = 0, GA_FIRST_REAL = 1, GA_MIDDLE = 2, GA_LAST = 3 };
+
+template <typename T, int MODE>
+struct GridAxis {
+  cplx<typename Work<T>::S>* g;  // the grid
+  const double* real;            // GA_FIRST_REAL: a real source instead (imaginary part 0)
+  cplx<T>* tile;                 // [GA_LINES][stride]
+  const cplx<T>* roots;          // exp(-2 pi i t / N)
+  T sg;
+  int a, b, c, stride, estep;
+  bool fwd;
+  __device__ __forceinline__ cplx<T> load(size_t i) const {
+    using S = typename Work<T>::S;
+    if constexpr (MODE == GA_FIRST_REAL) return Work<T>::in(mk((S)real[i], (S)0));
+    else if constexpr (MODE == GA_FIRST) return Work<T>::in(g[i]);
+    else return *reinterpret_cast<const cplx<T>*>(g + i);
+  }
+  __device__ __forceinline__ void store(size_t i, cplx<T> v) const {
+    if constexpr (MODE == GA_LAST) g[i] = Work<T>::out(v);
+    else *reinterpret_cast<cplx<T>*>(g + i) = v;
+  }
+  __device__ __forceinline__ cplx<T> twiddle(cplx<T> v, int t) const {
+    const cplx<T> w = roots[t];
+    return v * (fwd ? w : conj(w));
+  }
+};
+
+template <int R, typename T, int MODE>
+__device__ __forceinline__ void axis_step1(const GridAxis<T, MODE>& x, size_t base, int l, int g) {
+  const int m = x.b * x.c;
+  cplx<T> v[R];
+#pragma unroll
+  for (int k = 0; k < R; ++k) v[k] = x.load(base + (size_t)(m * k + g) * x.estep);
+  if constexpr (R > 1) Bfly<T, R>::run(v, x.sg, x.roots, m);
+  cplx<T>* o = x.tile + l * x.stride + g;
+#pragma unroll
+  for (int k = 0; k < R; ++k) o[m * k] = k > 0 && g > 0 ? x.twiddle(v[k], g * k) : v[k];
+}
+template <int R, typename T, int MODE>
+__device__ __forceinline__ void axis_step2(const GridAxis<T, MODE>& x, int l, int k1, int h) {
+  cplx<T>* o = x.tile + l * x.stride + x.b * x.c * k1 + h;
+  cplx<T> v[R];
+#pragma unroll
+  for (int k = 0; k < R; ++k) v[k] = o[x.c * k];
+  if constexpr (R > 1) Bfly<T, R>::run(v, x.sg, x.roots, x.a * x.c);
+#pragma unroll
+  for (int k = 0; k < R; ++k) o[x.c * k] = k > 0 && h > 0 ? x.twiddle(v[k], x.a * h * k) : v[k];
+}
+template <int R, typename T, int MODE>
+__device__ __forceinline__ void axis_step3(const GridAxis<T, MODE>& x, size_t base, int l, int k1, int k2) {
+  cplx<T> v[R];
+  const cplx<T>* in = x.tile + l * x.stride + R * (x.b * k1 + k2);
+#pragma unroll
+  for (int k = 0; k < R; ++k) v[k] = in[k];
+  if constexpr (R > 1) Bfly<T, R>::run(v, x.sg, x.roots, x.a * x.b);
+#pragma unroll
+  for (int k = 0; k < R; ++k) x.store(base + (size_t)(k1 + x.a * (k2 + x.b * k)) * x.estep, v[k]);
+}
+
+#define SGO_GRID_RADIX(r, F, ...)    \
+  switch (r) {                       \
+    case 1: F<1>(__VA_ARGS__); break; \
+    case 2: F<2>(__VA_ARGS__); break; \
+    case 3: F<3>(__VA_ARGS__); break; \
+    case 4: F<4>(__VA_ARGS__); break; \
+    case 5: F<5>(__VA_ARGS__); break; \
+    case 6: F<6>(__VA_ARGS__); break; \
+    case 8: F<8>(__VA_ARGS__); break; \
+    case 9: F<9>(__VA_ARGS__); break; \
+  }
+
+// axis 0: x, 1: y (contiguous), 2: z
+template <typename T, int MODE>
+__global__ void __launch_bounds__(GA_THREADS, 7) k_grid_axis(KArgs ka, int which, int sign, int axis) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  const int p = locate(ka.start, ka.nprob, blockIdx.x);
+  if (!ka.active[p]) return;
+  const Prob& P = ka.probs[p];
+  const int n1 = P.n1, n2 = P.n2, n12 = n1 * n2;
+  const int n = axis == 0 ? n1 : axis == 1 ? n2 : P.n3, nl = P.ngrid / n;
+  GridAxis<T, MODE> x;
+  grid_factors(n, &x.a, &x.b, &x.c);
+  x.g = grid_of<T>(P, which);
+  x.real = P.rho_out;
+  x.stride = n | 1;
+  x.tile = reinterpret_cast<cplx<T>*>(smem_raw);
+  cplx<T>* roots = x.tile + GA_LINES * x.stride;
+  x.roots = roots;
+  x.sg = sign < 0 ? T(-1) : T(1);
+  x.fwd = sign < 0;
+  x.estep = axis == 0 ? n2 : axis == 1 ? 1 : n12;
+  load_roots<T>(roots, P, axis == 0 ? 0 : axis == 1 ? n1 : n1 + n2, n);
+  __syncthreads();
+  const int l0 = (blockIdx.x - ka.start[p]) * GA_LINES;
+  // neighbouring threads on neighbouring addresses: along the line for y, across lines otherwise
+  auto split = [&](int t, int groups, int* l, int* grp) {
+    *l = axis == 1 ? t / groups : t % GA_LINES;
+    *grp = axis == 1 ? t - *l * groups : t / GA_LINES;
+    return l0 + *l < nl;
+  };
+  auto base = [&](int l) -> size_t {
+    const int id = l0 + l;
+    if (axis == 2) return id;
+    if (axis == 1) return (size_t)id * n2;
+    const int z = id / n2;
+    return (size_t)z * n12 + (id - z * n2);
+  };
+  int l, g;
+  const int m = x.b * x.c, ab = x.a * x.b, ac = x.a * x.c;
+  for (int t = threadIdx.x; t < GA_LINES * m; t += GA_THREADS)
+    if (split(t, m, &l, &g)) SGO_GRID_RADIX(x.a, axis_step1, x, base(l), l, g)
+  __syncthreads();
+  if (x.b > 1) {
+    for (int t = threadIdx.x; t < GA_LINES * ac; t += GA_THREADS)
+      if (split(t, ac, &l, &g)) SGO_GRID_RADIX(x.b, axis_step2, x, l, g / x.c, g % x.c)
+    __syncthreads();
+  }
+  // (consecutive groups k1 + A k2 on consecutive outputs)
+  for (int t = threadIdx.x; t < GA_LINES * ab; t += GA_THREADS)
+    if (split(t, ab, &l, &g)) SGO_GRID_RADIX(x.c, axis_step3, x, base(l), l, g % x.a, g / x.a)
+}
+
 // Line blocks of the grid transform for planes too large for one CTA: along x (axis 0:
 // length N1, element stride N2, lines (z, i2)) or y (axis 1: length N2, contiguous, lines
 // (z, i1)), QZ lines per CTA, loads and stores coalesced across the lines' fast index.
@@ -590,6 +733,21 @@ void launch_grid_line_fft(const Launch& L, int which, int sign, int axis) {
   size_t sm = (size_t)(2 * QZ + 1) * n * sizeof(cplx<T>);
   k_grid_line_fft<T><<<L.map.total, ZCOL_THREADS, sm, L.stream>>>(L.ka, which, sign, axis);
 }
+int grid_axis_ctas(int n1, int n2, int n3, int axis) {
+  const int n = axis == 0 ? n1 : axis == 1 ? n2 : n3;
+  return (n1 * n2 * n3 / n + GA_LINES - 1) / GA_LINES;
+}
+template <typename T>
+void launch_grid_axis(const Launch& L, int which, int sign, int axis, int step, bool real_src) {
+  if (!L.map.total) return;
+  const int n = axis == 0 ? L.max_n1 : axis == 1 ? L.max_n2 : L.max_n3;
+  const size_t sm = (size_t)(GA_LINES * (n | 1) + GA_LINES + n) * sizeof(cplx<T>);
+  auto* fn = step == 2 ? k_grid_axis<T, GA_LAST> : step == 1 ? k_grid_axis<T, GA_MIDDLE>
+             : real_src ? k_grid_axis<T, GA_FIRST_REAL> : k_grid_axis<T, GA_FIRST>;
+  fn<<<L.map.total, GA_THREADS, sm, L.stream>>>(L.ka, which, sign, axis);
+}
+template void launch_grid_axis<double>(const Launch&, int, int, int, int, bool);
+template void launch_grid_axis<ff>(const Launch&, int, int, int, int, bool);
 template <typename T>
 void launch_grid_plane_fft(const Launch& L, int which, int sign) {
   if (!L.map.total) return;
@@ -622,15 +780,20 @@ void fft_set_smem_limits(size_t bytes) {
   cudaFuncSetAttribute(k_grid_plane_fft<ff>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
   cudaFuncSetAttribute(k_grid_z_fft<ff>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
   cudaFuncSetAttribute(k_grid_line_fft<ff>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
-  cudaFuncSetAttribute(k_grid_plane_fft<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
-  cudaFuncSetAttribute(k_grid_z_fft<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
-  cudaFuncSetAttribute(k_grid_line_fft<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
   cudaFuncSetAttribute(k_big_y<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
   cudaFuncSetAttribute(k_big_y<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
   cudaFuncSetAttribute(k_big_x<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
   cudaFuncSetAttribute(k_big_x<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
   cudaFuncSetAttribute(k_big_density<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
   cudaFuncSetAttribute(k_big_density<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+  cudaFuncSetAttribute(k_grid_axis<double, GA_FIRST>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+  cudaFuncSetAttribute(k_grid_axis<double, GA_FIRST_REAL>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+  cudaFuncSetAttribute(k_grid_axis<double, GA_MIDDLE>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+  cudaFuncSetAttribute(k_grid_axis<double, GA_LAST>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+  cudaFuncSetAttribute(k_grid_axis<ff, GA_FIRST>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+  cudaFuncSetAttribute(k_grid_axis<ff, GA_FIRST_REAL>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+  cudaFuncSetAttribute(k_grid_axis<ff, GA_MIDDLE>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+  cudaFuncSetAttribute(k_grid_axis<ff, GA_LAST>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
   plane_vpsi_reg_set_smem_limits(bytes);
   plane_ms_set_smem_limits(bytes);
   zreg_set_smem_limits(bytes);
@@ -641,11 +804,8 @@ template void launch_wave_to_cols<float>(const Launch&, int);
 template void launch_wave_to_cols<double>(const Launch&, int);
 template void launch_cols_to_wave<float>(const Launch&, int, int);
 template void launch_cols_to_wave<double>(const Launch&, int, int);
-template void launch_grid_line_fft<float>(const Launch&, int, int, int);
 template void launch_grid_line_fft<double>(const Launch&, int, int, int);
-template void launch_grid_plane_fft<float>(const Launch&, int, int);
 template void launch_grid_plane_fft<double>(const Launch&, int, int);
-template void launch_grid_z_fft<float>(const Launch&, int, int);
 template void launch_grid_z_fft<double>(const Launch&, int, int);
 template void launch_grid_line_fft<ff>(const Launch&, int, int, int);
 template void launch_grid_plane_fft<ff>(const Launch&, int, int);

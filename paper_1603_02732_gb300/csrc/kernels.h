@@ -89,6 +89,34 @@ template <typename T> void launch_plane_density(const Launch& L, const double* o
 // same memory as single-precision complex)
 // T: float (FP32 grids), double (FP64), ff (float-float arithmetic on FP64 grids, ff.cuh)
 struct ff;
+// n = a b c with short DFTs for each (b = 1 where two of at most 6 are enough), the largest factor as
+// small as possible: every smooth length up to 216 that the transforms meet
+inline __host__ __device__ bool grid_factors(int n, int* a, int* b, int* c) {
+  const int r[8] = {1, 2, 3, 4, 5, 6, 8, 9};
+  for (int k = 0; k < 8; ++k)          // the largest factor, last
+    for (int j = 0; j <= k; ++j)       // two factors
+      if (k < 6 && r[j] * r[k] == n) {
+        *a = r[j];
+        *b = 1;
+        *c = r[k];
+        return true;
+      } else if (n % (r[j] * r[k]) == 0) {  // or three
+        const int q = n / (r[j] * r[k]);
+        for (int i = 1; i <= j; ++i)
+          if (r[i] == q) {
+            *a = r[i];
+            *b = r[j];
+            *c = r[k];
+            return true;
+          }
+      }
+  return false;
+}
+int grid_axis_ctas(int n1, int n2, int n3, int axis);
+// step 0, 1, 2: the first, second, third axis of a transform; real_src: the first one reads rho_out
+// (imaginary part 0) instead of the grid
+template <typename T> void launch_grid_axis(const Launch& L, int which, int sign, int axis, int step, bool real_src);
+// (grids with a length that has none: whole planes, z lines, or line blocks)
 template <typename T> void launch_grid_plane_fft(const Launch& L, int which, int sign);
 template <typename T> void launch_grid_z_fft(const Launch& L, int which, int sign);
 template <typename T> void launch_grid_line_fft(const Launch& L, int which, int sign, int axis);  // axis 0: x, 1: y

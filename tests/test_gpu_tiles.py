@@ -98,3 +98,20 @@ def test_density_sizes_mixed(sgo, grid, bands, ecut):
     rho /= abs(np.linalg.det(st.cell))
     got = ctx.density_of(psi, occ)
     assert np.abs(got - rho).max() < 2e-6 * rho.max()
+
+
+# every radix of the axis transforms in every step, odd and even lengths, lines that do not fill a
+# block, and a grid with a length that has no such form (250: the plane and line-block kernels)
+@pytest.mark.parametrize("grid", [(5, 9, 10), (27, 15, 16), (75, 81, 6), (96, 100, 8), (108, 10, 128), (135, 9, 144),
+                                  (10, 162, 9), (9, 10, 200), (64, 72, 45), (10, 250, 9)])
+@pytest.mark.parametrize("precision", ["fp64", "mixed"])
+def test_grid_transform_lengths(sgo, grid, precision):
+    """Both signs against NumPy: 1e-12 of the largest value (float-float keeps 44 bits, 6e-14, through
+    fewer than 16 sums a value)."""
+    st = dataclasses.replace(workloads.tiny(nat=1, ecut=0.6, kT=0.0, nbands=2), fft=grid)
+    ctx = sgo.Context(st, precision=precision, extra_bands=0)
+    rng = np.random.default_rng(6)
+    x = rng.normal(size=grid) + 1j * rng.normal(size=grid)
+    for sign in (-1, 1):
+        ref = np.fft.fftn(x) if sign < 0 else np.fft.ifftn(x) * x.size
+        assert np.abs(ctx.grid_fft(x, sign) - ref).max() < 1e-12 * np.abs(ref).max()
