@@ -20,6 +20,9 @@ LIB = os.path.join(HERE, "libsgo.so")
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 FLAGS = ["-std=c++17", "-O3", "-lineinfo", "-Xcompiler", "-fPIC", "-Xcompiler", "-fvisibility=hidden",
          "--expt-relaxed-constexpr", "-I", os.path.join(ROOT, "include")]
+# k_rr_td.cu writes its fused multiply-adds itself: a member's results must not depend on which
+# instantiation of the kernel its batch selects, and the compiler fuses them differently
+FILE_FLAGS = {"k_rr_td.cu": ["-fmad=false"]}
 SOURCES = ["k_fft.cu", "k_plane_vpsi.cu", "k_plane_ms.cu", "k_cols_reg.cu", "k_pair_reg.cu", "k_linalg.cu", "k_rr_td.cu", "k_grid.cu", "k_setup.cu", "engine.cu",
            "capi.cu", "noalloc.cu", "k_gemm_tc.cu", "relax.cpp", "de.cpp"]
 
@@ -36,7 +39,7 @@ def nvcc() -> str:
 
 def _compile(src: str) -> str:
     obj = os.path.join(BUILD, os.path.splitext(src)[0] + ".o")
-    cmd = [nvcc(), *ARCH, *FLAGS, "-c", os.path.join(CSRC, src), "-o", obj]
+    cmd = [nvcc(), *ARCH, *FLAGS, *FILE_FLAGS.get(src, []), "-c", os.path.join(CSRC, src), "-o", obj]
     r = subprocess.run(cmd, capture_output=True, text=True)
     if r.returncode != 0:
         raise RuntimeError(f"nvcc failed for {src}:\n{r.stderr}")

@@ -1004,7 +1004,7 @@ Engine::Engine(const std::vector<sgo_ctx*>& ctxs, cudaStream_t stream) : ctx_(ct
   }
   const sgo_opts& o0 = ctxs[0]->opts;
   wait_ns_ = o0.watchdog_ms > 0.0 ? (long long)(o0.watchdog_ms * 1e6) : 2000000000LL;
-  // subspace diagonalisation: one CTA per member up to rr_td_max bands (192 on the mixed path,
+  // subspace diagonalisation: k_rr_td.cu per member up to rr_td_max bands (192 on the mixed path,
   // 128 in FP64), beyond (or when asked for) one thread-block cluster per member (k_rr_cluster)
   // (the block Davidson steps diagonalise the 2 n_b block [X, W])
   davidson_ = o0.eigensolver == 1;

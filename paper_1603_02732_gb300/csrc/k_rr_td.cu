@@ -1,4 +1,4 @@
-// Rayleigh-Ritz of one CTA per problem (orthonormalisation + subspace diagonalisation of
+// Rayleigh-Ritz of one CTA or one cluster of CTAs per problem (orthonormalisation + subspace diagonalisation of
 // Algorithm 1): S = L L^T, C = L^-1 Hs L^-T, C = V diag(eps) V^T, Tm = L^-T V, so that X Tm is
 // orthonormal and diagonalises H in the subspace.  T = float on the mixed path, double on the
 // plain one.
@@ -29,10 +29,15 @@
 // lane j mod 32 (few warps with 8 to 16 rows each: the overhead of a step is paid per warp); the
 // Cholesky needs one barrier per RPW columns, the tridiagonalisation two per column, the
 // substitutions and the back transformation none (a warp owns whole columns).
-// Measured, mean per launch over an evaluation, Jacobi kernels before -> now: FP32 70 bands 299 ->
-// 258 us, 91 bands 553 -> 335 us, 86 bands in 64 members 484 -> 294 us, 169 bands (an 8-CTA cluster
-// before) 3565 -> 1403 us, 10 bands 31 -> 39 us; FP64 24 bands 317 -> 289 us, 70 bands 2500 -> 1883
-// us, up to 80 bands in six members 3550 -> 2115 us.
+// In a cluster the rows are dealt to the CTAs' warps in order; a CTA has its own copy of L, the
+// reflectors and the vectors, into which their owner writes (Team::put), and takes the roots, merge
+// columns and vectors of its own rows.  The leaves and the sorting are done by every CTA alike.
+// Results do not depend on the number of CTAs or warps (the sums over lanes have one shape, fused
+// multiply-adds are written out).
+// Measured, mean per launch over an evaluation, Jacobi kernels -> one CTA -> now: FP32 70 bands 299 ->
+// 256 us (one CTA), 91 bands 553 -> 335 us (one CTA), 169 bands (an 8-CTA cluster before) 3565 -> 1403
+// -> 990 us, 10 bands 31 -> 38 us (one CTA); FP64 24 bands 317 -> 288 -> 205 us, 70 bands 2500 ->
+// 1883 -> 762 us, up to 80 bands in six members 3550 -> 2118 -> 818 us.
 #include "kernels.h"
 
 namespace sgo {
@@ -95,7 +100,7 @@ __device__ __forceinline__ double td_rsqrt(double x) {  // two Newton steps on t
 template <typename T>
 __device__ __forceinline__ T wsum(T v) {
 #pragma unroll
-  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+  for (int o = 16; o > 0; o >>= 1) v = v + __shfl_xor_sync(0xffffffffu, v, o);
   return v;
 }
 
@@ -124,7 +129,7 @@ __device__ __forceinline__ T fold_sums(const T (&in)[R], int lane) {
       }
   }
 #pragma unroll
-  for (; o > 0; o >>= 1) v[0] += __shfl_xor_sync(0xffffffffu, v[0], o);
+  for (; o > 0; o >>= 1) v[0] = v[0] + __shfl_xor_sync(0xffffffffu, v[0], o);
   return v[0];
 }
 constexpr int log2i(int w) { return w <= 1 ? 0 : 1 + log2i(w / 2); }
@@ -135,7 +140,7 @@ __host__ __device__ constexpr int fold_shift() { return log2i(W) - fold_bits<R>(
 // sum over the g lanes of a root
 template <typename T>
 __device__ __forceinline__ T gsum(T v, int g) {
-  for (int o = g >> 1; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+  for (int o = g >> 1; o > 0; o >>= 1) v = v + __shfl_xor_sync(0xffffffffu, v, o);
   return v;
 }
 
@@ -145,9 +150,9 @@ __device__ __forceinline__ T gsum(T v, int g) {
 template <typename T>
 __device__ __forceinline__ T two_pole_root(T c, T s, T S, T w, bool right) {
   if (S == T(0)) return s * td_rcp(c);
-  const T b = right ? s + S - c * w : c * w + s + S;
+  const T b = right ? fma(-c, w, s + S) : fma(c, w, s) + S;
   const T d = right ? -S * w : s * w;
-  const T disc = b * b - T(4) * c * d;
+  const T disc = fma(b, b, -(T(4) * c * d));
   const T r = sqrt(disc > T(0) ? disc : T(0));
   const T num = b >= T(0) ? T(2) * d : b - r, den = b >= T(0) ? b + r : T(2) * c;
   return num * td_rcp(den);
@@ -198,7 +203,8 @@ __device__ __forceinline__ bool secular(const PO& pole, const F* zw, int lo, int
         done = true;
       } else {
         const F dl = pl - x, dr = ql - x;
-        const F c = f - dl * dp - (last ? F(0) : dr * dq);
+        F c = fma(-dl, dp, f);
+        if (!last) c = fma(-dr, dq, c);
         F y = two_pole_root(c, dl * dl * dp, last ? F(0) : dr * dr * dq, w, right);
         const bool in = y > a && y < b;
         if (!in) y = a == F(0) ? b * F(0.01) : b == F(0) ? a * F(0.01) : F(0.5) * (a + b);
@@ -242,36 +248,36 @@ __device__ __forceinline__ void td_leaf(T (&d)[M], T (&e)[M], T (&z)[M], int m0,
       for (int i = 0; i < M; ++i)
         if (i == m) dm = d[i];
       T g = (dl1 - dl) * td_rcp(T(2) * el);
-      g = dm - dl + el * td_rcp(g + copysign(sqrt(g * g + T(1)), g));
+      g = fma(el, td_rcp(g + copysign(sqrt(fma(g, g, T(1))), g)), dm - dl);
       T s = T(1), c = T(1), q = T(0);
       bool cut = false;  // an exact zero ended the sweep early
 #pragma unroll
       for (int i = M - 2; i >= 0; --i)
         if (i < m && i >= l && !cut) {
-          const T f = s * e[i], b = c * e[i], h = f * f + g * g;
+          const T f = s * e[i], b = c * e[i], h = fma(f, f, g * g);
           const T ir = td_rsqrt(h);
           if (h > TdNum<T>::floor) {
             e[i + 1] = h * ir;
             s = f * ir;
             c = g * ir;
             g = d[i + 1] - q;
-            const T r = (d[i] - g) * s + T(2) * c * b;
+            const T r = fma(d[i] - g, s, T(2) * c * b);
             q = s * r;
             d[i + 1] = g + q;
-            g = c * r - b;
+            g = fma(c, r, -b);
             const T zi = z[i + 1];
-            z[i + 1] = s * z[i] + c * zi;
-            z[i] = c * z[i] - s * zi;
+            z[i + 1] = fma(s, z[i], c * zi);
+            z[i] = fma(c, z[i], -(s * zi));
           } else {
             e[i + 1] = T(0);
-            d[i + 1] -= q;
+            d[i + 1] = d[i + 1] - q;
             cut = true;
           }
         }
 #pragma unroll
       for (int i = 0; i < M; ++i) {
         if (i == l && !cut) {
-          d[i] -= q;
+          d[i] = d[i] - q;
           e[i] = g;
         }
         if (i == m) e[i] = T(0);
@@ -280,9 +286,58 @@ __device__ __forceinline__ void td_leaf(T (&d)[M], T (&e)[M], T (&z)[M], int m0,
   }
 }
 
-__device__ __forceinline__ void bar_matrix(int threads) {
-  asm volatile("bar.sync 1, %0;" ::"r"(threads) : "memory");
-}
+// The CTAs of a problem: writes to every CTA's copy of a shared variable, barriers over all of them
+// (CL = 1: the CTA's own copy, the matrix warps).
+template <int CL>
+struct Team {
+  unsigned off[CL];  // from a shared address to CTA r's copy of it
+  int rank;
+  __device__ __forceinline__ void init(void* smem) {
+    rank = 0;
+    off[0] = 0;
+    if constexpr (CL > 1) {
+      asm("mov.u32 %0, %%cluster_ctarank;" : "=r"(rank));
+      const unsigned a = (unsigned)__cvta_generic_to_shared(smem);
+#pragma unroll
+      for (int r = 0; r < CL; ++r) {
+        unsigned b;
+        asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(b) : "r"(a), "r"(r));
+        off[r] = b - a;
+      }
+    }
+  }
+  static __device__ __forceinline__ void st(unsigned a, float v) {
+    asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(a), "f"(v) : "memory");
+  }
+  static __device__ __forceinline__ void st(unsigned a, double v) {
+    asm volatile("st.shared::cluster.f64 [%0], %1;" ::"r"(a), "d"(v) : "memory");
+  }
+  static __device__ __forceinline__ void st(unsigned a, int v) {
+    asm volatile("st.shared::cluster.s32 [%0], %1;" ::"r"(a), "r"(v) : "memory");
+  }
+  template <typename X>
+  __device__ __forceinline__ void put(X* p, X v) const {  // *p = v in every CTA
+    if constexpr (CL == 1) {
+      *p = v;
+    } else {
+      const unsigned a = (unsigned)__cvta_generic_to_shared(p);
+#pragma unroll
+      for (int r = 0; r < CL; ++r) st(a + off[r], v);
+    }
+  }
+  __device__ __forceinline__ void barrier() const {  // all threads of all CTAs
+    if constexpr (CL == 1) {
+      __syncthreads();
+    } else {
+      asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+      asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+    }
+  }
+  __device__ __forceinline__ void matrix_barrier(int threads) const {  // the matrix warps of all CTAs
+    if constexpr (CL == 1) asm volatile("bar.sync 1, %0;" ::"r"(threads) : "memory");
+    else barrier();
+  }
+};
 
 // R consecutive shared values (aligned to R values or 16 bytes) as vector loads
 template <typename T, int R>
@@ -317,19 +372,24 @@ __host__ __device__ inline size_t td_vec_bytes(int n, size_t ts) {
 // all: L, the reflectors, U and Z in shared memory; else L, the reflectors and the transposes go
 // through the member's global scratch (3 n^2 elements) and share U's place in turn.  FP32 keeps C
 // and the factors of the correction's products in the scratch too (rr_td_scratch_bytes).
-template <typename T, int NR, int MW, int NW>
+template <typename T, int NR, int MW, int NW, int CL>
 __global__ void __launch_bounds__(32 * NW, 1)
     k_rr_td(KArgs ka, T* gscratch, size_t gstride, int all, int blk) {
-  constexpr int RPW = 32 * NR / MW, NT = 32 * NW, MT = 32 * MW;
+  static_assert(CL == 1 || MW == NW, "in a cluster every warp is a matrix warp");
+  constexpr int RPW = 32 * NR / (MW * CL), NT = 32 * NW, MT = 32 * MW;
+  static_assert(RPW * MW * CL == 32 * NR && RPW % 2 == 0, "whole vectors of rows");
   using N = TdNum<T>;
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  const int p = blockIdx.x;
+  const int p = blockIdx.x / CL;
   if (!ka.active[p]) return;
   const Prob& P = ka.probs[p];
+  Team<CL> team;
+  team.init(smem_raw);
   const int n = blk * P.nb, ns = n | 1, zs = td_zs(n), us = td_us(n), vn = td_vn(n);
   const double* Sin = blk == 2 ? P.S2 : P.S;
   const double* Hin = blk == 2 ? P.H2 : P.Hs;
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int tid = threadIdx.x, lane = tid & 31, lwarp = tid >> 5;
+  const int warp = team.rank * MW + lwarp;  // (a matrix warp's number)
   // vectors
   T* dk = reinterpret_cast<T*>(smem_raw);  // 1 / (1 + d_k); 0 marks a left-out direction
   T* vbuf = dk + vn;                       // [2][vn] Householder vectors in turn
@@ -360,12 +420,13 @@ __global__ void __launch_bounds__(32 * NW, 1)
   T* gC = all ? gW : gV + (size_t)n * n;                               // (FP32) C
   T* gS = gW + ((all ? 1 : 4) * (size_t)n * n + 3) / 4 * 4;            // (FP32) [MW][n][RPW], 16-byte aligned
   if (tid < 16) flags[tid] = 0;
-  __syncthreads();
+  team.barrier();
 
   // row i = i0 + a, column (or, for column-owning steps, row) j = lane + 32 c
   const int i0 = warp * RPW;
+  const int c0 = team.rank * MW * RPW, c1 = CL == 1 ? n : min(n, c0 + MW * RPW);  // the CTA's rows
   T A[RPW][NR];
-  if (warp < MW) {
+  if (CL > 1 || lwarp < MW) {
     // ---- 1. Cholesky: a warp factors its RPW columns, one barrier, the others update ----
 #pragma unroll
     for (int a = 0; a < RPW; ++a)
@@ -401,15 +462,15 @@ __global__ void __launch_bounds__(32 * NW, 1)
           const bool bad = !drop && !(x > T(-0.999));
           const T inv = drop ? T(0) : td_rsqrt(T(1) + (bad ? T(-0.999) : x));
           if (lane == 0) {
-            dk[k] = inv;
-            if (bad) flags[0] = 1;
-            if (drop) flags[1] = 1;
+            team.put(&dk[k], inv);
+            if (bad) team.put(&flags[0], 1);
+            if (drop) team.put(&flags[1], 1);
           }
 #pragma unroll
           for (int c = 0; c < NR; ++c) {
             const int j = lane + 32 * c;
             row[c] = j > k && j < n ? row[c] * inv : T(0);
-            if (j < n) Lb[(size_t)k * ns + j] = row[c];
+            if (j < n) team.put(&Lb[(size_t)k * ns + j], row[c]);
           }
           __syncwarp();
 #pragma unroll
@@ -417,11 +478,11 @@ __global__ void __launch_bounds__(32 * NW, 1)
             if (b > a) {
               const T li = i0 + b < n ? Lb[(size_t)k * ns + i0 + b] : T(0);
 #pragma unroll
-              for (int c = 0; c < NR; ++c) A[b][c] -= li * row[c];
+              for (int c = 0; c < NR; ++c) A[b][c] = fma(-li, row[c], A[b][c]);
             }
         }
       }
-      bar_matrix(MT);
+      team.matrix_barrier(MT);
       if (warp > pw && i0 < n) {
         for (int k = pw * RPW; k < (pw + 1) * RPW; ++k) {
           T lj[NR];
@@ -432,7 +493,7 @@ __global__ void __launch_bounds__(32 * NW, 1)
             const T li = i0 + a < n ? Lb[(size_t)k * ns + i0 + a] : T(0);
 #pragma unroll
             for (int c = 0; c < NR; ++c)
-              if (32 * c + 31 >= i0) A[a][c] -= li * lj[c];
+              if (32 * c + 31 >= i0) A[a][c] = fma(-li, lj[c], A[a][c]);
           }
         }
       }
@@ -457,7 +518,7 @@ __global__ void __launch_bounds__(32 * NW, 1)
 #pragma unroll
           for (int c = ck; c < NR; ++c)
 #pragma unroll
-            for (int a = 0; a < RPW; ++a) X[a][c] -= l[c] * x[a];
+            for (int a = 0; a < RPW; ++a) X[a][c] = fma(-l[c], x[a], X[a][c]);
         }
       }
     };
@@ -475,26 +536,38 @@ __global__ void __launch_bounds__(32 * NW, 1)
     // transpose through U's place (or the global scratch, where L occupies it)
     T* const Tb = all ? Ub : gW;
     const int ts = all ? ns : n;
-    auto put = [&]() {  // Tb[i][j] = A
+    auto put = [&]() {  // Tb[i][j] = A (in a cluster, for the CTA of row j)
 #pragma unroll
       for (int a = 0; a < RPW; ++a)
 #pragma unroll
         for (int c = 0; c < NR; ++c)
-          if (i0 + a < n && lane + 32 * c < n) Tb[(size_t)(i0 + a) * ts + lane + 32 * c] = A[a][c];
+          if (i0 + a < n && lane + 32 * c < n) {
+            T* const q = &Tb[(size_t)(i0 + a) * ts + lane + 32 * c];
+            if (CL == 1 || !all) {
+              *q = A[a][c];
+            } else {
+              const int to = (lane + 32 * c) / (MW * RPW);
+              unsigned o = 0;
+#pragma unroll
+              for (int r = 0; r < CL; ++r)
+                if (r == to) o = team.off[r];
+              Team<CL>::st((unsigned)__cvta_generic_to_shared(q) + o, A[a][c]);
+            }
+          }
     };
     put();
-    bar_matrix(MT);
+    team.matrix_barrier(MT);
 #pragma unroll
     for (int a = 0; a < RPW; ++a)
 #pragma unroll
       for (int c = 0; c < NR; ++c)
         A[a][c] = i0 + a < n && lane + 32 * c < n ? Tb[(size_t)(lane + 32 * c) * ts + i0 + a] : T(0);
     if (i0 < n) forward(A);
-    bar_matrix(MT);
+    team.matrix_barrier(MT);
     put();
     if (!all)  // L is needed again at the end; its place is U's
-      for (int e = tid; e < n * n; e += MT) gL[e] = Lb[(size_t)(e / n) * ns + e % n];
-    bar_matrix(MT);
+      for (int e = team.rank * MT + tid; e < n * n; e += CL * MT) gL[e] = Lb[(size_t)(e / n) * ns + e % n];
+    team.matrix_barrier(MT);
     T rs = T(0);  // largest row sum of |C|
 #pragma unroll
     for (int a = 0; a < RPW; ++a) {
@@ -507,9 +580,9 @@ __global__ void __launch_bounds__(32 * NW, 1)
       if (flags[1]) rs = fmax(rs, wsum(s));
     }
     if (flags[1]) {  // (blk = 2) left-out directions above the spectrum
-      if (lane == 0) red[warp] = rs;
-      bar_matrix(MT);
-      for (int w = 0; w < MW; ++w) rs = fmax(rs, red[w]);
+      if (lane == 0) team.put(&red[warp], rs);
+      team.matrix_barrier(MT);
+      for (int w = 0; w < MW * CL; ++w) rs = fmax(rs, red[w]);
 #pragma unroll
       for (int a = 0; a < RPW; ++a)
 #pragma unroll
@@ -544,20 +617,20 @@ __global__ void __launch_bounds__(32 * NW, 1)
 #pragma unroll
         for (int c = 0; c < NR; ++c) {
           if (lane + 32 * c <= k + 1) x[c] = T(0);
-          sg += x[c] * x[c];
+          sg = fma(x[c], x[c], sg);
         }
         sg = wsum(sg);
         T beta = x1, f = T(0), tk = T(0);
         if (sg > T(0)) {
-          const T s2 = x1 * x1 + sg, r = td_rsqrt(s2), m = s2 * r;  // |x| = m
+          const T s2 = fma(x1, x1, sg), r = td_rsqrt(s2), m = s2 * r;  // |x| = m
           beta = x1 > T(0) ? -m : m;
           f = td_rcp(x1 - beta);
-          tk = T(1) + fabs(x1) * r;
+          tk = fma(fabs(x1), r, T(1));
         }
-        if (lane == (k & 31)) dg[k] = dd;
+        if (lane == (k & 31)) team.put(&dg[k], dd);
         if (lane == 0) {
-          eo[k] = beta;
-          tau[k] = tk;
+          team.put(&eo[k], beta);
+          team.put(&tau[k], tk);
         }
         T* vd = all ? Vb + (size_t)k * ns : gV + (size_t)k * n;
 #pragma unroll
@@ -565,12 +638,13 @@ __global__ void __launch_bounds__(32 * NW, 1)
           const int j = lane + 32 * c;
           const T vj = j == k + 1 ? T(1) : x[c] * f;
           if (j < n) {
-            v[j] = vj;
-            vd[j] = vj;
+            team.put(&v[j], vj);
+            if (all) team.put(&vd[j], vj);
+            else vd[j] = vj;
           }
         }
       }
-      bar_matrix(MT);
+      team.matrix_barrier(MT);
       const T tk = tau[k];
       if (tk == T(0)) continue;  // (uniform) nothing to eliminate
       const bool busy = i0 + RPW - 1 > k && i0 < n;
@@ -585,25 +659,25 @@ __global__ void __launch_bounds__(32 * NW, 1)
         for (int c = 0; c < NR; ++c)
           if (32 * c + 31 > k)
 #pragma unroll
-            for (int a = 0; a < RPW; ++a) q[a] += A[a][c] * vj[c];
+            for (int a = 0; a < RPW; ++a) q[a] = fma(A[a][c], vj[c], q[a]);
         const T s = fold_sums<T, RPW, 32>(q, lane);
         constexpr int S = fold_shift<RPW, 32>();
         const int a = lane >> S;
-        if ((lane & ((1 << S) - 1)) == 0 && a < RPW && i0 + a < n) pv[i0 + a] = s;
+        if ((lane & ((1 << S) - 1)) == 0 && a < RPW && i0 + a < n) team.put(&pv[i0 + a], s);
       }
-      bar_matrix(MT);
+      team.matrix_barrier(MT);
       if (busy) {
         T pj[NR], kk = T(0);
 #pragma unroll
         for (int c = 0; c < NR; ++c) {
           const int j = lane + 32 * c;
           pj[c] = j > k && j < n ? pv[j] : T(0);
-          kk += pj[c] * vj[c];
+          kk = fma(pj[c], vj[c], kk);
         }
         kk = T(0.5) * tk * wsum(kk);
 #pragma unroll
         for (int c = 0; c < NR; ++c) {
-          pj[c] = tk * (pj[c] - kk * vj[c]);  // w_j
+          pj[c] = tk * fma(-kk, vj[c], pj[c]);  // w_j
           const int j = lane + 32 * c;
           if (j >= i0 && j < i0 + RPW && j < n) wv[j] = pj[c];
         }
@@ -625,13 +699,14 @@ __global__ void __launch_bounds__(32 * NW, 1)
       for (int c = 0; c < NR; ++c) {
         const int i = i0 + a, j = lane + 32 * c;
         if (i < n && i + 2 >= n && j < n) {
-          if (i == j) dg[i] = A[a][c];
-          if (i == n - 2 && j == n - 1) eo[i] = A[a][c];
+          if (i == j) team.put(&dg[i], A[a][c]);
+          if (i == n - 2 && j == n - 1) team.put(&eo[i], A[a][c]);
         }
       }
   }
-  __syncthreads();
-  // ---- 4. divide and conquer ----
+  team.barrier();
+  // ---- 4. divide and conquer (in a cluster, the leaves, sorting and poles in every CTA alike; a CTA
+  // takes the roots, weights and vectors of its own rows) ----
   constexpr int TD_LEAF = td_leaf_rows<T>();
   // blocks: at shift sh, block q holds the indices (q n) >> sh .. ((q + 1) n) >> sh.  The leaves are
   // the blocks of at most TD_LEAF rows, torn apart at their ends (d -= |e| on either side of a
@@ -644,7 +719,7 @@ __global__ void __launch_bounds__(32 * NW, 1)
     }
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) nm = fmax(nm, __shfl_xor_sync(0xffffffffu, nm, o));
-    if (lane == 0) red[warp] = nm;
+    if (lane == 0) red[lwarp] = nm;
   }
   __syncthreads();
   T norm = T(0);
@@ -652,8 +727,8 @@ __global__ void __launch_bounds__(32 * NW, 1)
   int lev = 0;  // merge levels
   while (((n + (1 << lev) - 1) >> lev) > TD_LEAF) ++lev;
   const T gap = N::eps * norm;
-  if (tid < (TD_LEAF << lev)) {  // TD_LEAF lanes per leaf
-    const int q = tid / TD_LEAF, r = tid % TD_LEAF;
+  for (int t = tid; t < (TD_LEAF << lev); t += NT) {  // TD_LEAF lanes per leaf
+    const int q = t / TD_LEAF, r = t % TD_LEAF;
     const int lo = (q * n) >> lev, hi = ((q + 1) * n) >> lev, m0 = hi - lo;
     T d[TD_LEAF], e[TD_LEAF], z[TD_LEAF];
 #pragma unroll
@@ -680,7 +755,7 @@ __global__ void __launch_bounds__(32 * NW, 1)
   __syncthreads();
   for (int i = tid; i < n; i += NT) dg[i] = nd[i];
   // the merged vectors: A[a][c] = component lane + 32 c of vector i0 + a
-  if (warp < MW)
+  if (CL > 1 || lwarp < MW)
 #pragma unroll
     for (int a = 0; a < RPW; ++a)
 #pragma unroll
@@ -690,8 +765,8 @@ __global__ void __launch_bounds__(32 * NW, 1)
     const int sh = lev - l - 1;
     const int g = td_lanes<T>((n + (1 << sh) - 1) >> sh, n);  // lanes per root
     const int sub = tid & (g - 1), GR = NT / g, root0 = tid / g;
-    const int slots = (n + GR - 1) / GR;
-    __syncthreads();
+    const int slots = (c1 - c0 + GR - 1) / GR;
+    team.barrier();
     // sort the poles of the two halves together
     for (int i = tid; i < n; i += NT) {
       const int q = (((i + 1) << sh) - 1) / n;  // the block of index i at this level
@@ -723,7 +798,19 @@ __global__ void __launch_bounds__(32 * NW, 1)
     __syncthreads();
     for (int i = tid; i < n; i += NT)
       if (i > (bk[i] & 1023) && !(ds[i] - ds[i - 1] >= gap)) flags[2] = 1;
-    for (int e = tid; e < n * us / (16 / (int)sizeof(T)); e += NT) reinterpret_cast<float4*>(Ub)[e] = make_float4(0.f, 0.f, 0.f, 0.f);
+    if constexpr (CL == 1) {
+      for (int e = tid; e < n * us / (16 / (int)sizeof(T)); e += NT) reinterpret_cast<float4*>(Ub)[e] = make_float4(0.f, 0.f, 0.f, 0.f);
+    } else {  // the CTA's own columns
+      constexpr int V = RPW % (16 / (int)sizeof(T)) ? 1 : 16 / (int)sizeof(T), CW = MW * RPW / V;
+      for (int e = tid; e < n * CW; e += NT) {
+        const int j = c0 + e % CW * V;
+        if (j < us) {
+          T* const q = &Ub[(size_t)(e / CW) * us + j];
+          if constexpr (V > 1) *reinterpret_cast<float4*>(q) = make_float4(0.f, 0.f, 0.f, 0.f);
+          else *q = T(0);
+        }
+      }
+    }
     __syncthreads();
     if (flags[2]) {  // (few or none) poles closer than rounding: one thread per block moves them apart
       for (int i = tid; i < n; i += NT) {
@@ -744,8 +831,8 @@ __global__ void __launch_bounds__(32 * NW, 1)
     }
     // roots
     for (int sl = 0; sl < slots; ++sl) {
-      const int i = sl * GR + root0;
-      const bool live = i < n;
+      const int i = c0 + sl * GR + root0;
+      const bool live = i < c1;
       const int b3 = bk[live ? i : n - 1], lo = b3 & 1023, mid = (b3 >> 10) & 1023, hi = b3 >> 20;
       const T rho = mid > lo && mid < hi ? fabs(eo[mid - 1]) : T(0);
       const bool solve = live && rho > T(0.01) * gap;
@@ -767,12 +854,12 @@ __global__ void __launch_bounds__(32 * NW, 1)
       F fm = 0.f;
       if (solve) {
         const auto po = fpole(ii);
-        for (int j = lo + sub; j < hi; j += g) fm += zf[j] * td_rcp(po(j) - hf);
+        for (int j = lo + sub; j < hi; j += g) fm = fma(zf[j], td_rcp(po(j) - hf), fm);
       }
       fm = gsum(fm, g) + 1.f;
       const bool right = !last && fm < 0.f;
       const int K = right ? ii + 1 : ii;
-      F xf = two_pole_root(fm + 2.f * (zf[ii] - (last ? 0.f : zf[nx])) * td_rcp(wf), zf[ii], last ? 0.f : zf[nx], wf, right);
+      F xf = two_pole_root(fma(2.f * (zf[ii] - (last ? 0.f : zf[nx])), td_rcp(wf), fm), zf[ii], last ? 0.f : zf[nx], wf, right);
       const F af = right ? -wf : 0.f, bf = right ? 0.f : wf;
       if (!(xf > af && xf < bf)) xf = right ? -0.5f * hf : 0.5f * hf;
       bool done = secular(fpole(K), zf, lo, hi, ii, sub, g, wf, right, last, af, bf, !solve,
@@ -784,18 +871,18 @@ __global__ void __launch_bounds__(32 * NW, 1)
         done = secular(Poles<T, T>{ds, ds[K]}, zw, lo, hi, ii, sub, g, w, right, last, a, b, !solve, TD_ITERS, &x);
       }
       if (live && sub == 0) {
-        kx[i] = solve ? K : -1;  // -1: the halves stay as they are
-        mu[i] = solve ? x : T(0);
-        nd[i] = solve ? ds[K] + x : ds[i];
-        if (solve && !done) atomicAdd(&flags[3], 1);
+        team.put(&kx[i], solve ? K : -1);  // -1: the halves stay as they are
+        team.put(&mu[i], solve ? x : T(0));
+        team.put(&nd[i], solve ? ds[K] + x : ds[i]);
+        if (solve && !done) team.put(&flags[3], 1);
       }
     }
-    __syncthreads();
+    team.barrier();
     // z from the roots: z_j^2 ~ (lam_last - ds_j) prod_{i<j} (lam_i - ds_j) / (ds_i - ds_j)
     //                          prod_{j<=i<last} (lam_i - ds_j) / (ds_{i+1} - ds_j), every factor positive
     for (int sl = 0; sl < slots; ++sl) {
-      const int j = sl * GR + root0;
-      const bool live = j < n && kx[j < n ? j : 0] >= 0;
+      const int j = c0 + sl * GR + root0;
+      const bool live = j < c1 && kx[j < c1 ? j : 0] >= 0;
       T pr = T(1);
       if (live) {
         const int lo = bk[j] & 1023, hi = bk[j] >> 20;
@@ -808,14 +895,14 @@ __global__ void __launch_bounds__(32 * NW, 1)
       for (int o = g >> 1; o > 0; o >>= 1) pr *= __shfl_xor_sync(0xffffffffu, pr, o);
       if (live && sub == 0) {
         const T q = sqrt(fmax(fabs(pr), N::floor));
-        zv[j] = zh[j] < T(0) ? -q : q;
+        team.put(&zv[j], zh[j] < T(0) ? -q : q);
       }
     }
-    __syncthreads();
+    team.barrier();
     // U[original index of pole j - lo][i] = z_j / (ds_j - lam_i), normalised
     for (int sl = 0; sl < slots; ++sl) {
-      const int i = sl * GR + root0;
-      const bool live = i < n;
+      const int i = c0 + sl * GR + root0;
+      const bool live = i < c1;
       const int b3 = bk[live ? i : n - 1], lo = b3 & 1023, hi = b3 >> 20;
       const int K = live ? kx[i] : -1;
       T s = T(0);
@@ -824,7 +911,7 @@ __global__ void __launch_bounds__(32 * NW, 1)
         for (int j = lo + sub; j < hi; j += g) {
           const T v = zv[j] * td_rcp((ds[j] - base) - m);
           Ub[(size_t)perm[j] * us + i] = v;
-          s += v * v;
+          s = fma(v, v, s);
         }
       }
       s = gsum(s, g);
@@ -837,7 +924,7 @@ __global__ void __launch_bounds__(32 * NW, 1)
     }
     __syncthreads();
     // vectors: component r of vector i = sum over the poles j of r's half, U[j][i] Z[j][r]
-    if (warp < MW && i0 < n) {
+    if ((CL > 1 || lwarp < MW) && i0 < n) {
 #pragma unroll
       for (int a = 0; a < RPW; ++a)
 #pragma unroll
@@ -863,32 +950,32 @@ __global__ void __launch_bounds__(32 * NW, 1)
             if (32 * c < j1 && 32 * c + 31 >= j0) {
               const T zr = on[c] ? z[c][(j - j0) * zs] : T(0);
 #pragma unroll
-              for (int a = 0; a < RPW; ++a) A[a][c] += u[a] * zr;
+              for (int a = 0; a < RPW; ++a) A[a][c] = fma(u[a], zr, A[a][c]);
             }
         }
         jh = j1;
       }
     }
-    __syncthreads();
+    team.barrier();
     for (int i = tid; i < n; i += NT) dg[i] = nd[i];
-    if (sh > 0 && warp < MW) {
+    if (sh > 0 && (CL > 1 || lwarp < MW)) {
 #pragma unroll
       for (int a = 0; a < RPW; ++a) {
         const int b3 = bk[min(i0 + a, n - 1)], lo = b3 & 1023, hi = b3 >> 20;
 #pragma unroll
         for (int c = 0; c < NR; ++c) {
           const int r = lane + 32 * c;
-          if (i0 + a < n && r >= lo && r < hi) Zb[(size_t)(i0 + a) * zs + r - lo] = A[a][c];
+          if (i0 + a < n && r >= lo && r < hi) team.put(&Zb[(size_t)(i0 + a) * zs + r - lo], A[a][c]);
         }
       }
     }
   }
-  __syncthreads();
+  team.barrier();
   // ---- 5. reflectors from the last to the first, then back substitution with L^T ----
-  if (warp >= MW) return;  // (the matrix warps go on alone)
+  if (CL == 1 && lwarp >= MW) return;  // (the matrix warps go on alone)
   if (!all) {
     for (int e = tid; e < (n - 2) * n; e += MT) Ub[(size_t)(e / n) * ns + e % n] = gV[e];
-    bar_matrix(MT);
+    team.matrix_barrier(MT);
   }
   if (i0 < n)
     for (int k = n - 3; k >= 0; --k) {
@@ -903,7 +990,7 @@ __global__ void __launch_bounds__(32 * NW, 1)
         if (32 * c + 31 > k) {
           if (lane + 32 * c < n) v[c] = Vb[(size_t)k * ns + lane + 32 * c];
 #pragma unroll
-          for (int a = 0; a < RPW; ++a) q[a] += v[c] * A[a][c];
+          for (int a = 0; a < RPW; ++a) q[a] = fma(v[c], A[a][c], q[a]);
         }
       }
       const T s = fold_sums<T, RPW, 32>(q, lane) * tk;
@@ -913,7 +1000,7 @@ __global__ void __launch_bounds__(32 * NW, 1)
       for (int c = 0; c < NR; ++c)
         if (32 * c + 31 > k)
 #pragma unroll
-          for (int a = 0; a < RPW; ++a) A[a][c] -= q[a] * v[c];
+          for (int a = 0; a < RPW; ++a) A[a][c] = fma(-q[a], v[c], A[a][c]);
     }
   if constexpr (sizeof(T) == 4) {
     // Correction in FP32.  The steps so far leave |V^T C V - diag| and |V^T V - I| near 2e-6, a few
@@ -955,7 +1042,7 @@ __global__ void __launch_bounds__(32 * NW, 1)
           const int r = lane + 32 * c;
           const T x = X[k * sk + r * sr];  // (lanes r >= n read on into what follows; their sums are not used)
 #pragma unroll
-          for (int a = 0; a < RPW; ++a) A[a][c] += u[a] * x;
+          for (int a = 0; a < RPW; ++a) A[a][c] = fma(u[a], x, A[a][c]);
         }
       }
     };
@@ -964,28 +1051,28 @@ __global__ void __launch_bounds__(32 * NW, 1)
       for (int a = 0; a < RPW; ++a)
 #pragma unroll
         for (int c = 0; c < NR; ++c)
-          if (i0 + a < n && lane + 32 * c < n) Ub[(lane + 32 * c) * us + i0 + a] = A[a][c];
+          if (i0 + a < n && lane + 32 * c < n) team.put(&Ub[(lane + 32 * c) * us + i0 + a], A[a][c]);
     };
-    bar_matrix(MT);  // (the reflectors are done with)
+    team.matrix_barrier(MT);  // (the reflectors are done with)
     put_vt();
     if (all)
       for (int e = tid; e < n * n; e += MT) Vb[(size_t)(e / n) * ns + e % n] = gC[e];
-    bar_matrix(MT);
+    team.matrix_barrier(MT);
     if (i0 < n) {
       product(Ub + i0, us, Xc, cs, 1);  // C v_j
 #pragma unroll
       for (int a = 0; a < RPW; ++a)
 #pragma unroll
-        for (int c = 0; c < NR; ++c) A[a][c] -= dg[min(i0 + a, n - 1)] * vt(a, c);
+        for (int c = 0; c < NR; ++c) A[a][c] = fma(-dg[min(i0 + a, n - 1)], vt(a, c), A[a][c]);
       stage();
     }
     if (all) {
-      bar_matrix(MT);
+      team.matrix_barrier(MT);
 #pragma unroll
       for (int a = 0; a < RPW; ++a)
 #pragma unroll
         for (int c = 0; c < NR; ++c)
-          if (i0 + a < n && lane + 32 * c < n) Vb[(i0 + a) * ns + lane + 32 * c] = vt(a, c);
+          if (i0 + a < n && lane + 32 * c < n) team.put(&Vb[(i0 + a) * ns + lane + 32 * c], vt(a, c));
     }
     if (i0 < n) {
       product(mine, RPW, Ub, us, 1);  // v_i.r_j
@@ -995,13 +1082,13 @@ __global__ void __launch_bounds__(32 * NW, 1)
         for (int c = 0; c < NR; ++c) {
           const int i = lane + 32 * c, j = i0 + a;
           const T y = A[a][c], lj = dg[min(j, n - 1)], dl = lj - dg[min(i, n - 1)];
-          if (i == j && i < n) nd[i] = lj + y;
+          if (i == j && i < n) team.put(&nd[i], lj + y);
           // (closer pairs stay as they are: their quotients are rounding)
           A[a][c] = i < n && fabs(dl) > T(5e-4) * norm && fabs(y) <= T(2e-3) * fabs(dl) ? y * td_rcp(dl) : T(0);
         }
       stage();
     }
-    if (all) bar_matrix(MT);
+    if (all) team.matrix_barrier(MT);
     if (i0 < n) {
       product(mine, RPW, Xv, xk, xr);
 #pragma unroll
@@ -1009,15 +1096,15 @@ __global__ void __launch_bounds__(32 * NW, 1)
 #pragma unroll
         for (int c = 0; c < NR; ++c) A[a][c] += vt(a, c);
     }
-    bar_matrix(MT);
+    team.matrix_barrier(MT);
     put_vt();
     if (all)
 #pragma unroll
       for (int a = 0; a < RPW; ++a)
 #pragma unroll
         for (int c = 0; c < NR; ++c)
-          if (i0 + a < n && lane + 32 * c < n) Vb[(i0 + a) * ns + lane + 32 * c] = A[a][c];
-    bar_matrix(MT);
+          if (i0 + a < n && lane + 32 * c < n) team.put(&Vb[(i0 + a) * ns + lane + 32 * c], A[a][c]);
+    team.matrix_barrier(MT);
     if (i0 < n) {
       product(Ub + i0, us, Ub, us, 1);  // v_i.v_j
 #pragma unroll
@@ -1033,12 +1120,12 @@ __global__ void __launch_bounds__(32 * NW, 1)
         for (int c = 0; c < NR; ++c) A[a][c] += vt(a, c);
     }
     for (int i = tid; i < n; i += MT) dg[i] = nd[i];
-    bar_matrix(MT);
+    team.matrix_barrier(MT);
   }
   if (!all) {
-    bar_matrix(MT);
+    team.matrix_barrier(MT);
     for (int e = tid; e < n * n; e += MT) Ub[(size_t)(e / n) * ns + e % n] = gL[e];
-    bar_matrix(MT);
+    team.matrix_barrier(MT);
   }
   if (i0 < n) {
 #pragma unroll
@@ -1062,7 +1149,7 @@ __global__ void __launch_bounds__(32 * NW, 1)
         for (int c = 0; c < NR; ++c)
           if (c <= ck)
 #pragma unroll
-            for (int a = 0; a < RPW; ++a) A[a][c] -= lr[c] * x[a];
+            for (int a = 0; a < RPW; ++a) A[a][c] = fma(-lr[c], x[a], A[a][c]);
       }
     }
     // ascending: the corrected eigenvalues of close pairs may have changed places
@@ -1095,7 +1182,7 @@ __global__ void __launch_bounds__(32 * NW, 1)
       if (lane == 0) P.eps[i] = (double)dg[i0 + a];
     }
   }
-  if (tid == 0) {
+  if (warp == 0 && lane == 0) {
     if (flags[3]) P.scal[SC_RRCAP] += 1.0;
     if (flags[0]) P.status[0] = 1;
   }
@@ -1119,31 +1206,61 @@ size_t rr_td_scratch_bytes(int n, size_t tsize) {
   return (big + (tsize == 4 ? nn + 8 + (size_t)n * (n + 16) : 0)) * tsize;
 }
 
-template <typename T, int NR, int MW, int NW>
+template <typename T, int NR, int MW, int NW, int CL>
 static void td_launch(const Launch& L, int n, unsigned char* scratch, size_t stride, int blk) {
   const bool all = td_smem(n, sizeof(T), true) <= TD_SMEM_MAX;
   const size_t smem = td_smem(n, sizeof(T), all);
-  cudaFuncSetAttribute(k_rr_td<T, NR, MW, NW>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  k_rr_td<T, NR, MW, NW><<<L.ka.nprob, 32 * NW, smem, L.stream>>>(L.ka, reinterpret_cast<T*>(scratch),
-                                                                  stride / sizeof(T), all ? 1 : 0, blk);
+  auto* fn = k_rr_td<T, NR, MW, NW, CL>;
+  cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = L.ka.nprob * CL;
+  cfg.blockDim = 32 * NW;
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = L.stream;
+  cudaLaunchAttribute at[1] = {};
+  at[0].id = cudaLaunchAttributeClusterDimension;
+  at[0].val.clusterDim.x = CL;
+  at[0].val.clusterDim.y = 1;
+  at[0].val.clusterDim.z = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = CL > 1 ? 1 : 0;
+  cudaLaunchKernelEx(&cfg, fn, L.ka, reinterpret_cast<T*>(scratch), stride / sizeof(T), all ? 1 : 0, blk);
 }
 
-// n: the largest subspace of the launch (n_b, or 2 n_b for blk = 2)
+// n: the largest subspace of the launch (n_b, or 2 n_b for blk = 2).  CTAs per problem: more of them
+// shorten the column-owning steps and, on the FP64 path, share the FP64 lanes' work; each barrier
+// costs 0.4 us more.  So a cluster wherever it is faster, while the launch leaves half the SMs to the
+// sub-batches that run beside it.  Measured, one problem, 1 / 4 / 8 CTAs: FP64 24 bands 269 / 219 / 191 us, 52 bands 851 / 550 /
+// 472, 70 bands 1825 / 925 / 724, 119 bands 5074 / 1953 / 1438; FP32 52 bands 141 / 185 / 195, 70
+// bands 237 / 279 / 297, 119 bands 525 / 502 / 526, 169 bands 1345 / 934 / 918.
 template <typename T>
 void launch_rr_td(const Launch& L, int n, unsigned char* scratch, size_t stride, int blk) {
-  // (FP32: 4 to 12 rows per warp, bound by issue and latency; FP64: 8 to 16 rows in as few warps as
-  // the registers allow, bound by the FP64 lanes, which every warp's own sums use too)
+  constexpr int SMS = 152 / 2;
+  const int np = L.ka.nprob;
+  // (FP32: 4 to 12 rows per warp, bound by issue and latency; FP64 in one CTA: 8 to 16 rows in as few
+  // warps as the registers allow, bound by the FP64 lanes, which every warp's own sums use too)
   if constexpr (sizeof(T) == 4) {
-    if (n <= 32) td_launch<T, 1, 8, 8>(L, n, scratch, stride, blk);
-    else if (n <= 64) td_launch<T, 2, 16, 16>(L, n, scratch, stride, blk);
-    else if (n <= 96) td_launch<T, 3, 16, 16>(L, n, scratch, stride, blk);
-    else if (n <= 128) td_launch<T, 4, 16, 16>(L, n, scratch, stride, blk);
-    else td_launch<T, 6, 16, 16>(L, n, scratch, stride, blk);
+    if (n <= 32) td_launch<T, 1, 8, 8, 1>(L, n, scratch, stride, blk);
+    else if (n <= 64) td_launch<T, 2, 16, 16, 1>(L, n, scratch, stride, blk);
+    else if (n <= 96) td_launch<T, 3, 16, 16, 1>(L, n, scratch, stride, blk);
+    else if (n <= 128) td_launch<T, 4, 16, 16, 1>(L, n, scratch, stride, blk);
+    else if (np * 4 <= SMS) td_launch<T, 6, 8, 8, 4>(L, n, scratch, stride, blk);
+    else td_launch<T, 6, 16, 16, 1>(L, n, scratch, stride, blk);
+  } else if (np * 8 <= SMS) {
+    if (n <= 32) td_launch<T, 1, 2, 2, 8>(L, n, scratch, stride, blk);
+    else if (n <= 64) td_launch<T, 2, 4, 4, 8>(L, n, scratch, stride, blk);
+    else if (n <= 96) td_launch<T, 3, 6, 6, 8>(L, n, scratch, stride, blk);
+    else td_launch<T, 4, 8, 8, 8>(L, n, scratch, stride, blk);
+  } else if (np * 4 <= SMS) {
+    if (n <= 32) td_launch<T, 1, 2, 2, 4>(L, n, scratch, stride, blk);
+    else if (n <= 64) td_launch<T, 2, 4, 4, 4>(L, n, scratch, stride, blk);
+    else if (n <= 96) td_launch<T, 3, 6, 6, 4>(L, n, scratch, stride, blk);
+    else td_launch<T, 4, 8, 8, 4>(L, n, scratch, stride, blk);
   } else {
-    if (n <= 32) td_launch<T, 1, 4, 8>(L, n, scratch, stride, blk);
-    else if (n <= 64) td_launch<T, 2, 8, 8>(L, n, scratch, stride, blk);
-    else if (n <= 96) td_launch<T, 3, 8, 8>(L, n, scratch, stride, blk);
-    else td_launch<T, 4, 8, 8>(L, n, scratch, stride, blk);
+    if (n <= 32) td_launch<T, 1, 4, 8, 1>(L, n, scratch, stride, blk);
+    else if (n <= 64) td_launch<T, 2, 8, 8, 1>(L, n, scratch, stride, blk);
+    else if (n <= 96) td_launch<T, 3, 8, 8, 1>(L, n, scratch, stride, blk);
+    else td_launch<T, 4, 8, 8, 1>(L, n, scratch, stride, blk);
   }
 }
 template void launch_rr_td<float>(const Launch&, int, unsigned char*, size_t, int);

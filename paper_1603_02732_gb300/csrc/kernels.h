@@ -221,7 +221,7 @@ template <typename T> void launch_random_init(const Launch& L, int xrole, unsign
 // rows >= nvec: zero, or (keep_tail) left as they are
 template <typename T> void launch_copy_in(const Launch& L, int role, const double* src, int nvec, bool keep_tail = false);
 template <typename T> void launch_copy_out(const Launch& L, int role, double* dst, int nvec);
-// subspace diagonalisation, one CTA per problem (k_rr_td.cu): T = float or double; n the largest
+// subspace diagonalisation, one CTA or cluster per problem (k_rr_td.cu): T = float or double; n the largest
 // subspace of the launch, at most rr_td_max(sizeof(T)); scratch of rr_td_scratch_bytes(n) bytes
 // per problem (none when it is 0)
 // blk = 1: the n_b x n_b subspace (S, Hs -> Tm); blk = 2: the 2 n_b block [X, W] of the block

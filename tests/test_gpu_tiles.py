@@ -115,3 +115,21 @@ def test_grid_transform_lengths(sgo, grid, precision):
     for sign in (-1, 1):
         ref = np.fft.fftn(x) if sign < 0 else np.fft.ifftn(x) * x.size
         assert np.abs(ctx.grid_fft(x, sign) - ref).max() < 1e-12 * np.abs(ref).max()
+
+
+# members per launch on either side of the eigensolve's cluster rule (8, 4 and 1 CTAs per problem)
+@pytest.mark.parametrize("members", [9, 10, 20])
+@pytest.mark.parametrize("precision,bands", [("fp64", 9), ("fp64", 40), ("mixed", 130)])
+def test_subspace_eigensolve_per_launch(sgo, members, precision, bands):
+    """The CTAs of a problem share its work without changing a sum: a member's F and spectrum after a
+    few iterations are bitwise those of a batch of two."""
+    st = _with_bands(workloads.tiny(nat=2, ecut=9.0, kT=0.01), bands)
+
+    def run(n):
+        ctxs = [sgo.Context(st, precision=precision, max_scf=4, autotune=0, sub_batches=1) for _ in range(n)]
+        F = sgo.Batch(ctxs).energy_forces()[0]
+        return F[0], ctxs[0].eigen()[0]
+
+    two, many = run(2), run(members)
+    assert two[0] == many[0]
+    assert np.array_equal(two[1], many[1])
