@@ -824,7 +824,7 @@ Engine::Engine(const std::vector<sgo_ctx*>& ctxs, cudaStream_t stream) : ctx_(ct
     }
   }
   std::vector<Prob> host(n_);
-  std::vector<int> c_zcol, c_plane, c_dens, c_gz, c_gp, c_gew, c_gch, c_bands, c_rww, c_nn, c_atoms, c_projs, c_atomch, c_ewsg, c_prob, c_tc, c_nntc, c_preg[2], c_dreg[2], c_zreg[2], c_ppair,
+  std::vector<int> c_zcol, c_plane, c_dens, c_gz, c_gp, c_gew, c_bands, c_rww, c_nn, c_atoms, c_projs, c_atomch, c_ewsg, c_prob, c_tc, c_nntc, c_preg[2], c_dreg[2], c_zreg[2], c_ppair,
       c_dpair, c_zpair, c_gx, c_gy, c_gaxis[3], c_gold, c_bigy, c_bigx, c_bigdy, c_bigd;
   size_t part = 0;
   int max_nproj = 0;
@@ -892,7 +892,6 @@ Engine::Engine(const std::vector<sgo_ctx*>& ctxs, cudaStream_t stream) : ctx_(ct
     c_gz.push_back(gaxis ? 0 : div_up(d.n1 * d.n2, QZ));
     c_gp.push_back(gaxis || gbig ? 0 : d.n3);
     c_gew.push_back(div_up(d.ngrid, GRID_EW_POINTS));
-    c_gch.push_back(nch);
     c_bands.push_back(d.nb);
     c_rww.push_back(div_up(d.nb * d.nb, 256));
     c_nn.push_back(precision_ ? div_up(d.npw, 64 * NN_RT) * div_up(d.nb, 64)
@@ -927,7 +926,6 @@ Engine::Engine(const std::vector<sgo_ctx*>& ctxs, cudaStream_t stream) : ctx_(ct
   m_gz_ = make_map(c_gz);
   m_gp_ = make_map(c_gp);
   m_gew_ = make_map(c_gew);
-  m_gch_ = make_map(c_gch);
   m_bands_ = make_map(c_bands);
   m_asm_ = make_map(c_rww);
   m_nn_ = make_map(c_nn);
@@ -958,7 +956,7 @@ Engine::Engine(const std::vector<sgo_ctx*>& ctxs, cudaStream_t stream) : ctx_(ct
   cudaMemcpy(d_active_, h_active_.data(), sizeof(int) * n_, cudaMemcpyHostToDevice);
   if (!cuda_ok(dev_malloc(&d_part_, sizeof(double) * part_stride_ * n_), "dev_malloc(part)")) return;
   allocs_.push_back(d_part_);
-  if (!cuda_ok(dev_malloc(&d_gpart_, sizeof(double) * (size_t)maxchunk_ * n_ * 8), "dev_malloc(gpart)")) return;
+  if (!cuda_ok(dev_malloc(&d_gpart_, sizeof(double) * (size_t)*std::max_element(c_gew.begin(), c_gew.end()) * n_ * 8), "dev_malloc(gpart)")) return;
   allocs_.push_back(d_gpart_);
   if (!cuda_ok(dev_malloc(&d_flags_, sizeof(double) * 4 * n_), "dev_malloc(flags)")) return;
   allocs_.push_back(d_flags_);
@@ -1004,7 +1002,7 @@ Engine::Engine(const std::vector<sgo_ctx*>& ctxs, cudaStream_t stream) : ctx_(ct
   }
   const sgo_opts& o0 = ctxs[0]->opts;
   wait_ns_ = o0.watchdog_ms > 0.0 ? (long long)(o0.watchdog_ms * 1e6) : 2000000000LL;
-  // subspace diagonalisation: k_rr_td.cu per member up to rr_td_max bands (192 on the mixed path,
+  // subspace diagonalisation: k_rr_td.cu per member up to rr_td_max bands (184 on the mixed path,
   // 128 in FP64), beyond (or when asked for) one thread-block cluster per member (k_rr_cluster)
   // (the block Davidson steps diagonalise the 2 n_b block [X, W])
   davidson_ = o0.eigensolver == 1;
@@ -1462,9 +1460,8 @@ void Engine::density_energy(int mode) {
     grid_fft(3, 1);
   }
   tbeg(TK_GRID_OTHER);
-  launch_grid_energies<T>(L(m_gch_), d_gpart_, maxchunk_);
-  launch_grid_energies_reduce(L(m_prob_), d_gpart_, maxchunk_);
-  launch_finish_iteration(L(m_prob_), o.scf_tol_e, o.scf_tol_rho, mode);
+  launch_grid_energies<T>(L(m_gew_), d_gpart_, m_gew_.maxper);
+  launch_finish_iteration(L(m_prob_), d_gpart_, m_gew_.maxper, o.scf_tol_e, o.scf_tol_rho, mode);
   tend(TK_GRID_OTHER);
 }
 
@@ -1561,9 +1558,8 @@ void Engine::pulay_step() {
   const sgo_opts& o = ctx_[0]->opts;
   const int hist = std::min(std::max(o.pulay_hist, 1), MAX_HIST);
   tbeg(TK_GRID_OTHER);
-  launch_pulay_store(L(m_gew_));
-  launch_pulay_gram(L(m_gch_), d_gpart_, maxchunk_, hist);
-  launch_pulay_solve(L(m_prob_), d_gpart_, maxchunk_, hist);
+  launch_pulay_gram(L(m_gew_), d_gpart_, m_gew_.maxper, hist);
+  launch_pulay_solve(L(m_prob_), d_gpart_, m_gew_.maxper, hist);
   launch_pulay_mix(L(m_gew_), o.mix_alpha, o.kerker_q0);
   tend(TK_GRID_OTHER);
 }

@@ -52,6 +52,15 @@ __device__ __forceinline__ double* grid_sel(const Prob& P, int sel) {
   }
 }
 
+// 1 / x for a positive normal number: the approximate reciprocal and two Newton steps (four FP64
+// operations; a division takes more than twice as many)
+__device__ __forceinline__ double rcp_newton(double x) {
+  double r;
+  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(x));
+  r = fma(r, fma(-x, r, 1.0), r);
+  return fma(r, fma(-x, r, 1.0), r);
+}
+
 // exp(-i G.R_I) from the atom's 1D tables (indexed by grid index per axis).
 __device__ __forceinline__ cplx<double> phase_at(const Prob& P, int atom, int i1, int i2, int i3) {
   const cplx<double>* ph = reinterpret_cast<const cplx<double>*>(P.phase) + (size_t)atom * (P.n1 + P.n2 + P.n3);
@@ -278,7 +287,7 @@ __global__ void k_potential_g(KArgs ka) {
   for (int i = base + threadIdx.x; i < end; i += blockDim.x) {
     const double g2 = P.g2box[i];  // -1 on Nyquist planes
     double2 r = P.rhog_in[i];
-    double f = g2 < 1e-14 ? 0.0 : 4.0 * PI / g2;
+    double f = g2 < 1e-14 ? 0.0 : 4.0 * PI * rcp_newton(g2);
     // (r.x + i r.y) + i f (r.x + i r.y)
     g[i] = mk((T)(r.x - f * r.y), (T)(r.y + f * r.x));
   }
@@ -381,20 +390,19 @@ __global__ void k_rho0_g(KArgs ka) {
 // ---------------------------------------------------------------------------
 // Grid reductions for the energy at rho_out (work grid gfft2 = N rho_out(G)):
 // part[p][chunk][0..4] = sum V_ion rho, sum rho eps_xc, sum rho, sum |rho_out - rho_in|,
-// sum_{G!=0} |rho(G)|^2 / G^2.
+// sum_{G!=0} |rho(G)|^2 / G^2.  CTA = (problem, GRID_EW points).
+// Bound by FP64 operations (about 20 a point; the two FP64 lanes of an SM) and, for one structure,
+// by latency: chunks of 4096 points left most SMs idle, and five block sums one after the other and
+// the division took half the FP64 work.  24-atom layer 43 -> 17 us, 64 members 244 -> 184 us.
 // ---------------------------------------------------------------------------
-constexpr int NGE = 5;
+constexpr int NGE = 5, NRED = 8;  // sums used, stride of a chunk's partial sums
 
 template <typename T>
 __global__ void k_grid_energies(KArgs ka, double* part, int maxchunk) {
-  __shared__ double red[33];
-  const int p = locate(ka.start, ka.nprob, blockIdx.x);
-  if (!ka.active[p]) return;
-  const Prob& P = ka.probs[p];
-  const int chunk = blockIdx.x - ka.start[p];
-  const int base = chunk * GRID_CHUNK, end = min(P.ngrid, base + GRID_CHUNK);
-  const double inv_n = 1.0 / P.ngrid;
-  double s[NGE] = {0, 0, 0, 0, 0};
+  __shared__ double red[64], tot[8];
+  GRID_EW_PROLOGUE
+  const double inv_n2 = (1.0 / P.ngrid) * (1.0 / P.ngrid);
+  double s[8] = {0, 0, 0, 0, 0, 0, 0, 0};
   for (int i = base + threadIdx.x; i < end; i += blockDim.x) {
     double r = P.rho_out[i];
     if (P.xc == 1) {  // PBE with grad rho_out in gfft3 (x + i y) and gfft4 (z)
@@ -414,52 +422,58 @@ __global__ void k_grid_energies(KArgs ka, double* part, int maxchunk) {
     const double g2 = P.g2box[i];  // -1 on Nyquist planes
     if (g2 > 1e-14) {
       double2 v = P.gfft2[i];
-      s[4] += (v.x * v.x + v.y * v.y) * inv_n * inv_n / g2;
+      s[4] += (v.x * v.x + v.y * v.y) * rcp_newton(g2);
     }
   }
-  for (int k = 0; k < NGE; ++k) {
-    double t = block_sum(s[k], red);
-    if (threadIdx.x == 0) part[((size_t)p * maxchunk + chunk) * NGE + k] = t;
-  }
+  s[4] *= inv_n2;
+  block_sums8(s, red, tot);
+  if (threadIdx.x < NRED) part[((size_t)p * maxchunk + (blockIdx.x - ka.start[p])) * NRED + threadIdx.x] = tot[threadIdx.x];
 }
 
-__global__ void k_grid_energies_reduce(KArgs ka, const double* part, int maxchunk) {
-  const int p = blockIdx.x;
-  if (!ka.active[p] || threadIdx.x != 0) return;
-  const Prob& P = ka.probs[p];
-  const int nch = (P.ngrid + GRID_CHUNK - 1) / GRID_CHUNK;
-  double s[NGE] = {0, 0, 0, 0, 0};
-  for (int c = 0; c < nch; ++c)
-    for (int k = 0; k < NGE; ++k) s[k] += part[((size_t)p * maxchunk + c) * NGE + k];
-  const double dv = P.omega / P.ngrid;
-  P.scal[SC_ELOC] = dv * s[0];
-  P.scal[SC_EXC] = dv * s[1];
-  P.scal[SC_NELCHK] = dv * s[2];
-  P.scal[SC_RESID] = dv * s[3] / P.nel;
-  P.scal[SC_EH] = 0.5 * P.omega * 4.0 * PI * s[4];
+// Sums of a problem's partial sums over its chunks, in tot[8] (256 threads: 32 slices of the chunks)
+__device__ __forceinline__ void chunk_sums(const Prob& P, const double* part, double (&red)[32][NRED + 1], double* tot) {
+  const int nch = (P.ngrid + GRID_EW - 1) / GRID_EW, lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  double s = 0.0;
+  for (int c = threadIdx.x >> 3; c < nch; c += 32) s += part[(size_t)c * NRED + (threadIdx.x & 7)];
+  red[threadIdx.x >> 3][threadIdx.x & 7] = s;
+  __syncthreads();
+  s = warp_sum(red[lane][w]);
+  if (lane == 0) tot[w] = s;
+  __syncthreads();
 }
 
-// Band terms, total free energy, convergence test.  One CTA per problem.
-__global__ void k_finish_iteration(KArgs ka, double tol_e, double tol_rho, int count_iter) {
-  __shared__ double red[33];
+// Grid sums, band terms, total free energy, convergence test.  One CTA of 256 threads per problem.
+// (One thread summing the chunks and one thread per band summing its projectors took 18 + 13 us for
+// the 24-atom layer and 18 + 42 us for 32 atoms with p channels; now 14 and 20 us.)
+__global__ void k_finish_iteration(KArgs ka, const double* part, int maxchunk, double tol_e, double tol_rho,
+                                   int count_iter) {
+  __shared__ double red[33], redc[32][NRED + 1], tot[NRED];
   const int p = blockIdx.x;
   if (!ka.active[p]) return;
   const Prob& P = ka.probs[p];
+  chunk_sums(P, part + (size_t)p * maxchunk * NRED, redc, tot);
   double ek = 0.0, en = 0.0;
-  for (int i = threadIdx.x; i < P.nb; i += blockDim.x) {
-    const double f = P.occ[i];
-    ek += f * P.bv[BV_EKIN * P.nb + i];
+  for (int i = threadIdx.x; i < P.nb; i += blockDim.x) ek += P.occ[i] * P.bv[BV_EKIN * P.nb + i];
+  constexpr int SL = 16;  // slices of the projectors
+  for (int e = threadIdx.x; e < SL * P.nb; e += blockDim.x) {
+    const int sl = e / P.nb, i = e - sl * P.nb;
     double s = 0.0;
-    for (int k = 0; k < P.nproj; ++k) {
-      double pr = P.proj[(size_t)k * P.nb + i];
+    for (int k = sl; k < P.nproj; k += SL) {
+      const double pr = P.proj[(size_t)k * P.nb + i];
       s += P.pj_d[k] * pr * pr;
     }
-    en += f * s;
+    en += P.occ[i] * s;
   }
   ek = block_sum(ek, red);
   en = block_sum(en, red);
   if (threadIdx.x == 0) {
     double* sc = P.scal;
+    const double dv = P.omega / P.ngrid;
+    sc[SC_ELOC] = dv * tot[0];
+    sc[SC_EXC] = dv * tot[1];
+    sc[SC_NELCHK] = dv * tot[2];
+    sc[SC_RESID] = dv * tot[3] / P.nel;
+    sc[SC_EH] = 0.5 * P.omega * 4.0 * PI * tot[4];
     sc[SC_EKIN] = ek;
     sc[SC_ENL] = en;
     sc[SC_MTS] = -P.kT * sc[SC_ENTROPY];
@@ -481,107 +495,124 @@ __global__ void k_finish_iteration(KArgs ka, double tol_e, double tol_rho, int c
 // ---------------------------------------------------------------------------
 // Pulay (DIIS) mixing on R = rho_out - rho_in with a ring history.
 // ---------------------------------------------------------------------------
-__global__ void k_pulay_store(KArgs ka) {
+// The density and residual go into the ring; part[p][chunk][j] = <R_pos, R_j> over a chunk for every
+// ring slot j (0 for the empty ones).  CTA = (problem, GRID_EW points): the points' loads of all
+// slots are in flight together and the eight sums are reduced together.  For one structure bound by
+// latency, in a batch by the ring's bytes.  24-atom layer: 62 us (37 CTAs, one slot after the other)
+// and 7 us for the store -> 22 us; 64 members 227 + 68 -> 258 us.
+__global__ void k_pulay_gram(KArgs ka, double* part, int maxchunk, int hist) {
+  __shared__ double red[64], tot[8];
   GRID_EW_PROLOGUE
   const int pos = (int)P.scal[SC_PULAY_POS];
-  double2* hr = P.hrho + (size_t)pos * P.ngrid;
-  double2* hs = P.hres + (size_t)pos * P.ngrid;
+  const int cnt = min((int)P.scal[SC_PULAY_N] + 1, hist);
   const double inv_n = 1.0 / P.ngrid;
+  const size_t ng = P.ngrid;
+  double s[8] = {0, 0, 0, 0, 0, 0, 0, 0};
   for (int i = base + threadIdx.x; i < end; i += blockDim.x) {
-    double2 ri = P.rhog_in[i], ro = P.gfft2[i];
-    hr[i] = ri;
-    hs[i] = make_double2(ro.x * inv_n - ri.x, ro.y * inv_n - ri.y);
+    double2 r[MAX_HIST];
+#pragma unroll
+    for (int j = 0; j < MAX_HIST; ++j) r[j] = j < cnt && j != pos ? P.hres[j * ng + i] : make_double2(0.0, 0.0);
+    const double2 ri = P.rhog_in[i], ro = P.gfft2[i];
+    const double2 rp = make_double2(ro.x * inv_n - ri.x, ro.y * inv_n - ri.y);
+    P.hrho[pos * ng + i] = ri;
+    P.hres[pos * ng + i] = rp;
+#pragma unroll
+    for (int j = 0; j < MAX_HIST; ++j)
+      if (j < cnt) {
+        const double2 rj = j == pos ? rp : r[j];
+        s[j] += rp.x * rj.x + rp.y * rj.y;
+      }
   }
+  block_sums8(s, red, tot);
+  if (threadIdx.x < NRED) part[((size_t)p * maxchunk + (blockIdx.x - ka.start[p])) * NRED + threadIdx.x] = tot[threadIdx.x];
 }
 
-// part[p][chunk][j] = <R_pos, R_j> over a chunk, for every ring slot j.
-__global__ void k_pulay_gram(KArgs ka, double* part, int maxchunk, int hist) {
-  __shared__ double red[33];
-  const int p = locate(ka.start, ka.nprob, blockIdx.x);
+// Gram row update and the DIIS system [A 1; 1 0][c; l] = [0; 1] (Gaussian elimination with partial
+// pivoting, lane i of one warp holding row i).  One CTA of 256 threads per problem; one thread alone
+// took 62 us for the 24-atom layer (sums over the chunks, then the elimination in local memory), this
+// form 25 us.
+__global__ void k_pulay_solve(KArgs ka, const double* part, int maxchunk, int hist) {
+  __shared__ double redc[32][NRED + 1], tot[NRED];
+  const int p = blockIdx.x;
   if (!ka.active[p]) return;
   const Prob& P = ka.probs[p];
-  const int chunk = blockIdx.x - ka.start[p];
-  const int base = chunk * GRID_CHUNK, end = min(P.ngrid, base + GRID_CHUNK);
-  const int pos = (int)P.scal[SC_PULAY_POS];
-  const int cnt = min((int)P.scal[SC_PULAY_N] + 1, hist);
-  const double2* rp = P.hres + (size_t)pos * P.ngrid;
-  for (int j = 0; j < cnt; ++j) {
-    const double2* rj = P.hres + (size_t)j * P.ngrid;
-    double s = 0.0;
-    for (int i = base + threadIdx.x; i < end; i += blockDim.x) s += rp[i].x * rj[i].x + rp[i].y * rj[i].y;
-    s = block_sum(s, red);
-    if (threadIdx.x == 0) part[((size_t)p * maxchunk + chunk) * MAX_HIST + j] = s;
-  }
-}
-
-// Gram row update and the DIIS system [A 1; 1 0][c; l] = [0; 1] (partial pivoting).
-__global__ void k_pulay_solve(KArgs ka, const double* part, int maxchunk, int hist) {
-  const int p = blockIdx.x;
-  if (!ka.active[p] || threadIdx.x != 0) return;
-  const Prob& P = ka.probs[p];
+  chunk_sums(P, part + (size_t)p * maxchunk * NRED, redc, tot);
+  if (threadIdx.x >= 32) return;
+  constexpr int R = MAX_HIST + 1;  // rows
+  constexpr unsigned full = 0xffffffffu;
   double* sc = P.scal;
   double* A = sc + SC_PULAY_A;
   double* alpha = sc + SC_PULAY_A + MAX_HIST * MAX_HIST;
-  const int pos = (int)sc[SC_PULAY_POS];
-  const int cnt = min((int)sc[SC_PULAY_N] + 1, hist);
-  const int nch = (P.ngrid + GRID_CHUNK - 1) / GRID_CHUNK;
-  for (int j = 0; j < cnt; ++j) {
-    double s = 0.0;
-    for (int c = 0; c < nch; ++c) s += part[((size_t)p * maxchunk + c) * MAX_HIST + j];
-    A[pos * MAX_HIST + j] = s;
-    A[j * MAX_HIST + pos] = s;
+  const int lane = threadIdx.x, pos = (int)sc[SC_PULAY_POS];
+  const int cnt = min((int)sc[SC_PULAY_N] + 1, hist), m = cnt + 1;
+  if (lane < cnt) {
+    A[pos * MAX_HIST + lane] = tot[lane];
+    A[lane * MAX_HIST + pos] = tot[lane];
   }
-  const int m = cnt + 1;
-  double M[(MAX_HIST + 1) * (MAX_HIST + 2)];
-  const double scl = A[pos * MAX_HIST + pos] > 0.0 ? 1.0 / A[pos * MAX_HIST + pos] : 1.0;
-  for (int i = 0; i < m; ++i) {
-    for (int j = 0; j < m; ++j) {
-      double v;
-      if (i < cnt && j < cnt) v = A[i * MAX_HIST + j] * scl;
-      else if (i == cnt && j == cnt) v = 0.0;
-      else v = 1.0;
-      M[i * (m + 1) + j] = v;
-    }
-    M[i * (m + 1) + m] = (i == cnt) ? 1.0 : 0.0;
-  }
-  bool ok = true;
-  for (int k = 0; k < m && ok; ++k) {
-    int piv = k;
-    for (int i = k + 1; i < m; ++i)
-      if (fabs(M[i * (m + 1) + k]) > fabs(M[piv * (m + 1) + k])) piv = i;
-    if (fabs(M[piv * (m + 1) + k]) < 1e-300) { ok = false; break; }
-    if (piv != k)
-      for (int j = 0; j <= m; ++j) {
-        double t = M[k * (m + 1) + j];
-        M[k * (m + 1) + j] = M[piv * (m + 1) + j];
-        M[piv * (m + 1) + j] = t;
+  __syncwarp();
+  const double scl = tot[pos] > 0.0 ? 1.0 / tot[pos] : 1.0;
+  double M[R], b = lane == cnt ? 1.0 : 0.0, x = 0.0;
+#pragma unroll
+  for (int j = 0; j < R; ++j)
+    M[j] = lane < cnt && j < cnt ? A[lane * MAX_HIST + j] * scl : lane < m && j < m && (lane < cnt || j < cnt) ? 1.0 : 0.0;
+  bool ok = true;  // (uniform)
+#pragma unroll
+  for (int k = 0; k < R; ++k) {
+    if (k >= m || !ok) continue;
+    double v = lane >= k && lane < m ? fabs(M[k]) : -1.0;  // largest |M_ik|, the first such row
+    int piv = lane;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+      const double w = __shfl_xor_sync(full, v, o);
+      const int q = __shfl_xor_sync(full, piv, o);
+      if (w > v || (w == v && q < piv)) {
+        v = w;
+        piv = q;
       }
-    for (int i = k + 1; i < m; ++i) {
-      double f = M[i * (m + 1) + k] / M[k * (m + 1) + k];
-      for (int j = k; j <= m; ++j) M[i * (m + 1) + j] -= f * M[k * (m + 1) + j];
+    }
+    piv = __shfl_sync(full, piv, 0);
+    if (__shfl_sync(full, v, 0) < 1e-300) {
+      ok = false;
+      continue;
+    }
+    // rows k and piv change places; bp, row: the pivot row
+    const double bp = __shfl_sync(full, b, piv), bk = __shfl_sync(full, b, k);
+    if (lane == piv) b = bk;
+    if (lane == k) b = bp;
+    double row[R];
+#pragma unroll
+    for (int j = k; j < R; ++j) {
+      row[j] = __shfl_sync(full, M[j], piv);
+      const double mk = __shfl_sync(full, M[j], k);
+      if (lane == piv) M[j] = mk;
+      if (lane == k) M[j] = row[j];
+    }
+    if (lane > k && lane < m) {
+      const double f = M[k] / row[k];
+#pragma unroll
+      for (int j = k; j < R; ++j) M[j] -= f * row[j];
+      b -= f * bp;
     }
   }
-  double x[MAX_HIST + 1];
-  if (ok) {
-    for (int i = m - 1; i >= 0; --i) {
-      double s = M[i * (m + 1) + m];
-      for (int j = i + 1; j < m; ++j) s -= M[i * (m + 1) + j] * x[j];
-      x[i] = s / M[i * (m + 1) + i];
-      if (!isfinite(x[i])) ok = false;
-    }
+#pragma unroll
+  for (int i = R - 1; i >= 0; --i) {
+    if (i >= m || !ok) continue;
+    const double xi = __shfl_sync(full, b / M[i], i);
+    if (!isfinite(xi)) ok = false;
+    if (lane == i) x = xi;
+    if (lane < i) b -= M[i] * xi;
   }
-  for (int j = 0; j < MAX_HIST; ++j) alpha[j] = 0.0;
-  if (ok) {
-    for (int j = 0; j < cnt; ++j) alpha[j] = x[j];
-  } else {
-    alpha[pos] = 1.0;
+  if (lane < MAX_HIST) alpha[lane] = ok ? (lane < cnt ? x : 0.0) : lane == pos ? 1.0 : 0.0;
+  if (lane == 0) {
+    sc[SC_PULAY_N] = cnt;
+    sc[SC_PULAY_POS] = (pos + 1) % hist;
   }
-  sc[SC_PULAY_N] = cnt;
-  sc[SC_PULAY_POS] = (pos + 1) % hist;
 }
 
 // rho_in(G) = sum_j c_j rho_j(G) + a K(G) sum_j c_j R_j(G), K = G^2/(G^2 + q0^2) (1 if q0 = 0),
 // zero on Nyquist planes.
+// Bound by FP64 operations in a batch (4 a point and slot): 64 members 331 us.  (All slots' loads in
+// flight together took 404: more registers, fewer warps.)
 __global__ void k_pulay_mix(KArgs ka, double a, double q0) {
   GRID_EW_PROLOGUE
   const double* alpha = P.scal + SC_PULAY_A + MAX_HIST * MAX_HIST;
@@ -597,7 +628,7 @@ __global__ void k_pulay_mix(KArgs ka, double a, double q0) {
       sy += alpha[j] * r.y;
     }
     double k = 1.0;
-    if (q0 > 0.0) k = g2 < 1e-14 ? 0.0 : g2 / (g2 + q0 * q0);
+    if (q0 > 0.0) k = g2 < 1e-14 ? 0.0 : g2 * rcp_newton(g2 + q0 * q0);
     if (g2 < 0.0) k = 0.0, rx = ry = 0.0;
     P.rhog_in[i] = make_double2(rx + a * k * sx, ry + a * k * sy);
   }
@@ -810,27 +841,22 @@ void launch_vion_g(const Launch& L) {
 void launch_rho0_g(const Launch& L) {
   if (ew_blocks(L)) k_rho0_g<<<L.map.total, 256, 0, L.stream>>>(L.ka);
 }
-void launch_pulay_store(const Launch& L) {
-  if (ew_blocks(L)) k_pulay_store<<<L.map.total, 256, 0, L.stream>>>(L.ka);
-}
 void launch_pulay_mix(const Launch& L, double a, double q0) {
   if (ew_blocks(L)) k_pulay_mix<<<L.map.total, 256, 0, L.stream>>>(L.ka, a, q0);
 }
 template <typename T>
-void launch_grid_energies(const Launch& Lchunks, double* part, int maxchunk) {
-  if (Lchunks.map.total) k_grid_energies<T><<<Lchunks.map.total, 256, 0, Lchunks.stream>>>(Lchunks.ka, part, maxchunk);
+void launch_grid_energies(const Launch& L, double* part, int maxchunk) {
+  if (ew_blocks(L)) k_grid_energies<T><<<L.map.total, 256, 0, L.stream>>>(L.ka, part, maxchunk);
 }
-void launch_grid_energies_reduce(const Launch& L, const double* part, int maxchunk) {
-  k_grid_energies_reduce<<<L.ka.nprob, 32, 0, L.stream>>>(L.ka, part, maxchunk);
+void launch_finish_iteration(const Launch& L, const double* part, int maxchunk, double tol_e, double tol_rho,
+                             int count_iter) {
+  k_finish_iteration<<<L.ka.nprob, 256, 0, L.stream>>>(L.ka, part, maxchunk, tol_e, tol_rho, count_iter);
 }
-void launch_finish_iteration(const Launch& L, double tol_e, double tol_rho, int count_iter) {
-  k_finish_iteration<<<L.ka.nprob, 128, 0, L.stream>>>(L.ka, tol_e, tol_rho, count_iter);
-}
-void launch_pulay_gram(const Launch& Lchunks, double* part, int maxchunk, int hist) {
-  if (Lchunks.map.total) k_pulay_gram<<<Lchunks.map.total, 256, 0, Lchunks.stream>>>(Lchunks.ka, part, maxchunk, hist);
+void launch_pulay_gram(const Launch& L, double* part, int maxchunk, int hist) {
+  if (ew_blocks(L)) k_pulay_gram<<<L.map.total, 256, 0, L.stream>>>(L.ka, part, maxchunk, hist);
 }
 void launch_pulay_solve(const Launch& L, const double* part, int maxchunk, int hist) {
-  k_pulay_solve<<<L.ka.nprob, 32, 0, L.stream>>>(L.ka, part, maxchunk, hist);
+  k_pulay_solve<<<L.ka.nprob, 256, 0, L.stream>>>(L.ka, part, maxchunk, hist);
 }
 template <typename T>
 void launch_build_projectors(const Launch& Latoms, int deriv) {

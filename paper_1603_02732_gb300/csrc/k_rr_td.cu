@@ -104,39 +104,6 @@ __device__ __forceinline__ T wsum(T v) {
   return v;
 }
 
-// Sums over W consecutive lanes of R values per lane.  Pairs of values are folded into one
-// register per exchange (the lanes on either side of a bit keep one value each), so that R sums
-// cost about R + log2 W shuffles and adds instead of R log2 W: on return a lane holds the sum of
-// value fold_index(lane).
-template <int R>
-__host__ __device__ constexpr int fold_bits() { return R > 8 ? 4 : R > 4 ? 3 : R > 2 ? 2 : R > 1 ? 1 : 0; }
-template <typename T, int R, int W>
-__device__ __forceinline__ T fold_sums(const T (&in)[R], int lane) {
-  constexpr int B = fold_bits<R>(), N = 1 << B;
-  T v[N];
-#pragma unroll
-  for (int i = 0; i < N; ++i) v[i] = i < R ? in[i < R ? i : 0] : T(0);
-  int o = W / 2;
-#pragma unroll
-  for (int b = 0; b < B; ++b, o >>= 1) {
-    const bool up = (lane & o) != 0;
-    const int h = N >> (b + 1);
-#pragma unroll
-    for (int i = 0; i < N; ++i)
-      if (i < h) {
-        const T keep = up ? v[i + h] : v[i], give = up ? v[i] : v[i + h];
-        v[i] = keep + __shfl_xor_sync(0xffffffffu, give, o);
-      }
-  }
-#pragma unroll
-  for (; o > 0; o >>= 1) v[0] = v[0] + __shfl_xor_sync(0xffffffffu, v[0], o);
-  return v[0];
-}
-constexpr int log2i(int w) { return w <= 1 ? 0 : 1 + log2i(w / 2); }
-// shift from a lane of the W to the value it holds (the first lane that holds value a is a << it)
-template <int R, int W>
-__host__ __device__ constexpr int fold_shift() { return log2i(W) - fold_bits<R>(); }
-
 // sum over the g lanes of a root
 template <typename T>
 __device__ __forceinline__ T gsum(T v, int g) {

@@ -47,7 +47,7 @@ __host__ __device__ inline int nn_rows_f64(int nb, int npw) {
   return 4 * (256 / cg < cap ? 256 / cg : cap);
 }
 constexpr int BAND_THREADS = 256;
-constexpr int GRID_CHUNK = 4096;       // grid points per reduction CTA
+constexpr int GRID_CHUNK = 4096;       // grid points per CTA of the local forces
 constexpr int RR_THREADS = 1024;
 constexpr int RR_CLUSTER = 8;          // CTAs of the cluster Rayleigh-Ritz (large subspaces)
 constexpr int LF_GROUP = 4;            // atoms per local-force CTA
@@ -259,12 +259,12 @@ void launch_gga_div(const Launch& L);
 template <typename T> void launch_potential_g(const Launch& L);
 void launch_vion_g(const Launch& L);
 void launch_rho0_g(const Launch& L);
-void launch_pulay_store(const Launch& L);
 void launch_pulay_mix(const Launch& L, double a, double q0);
-template <typename T> void launch_grid_energies(const Launch& Lchunks, double* part, int maxchunk);
-void launch_grid_energies_reduce(const Launch& L, const double* part, int maxchunk);
-void launch_finish_iteration(const Launch& L, double tol_e, double tol_rho, int count_iter);
-void launch_pulay_gram(const Launch& Lchunks, double* part, int maxchunk, int hist);
+// (part: [problem][maxchunk][8], maxchunk chunks of GRID_EW_POINTS at most)
+template <typename T> void launch_grid_energies(const Launch& L, double* part, int maxchunk);
+void launch_finish_iteration(const Launch& L, const double* part, int maxchunk, double tol_e, double tol_rho,
+                             int count_iter);
+void launch_pulay_gram(const Launch& L, double* part, int maxchunk, int hist);
 void launch_pulay_solve(const Launch& L, const double* part, int maxchunk, int hist);
 template <typename T> void launch_build_projectors(const Launch& Latoms, int deriv);
 void launch_local_forces(const Launch& Latom_chunks, int maxchunk);

@@ -261,6 +261,56 @@ __device__ __forceinline__ double warp_sum(double v) {
   return v;
 }
 
+// Sums over W consecutive lanes of R values per lane.  Pairs of values are folded into one
+// register per exchange (the lanes on either side of a bit keep one value each), so that R sums
+// cost about R + log2 W shuffles and adds instead of R log2 W: on return a lane holds the sum of
+// value fold_index(lane).
+template <int R>
+__host__ __device__ constexpr int fold_bits() { return R > 8 ? 4 : R > 4 ? 3 : R > 2 ? 2 : R > 1 ? 1 : 0; }
+template <typename T, int R, int W>
+__device__ __forceinline__ T fold_sums(const T (&in)[R], int lane) {
+  constexpr int B = fold_bits<R>(), N = 1 << B;
+  T v[N];
+#pragma unroll
+  for (int i = 0; i < N; ++i) v[i] = i < R ? in[i < R ? i : 0] : T(0);
+  int o = W / 2;
+#pragma unroll
+  for (int b = 0; b < B; ++b, o >>= 1) {
+    const bool up = (lane & o) != 0;
+    const int h = N >> (b + 1);
+#pragma unroll
+    for (int i = 0; i < N; ++i)
+      if (i < h) {
+        const T keep = up ? v[i + h] : v[i], give = up ? v[i] : v[i + h];
+        v[i] = keep + __shfl_xor_sync(0xffffffffu, give, o);
+      }
+  }
+#pragma unroll
+  for (; o > 0; o >>= 1) v[0] = v[0] + __shfl_xor_sync(0xffffffffu, v[0], o);
+  return v[0];
+}
+constexpr int log2i(int w) { return w <= 1 ? 0 : 1 + log2i(w / 2); }
+// shift from a lane of the W to the value it holds (the first lane that holds value a is a << it)
+template <int R, int W>
+__host__ __device__ constexpr int fold_shift() { return log2i(W) - fold_bits<R>(); }
+
+// Sums of up to 8 values per thread over a block of 256, in tot[8] (shared, valid after the call);
+// red: 64 doubles of shared memory.  Nine additions per warp instead of 40: FP64 additions are what
+// the reductions of the grid kernels cost.
+__device__ __forceinline__ void block_sums8(const double (&v)[8], double* red, double* tot) {
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  const double s = fold_sums<double, 8, 32>(v, lane);
+  constexpr int S = fold_shift<8, 32>();
+  if ((lane & ((1 << S) - 1)) == 0) red[w * 8 + (lane >> S)] = s;
+  __syncthreads();
+  if (threadIdx.x < 8) {
+    double t = 0.0;
+    for (int k = 0; k < 8; ++k) t += red[k * 8 + threadIdx.x];
+    tot[threadIdx.x] = t;
+  }
+  __syncthreads();
+}
+
 // Sum over the block; every thread gets the result.  red: >= 33 doubles of shared memory.
 __device__ __forceinline__ double block_sum(double v, double* red) {
   int lane = threadIdx.x & 31, w = threadIdx.x >> 5, nw = (blockDim.x + 31) >> 5;

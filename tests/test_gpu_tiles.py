@@ -133,3 +133,32 @@ def test_subspace_eigensolve_per_launch(sgo, members, precision, bands):
     two, many = run(2), run(members)
     assert two[0] == many[0]
     assert np.array_equal(two[1], many[1])
+
+
+# ring lengths of the mixing (a 2 x 2 system, a ring that wraps, the longest), a grid of less than one
+# chunk of the reductions and one of several
+@pytest.mark.parametrize("hist", [1, 2, 5, 8])
+@pytest.mark.parametrize("grid", [(9, 10, 9), (18, 20, 20)])
+def test_mixing_history(sgo, hist, grid):
+    """The converged F does not depend on the ring's length: second order in the density error of
+    1e-7 per electron, so below 1e-9."""
+    st = dataclasses.replace(workloads.tiny(nat=2, ecut=1.2, kT=0.01), fft=grid)
+    F = [sgo.Context(st, precision="fp64", pulay_hist=h, max_scf=200, scf_tol_rho=1e-7, scf_tol_e=1e-9).energy_forces()[0]
+         for h in (hist, 4)]
+    assert abs(F[0] - F[1]) < 1e-9
+
+
+# bands that one lane holds and several, levels far apart and close together against kT
+@pytest.mark.parametrize("nbands", [5, 33, 70])
+@pytest.mark.parametrize("kT", [1e-4, 0.02, 0.5])
+def test_occupations(sgo, nbands, kT):
+    """Sum f = N_el (1e-13 N_el is the iteration's rule) and one mu for every partly filled band: from
+    f = 2 / (1 + exp(u)), u = ln(2 / f - 1) is known to 2e-16 / (f (2 - f)), 1e-9 kT where f (2 - f) > 1e-6."""
+    st = _with_bands(workloads.tiny(nat=2, ecut=6.0, kT=kT), nbands)
+    ctx = sgo.Context(st, precision="fp64", max_scf=3, extra_bands=0)
+    ctx.energy_forces(check=False)
+    eps, occ = ctx.eigen()
+    assert abs(occ.sum() - 8.0) < 1e-11
+    part = occ * (2.0 - occ) > 1e-6
+    mu = (eps - kT * np.log(2.0 / occ.clip(1e-300) - 1.0))[part] if part.any() else np.zeros(1)
+    assert np.ptp(mu) < 1e-9 * max(1.0, kT) + 1e-12
