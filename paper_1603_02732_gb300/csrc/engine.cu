@@ -870,7 +870,7 @@ Engine::Engine(const std::vector<sgo_ctx*>& ctxs, cudaStream_t stream) : ctx_(ct
       return;
     }
     c_plane.push_back(preg || ppair || pp.pbig ? 0 : d.npair * d.n3);
-    c_dens.push_back(dreg || dpair || pp.dbig ? 0 : d.n3);
+    c_dens.push_back(dreg || dpair || pp.dbig ? 0 : DENS_CLUSTER * d.n3);
     c_bigy.push_back(pp.pbig ? big_y_ctas(d.npair, d.n3, d.m1max) : 0);
     c_bigx.push_back(pp.pbig ? big_x_ctas(d.npair, d.n3, d.n2) : 0);
     c_bigdy.push_back(pp.dbig ? big_y_ctas(d.npair, d.n3, d.m1max) : 0);

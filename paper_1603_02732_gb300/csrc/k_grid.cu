@@ -444,7 +444,7 @@ __device__ __forceinline__ void chunk_sums(const Prob& P, const double* part, do
 
 // Grid sums, band terms, total free energy, convergence test.  One CTA of 256 threads per problem.
 // (One thread summing the chunks and one thread per band summing its projectors took 18 + 13 us for
-// the 24-atom layer and 18 + 42 us for 32 atoms with p channels; now 14 and 20 us.)
+// the 24-atom layer and 18 + 42 us for 32 atoms with p channels; now 15 and 25 us.)
 __global__ void k_finish_iteration(KArgs ka, const double* part, int maxchunk, double tol_e, double tol_rho,
                                    int count_iter) {
   __shared__ double red[33], redc[32][NRED + 1], tot[NRED];

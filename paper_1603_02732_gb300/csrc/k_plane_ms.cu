@@ -71,10 +71,6 @@ __host__ __device__ inline int ms_q(int n1, int n2, int n3) {
 }
 
 // Density pass: whole rows plus the float-float sums of a plane
-// CTAs that share a block of planes.  Measured with 2 / 4 / 8: 24-atom layer 73 / 47 / 56 us, 13-atom
-// cluster 136 / 90 / 109, folded 2x2x2 mesh 180 / 116 / 125, 8 members of 8 atoms 34 / 28 / 38, 64
-// members 657 / 723 / 967 (21 members, a sub-batch: 315 / 317 / 396), 8-atom crystal 26 / 18 / 15.
-constexpr int DENS_CLUSTER = 4;
 __host__ __device__ inline size_t ms_dens_plane_bytes(int n1, int n2) {
   return (size_t)n1 * (n2 | 1) * 8 + (size_t)n1 * n2 * 8;
 }
@@ -400,7 +396,7 @@ __global__ void __launch_bounds__(PLANE_MS_THREADS, PLANE_MS_MINB) k_plane_vpsi_
 // one FP64 addition per point and band pair alone would take as long as the whole pass.
 // Before, one CTA per block of planes looped over all band pairs, a thread per line (255 registers,
 // one CTA per SM, FP64 sums): the 24-atom layer 367 us, the 72^3 cluster 702 us, the folded mesh
-// 1188 us, 64 members 1370 us (now: at DENS_CLUSTER).
+// 1188 us, 64 members 1370 us (now: at DENS_CLUSTER in kernels.h).
 __global__ void __launch_bounds__(PLANE_MS_THREADS, PLANE_MS_MINB) k_plane_density_ms(KArgs ka, const double* occ_override) {
   namespace cg = cooperative_groups;
   cg::cluster_group cluster = cg::this_cluster();
