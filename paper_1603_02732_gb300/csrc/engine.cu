@@ -716,7 +716,13 @@ WorkMap Engine::make_map(const std::vector<int>& counts) {
 
 // Maps of the GEMMs whose CTA counts follow the tile knobs.
 void Engine::build_gemm_maps() {
-  std::vector<int> ww, bw, dw, tc, nntc, red[3][2];
+  std::vector<int> ww, bw, dw, tc, nntc[2], red[3][2];
+  // tiles per NN CTA: at most the knob, fewer while one launch has less than a CTA per SM (one matrix
+  // pair or four; each CTA's fixed part, the image and the barriers, is worth about four tiles).  The
+  // sums do not depend on it.  24-atom layer, 15 CTAs per pair at the knob's 4: 21 -> 13 us a launch
+  int tiles = 0;
+  for (auto* c : ctx_) tiles += div_up(c->d.npw, 128);
+  for (int k = 0; k < 2; ++k) nn_tiles_[k] = std::min(nn_tpc_, div_up(tiles * (k ? 4 : 1), 152));
   for (auto* c : ctx_) {
     const Prob& d = c->d;
     const int nsplit = div_up(d.npw, tn_kc_ > 0 ? tn_kc_ : tn_kc_f64(d.npw));
@@ -725,7 +731,7 @@ void Engine::build_gemm_maps() {
     bw.push_back(ta * tw * nsplit);
     dw.push_back(td * tw * nsplit);
     tc.push_back(div_up(d.npw, tc_kc_));
-    nntc.push_back(div_up(div_up(d.npw, 128), nn_tpc_));
+    for (int k = 0; k < 2; ++k) nntc[k].push_back(div_up(div_up(d.npw, 128), nn_tiles_[k]));
     const int nin[3] = {d.nb, d.nproj, 3 * d.nproj};
     for (int k = 0; k < 3; ++k)
       for (int t = 0; t < 2; ++t)
@@ -733,7 +739,8 @@ void Engine::build_gemm_maps() {
   }
   // one buffer and one copy for all of them (the autotuner rebuilds them for every candidate)
   std::vector<std::pair<WorkMap*, const std::vector<int>*>> maps = {
-      {&m_tn_[OPK_WB], &ww}, {&m_tn_[OPK_B], &bw}, {&m_tn_[OPK_DB], &dw}, {&m_tc_, &tc}, {&m_nntc_, &nntc}};
+      {&m_tn_[OPK_WB], &ww}, {&m_tn_[OPK_B], &bw}, {&m_tn_[OPK_DB], &dw}, {&m_tc_, &tc},
+      {&m_nntc_[0], &nntc[0]}, {&m_nntc_[1], &nntc[1]}};
   for (int k = 0; k < 3; ++k)
     for (int t = 0; t < 2; ++t) maps.push_back({&m_red_[k][t], &red[k][t]});
   const size_t len = ctx_.size() + 1;
@@ -1208,8 +1215,9 @@ void Engine::nn_pairs(int akind, const RolePairs& rp, int msel, double alpha, do
   tbeg(kind);
   if (sizeof(T) == 4 && nn_tc_ok_[akind]) {
     if (!image_ready) launch_nn_image(L(m_prob_), akind, msel, d_nnimg_, nnimg_stride_);
-    launch_gemm_nn_tc(L(m_nntc_), d_tmaps_, d_nnimg_, nnimg_stride_, nnimg_max_[akind], akind, rp, alpha, beta,
-                      nn_tpc_);
+    const int k = rp.n > 1;
+    launch_gemm_nn_tc(L(m_nntc_[k]), d_tmaps_, d_nnimg_, nnimg_stride_, nnimg_max_[akind], akind, rp, alpha, beta,
+                      nn_tiles_[k]);
   } else {
     launch_gemm_nn<T>(L(m_nn_), akind, rp, msel, alpha, beta);
   }

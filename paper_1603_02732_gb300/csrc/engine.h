@@ -186,7 +186,7 @@ class Engine {
   std::vector<void*> allocs_;
   int max_n1_ = 0, max_n2_ = 0, max_n3_ = 0, max_n12_ = 0, max_nb_ = 0, plane_threads_ = 128;
   WorkMap m_zcol_, m_plane_, m_dens_, m_gz_, m_gp_, m_gew_, m_bands_, m_tn_[3], m_red_[3][2], m_asm_,
-      m_nn_, m_atoms_, m_projs_, m_atomch_, m_ewsg_, m_prob_, m_tc_, m_nntc_;
+      m_nn_, m_atoms_, m_projs_, m_atomch_, m_ewsg_, m_prob_, m_tc_, m_nntc_[2];
   WorkMap m_preg_[2], m_dreg_[2], m_zreg_[2];  // register-FFT plane / column kernels, per size class
   size_t preg_smem_[2] = {0, 0}, dreg_smem_[2] = {0, 0}, zreg_smem_[2] = {0, 0};
   WorkMap m_ppair_, m_dpair_, m_zpair_;         // lane-pair register FFT kernels (lengths 96-128)
@@ -234,6 +234,7 @@ class Engine {
   bool use_graph_ = false;
   // GEMM tile knobs: K chunk of the tensor-core TN, 128-wave tiles per NN CTA, K chunk of
   // the CUDA-core TN; the maps that depend on them
+  int nn_tiles_[2] = {NN_TPC, NN_TPC};  // tiles per NN CTA (see build_gemm_maps): one role pair, several
   int tc_kc_ = TC_KC, nn_tpc_ = NN_TPC, tn_kc_ = TN_KC;  // (tn_kc_ 0 on the FP64 path: tn_kc_f64)
   void build_gemm_maps();
   int* d_gmaps_ = nullptr;      // their start indices

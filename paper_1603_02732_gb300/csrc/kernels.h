@@ -84,9 +84,10 @@ enum { DD_S = 0, DD_HS, DD_CM, DD_TM, DD_PROJ, DD_DPROJ, DD_PROJ_D };
 template <typename T> void launch_wave_to_cols(const Launch& L, int src);
 template <typename T> void launch_cols_to_wave(const Launch& L, int src, int dst);
 template <typename T> void launch_plane_vpsi(const Launch& L);
-// CTAs of the density pass that share a plane or a block of planes.  Measured (k_plane_ms.cu) with 2 / 4 / 8: 24-atom layer 73 / 47 / 56 us, 13-atom
-// cluster 136 / 90 / 109, folded 2x2x2 mesh 180 / 116 / 125, 8 members of 8 atoms 34 / 28 / 38, 64
-// members 657 / 723 / 967 (21 members, a sub-batch: 315 / 317 / 396), 8-atom crystal 26 / 18 / 15.
+// CTAs of the density pass that share a plane or a block of planes.  Measured (k_plane_ms.cu) with
+// 2 / 4 / 8: 24-atom layer 73 / 47 / 56 us, 13-atom cluster 136 / 90 / 109, folded 2x2x2 mesh 180 /
+// 116 / 125, 8 members of 8 atoms 34 / 28 / 38, 64 members 657 / 723 / 967 (21 members, a sub-batch:
+// 315 / 317 / 396), 8-atom crystal 26 / 18 / 15.
 constexpr int DENS_CLUSTER = 4;
 template <typename T> void launch_plane_density(const Launch& L, const double* occ_override);
 // grid transforms of the work grids (T = double; T = float views the first half of the

@@ -44,6 +44,22 @@ def test_subspace_products_at_tile_edges(sgo, name, bands, precision, tol):
     assert (np.abs(out - ref) / (1.5 * (np.abs(m).T @ np.abs(x)) + 0.5 * np.abs(y))).max() <= tol
 
 
+# the tensor-core rotation: one tile of plane waves and many, output bands on either side of the 16s and
+# 32s of the matrix image, the largest
+@pytest.mark.parametrize("name,bands", [("tiny", 5), ("tiny", 16), ("tiny", 17), ("tiny", 33), ("tiny", 124), ("de", 81), ("layer", 49)])
+def test_block_update_tensor_cores(sgo, name, bands):
+    """Y <- alpha M^T X + beta Y in 3xTF32, relative to the sums of magnitudes: the split keeps 21 bits of
+    each factor and drops lo lo, 4e-7, and FP32 sums of up to 124 terms add 1e-6 at most."""
+    base = dict(tiny=workloads.tiny(nat=2, ecut=6.0), de=workloads.de_candidate(44), layer=workloads.honeycomb24())[name]
+    ctx = sgo.Context(_with_bands(base, bands), precision="mixed")
+    rng = np.random.default_rng(32)
+    x, y = rng.normal(size=(2, bands, ctx.npw))
+    m = rng.normal(size=(bands, bands))
+    out = ctx.block_update(x, m, -1.5, 0.5, y)
+    ref = -1.5 * (m.T @ x) + 0.5 * y
+    assert (np.abs(out - ref) / (1.5 * (np.abs(m).T @ np.abs(x)) + 0.5 * np.abs(y))).max() <= 2e-6
+
+
 # carried bands (requested + 4 + requested / 32): one leaf and two of the divide and conquer, the
 # edges of every size class, the largest subspace of one CTA, and beyond it in FP64
 @pytest.mark.parametrize("carried", [9, 16, 17, 32, 33, 64, 65, 96, 97, 128, 129, 184])
