@@ -88,6 +88,7 @@ class Engine {
   sgo_status grid_transform(int sign, const double* in, double* out);
   sgo_status subspace(int nvec, const double* x, const double* y, double* c);
   sgo_status block_update(int nvec, const double* x, const double* m, double alpha, double beta, double* y);
+  void projector_terms();
   sgo_status structure_terms();
   // Live CUDA-event timing of one kernel class (see kTimerNames) over subsequent runs.
   bool timer_select(const char* name);
