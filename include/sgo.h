@@ -127,10 +127,10 @@ typedef struct {
                              requested bands get headroom; occupations, eigenvalues, energies and
                              the eig_tol test cover the requested bands only (-1, default:
                              4 + nbands / 32; 0 = none) */
-  int rr_cluster;         /* subspace diagonalisation kernel: -1 (default) or 0 one CTA per member up
-                             to 184 bands (FP64: 128), beyond a thread-block cluster of 8 CTAs per
-                             member; 1 = always the cluster.  Taken from the first member of a
-                             batch. */
+  int rr_cluster;         /* subspace diagonalisation kernel: -1 (default) or 0 the tridiagonal one
+                             (one CTA or a small cluster per member) up to 184 bands (FP64: 128),
+                             beyond it the Jacobi one on a cluster of 8 CTAs per member; 1 = always
+                             the latter.  Taken from the first member of a batch. */
   int eigensolver;        /* 0 (default): Algorithm 1's all-band CG steps (Sec. II D): per band a
                              preconditioned, conjugated, projected search direction, a line
                              minimisation, then a Rayleigh-Ritz over the n_b bands.  1: block
