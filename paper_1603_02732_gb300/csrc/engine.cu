@@ -8,6 +8,7 @@
 #include <cmath>
 #include <cstring>
 #include <mutex>
+#include <type_traits>
 #include <unordered_map>
 
 #include "engine.h"
@@ -856,11 +857,13 @@ Engine::Engine(const std::vector<sgo_ctx*>& ctxs, cudaStream_t stream) : ctx_(ct
     if (zreg) zreg_smem_[zreg_class(d.n3)] = std::max(zreg_smem_[zreg_class(d.n3)], zreg_smem(d.n3));
     c_zpair.push_back(zpair ? zpair_ctas(d.ncp, d.npair) : 0);
     if (zpair) zpair_smem_ = std::max(zpair_smem_, zpair_smem(d.n3));
-    // FP64 grid transforms: a whole plane per CTA when two planes fit in shared memory,
-    // otherwise line blocks along x and y
-    // (all of it only for grids with a length that has no such transform, see k_grid_axis)
+    // grid transforms: the FP64 path one axis a launch where every length has short factors
+    // (k_grid_axis); else, and on the mixed path, a whole plane per CTA when two planes fit in
+    // shared memory, line blocks along x and y when they do not.  (The mixed path's results are
+    // pinned to the bits of these kernels: its SCF stops near the FP32 floor, where any other
+    // rounding moves the stop of one small metallic cluster in eight and its forces by 1e-5 to 3e-5.)
     int fa, fb, fc;
-    const bool gaxis = grid_factors(d.n1, &fa, &fb, &fc) && grid_factors(d.n2, &fa, &fb, &fc) &&
+    const bool gaxis = precision_ == 0 && grid_factors(d.n1, &fa, &fb, &fc) && grid_factors(d.n2, &fa, &fb, &fc) &&
                        grid_factors(d.n3, &fa, &fb, &fc);
     const bool gbig = !gaxis && (size_t)(2 * d.n1 * d.n2 + d.n1 + d.n2) * 16 > 220 * 1024;
     for (int k = 0; k < 3; ++k) c_gaxis[k].push_back(gaxis ? grid_axis_ctas(d.n1, d.n2, d.n3, k) : 0);
@@ -1165,11 +1168,12 @@ void Engine::grid_fft(int which, int sign, int real_src) {
 template <typename T>
 void Engine::grid_fft_raw(int which, int sign, int real_src) {
   // forward: y, x, z; inverse: z, x, y
-  for (int k = 0; k < 3; ++k) {
-    const int axis = sign < 0 ? (k == 0 ? 1 : k == 1 ? 0 : 2) : (k == 0 ? 2 : k == 1 ? 0 : 1);
-    launch_grid_axis<T>(L(m_gaxis_[axis]), which, sign, axis, k, real_src != 0);
-  }
-  // grids with a length that has no such transform: planes (y, x), large ones by line
+  if constexpr (std::is_same_v<T, double>)
+    for (int k = 0; k < 3; ++k) {
+      const int axis = sign < 0 ? (k == 0 ? 1 : k == 1 ? 0 : 2) : (k == 0 ? 2 : k == 1 ? 0 : 1);
+      launch_grid_axis(L(m_gaxis_[axis]), which, sign, axis, k == 0 && real_src != 0);
+    }
+  // the mixed path, and grids with a length that has no such transform: planes (y, x), large ones by line
   // blocks, and z lines
   auto planes = [&](int sg) {
     launch_grid_plane_fft<T>(L(m_gp_), which, sg);

@@ -298,9 +298,7 @@ __global__ void __launch_bounds__(PLANE_THREADS, sizeof(T) == 4 ? PLANE_MIN_BLOC
 // Full FP64 complex grid transforms (in place): plane pass (x and y) and z pass.
 // which: 0 = gfft, 1 = gfft2, 2 = gfft3, 3 = gfft4 (the PBE grids).
 // ---------------------------------------------------------------------------
-// The work grids in the storage precision of a transform: FP64 complex (double and
-// float-float), or (FP32) the first half of the same memory viewed as single-precision
-// complex.
+// The work grids in the storage precision of a transform: FP64 complex (double and float-float).
 template <typename T>
 __device__ __forceinline__ cplx<typename Work<T>::S>* grid_of(const Prob& P, int which) {
   double2* const g[4] = {P.gfft, P.gfft2, P.gfft3, P.gfft4};
@@ -357,83 +355,71 @@ __global__ void __launch_bounds__(ZCOL_THREADS) k_grid_z_fft(KArgs ka, int which
 }
 
 // ---------------------------------------------------------------------------
-// Grid transform along one axis, lengths N = A B C with short DFTs (grid_factors; B = 1 where two
-// are enough).  With M = B C, W_n = exp(s 2 pi i / n):
+// FP64 grid transform along one axis (FP64 path), lengths N = A B C with short DFTs (grid_factors;
+// B = 1 where two are enough).  With M = B C, W_n = exp(s 2 pi i / n):
 //   step 1, group g < M:      Y[M k1 + g] = W_N^(g k1) sum_{n1 < A} x[M n1 + g] W_A^(n1 k1)
 //   step 2, (k1 < A, h < C):  Z[M k1 + C k2 + h] = W_M^(h k2) sum_{n2 < B} Y[M k1 + C n2 + h] W_B^(n2 k2)
 //   step 3, (k1 < A, k2 < B): X[k1 + A (k2 + B k3)] = sum_{h < C} Z[M k1 + C k2 + h] W_C^(h k3)
-// CTA = (problem, GA_LINES lines): step 1 reads global memory, step 3 writes it, the lines stay in
-// shared memory in between.  Between the axes of a float-float transform the grid holds the float
-// pairs themselves: converting FP64 takes four FP64-rate instructions a value (MODE, a template
-// parameter so that no conversion is executed and then not used).
-// Bound by latency and instruction fetch (about 250 FP32 instructions a point and axis in
-// float-float, straight-line code per DFT), so short DFTs, whose code stays in the instruction
-// cache, few registers and many small CTAs: 648 for one axis of a 72^3 grid.  A whole transform,
-// against the kernels below (one CTA a plane, then blocks of z lines, general radix loops):
-// 72^3 123 -> 69 us, a 24-atom layer 87 -> 49, 8 atoms 51 -> 31, 64 structures in a batch
-// 537 -> 427 (FP64: the layer 85 -> 50, 8 atoms 43 -> 27).  Two steps with DFTs up to 16 took
-// 118 us and 760 us for the first and the batch, 13 % of the issue slots used; 16 lines a CTA
-// 74 and 354; 64 threads 76 and 403; 64 registers 69 and 411.
+// CTA = (problem, GA_LINES lines): step 1 reads global memory (REAL: rho_out instead of the grid),
+// step 3 writes it, the lines stay in shared memory in between.
+// Bound by the FP64 lanes and by latency, so many small CTAs; short DFTs, whose straight-line code
+// stays in the instruction cache, and few registers.  A whole transform, against the kernels above
+// (one CTA a plane, then blocks of z lines): 24-atom layer 85 -> 50 us, 8 atoms 43 -> 27.
+// The mixed path stays with those: its results are pinned to the bits of their radix order (see
+// Engine::Engine).
 // ---------------------------------------------------------------------------
 constexpr int GA_LINES = 8;      // lines per CTA
 constexpr int GA_THREADS = 128;
-enum { GA_FIRST = 0, GA_FIRST_REAL = 1, GA_MIDDLE = 2, GA_LAST = 3 };
 
-template <typename T, int MODE>
+template <bool REAL>
 struct GridAxis {
-  cplx<typename Work<T>::S>* g;  // the grid
-  const double* real;            // GA_FIRST_REAL: a real source instead (imaginary part 0)
-  cplx<T>* tile;                 // [GA_LINES][stride]
-  const cplx<T>* roots;          // exp(-2 pi i t / N)
-  T sg;
+  cplx<double>* g;            // the grid
+  const double* real;         // REAL: the source of step 1 (imaginary part 0)
+  cplx<double>* tile;         // [GA_LINES][stride]
+  const cplx<double>* roots;  // exp(-2 pi i t / N)
+  double sg;
   int a, b, c, stride, estep;
   bool fwd;
-  __device__ __forceinline__ cplx<T> load(size_t i) const {
-    using S = typename Work<T>::S;
-    if constexpr (MODE == GA_FIRST_REAL) return Work<T>::in(mk((S)real[i], (S)0));
-    else if constexpr (MODE == GA_FIRST) return Work<T>::in(g[i]);
-    else return *reinterpret_cast<const cplx<T>*>(g + i);
+  __device__ __forceinline__ cplx<double> load(size_t i) const {
+    if constexpr (REAL) return mk(real[i], 0.0);
+    else return g[i];
   }
-  __device__ __forceinline__ void store(size_t i, cplx<T> v) const {
-    if constexpr (MODE == GA_LAST) g[i] = Work<T>::out(v);
-    else *reinterpret_cast<cplx<T>*>(g + i) = v;
-  }
-  __device__ __forceinline__ cplx<T> twiddle(cplx<T> v, int t) const {
-    const cplx<T> w = roots[t];
+  __device__ __forceinline__ cplx<double> twiddle(cplx<double> v, int t) const {
+    const cplx<double> w = roots[t];
     return v * (fwd ? w : conj(w));
   }
 };
 
-template <int R, typename T, int MODE>
-__device__ __forceinline__ void axis_step1(const GridAxis<T, MODE>& x, size_t base, int l, int g) {
+template <int R, bool REAL>
+__device__ __forceinline__ void axis_step1(const GridAxis<REAL>& x, size_t base, int l, int g) {
   const int m = x.b * x.c;
-  cplx<T> v[R];
+  cplx<double> v[R];
 #pragma unroll
   for (int k = 0; k < R; ++k) v[k] = x.load(base + (size_t)(m * k + g) * x.estep);
-  if constexpr (R > 1) Bfly<T, R>::run(v, x.sg, x.roots, m);
-  cplx<T>* o = x.tile + l * x.stride + g;
+  if constexpr (R > 1) Bfly<double, R>::run(v, x.sg, x.roots, m);
+  cplx<double>* o = x.tile + l * x.stride + g;
 #pragma unroll
   for (int k = 0; k < R; ++k) o[m * k] = k > 0 && g > 0 ? x.twiddle(v[k], g * k) : v[k];
 }
-template <int R, typename T, int MODE>
-__device__ __forceinline__ void axis_step2(const GridAxis<T, MODE>& x, int l, int k1, int h) {
-  cplx<T>* o = x.tile + l * x.stride + x.b * x.c * k1 + h;
-  cplx<T> v[R];
+template <int R, bool REAL>
+__device__ __forceinline__ void axis_step2(const GridAxis<REAL>& x, int l, int k1, int h) {
+  cplx<double>* o = x.tile + l * x.stride + x.b * x.c * k1 + h;
+  cplx<double> v[R];
 #pragma unroll
   for (int k = 0; k < R; ++k) v[k] = o[x.c * k];
-  if constexpr (R > 1) Bfly<T, R>::run(v, x.sg, x.roots, x.a * x.c);
+  if constexpr (R > 1) Bfly<double, R>::run(v, x.sg, x.roots, x.a * x.c);
 #pragma unroll
   for (int k = 0; k < R; ++k) o[x.c * k] = k > 0 && h > 0 ? x.twiddle(v[k], x.a * h * k) : v[k];
 }
-template <int R, typename T, int MODE>
-__device__ __forceinline__ void axis_step3(const GridAxis<T, MODE>& x, size_t base, int l, int k1, int k2) {
-  cplx<T> v[R];
-  const cplx<T>* in = x.tile + l * x.stride + R * (x.b * k1 + k2);
+template <int R, bool REAL>
+__device__ __forceinline__ void axis_step3(const GridAxis<REAL>& x, size_t base, int l, int k1, int k2) {
+  cplx<double> v[R];
+  const cplx<double>* in = x.tile + l * x.stride + R * (x.b * k1 + k2);
 #pragma unroll
   for (int k = 0; k < R; ++k) v[k] = in[k];
-  if constexpr (R > 1) Bfly<T, R>::run(v, x.sg, x.roots, x.a * x.b);
+  if constexpr (R > 1) Bfly<double, R>::run(v, x.sg, x.roots, x.a * x.b);
 #pragma unroll
-  for (int k = 0; k < R; ++k) x.store(base + (size_t)(k1 + x.a * (k2 + x.b * k)) * x.estep, v[k]);
+  for (int k = 0; k < R; ++k) x.g[base + (size_t)(k1 + x.a * (k2 + x.b * k)) * x.estep] = v[k];
 }
 
 #define SGO_GRID_RADIX(r, F, ...)    \
@@ -449,7 +435,7 @@ __device__ __forceinline__ void axis_step3(const GridAxis<T, MODE>& x, size_t ba
   }
 
 // axis 0: x, 1: y (contiguous), 2: z
-template <typename T, int MODE>
+template <bool REAL>
 __global__ void __launch_bounds__(GA_THREADS, 7) k_grid_axis(KArgs ka, int which, int sign, int axis) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const int p = locate(ka.start, ka.nprob, blockIdx.x);
@@ -457,18 +443,18 @@ __global__ void __launch_bounds__(GA_THREADS, 7) k_grid_axis(KArgs ka, int which
   const Prob& P = ka.probs[p];
   const int n1 = P.n1, n2 = P.n2, n12 = n1 * n2;
   const int n = axis == 0 ? n1 : axis == 1 ? n2 : P.n3, nl = P.ngrid / n;
-  GridAxis<T, MODE> x;
+  GridAxis<REAL> x;
   grid_factors(n, &x.a, &x.b, &x.c);
-  x.g = grid_of<T>(P, which);
+  x.g = grid_of<double>(P, which);
   x.real = P.rho_out;
   x.stride = n | 1;
-  x.tile = reinterpret_cast<cplx<T>*>(smem_raw);
-  cplx<T>* roots = x.tile + GA_LINES * x.stride;
+  x.tile = reinterpret_cast<cplx<double>*>(smem_raw);
+  cplx<double>* roots = x.tile + GA_LINES * x.stride;
   x.roots = roots;
-  x.sg = sign < 0 ? T(-1) : T(1);
+  x.sg = sign < 0 ? -1.0 : 1.0;
   x.fwd = sign < 0;
   x.estep = axis == 0 ? n2 : axis == 1 ? 1 : n12;
-  load_roots<T>(roots, P, axis == 0 ? 0 : axis == 1 ? n1 : n1 + n2, n);
+  load_roots<double>(roots, P, axis == 0 ? 0 : axis == 1 ? n1 : n1 + n2, n);
   __syncthreads();
   const int l0 = (blockIdx.x - ka.start[p]) * GA_LINES;
   // neighbouring threads on neighbouring addresses: along the line for y, across lines otherwise
@@ -761,17 +747,13 @@ int grid_axis_ctas(int n1, int n2, int n3, int axis) {
   const int n = axis == 0 ? n1 : axis == 1 ? n2 : n3;
   return (n1 * n2 * n3 / n + GA_LINES - 1) / GA_LINES;
 }
-template <typename T>
-void launch_grid_axis(const Launch& L, int which, int sign, int axis, int step, bool real_src) {
+void launch_grid_axis(const Launch& L, int which, int sign, int axis, bool real_src) {
   if (!L.map.total) return;
   const int n = axis == 0 ? L.max_n1 : axis == 1 ? L.max_n2 : L.max_n3;
-  const size_t sm = (size_t)(GA_LINES * (n | 1) + GA_LINES + n) * sizeof(cplx<T>);
-  auto* fn = step == 2 ? k_grid_axis<T, GA_LAST> : step == 1 ? k_grid_axis<T, GA_MIDDLE>
-             : real_src ? k_grid_axis<T, GA_FIRST_REAL> : k_grid_axis<T, GA_FIRST>;
+  const size_t sm = (size_t)(GA_LINES * (n | 1) + GA_LINES + n) * sizeof(cplx<double>);
+  auto* fn = real_src ? k_grid_axis<true> : k_grid_axis<false>;
   fn<<<L.map.total, GA_THREADS, sm, L.stream>>>(L.ka, which, sign, axis);
 }
-template void launch_grid_axis<double>(const Launch&, int, int, int, int, bool);
-template void launch_grid_axis<ff>(const Launch&, int, int, int, int, bool);
 template <typename T>
 void launch_grid_plane_fft(const Launch& L, int which, int sign) {
   if (!L.map.total) return;
@@ -810,14 +792,8 @@ void fft_set_smem_limits(size_t bytes) {
   cudaFuncSetAttribute(k_big_x<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
   cudaFuncSetAttribute(k_big_density<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
   cudaFuncSetAttribute(k_big_density<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
-  cudaFuncSetAttribute(k_grid_axis<double, GA_FIRST>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
-  cudaFuncSetAttribute(k_grid_axis<double, GA_FIRST_REAL>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
-  cudaFuncSetAttribute(k_grid_axis<double, GA_MIDDLE>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
-  cudaFuncSetAttribute(k_grid_axis<double, GA_LAST>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
-  cudaFuncSetAttribute(k_grid_axis<ff, GA_FIRST>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
-  cudaFuncSetAttribute(k_grid_axis<ff, GA_FIRST_REAL>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
-  cudaFuncSetAttribute(k_grid_axis<ff, GA_MIDDLE>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
-  cudaFuncSetAttribute(k_grid_axis<ff, GA_LAST>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+  cudaFuncSetAttribute(k_grid_axis<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+  cudaFuncSetAttribute(k_grid_axis<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
   plane_vpsi_reg_set_smem_limits(bytes);
   plane_ms_set_smem_limits(bytes);
   zreg_set_smem_limits(bytes);

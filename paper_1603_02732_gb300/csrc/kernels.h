@@ -90,12 +90,11 @@ template <typename T> void launch_plane_vpsi(const Launch& L);
 // 315 / 317 / 396), 8-atom crystal 26 / 18 / 15.
 constexpr int DENS_CLUSTER = 4;
 template <typename T> void launch_plane_density(const Launch& L, const double* occ_override);
-// grid transforms of the work grids (T = double; T = float views the first half of the
-// same memory as single-precision complex)
-// T: float (FP32 grids), double (FP64), ff (float-float arithmetic on FP64 grids, ff.cuh)
+// grid transforms of the work grids, T: double, or ff (float-float arithmetic on FP64 grids, ff.cuh)
 struct ff;
 // n = a b c with short DFTs for each (b = 1 where two of at most 6 are enough), the largest factor as
-// small as possible: every smooth length up to 216 that the transforms meet
+// small as possible.  Of the lengths 2^i 3^j 5^k up to 729 only 250, 300, 375, 400, 450, 480, 500, 540,
+// 600, 625, 640, 675 and 720 have none.
 inline __host__ __device__ bool grid_factors(int n, int* a, int* b, int* c) {
   const int r[8] = {1, 2, 3, 4, 5, 6, 8, 9};
   for (int k = 0; k < 8; ++k)          // the largest factor, last
@@ -118,10 +117,9 @@ inline __host__ __device__ bool grid_factors(int n, int* a, int* b, int* c) {
   return false;
 }
 int grid_axis_ctas(int n1, int n2, int n3, int axis);
-// step 0, 1, 2: the first, second, third axis of a transform; real_src: the first one reads rho_out
-// (imaginary part 0) instead of the grid
-template <typename T> void launch_grid_axis(const Launch& L, int which, int sign, int axis, int step, bool real_src);
-// (grids with a length that has none: whole planes, z lines, or line blocks)
+// (FP64) real_src: reads rho_out (imaginary part 0) instead of the grid
+void launch_grid_axis(const Launch& L, int which, int sign, int axis, bool real_src);
+// (the mixed path, and grids with a length that has none: whole planes, z lines, or line blocks)
 template <typename T> void launch_grid_plane_fft(const Launch& L, int which, int sign);
 template <typename T> void launch_grid_z_fft(const Launch& L, int which, int sign);
 template <typename T> void launch_grid_line_fft(const Launch& L, int which, int sign, int axis);  // axis 0: x, 1: y
