@@ -23,7 +23,7 @@ FLAGS = ["-std=c++17", "-O3", "-lineinfo", "-Xcompiler", "-fPIC", "-Xcompiler", 
 # k_rr_td.cu writes its fused multiply-adds itself: a member's results must not depend on which
 # instantiation of the kernel its batch selects, and the compiler fuses them differently
 FILE_FLAGS = {"k_rr_td.cu": ["-fmad=false"]}
-SOURCES = ["k_fft.cu", "k_plane_vpsi.cu", "k_plane_ms.cu", "k_cols_reg.cu", "k_pair_reg.cu", "k_linalg.cu", "k_rr_td.cu", "k_grid.cu", "k_setup.cu", "engine.cu",
+SOURCES = ["k_fft.cu", "k_plane_vpsi.cu", "k_plane_ms.cu", "k_plane_density.cu", "k_cols_reg.cu", "k_pair_reg.cu", "k_linalg.cu", "k_rr_td.cu", "k_grid.cu", "k_setup.cu", "engine.cu",
            "capi.cu", "noalloc.cu", "k_gemm_tc.cu", "relax.cpp", "de.cpp"]
 
 

@@ -284,7 +284,7 @@ PlanePaths plane_paths(const Prob& d, int precision) {
   const size_t cap = 220 * 1024;
   PlanePaths q;
   q.preg = precision == 1 && plane_reg_ok(d.n1, d.n2) && plane_reg_smem(d.n1, d.n2, d.m1max) <= cap;
-  q.dreg = q.preg && plane_density_ms_smem(d.n1, d.n2, d.n3) <= cap;
+  q.dreg = q.preg && plane_density_reg_smem(d.n1, d.n2, d.m1max) <= cap;
   q.ppair = precision == 1 && !q.preg && pair_plane_ok(d.n1, d.n2) && pair_plane_smem(d.n1, d.n2, d.m1max) <= cap;
   q.dpair = q.ppair && pair_density_smem(d.n1, d.n2, d.m1max) <= cap;
   q.psmem = (size_t)(2 * d.n1 * d.n2 + d.n1 + d.n2) * 16 <= cap && d.n1 * d.n2 <= 8192;
@@ -880,7 +880,7 @@ Engine::Engine(const std::vector<sgo_ctx*>& ctxs, cudaStream_t stream) : ctx_(ct
       return;
     }
     c_plane.push_back(preg || ppair || pp.pbig ? 0 : d.npair * d.n3);
-    c_dens.push_back(dreg || dpair || pp.dbig ? 0 : DENS_CLUSTER * d.n3);
+    c_dens.push_back(dreg || dpair || pp.dbig ? 0 : (precision_ ? dens_cluster<float>() : dens_cluster<double>()) * d.n3);
     c_bigy.push_back(pp.pbig ? big_y_ctas(d.npair, d.n3, d.m1max) : 0);
     c_bigx.push_back(pp.pbig ? big_x_ctas(d.npair, d.n3, d.n2) : 0);
     c_bigdy.push_back(pp.dbig ? big_y_ctas(d.npair, d.n3, d.m1max) : 0);
@@ -893,12 +893,12 @@ Engine::Engine(const std::vector<sgo_ctx*>& ctxs, cudaStream_t stream) : ctx_(ct
       c_preg[k].push_back(pcls != k ? 0
                           : kPlaneMultiPass ? plane_ms_ctas(d.n1, d.n2, d.n3, d.npair)
                                             : plane_reg_ctas(d.n2, d.n3, d.npair));
-      c_dreg[k].push_back(dreg && pcls == k ? plane_density_ms_ctas(d.n1, d.n2, d.n3) : 0);
+      c_dreg[k].push_back(dreg && pcls == k ? plane_density_reg_ctas(d.n2, d.n3) : 0);
     }
     if (preg)
       preg_smem_[pcls] = std::max(preg_smem_[pcls], kPlaneMultiPass ? plane_ms_smem(d.n1, d.n2, d.n3)
                                                                     : plane_reg_smem(d.n1, d.n2, d.m1max));
-    if (dreg) dreg_smem_[pcls] = std::max(dreg_smem_[pcls], plane_density_ms_smem(d.n1, d.n2, d.n3));
+    if (dreg) dreg_smem_[pcls] = std::max(dreg_smem_[pcls], plane_density_reg_smem(d.n1, d.n2, d.m1max));
     c_gz.push_back(gaxis ? 0 : div_up(d.n1 * d.n2, QZ));
     c_gp.push_back(gaxis || gbig ? 0 : d.n3);
     c_gew.push_back(div_up(d.ngrid, GRID_EW_POINTS));
@@ -1462,7 +1462,7 @@ void Engine::density_energy(int mode) {
   wave_to_cols<T>(WB_X);
   tbeg(TK_PLANE_DENSITY);
   launch_plane_density<T>(L(m_dens_), nullptr);
-  for (int k = 0; k < 2; ++k) launch_plane_density_ms(L(m_dreg_[k]), dreg_smem_[k], nullptr);
+  for (int k = 0; k < 2; ++k) launch_plane_density_reg(L(m_dreg_[k]), k, dreg_smem_[k], nullptr);
   launch_plane_density_pair(L(m_dpair_), dpair_smem_, nullptr);
   launch_big_y<T>(L(m_bigdy_), 1, 1, nullptr);
   launch_big_density<T>(L(m_bigd_), nullptr);
@@ -1875,7 +1875,7 @@ sgo_status Engine::density(int nvec, const double* psi, const double* occ, doubl
     launch_copy_in<float>(L(m_bands_), WB_W, dpsi, nvec);
     wave_to_cols<float>(WB_W);
     launch_plane_density<float>(L(m_dens_), docc);
-    for (int k = 0; k < 2; ++k) launch_plane_density_ms(L(m_dreg_[k]), dreg_smem_[k], docc);
+    for (int k = 0; k < 2; ++k) launch_plane_density_reg(L(m_dreg_[k]), k, dreg_smem_[k], docc);
     launch_plane_density_pair(L(m_dpair_), dpair_smem_, docc);
     launch_big_y<float>(L(m_bigdy_), 1, 1, docc);
     launch_big_density<float>(L(m_bigd_), docc);

@@ -242,10 +242,10 @@ __global__ void __launch_bounds__(PLANE_THREADS, sizeof(T) == 4 ? PLANE_MIN_BLOC
 
 // ---------------------------------------------------------------------------
 // Per (problem, z): rho(r) = (1/Omega) sum_pairs f_a Re^2 + f_b Im^2, summed in FP64 in shared memory.
-// A cluster of DENS_CLUSTER CTAs takes a plane, CTA r of it the pairs r, r + DENS_CLUSTER, ...; their
+// A cluster of CL = dens_cluster<T>() CTAs takes a plane, CTA r of it the pairs r, r + CL, ...; their
 // sums are added in rank order through distributed shared memory, each CTA a share of the points.
-// Bound by the FP64 operations of the transforms (FP64 path).  One CTA a plane left most SMs idle:
-// FP64 24-atom layer 1020 -> 673 us, 8 atoms 215 -> 74 us, six members 1917 -> 1386 us.
+// FP64 path: bound by the FP64 operations of the transforms; one CTA a plane left most SMs idle
+// (24-atom layer 1020 -> 673 us, 8 atoms 215 -> 74 us, six members 1917 -> 1386 us).
 // ---------------------------------------------------------------------------
 template <typename T>
 __global__ void __launch_bounds__(PLANE_THREADS, sizeof(T) == 4 ? PLANE_MIN_BLOCKS : 2) k_plane_density(KArgs ka, const double* occ_override) {
@@ -255,7 +255,8 @@ __global__ void __launch_bounds__(PLANE_THREADS, sizeof(T) == 4 ? PLANE_MIN_BLOC
   const Prob& P = ka.probs[p];
   namespace cg = cooperative_groups;
   cg::cluster_group cluster = cg::this_cluster();
-  const int local = blockIdx.x - ka.start[p], z = local / DENS_CLUSTER, rank = local - z * DENS_CLUSTER;
+  constexpr int CL = dens_cluster<T>();
+  const int local = blockIdx.x - ka.start[p], z = local / CL, rank = local - z * CL;
   const int n1 = P.n1, n2 = P.n2, n12 = n1 * n2;
   cplx<T>* b0 = reinterpret_cast<cplx<T>*>(smem_raw);
   cplx<T>* b1 = b0 + n12;
@@ -268,7 +269,7 @@ __global__ void __launch_bounds__(PLANE_THREADS, sizeof(T) == 4 ? PLANE_MIN_BLOC
   for (int t = threadIdx.x; t < n12; t += blockDim.x) acc[t] = 0.0;
   const int mx = P.m1max;
   const LineMap rows{mx + 1, n1 - 2 * mx - 1};
-  for (int pair = rank; pair < P.npair; pair += DENS_CLUSTER) {
+  for (int pair = rank; pair < P.npair; pair += CL) {
     const double fa = occ[2 * pair];
     const double fb = (2 * pair + 1 < P.nb) ? occ[2 * pair + 1] : 0.0;
     if (fa == 0.0 && fb == 0.0) continue;  // uniform across the block
@@ -286,9 +287,9 @@ __global__ void __launch_bounds__(PLANE_THREADS, sizeof(T) == 4 ? PLANE_MIN_BLOC
   cluster.sync();
   const double io = 1.0 / P.omega;
   double* rho = P.rho_out + (size_t)z * n12;
-  for (int t = rank * blockDim.x + threadIdx.x; t < n12; t += DENS_CLUSTER * blockDim.x) {
+  for (int t = rank * blockDim.x + threadIdx.x; t < n12; t += CL * blockDim.x) {
     double s = cluster.map_shared_rank(acc, 0)[t];
-    for (int r = 1; r < DENS_CLUSTER; ++r) s += cluster.map_shared_rank(acc, r)[t];
+    for (int r = 1; r < CL; ++r) s += cluster.map_shared_rank(acc, r)[t];
     rho[t] = s * io;
   }
   cluster.sync();  // no CTA leaves while another may still read its sums
@@ -729,7 +730,7 @@ void launch_plane_density(const Launch& L, const double* occ_override) {
   cfg.stream = L.stream;
   cudaLaunchAttribute at[1];
   at[0].id = cudaLaunchAttributeClusterDimension;
-  at[0].val.clusterDim.x = DENS_CLUSTER;
+  at[0].val.clusterDim.x = dens_cluster<T>();
   at[0].val.clusterDim.y = 1;
   at[0].val.clusterDim.z = 1;
   cfg.attrs = at;
@@ -768,7 +769,7 @@ void launch_grid_z_fft(const Launch& L, int which, int sign) {
 }
 
 bool fft_reg_init() {
-  return plane_vpsi_reg_init() && zreg_init() && pair_reg_init() && plane_ms_init();
+  return plane_vpsi_reg_init() && plane_density_reg_init() && zreg_init() && pair_reg_init() && plane_ms_init();
 }
 
 void fft_set_smem_limits(size_t bytes) {
@@ -796,6 +797,7 @@ void fft_set_smem_limits(size_t bytes) {
   cudaFuncSetAttribute(k_grid_axis<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
   plane_vpsi_reg_set_smem_limits(bytes);
   plane_ms_set_smem_limits(bytes);
+  plane_density_reg_set_smem_limits(bytes);
   zreg_set_smem_limits(bytes);
   pair_reg_set_smem_limits(bytes);
 }

@@ -21,9 +21,6 @@
 // the occupied rows are read), times V_eff/N at (x, y), x forward (only the occupied rows are
 // written); y forward (transposed -> natural); the compact columns go back.  Rows are padded
 // to n2 | 1 entries so that threads walking down columns or across rows hit distinct banks.
-#include <cooperative_groups.h>
-
-#include "ff.cuh"
 #include "fft_reg.cuh"
 #include "kernels.h"
 
@@ -66,16 +63,6 @@ __host__ __device__ inline size_t ms_table_bytes(int n1, int n2) { return (size_
 constexpr size_t kMsPlaneBudget = PLANE_MS_BUDGET_KB * 1024;  // planes per CTA: as many as fit (at least one)
 __host__ __device__ inline int ms_q(int n1, int n2, int n3) {
   int q = (int)(kMsPlaneBudget / ms_plane_bytes(n1, n2));
-  q = q < 1 ? 1 : (q > 8 ? 8 : q);
-  return q < n3 ? q : n3;
-}
-
-// Density pass: whole rows plus the float-float sums of a plane
-__host__ __device__ inline size_t ms_dens_plane_bytes(int n1, int n2) {
-  return (size_t)n1 * (n2 | 1) * 8 + (size_t)n1 * n2 * 8;
-}
-__host__ __device__ inline int ms_dens_q(int n1, int n2, int n3) {
-  int q = (int)(kMsPlaneBudget / ms_dens_plane_bytes(n1, n2));
   q = q < 1 ? 1 : (q > 8 ? 8 : q);
   return q < n3 ? q : n3;
 }
@@ -164,9 +151,10 @@ __device__ __forceinline__ void ms_y_fwd(const MsPlanes& p) {
   __syncthreads();
 }
 
-// first pass of the x inverse (n1 = A B), one line per column of the CTA's planes, occupied rows in
+// x lines (n1 = A B), one per column of the CTA's planes: inverse (occupied rows in),
+// times V_eff / N, forward (occupied rows out)
 template <int A, int B>
-__device__ __forceinline__ void ms_x_inv1(const MsPlanes& p) {
+__device__ __forceinline__ void ms_x(const MsPlanes& p) {
   const int nl = p.nq * p.n2, P2 = p.P2;
   const float inv_nl = 1.f / (float)nl;
   for (int t = threadIdx.x; t < B * nl; t += blockDim.x) {
@@ -184,14 +172,6 @@ __device__ __forceinline__ void ms_x_inv1(const MsPlanes& p) {
     for (int k1 = 0; k1 < A; ++k1) col[(B * k1 + g) * P2] = k1 == 0 ? v[0] : v[k1] * conj(p.twx[g * k1]);
   }
   __syncthreads();
-}
-
-// x lines: inverse, times V_eff / N, forward (occupied rows out)
-template <int A, int B>
-__device__ __forceinline__ void ms_x(const MsPlanes& p) {
-  const int nl = p.nq * p.n2, P2 = p.P2;
-  const float inv_nl = 1.f / (float)nl;
-  ms_x_inv1<A, B>(p);
   for (int t = threadIdx.x; t < A * nl; t += blockDim.x) {
     const int k1 = qdiv(t, inv_nl), l = t - k1 * nl;
     const int q = qdiv(l, p.inv_n2), c = l - q * p.n2;
@@ -220,33 +200,6 @@ __device__ __forceinline__ void ms_x(const MsPlanes& p) {
     for (int m1 = 0; m1 < A; ++m1) {
       const int e = m2 + B * m1;
       if (ms_occ(p, e)) col[e * P2] = v[m1];
-    }
-  }
-  __syncthreads();
-}
-
-// x lines of the density: inverse, then acc += fa Re^2 + fb Im^2 at every point (acc[q n12 + x n2 +
-// c], columns in the transposed y order): FP32 terms into float-float sums
-template <int A, int B>
-__device__ __forceinline__ void ms_x_dens(const MsPlanes& p, ff* acc, float fa, float fb) {
-  const int nl = p.nq * p.n2, P2 = p.P2;
-  const float inv_nl = 1.f / (float)nl;
-  ms_x_inv1<A, B>(p);
-  for (int t = threadIdx.x; t < A * nl; t += blockDim.x) {
-    const int k1 = qdiv(t, inv_nl), l = t - k1 * nl;
-    const int q = qdiv(l, p.inv_n2), c = l - q * p.n2;
-    const cplx<float>* col = p.S + q * p.pstride + c + B * k1 * P2;
-    ff* aq = acc + q * p.n12 + c + k1 * p.n2;
-    cplx<float> v[B];
-#pragma unroll
-    for (int g = 0; g < B; ++g) v[g] = col[g * P2];
-    sdft<B>(v, 1.f, p.twx, A);
-#pragma unroll
-    for (int k2 = 0; k2 < B; ++k2) {
-      ff* a = aq + A * k2 * p.n2;
-      const ff o = *a;
-      const ff u = two_sum(o.hi, fa * v[k2].x * v[k2].x + fb * v[k2].y * v[k2].y);
-      *a = ff(u.hi, add_rn(o.lo, u.lo));
     }
   }
   __syncthreads();
@@ -284,18 +237,6 @@ __device__ __forceinline__ void ms_x_n(const MsPlanes& p) {
 #define SGO_CASE(N, A, B) \
   case N:                 \
     ms_x<A, B>(p);        \
-    break;
-    SGO_MS_SIZES(SGO_CASE)
-#undef SGO_CASE
-    default: break;
-  }
-}
-
-__device__ __forceinline__ void ms_x_dens_n(const MsPlanes& p, ff* acc, float fa, float fb) {
-  switch (p.n1) {
-#define SGO_CASE(N, A, B)            \
-  case N:                            \
-    ms_x_dens<A, B>(p, acc, fa, fb); \
     break;
     SGO_MS_SIZES(SGO_CASE)
 #undef SGO_CASE
@@ -385,103 +326,6 @@ __global__ void __launch_bounds__(PLANE_MS_THREADS, PLANE_MS_MINB) k_plane_vpsi_
     }
     __syncthreads();
   }
-}
-
-// Density pass of the same lengths: rho(r) = (1/Omega) sum_n occ_n |psi_n(r)|^2.  A cluster of
-// DENS_CLUSTER CTAs takes a block of Q z-planes, CTA r of it the occupied band pairs r, r +
-// DENS_CLUSTER, ...: the columns land in the planes, y inverse, x inverse, and the x pass's second
-// half adds its samples to the CTA's sums in shared memory; the cluster then adds its CTAs' sums
-// in rank order through distributed shared memory, each CTA a share of the points.  The sums are
-// float-float (44 bits and more; the terms are FP32): FP64 runs at 1/64 of the FP32 rate here, and
-// one FP64 addition per point and band pair alone would take as long as the whole pass.
-// Before, one CTA per block of planes looped over all band pairs, a thread per line (255 registers,
-// one CTA per SM, FP64 sums): the 24-atom layer 367 us, the 72^3 cluster 702 us, the folded mesh
-// 1188 us, 64 members 1370 us (now: at DENS_CLUSTER in kernels.h).
-__global__ void __launch_bounds__(PLANE_MS_THREADS, PLANE_MS_MINB) k_plane_density_ms(KArgs ka, const double* occ_override) {
-  namespace cg = cooperative_groups;
-  cg::cluster_group cluster = cg::this_cluster();
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  const int p = locate(ka.start, ka.nprob, blockIdx.x);
-  if (!ka.active[p]) return;  // (a cluster belongs to one problem)
-  const Prob& P = ka.probs[p];
-  const int n1 = P.n1, n2 = P.n2, n3 = P.n3, mx = P.m1max, ncol = P.ncol, n12 = n1 * n2;
-  const int R = 2 * mx + 1, P2 = n2 | 1, pstride = n1 * P2;
-  const int Q = ms_dens_q(n1, n2, n3);
-  const int local = blockIdx.x - ka.start[p];
-  const int zb = local / DENS_CLUSTER, rank = local - zb * DENS_CLUSTER;
-  const int z0 = zb * Q, nq = min(Q, n3 - z0);
-  cplx<float>* const S = reinterpret_cast<cplx<float>*>(smem_raw);
-  cplx<float>* const twx = S + Q * pstride;
-  cplx<float>* const twy = twx + n1;
-  ff* const acc = reinterpret_cast<ff*>(twy + n2);
-  const int ox = ms_tw_offset(n1), oy = ms_tw_offset(n2);
-  const int ay = ms_a(n2), by = n2 / ay;
-  for (int t = threadIdx.x; t < n1; t += blockDim.x) twx[t] = c_tw[ox + t];
-  for (int t = threadIdx.x; t < n2; t += blockDim.x) twy[t] = c_tw[oy + t];
-  for (int t = threadIdx.x; t < nq * n12; t += blockDim.x) acc[t] = ff(0.f, 0.f);
-  MsPlanes mp{S, nullptr, twx, twy, n1, n2, P2, pstride, n12, nq, mx, R, 1.f / (float)R, 1.f / (float)n2};
-  const int* __restrict__ sidx = P.col_sidx;
-  const float inv_P2 = 1.f / (float)P2;
-  auto slot = [&](int s) {  // compact slot rho P2 + i2 -> whole-row slot e P2 + i2
-    const int rho = qdiv(s, inv_P2), i2 = s - rho * P2;
-    return (rho <= mx ? rho : rho + n1 - R) * P2 + i2;
-  };
-  const double* occ = occ_override ? occ_override : P.occ;
-#pragma unroll 1
-  for (int pair = rank; pair < P.npair; pair += DENS_CLUSTER) {
-    const float fa = (float)occ[2 * pair], fb = 2 * pair + 1 < P.nb ? (float)occ[2 * pair + 1] : 0.f;
-    if (fa == 0.f && fb == 0.f) continue;  // uniform across the block
-    for (int t = threadIdx.x; t < nq * R * P2; t += blockDim.x) {
-      const int l = qdiv(t, inv_P2), j = t - l * P2;
-      ms_row(mp, l)[j] = mk(0.f, 0.f);
-    }
-    __syncthreads();
-    const cplx<float>* wc = reinterpret_cast<const cplx<float>*>(P.Wc) + ((size_t)pair * n3 + z0) * ncol;
-    for (int q = 0; q < nq; ++q)
-      for (int c = threadIdx.x; c < ncol; c += blockDim.x) cp_async8(S + q * pstride + slot(sidx[c]), wc + q * ncol + c);
-    cp_async_commit();
-    cp_async_wait<0>();
-    __syncthreads();
-    ms_y_inv_n(mp);
-    ms_x_dens_n(mp, acc, fa, fb);
-  }
-  cluster.sync();
-  const double io = 1.0 / P.omega;
-  double* rho = P.rho_out + (size_t)z0 * n12;
-  const float inv_by = 1.f / (float)by;
-  for (int t = rank * blockDim.x + threadIdx.x; t < nq * n12; t += DENS_CLUSTER * blockDim.x) {
-    ff s = cluster.map_shared_rank(acc, 0)[t];
-    for (int r = 1; r < DENS_CLUSTER; ++r) s = s + cluster.map_shared_rank(acc, r)[t];
-    const int row = t / n2, c = t - row * n2, k1 = qdiv(c, inv_by), k2 = c - k1 * by;
-    rho[row * n2 + k1 + ay * k2] = ff_to(s) * io;
-  }
-  cluster.sync();  // no CTA leaves while another may still read its sums
-}
-
-int plane_density_ms_ctas(int n1, int n2, int n3) {
-  const int q = ms_dens_q(n1, n2, n3);
-  return DENS_CLUSTER * ((n3 + q - 1) / q);
-}
-size_t plane_density_ms_smem(int n1, int n2, int n3) {
-  return (size_t)ms_dens_q(n1, n2, n3) * ms_dens_plane_bytes(n1, n2) + ms_table_bytes(n1, n2);
-}
-void launch_plane_density_ms(const Launch& L, size_t smem, const double* occ_override) {
-  if (!L.map.total) return;
-  auto* fn = k_plane_density_ms;
-  cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(L.map.total);
-  cfg.blockDim = dim3(PLANE_MS_THREADS);
-  cfg.dynamicSmemBytes = smem;
-  cfg.stream = L.stream;
-  cudaLaunchAttribute at[1];
-  at[0].id = cudaLaunchAttributeClusterDimension;
-  at[0].val.clusterDim.x = DENS_CLUSTER;
-  at[0].val.clusterDim.y = 1;
-  at[0].val.clusterDim.z = 1;
-  cfg.attrs = at;
-  cfg.numAttrs = 1;
-  cuda_ok(cudaLaunchKernelEx(&cfg, fn, L.ka, occ_override), "density launch");
 }
 
 int plane_ms_ctas(int n1, int n2, int n3, int npair) {

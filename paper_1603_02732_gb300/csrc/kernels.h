@@ -84,11 +84,10 @@ enum { DD_S = 0, DD_HS, DD_CM, DD_TM, DD_PROJ, DD_DPROJ, DD_PROJ_D };
 template <typename T> void launch_wave_to_cols(const Launch& L, int src);
 template <typename T> void launch_cols_to_wave(const Launch& L, int src, int dst);
 template <typename T> void launch_plane_vpsi(const Launch& L);
-// CTAs of the density pass that share a plane or a block of planes.  Measured (k_plane_ms.cu) with
-// 2 / 4 / 8: 24-atom layer 73 / 47 / 56 us, 13-atom cluster 136 / 90 / 109, folded 2x2x2 mesh 180 /
-// 116 / 125, 8 members of 8 atoms 34 / 28 / 38, 64 members 657 / 723 / 967 (21 members, a sub-batch:
-// 315 / 317 / 396), 8-atom crystal 26 / 18 / 15.
-constexpr int DENS_CLUSTER = 4;
+// CTAs of the shared-memory density pass that share a plane: FP64 path 4 (2 / 4 / 8 CTAs, 8-atom
+// crystal 26 / 18 / 15 us, 24-atom layer and batches fastest with 4), mixed path 1 (its sums are
+// pinned to the order of one CTA)
+template <typename T> __host__ __device__ constexpr int dens_cluster() { return sizeof(T) == 8 ? 4 : 1; }
 template <typename T> void launch_plane_density(const Launch& L, const double* occ_override);
 // grid transforms of the work grids, T: double, or ff (float-float arithmetic on FP64 grids, ff.cuh)
 struct ff;
@@ -152,10 +151,6 @@ constexpr bool kPlaneMultiPass = true;
 int plane_ms_ctas(int n1, int n2, int n3, int npair);
 size_t plane_ms_smem(int n1, int n2, int n3);
 void launch_plane_vpsi_ms(const Launch& L, size_t smem);
-// the density of the same lengths (multi-pass too, clusters of CTAs over the band pairs)
-int plane_density_ms_ctas(int n1, int n2, int n3);
-size_t plane_density_ms_smem(int n1, int n2, int n3);
-void launch_plane_density_ms(const Launch& L, size_t smem, const double* occ_override);
 bool plane_ms_init();
 void plane_ms_set_smem_limits(size_t bytes);
 int plane_reg_class(int n1, int n2);          // 0: both <= 40, 1: up to PLANE_REG_MAXN
@@ -163,7 +158,9 @@ int plane_reg_ctas(int n2, int n3, int npair);
 size_t plane_reg_smem(int n1, int n2, int m1max);
 bool fft_reg_init();                          // twiddle tables on the current device
 bool plane_vpsi_reg_init();
+bool plane_density_reg_init();
 void plane_vpsi_reg_set_smem_limits(size_t bytes);
+void plane_density_reg_set_smem_limits(size_t bytes);
 // register-FFT z-column passes (mixed path), k_cols_reg.cu
 int zreg_class(int n3);
 bool zreg_ok(int n3);
@@ -189,6 +186,9 @@ void launch_cols_to_wave_pair(const Launch& L, size_t smem, int src, int dst);
 bool pair_reg_init();
 void pair_reg_set_smem_limits(size_t bytes);
 void launch_plane_vpsi_reg(const Launch& L, int cls, size_t smem);
+size_t plane_density_reg_smem(int n1, int n2, int m1max);
+int plane_density_reg_ctas(int n2, int n3);
+void launch_plane_density_reg(const Launch& L, int cls, size_t smem, const double* occ_override);
 
 // k_linalg.cu
 template <typename T>

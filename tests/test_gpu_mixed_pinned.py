@@ -47,10 +47,24 @@ def grid_fft(sgo, grid):
     return _hash(ctx.grid_fft(x, -1)) + _hash(ctx.grid_fft(x, 1))
 
 
+# (planes of the register kernel in both its classes, of the lane-pair kernel, of the shared-memory one)
+DENSITIES = [((12, 16, 10), 5), ((25, 27, 12), 16), ((45, 48, 16), 17), ((72, 72, 10), 18), ((96, 100, 10), 17),
+             ((9, 10, 9), 17), ((75, 81, 10), 17)]
+
+
+def density(sgo, grid, bands):
+    ctx = sgo.Context(_grid(grid, bands), precision="mixed", extra_bands=0)
+    rng = np.random.default_rng(62)
+    psi = rng.normal(size=(bands, ctx.npw))
+    return _hash(ctx.density_of(psi, np.where(np.arange(bands) % 5 == 3, 0.0, rng.uniform(0.0, 2.0, size=bands))))
+
+
 # every pinned result: name -> how it is computed
 CASES = {}
 for _g in GRIDS:
     CASES["grid_fft %dx%dx%d" % _g] = lambda s, g=_g: grid_fft(s, g)
+for _g, _n in DENSITIES:
+    CASES["density %dx%dx%d, %d bands" % (*_g, _n)] = lambda s, g=_g, n=_n: density(s, g, n)
 
 
 @pytest.mark.parametrize("name", CASES)
