@@ -736,7 +736,7 @@ void Engine::build_gemm_maps() {
     const int nin[3] = {d.nb, d.nproj, 3 * d.nproj};
     for (int k = 0; k < 3; ++k)
       for (int t = 0; t < 2; ++t)
-        red[k][t].push_back(div_up(nin[k] * d.nb, 256 / tn_reduce_lanes(t ? tc.back() : nsplit)));
+        red[k][t].push_back(div_up(nin[k] * d.nb, 256 / tn_reduce_lanes(t ? tc_kc_ : tn_kc_, nsplit)));
   }
   // one buffer and one copy for all of them (the autotuner rebuilds them for every candidate)
   std::vector<std::pair<WorkMap*, const std::vector<int>*>> maps = {

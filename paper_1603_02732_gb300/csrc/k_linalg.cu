@@ -149,7 +149,7 @@ __global__ void __launch_bounds__(256) k_gemm_tn(KArgs ka, int akind, int arole,
   const int ti0 = 4 * bi * pa, tj0 = 4 * bj * pb;
   const int ca = min(pa, ga - bi * pa), cb = min(pb, gb - bj * pb);  // tiles of this block
   const int nt = tri ? ca * (ca + 1) / 2 : ca * cb;
-  const int ks = 256 / nt;
+  const int ks = sizeof(T) == 8 ? 256 / nt : 1;
   const int k0 = split * kc, k1 = min(P.npw, k0 + kc);
   const int t = threadIdx.x;
   const int tile = t % nt, slice = t / nt;
@@ -240,11 +240,10 @@ __global__ void __launch_bounds__(256) k_gemm_tn(KArgs ka, int akind, int arole,
 }
 
 // Sum the partials of every output: CTA = (problem, chunk of 256 / L outputs), L =
-// tn_reduce_lanes(nsplit) threads per output taking every L-th partial, added in order.
+// tn_reduce_lanes(kc, nsplit) threads per output taking every L-th partial, added in order.
 // sym: A^T A from k_gemm_tn, whose tiles below the diagonal were not computed (read mirrored).
-// L keeps the serial chain of loads at about eight: with one thread per output the 83
-// partials of the 24-atom layer's FP64 products would be one chain of 83 (11.9 -> 7 us there
-// on the mixed path's 42).
+// L keeps the serial chain of loads at about eight on the FP64 path: with one thread per output
+// the 83 partials of the 24-atom layer's products would be one chain of 83.
 __global__ void k_gemm_tn_reduce(KArgs ka, int akind, int bkind, int dst, const double* part_base, size_t part_stride,
                                  int kc_arg, int sym) {
   __shared__ double red[256];
@@ -253,7 +252,7 @@ __global__ void k_gemm_tn_reduce(KArgs ka, int akind, int bkind, int dst, const 
   const Prob& P = ka.probs[p];
   const int na = opnd_count(P, akind), nbv = opnd_count(P, bkind);
   const int kc = kc_arg > 0 ? kc_arg : tn_kc_f64(P.npw);
-  const int nsplit = (P.npw + kc - 1) / kc, L = tn_reduce_lanes(nsplit), no = 256 / L;
+  const int nsplit = (P.npw + kc - 1) / kc, L = tn_reduce_lanes(kc_arg, nsplit), no = 256 / L;
   const int lo = threadIdx.x % no, sl = threadIdx.x / no;
   const int o = (blockIdx.x - ka.start[p]) * no + lo;
   const bool in = o < na * nbv;

@@ -35,9 +35,12 @@ __host__ __device__ inline int tn_block_groups(int n) { return ((n + 3) / 4 + tn
 // crystal 264 -> 10.7 us, the layer 437 -> 106 us, six uneven members 555 -> 204 us (chunks of
 // 256 and whole 64 x 64 tiles before).
 __host__ __device__ inline int tn_kc_f64(int npw) { return npw < 4096 ? 32 : npw < 8192 ? 64 : 128; }
-// Threads that share one output of the split-K reduction (a power of two up to 8, about eight
-// partials each)
-__host__ __device__ inline int tn_reduce_lanes(int nsplit) { return nsplit < 16 ? 1 : nsplit < 32 ? 2 : nsplit < 64 ? 4 : 8; }
+// Threads that share one output of the split-K reduction: on the FP64 path (kc 0) a power of two up to
+// 8, about eight partials each; one where the chunk is given (the mixed path, whose results are pinned
+// to that order)
+__host__ __device__ inline int tn_reduce_lanes(int kc, int nsplit) {
+  return kc > 0 || nsplit < 16 ? 1 : nsplit < 32 ? 2 : nsplit < 64 ? 4 : 8;
+}
 // Rows of an FP64 NN CTA: as many groups of 4 as give each of 256 threads a 4 x 4 tile, at most
 // 8 groups while a structure has few plane waves (so that it fills the GPU).  Mean per launch
 // (1 to 4 products): the 8-atom crystal 95 -> 15 us, the 24-atom layer 460 -> 189 us (1.1

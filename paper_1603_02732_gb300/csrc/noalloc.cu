@@ -104,7 +104,7 @@ sgo_status run(sgo_ctx* c, const double* veff, int nvec, const double* psi, doub
   }
   const int counts[NMAP] = {d.npair * div_up(d.ncp, QCP), d.npair * d.n3, d.nb, d.natom,
                             tn_blocks(d.nproj) * tn_blocks(d.nb) * nsplit,
-                            div_up(d.nproj * d.nb, 256 / tn_reduce_lanes(nsplit)),
+                            div_up(d.nproj * d.nb, 256 / tn_reduce_lanes(TN_KC, nsplit)),
                             sizeof(T) == 4 ? div_up(d.npw, 64 * NN_RT) * div_up(d.nb, 64)
                                            : div_up(d.npw, nn_rows_f64(d.nb, d.npw)) * tn_blocks(d.nb),
                             div_up(d.ngrid, GRID_EW_POINTS), d.nproj};

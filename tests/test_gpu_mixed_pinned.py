@@ -59,12 +59,28 @@ def density(sgo, grid, bands):
     return _hash(ctx.density_of(psi, np.where(np.arange(bands) % 5 == 3, 0.0, rng.uniform(0.0, 2.0, size=bands))))
 
 
+PRODUCTS = [("tiny", 13, 0), ("tiny", 60, 0), ("tiny", 121, 0), ("de", 81, 0), ("de", 81, 1), ("layer", 64, 0), ("layer", 64, 1)]
+
+
+def products(sgo, name, bands, tensor_cores):
+    """Psi^T Y, Psi^T Psi and Psi M + Y of the subspace, and H Psi."""
+    base = dict(tiny=workloads.tiny(nat=2, ecut=6.0), de=workloads.de_candidate(44), layer=workloads.honeycomb24())[name]
+    ctx = sgo.Context(dataclasses.replace(base, nbands=bands), precision="mixed", gemm_tc=tensor_cores)
+    rng = np.random.default_rng(63)
+    x, y = rng.normal(size=(2, bands, ctx.npw))
+    m = rng.normal(size=(bands, bands))
+    h = ctx.apply_hamiltonian(rng.normal(size=base.fft), x)
+    return _hash(ctx.subspace_matrix(x, y)) + _hash(ctx.subspace_matrix(x, x)) + _hash(ctx.block_update(x, m, -1.5, 0.5, y)) + _hash(h)
+
+
 # every pinned result: name -> how it is computed
 CASES = {}
 for _g in GRIDS:
     CASES["grid_fft %dx%dx%d" % _g] = lambda s, g=_g: grid_fft(s, g)
 for _g, _n in DENSITIES:
     CASES["density %dx%dx%d, %d bands" % (*_g, _n)] = lambda s, g=_g, n=_n: density(s, g, n)
+for _p in PRODUCTS:
+    CASES["products %s, %d bands, gemm_tc=%d" % _p] = lambda s, p=_p: products(s, *p)
 
 
 @pytest.mark.parametrize("name", CASES)
