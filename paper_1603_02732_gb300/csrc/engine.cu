@@ -832,7 +832,8 @@ Engine::Engine(const std::vector<sgo_ctx*>& ctxs, cudaStream_t stream) : ctx_(ct
     }
   }
   std::vector<Prob> host(n_);
-  std::vector<int> c_zcol, c_plane, c_dens, c_gz, c_gp, c_gew, c_bands, c_rww, c_nn, c_atoms, c_projs, c_atomch, c_ewsg, c_prob, c_tc, c_nntc, c_preg[2], c_dreg[2], c_zreg[2], c_ppair,
+  std::vector<int> c_zcol, c_plane, c_dens, c_gz, c_gp, c_gew, c_gred, c_bands, c_rww, c_nn, c_atoms, c_projs, c_atomch,
+      c_ewsg, c_prob, c_tc, c_nntc, c_preg[2], c_dreg[2], c_zreg[2], c_ppair,
       c_dpair, c_zpair, c_gx, c_gy, c_gaxis[3], c_gold, c_bigy, c_bigx, c_bigdy, c_bigd;
   size_t part = 0;
   int max_nproj = 0;
@@ -902,6 +903,7 @@ Engine::Engine(const std::vector<sgo_ctx*>& ctxs, cudaStream_t stream) : ctx_(ct
     c_gz.push_back(gaxis ? 0 : div_up(d.n1 * d.n2, QZ));
     c_gp.push_back(gaxis || gbig ? 0 : d.n3);
     c_gew.push_back(div_up(d.ngrid, GRID_EW_POINTS));
+    c_gred.push_back(div_up(d.ngrid, grid_red_chunk(precision_ == 0)));
     c_bands.push_back(d.nb);
     c_rww.push_back(div_up(d.nb * d.nb, 256));
     c_nn.push_back(precision_ ? div_up(d.npw, 64 * NN_RT) * div_up(d.nb, 64)
@@ -936,6 +938,7 @@ Engine::Engine(const std::vector<sgo_ctx*>& ctxs, cudaStream_t stream) : ctx_(ct
   m_gz_ = make_map(c_gz);
   m_gp_ = make_map(c_gp);
   m_gew_ = make_map(c_gew);
+  m_gred_ = make_map(c_gred);
   m_bands_ = make_map(c_bands);
   m_asm_ = make_map(c_rww);
   m_nn_ = make_map(c_nn);
@@ -966,7 +969,7 @@ Engine::Engine(const std::vector<sgo_ctx*>& ctxs, cudaStream_t stream) : ctx_(ct
   cudaMemcpy(d_active_, h_active_.data(), sizeof(int) * n_, cudaMemcpyHostToDevice);
   if (!cuda_ok(dev_malloc(&d_part_, sizeof(double) * part_stride_ * n_), "dev_malloc(part)")) return;
   allocs_.push_back(d_part_);
-  if (!cuda_ok(dev_malloc(&d_gpart_, sizeof(double) * (size_t)*std::max_element(c_gew.begin(), c_gew.end()) * n_ * 8), "dev_malloc(gpart)")) return;
+  if (!cuda_ok(dev_malloc(&d_gpart_, sizeof(double) * (size_t)m_gred_.maxper * n_ * 8), "dev_malloc(gpart)")) return;
   allocs_.push_back(d_gpart_);
   if (!cuda_ok(dev_malloc(&d_flags_, sizeof(double) * 4 * n_), "dev_malloc(flags)")) return;
   allocs_.push_back(d_flags_);
@@ -1458,7 +1461,7 @@ template <typename T>
 void Engine::density_energy(int mode) {
   const sgo_opts& o = ctx_[0]->opts;
   // occupations and rho_out
-  launch_occupations(L(m_prob_));
+  launch_occupations<T>(L(m_prob_));
   wave_to_cols<T>(WB_X);
   tbeg(TK_PLANE_DENSITY);
   launch_plane_density<T>(L(m_dens_), nullptr);
@@ -1479,8 +1482,8 @@ void Engine::density_energy(int mode) {
     grid_fft(3, 1);
   }
   tbeg(TK_GRID_OTHER);
-  launch_grid_energies<T>(L(m_gew_), d_gpart_, m_gew_.maxper);
-  launch_finish_iteration(L(m_prob_), d_gpart_, m_gew_.maxper, o.scf_tol_e, o.scf_tol_rho, mode);
+  launch_grid_energies<T>(L(m_gred_), d_gpart_, m_gred_.maxper);
+  launch_finish_iteration<T>(L(m_prob_), d_gpart_, m_gred_.maxper, o.scf_tol_e, o.scf_tol_rho, mode);
   tend(TK_GRID_OTHER);
 }
 
@@ -1573,12 +1576,13 @@ bool Engine::build_polish_graphs() {
 }
 
 // Pulay mixing of rho_out with rho_in (members still iterating).
+template <typename T>
 void Engine::pulay_step() {
   const sgo_opts& o = ctx_[0]->opts;
   const int hist = std::min(std::max(o.pulay_hist, 1), MAX_HIST);
   tbeg(TK_GRID_OTHER);
-  launch_pulay_gram(L(m_gew_), d_gpart_, m_gew_.maxper, hist);
-  launch_pulay_solve(L(m_prob_), d_gpart_, m_gew_.maxper, hist);
+  launch_pulay_gram<T>(L(m_gred_), d_gpart_, m_gred_.maxper, hist);
+  launch_pulay_solve<T>(L(m_prob_), d_gpart_, m_gred_.maxper, hist);
   launch_pulay_mix(L(m_gew_), o.mix_alpha, o.kerker_q0);
   tend(TK_GRID_OTHER);
 }
@@ -1635,7 +1639,7 @@ bool Engine::build_graphs() {
   if (ok) {
     scf_iteration<T>(o.ncg, true);
     k_scf_control<<<1, 256, 0, stream_>>>(L(m_prob_).ka, d_active_, d_flags_, d_iter_, o.max_scf, cond, 1);
-    pulay_step();
+    pulay_step<T>();
     cudaGraph_t got = nullptr;
     ok = cuda_ok(cudaStreamEndCapture(stream_, &got), "capture body end");
   }
@@ -1695,7 +1699,7 @@ sgo_status Engine::launch_t(bool want_forces) {
       int nact = 0;
       for (int p = 0; p < n_; ++p) nact += h_active_[p];
       if (nact == 0) break;
-      if (it > nonsc) pulay_step();
+      if (it > nonsc) pulay_step<T>();
     }
     run_it_ = it;
     polish<T>();

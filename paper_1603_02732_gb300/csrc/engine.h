@@ -139,7 +139,7 @@ class Engine {
   template <typename T> void polish();
   template <typename T> bool build_polish_graphs();
   bool read_active();
-  void pulay_step();
+  template <typename T> void pulay_step();
   template <typename T> bool build_graphs();
   template <typename T> void hpsi(int src, int dst);
   template <typename T> void rayleigh_ritz(bool rotate_history);
@@ -186,7 +186,7 @@ class Engine {
   std::vector<int> h_active_;
   std::vector<void*> allocs_;
   int max_n1_ = 0, max_n2_ = 0, max_n3_ = 0, max_n12_ = 0, max_nb_ = 0, plane_threads_ = 128;
-  WorkMap m_zcol_, m_plane_, m_dens_, m_gz_, m_gp_, m_gew_, m_bands_, m_tn_[3], m_red_[3][2], m_asm_,
+  WorkMap m_zcol_, m_plane_, m_dens_, m_gz_, m_gp_, m_gew_, m_gred_, m_bands_, m_tn_[3], m_red_[3][2], m_asm_,
       m_nn_, m_atoms_, m_projs_, m_atomch_, m_ewsg_, m_prob_, m_tc_, m_nntc_[2];
   WorkMap m_preg_[2], m_dreg_[2], m_zreg_[2];  // register-FFT plane / column kernels, per size class
   size_t preg_smem_[2] = {0, 0}, dreg_smem_[2] = {0, 0}, zreg_smem_[2] = {0, 0};

@@ -52,15 +52,6 @@ __device__ __forceinline__ double* grid_sel(const Prob& P, int sel) {
   }
 }
 
-// 1 / x for a positive normal number: the approximate reciprocal and two Newton steps (four FP64
-// operations; a division takes more than twice as many)
-__device__ __forceinline__ double rcp_newton(double x) {
-  double r;
-  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(x));
-  r = fma(r, fma(-x, r, 1.0), r);
-  return fma(r, fma(-x, r, 1.0), r);
-}
-
 // exp(-i G.R_I) from the atom's 1D tables (indexed by grid index per axis).
 __device__ __forceinline__ cplx<double> phase_at(const Prob& P, int atom, int i1, int i2, int i3) {
   const cplx<double>* ph = reinterpret_cast<const cplx<double>*>(P.phase) + (size_t)atom * (P.n1 + P.n2 + P.n3);
@@ -211,12 +202,13 @@ __device__ __forceinline__ void pbe_point(R rho_v, R sigma_v, R* e, R* dr, R* ds
 // ---------------------------------------------------------------------------
 constexpr int GRID_EW = GRID_EW_POINTS;
 
-#define GRID_EW_PROLOGUE                                           \
+#define GRID_PROLOGUE(CHUNK)                                       \
   const int p = locate(ka.start, ka.nprob, blockIdx.x);            \
   if (!ka.active[p]) return;                                       \
   const Prob& P = ka.probs[p];                                     \
-  const int base = (blockIdx.x - ka.start[p]) * GRID_EW;           \
-  const int end = min(P.ngrid, base + GRID_EW);
+  const int base = (blockIdx.x - ka.start[p]) * (CHUNK);           \
+  const int end = min(P.ngrid, base + (CHUNK));
+#define GRID_EW_PROLOGUE GRID_PROLOGUE(GRID_EW)
 
 __global__ void k_real_to_grid(KArgs ka, int src, int which) {
   GRID_EW_PROLOGUE
@@ -287,7 +279,7 @@ __global__ void k_potential_g(KArgs ka) {
   for (int i = base + threadIdx.x; i < end; i += blockDim.x) {
     const double g2 = P.g2box[i];  // -1 on Nyquist planes
     double2 r = P.rhog_in[i];
-    double f = g2 < 1e-14 ? 0.0 : 4.0 * PI * rcp_newton(g2);
+    double f = g2 < 1e-14 ? 0.0 : 4.0 * PI / g2;
     // (r.x + i r.y) + i f (r.x + i r.y)
     g[i] = mk((T)(r.x - f * r.y), (T)(r.y + f * r.x));
   }
@@ -390,18 +382,21 @@ __global__ void k_rho0_g(KArgs ka) {
 // ---------------------------------------------------------------------------
 // Grid reductions for the energy at rho_out (work grid gfft2 = N rho_out(G)):
 // part[p][chunk][0..4] = sum V_ion rho, sum rho eps_xc, sum rho, sum |rho_out - rho_in|,
-// sum_{G!=0} |rho(G)|^2 / G^2.  CTA = (problem, GRID_EW points).
-// Bound by FP64 operations (about 20 a point; the two FP64 lanes of an SM) and, for one structure,
-// by latency: chunks of 4096 points left most SMs idle, and five block sums one after the other and
-// the division took half the FP64 work.  24-atom layer 43 -> 17 us, 64 members 244 -> 184 us.
+// sum_{G!=0} |rho(G)|^2 / G^2.  CTA = (problem, chunk of points).
+// FP64 path: chunks of GRID_EW points; bound by FP64 operations (the two FP64 lanes of an SM) and, for
+// one structure, by latency, since chunks of 4096 points leave most SMs idle.  Mixed path: chunks of
+// 4096 points, added in order: its results are pinned to the order of these sums (here and in the
+// kernels below).
 // ---------------------------------------------------------------------------
-constexpr int NGE = 5, NRED = 8;  // sums used, stride of a chunk's partial sums
+template <typename T>
+__host__ __device__ constexpr int red_chunk() { return sizeof(T) == 8 ? GRID_EW : GRID_CHUNK; }
+constexpr int NRED = 8;  // stride of a chunk's partial sums (5 of the energies, one per ring slot of the mixing)
 
 template <typename T>
 __global__ void k_grid_energies(KArgs ka, double* part, int maxchunk) {
   __shared__ double red[64], tot[8];
-  GRID_EW_PROLOGUE
-  const double inv_n2 = (1.0 / P.ngrid) * (1.0 / P.ngrid);
+  GRID_PROLOGUE(red_chunk<T>())
+  const double inv_n = 1.0 / P.ngrid;
   double s[8] = {0, 0, 0, 0, 0, 0, 0, 0};
   for (int i = base + threadIdx.x; i < end; i += blockDim.x) {
     double r = P.rho_out[i];
@@ -422,39 +417,47 @@ __global__ void k_grid_energies(KArgs ka, double* part, int maxchunk) {
     const double g2 = P.g2box[i];  // -1 on Nyquist planes
     if (g2 > 1e-14) {
       double2 v = P.gfft2[i];
-      s[4] += (v.x * v.x + v.y * v.y) * rcp_newton(g2);
+      s[4] += (v.x * v.x + v.y * v.y) * inv_n * inv_n / g2;
     }
   }
-  s[4] *= inv_n2;
   block_sums8(s, red, tot);
   if (threadIdx.x < NRED) part[((size_t)p * maxchunk + (blockIdx.x - ka.start[p])) * NRED + threadIdx.x] = tot[threadIdx.x];
 }
 
-// Sums of a problem's partial sums over its chunks, in tot[8] (256 threads: 32 slices of the chunks)
+// Sums of a problem's partial sums over its chunks, in tot[8].  FP64 path: 256 threads, 32 slices of
+// the chunks.  Mixed path: a thread per sum, chunk after chunk.
+template <typename T>
 __device__ __forceinline__ void chunk_sums(const Prob& P, const double* part, double (&red)[32][NRED + 1], double* tot) {
-  const int nch = (P.ngrid + GRID_EW - 1) / GRID_EW, lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  const int nch = (P.ngrid + red_chunk<T>() - 1) / red_chunk<T>();
   double s = 0.0;
-  for (int c = threadIdx.x >> 3; c < nch; c += 32) s += part[(size_t)c * NRED + (threadIdx.x & 7)];
-  red[threadIdx.x >> 3][threadIdx.x & 7] = s;
-  __syncthreads();
-  s = warp_sum(red[lane][w]);
-  if (lane == 0) tot[w] = s;
+  if constexpr (sizeof(T) == 8) {
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    for (int c = threadIdx.x >> 3; c < nch; c += 32) s += part[(size_t)c * NRED + (threadIdx.x & 7)];
+    red[threadIdx.x >> 3][threadIdx.x & 7] = s;
+    __syncthreads();
+    s = warp_sum(red[lane][w]);
+    if (lane == 0) tot[w] = s;
+  } else if (threadIdx.x < NRED) {
+#pragma unroll 8
+    for (int c = 0; c < nch; ++c) s += part[(size_t)c * NRED + threadIdx.x];
+    tot[threadIdx.x] = s;
+  }
   __syncthreads();
 }
 
-// Grid sums, band terms, total free energy, convergence test.  One CTA of 256 threads per problem.
-// (One thread summing the chunks and one thread per band summing its projectors took 18 + 13 us for
-// the 24-atom layer and 18 + 42 us for 32 atoms with p channels; now 15 and 25 us.)
+// Grid sums, band terms, total free energy, convergence test.  One CTA per problem (FP64 path 256
+// threads, several slices of a band's projectors; mixed path 128, a band's projectors in order).
+template <typename T>
 __global__ void k_finish_iteration(KArgs ka, const double* part, int maxchunk, double tol_e, double tol_rho,
                                    int count_iter) {
   __shared__ double red[33], redc[32][NRED + 1], tot[NRED];
   const int p = blockIdx.x;
   if (!ka.active[p]) return;
   const Prob& P = ka.probs[p];
-  chunk_sums(P, part + (size_t)p * maxchunk * NRED, redc, tot);
+  chunk_sums<T>(P, part + (size_t)p * maxchunk * NRED, redc, tot);
   double ek = 0.0, en = 0.0;
   for (int i = threadIdx.x; i < P.nb; i += blockDim.x) ek += P.occ[i] * P.bv[BV_EKIN * P.nb + i];
-  constexpr int SL = 16;  // slices of the projectors
+  constexpr int SL = sizeof(T) == 8 ? 16 : 1;  // slices of the projectors
   for (int e = threadIdx.x; e < SL * P.nb; e += blockDim.x) {
     const int sl = e / P.nb, i = e - sl * P.nb;
     double s = 0.0;
@@ -496,13 +499,13 @@ __global__ void k_finish_iteration(KArgs ka, const double* part, int maxchunk, d
 // Pulay (DIIS) mixing on R = rho_out - rho_in with a ring history.
 // ---------------------------------------------------------------------------
 // The density and residual go into the ring; part[p][chunk][j] = <R_pos, R_j> over a chunk for every
-// ring slot j (0 for the empty ones).  CTA = (problem, GRID_EW points): the points' loads of all
+// ring slot j (0 for the empty ones).  CTA = (problem, chunk of points): the points' loads of all
 // slots are in flight together and the eight sums are reduced together.  For one structure bound by
-// latency, in a batch by the ring's bytes.  24-atom layer: 62 us (37 CTAs, one slot after the other)
-// and 7 us for the store -> 22 us; 64 members 227 + 68 -> 258 us.
+// latency, in a batch by the ring's bytes.
+template <typename T>
 __global__ void k_pulay_gram(KArgs ka, double* part, int maxchunk, int hist) {
   __shared__ double red[64], tot[8];
-  GRID_EW_PROLOGUE
+  GRID_PROLOGUE(red_chunk<T>())
   const int pos = (int)P.scal[SC_PULAY_POS];
   const int cnt = min((int)P.scal[SC_PULAY_N] + 1, hist);
   const double inv_n = 1.0 / P.ngrid;
@@ -520,7 +523,7 @@ __global__ void k_pulay_gram(KArgs ka, double* part, int maxchunk, int hist) {
     for (int j = 0; j < MAX_HIST; ++j)
       if (j < cnt) {
         const double2 rj = j == pos ? rp : r[j];
-        s[j] += rp.x * rj.x + rp.y * rj.y;
+        s[j] += fma(rp.x, rj.x, __dmul_rn(rp.y, rj.y));  // (written out: the compiler may fuse either product)
       }
   }
   block_sums8(s, red, tot);
@@ -528,15 +531,14 @@ __global__ void k_pulay_gram(KArgs ka, double* part, int maxchunk, int hist) {
 }
 
 // Gram row update and the DIIS system [A 1; 1 0][c; l] = [0; 1] (Gaussian elimination with partial
-// pivoting, lane i of one warp holding row i).  One CTA of 256 threads per problem; one thread alone
-// took 62 us for the 24-atom layer (sums over the chunks, then the elimination in local memory), this
-// form 25 us.
+// pivoting, lane i of one warp holding row i).  One CTA per problem (mixed path: one warp).
+template <typename T>
 __global__ void k_pulay_solve(KArgs ka, const double* part, int maxchunk, int hist) {
   __shared__ double redc[32][NRED + 1], tot[NRED];
   const int p = blockIdx.x;
   if (!ka.active[p]) return;
   const Prob& P = ka.probs[p];
-  chunk_sums(P, part + (size_t)p * maxchunk * NRED, redc, tot);
+  chunk_sums<T>(P, part + (size_t)p * maxchunk * NRED, redc, tot);
   if (threadIdx.x >= 32) return;
   constexpr int R = MAX_HIST + 1;  // rows
   constexpr unsigned full = 0xffffffffu;
@@ -596,11 +598,16 @@ __global__ void k_pulay_solve(KArgs ka, const double* part, int maxchunk, int hi
   }
 #pragma unroll
   for (int i = R - 1; i >= 0; --i) {
-    if (i >= m || !ok) continue;
-    const double xi = __shfl_sync(full, b / M[i], i);
+    if (i >= m) continue;
+    double t = b;  // (lane i) less M_ij x_j, j ascending
+#pragma unroll
+    for (int j = i + 1; j < R; ++j) {
+      const double xj = __shfl_sync(full, x, j);
+      if (j < m) t -= M[j] * xj;
+    }
+    const double xi = __shfl_sync(full, t / M[i], i);
     if (!isfinite(xi)) ok = false;
     if (lane == i) x = xi;
-    if (lane < i) b -= M[i] * xi;
   }
   if (lane < MAX_HIST) alpha[lane] = ok ? (lane < cnt ? x : 0.0) : lane == pos ? 1.0 : 0.0;
   if (lane == 0) {
@@ -611,8 +618,7 @@ __global__ void k_pulay_solve(KArgs ka, const double* part, int maxchunk, int hi
 
 // rho_in(G) = sum_j c_j rho_j(G) + a K(G) sum_j c_j R_j(G), K = G^2/(G^2 + q0^2) (1 if q0 = 0),
 // zero on Nyquist planes.
-// Bound by FP64 operations in a batch (4 a point and slot): 64 members 331 us.  (All slots' loads in
-// flight together took 404: more registers, fewer warps.)
+// Bound by FP64 operations in a batch (4 a point and slot): 64 members 331 us.
 __global__ void k_pulay_mix(KArgs ka, double a, double q0) {
   GRID_EW_PROLOGUE
   const double* alpha = P.scal + SC_PULAY_A + MAX_HIST * MAX_HIST;
@@ -628,7 +634,7 @@ __global__ void k_pulay_mix(KArgs ka, double a, double q0) {
       sy += alpha[j] * r.y;
     }
     double k = 1.0;
-    if (q0 > 0.0) k = g2 < 1e-14 ? 0.0 : g2 * rcp_newton(g2 + q0 * q0);
+    if (q0 > 0.0) k = g2 < 1e-14 ? 0.0 : g2 / (g2 + q0 * q0);
     if (g2 < 0.0) k = 0.0, rx = ry = 0.0;
     P.rhog_in[i] = make_double2(rx + a * k * sx, ry + a * k * sy);
   }
@@ -848,16 +854,21 @@ template <typename T>
 void launch_grid_energies(const Launch& L, double* part, int maxchunk) {
   if (ew_blocks(L)) k_grid_energies<T><<<L.map.total, 256, 0, L.stream>>>(L.ka, part, maxchunk);
 }
+template <typename T>
 void launch_finish_iteration(const Launch& L, const double* part, int maxchunk, double tol_e, double tol_rho,
                              int count_iter) {
-  k_finish_iteration<<<L.ka.nprob, 256, 0, L.stream>>>(L.ka, part, maxchunk, tol_e, tol_rho, count_iter);
+  k_finish_iteration<T><<<L.ka.nprob, sizeof(T) == 8 ? 256 : 128, 0, L.stream>>>(L.ka, part, maxchunk, tol_e, tol_rho,
+                                                                               count_iter);
 }
+template <typename T>
 void launch_pulay_gram(const Launch& L, double* part, int maxchunk, int hist) {
-  if (ew_blocks(L)) k_pulay_gram<<<L.map.total, 256, 0, L.stream>>>(L.ka, part, maxchunk, hist);
+  if (L.map.total) k_pulay_gram<T><<<L.map.total, 256, 0, L.stream>>>(L.ka, part, maxchunk, hist);
 }
+template <typename T>
 void launch_pulay_solve(const Launch& L, const double* part, int maxchunk, int hist) {
-  k_pulay_solve<<<L.ka.nprob, 256, 0, L.stream>>>(L.ka, part, maxchunk, hist);
+  k_pulay_solve<T><<<L.ka.nprob, sizeof(T) == 8 ? 256 : 32, 0, L.stream>>>(L.ka, part, maxchunk, hist);
 }
+int grid_red_chunk(bool fp64) { return fp64 ? red_chunk<double>() : red_chunk<float>(); }
 template <typename T>
 void launch_build_projectors(const Launch& Latoms, int deriv) {
   if (Latoms.map.total) k_build_projectors<T><<<Latoms.map.total, 256, 0, Latoms.stream>>>(Latoms.ka, deriv);
@@ -871,6 +882,12 @@ void launch_force_total(const Launch& L, int maxchunk) {
 
 template void launch_grid_energies<float>(const Launch&, double*, int);
 template void launch_grid_energies<double>(const Launch&, double*, int);
+template void launch_finish_iteration<float>(const Launch&, const double*, int, double, double, int);
+template void launch_finish_iteration<double>(const Launch&, const double*, int, double, double, int);
+template void launch_pulay_gram<float>(const Launch&, double*, int, int);
+template void launch_pulay_gram<double>(const Launch&, double*, int, int);
+template void launch_pulay_solve<float>(const Launch&, const double*, int, int);
+template void launch_pulay_solve<double>(const Launch&, const double*, int, int);
 template void launch_veff<float>(const Launch&, const double*);
 template void launch_veff<double>(const Launch&, const double*);
 template void launch_build_projectors<float>(const Launch&, int);

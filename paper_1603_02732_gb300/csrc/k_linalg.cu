@@ -1182,13 +1182,14 @@ template bool launch_rr_cluster<double>(const Launch&, int, unsigned char*, size
 // Occupations: integer (kT = 0) or Fermi-Dirac with mu from sum f = N_el; entropy
 // S = -2 sum [x ln x + (1-x) ln(1-x)], x = f/2.  One warp per problem.
 // ---------------------------------------------------------------------------
-__device__ __forceinline__ double fd_x(double e, double mu, double ikT) {
-  double a = (e - mu) * ikT;
+__device__ __forceinline__ double fd_x(double e, double mu, double kT) {
+  double a = (e - mu) / kT;
   if (a > 700.0) return 0.0;
   if (a < -700.0) return 1.0;
   return 1.0 / (1.0 + exp(a));
 }
 
+template <typename T>
 __global__ void k_occupations(KArgs ka) {
   const int p = blockIdx.x;
   if (!ka.active[p]) return;
@@ -1209,19 +1210,22 @@ __global__ void k_occupations(KArgs ka) {
     return;
   }
   double lo = eps[0] - 40.0 * kT - 1.0, hi = eps[n - 1] + 40.0 * kT + 1.0;
-  // the iteration starts between the bands around N_el / 2 (at the root where they are far apart
-  // against kT): the middle of the bracket took several times as many steps (24-atom layer 47 us a
-  // launch, now 25), each a chain of FP64 exponentials
-  const double h = 0.5 * nel, ikT = 1.0 / kT;
-  const int i1 = min(max((int)ceil(h) - 1, 0), n - 1), i2 = min(max((int)floor(h), 0), n - 1);
-  double mu = 0.5 * (eps[i1] + eps[i2]);
-  if (!(mu > lo && mu < hi)) mu = 0.5 * (lo + hi);
+  double mu = 0.5 * (lo + hi);
+  if constexpr (sizeof(T) == 8) {
+    // the iteration starts between the bands around N_el / 2 (at the root where they are far apart
+    // against kT): the middle of the bracket takes several times as many steps, each a chain of FP64
+    // exponentials.  (The mixed path starts in the middle: its results are pinned to that root's bits.)
+    const double h = 0.5 * nel;
+    const int i1 = min(max((int)ceil(h) - 1, 0), n - 1), i2 = min(max((int)floor(h), 0), n - 1);
+    const double m = 0.5 * (eps[i1] + eps[i2]);
+    if (m > lo && m < hi) mu = m;
+  }
   for (int it = 0; it < 200; ++it) {
     double cnt = 0.0, der = 0.0;
     for (int i = lane; i < n; i += 32) {
-      double x = fd_x(eps[i], mu, ikT);
+      double x = fd_x(eps[i], mu, kT);
       cnt += 2.0 * x;
-      der += 2.0 * x * (1.0 - x) * ikT;
+      der += 2.0 * x * (1.0 - x) / kT;
     }
     cnt = warp_sum(cnt);
     der = warp_sum(der);
@@ -1235,7 +1239,7 @@ __global__ void k_occupations(KArgs ka) {
   }
   double ent = 0.0;
   for (int i = lane; i < n; i += 32) {
-    double x = fd_x(eps[i], mu, ikT);
+    double x = fd_x(eps[i], mu, kT);
     P.occ[i] = 2.0 * x;
     if (x > 0.0) ent += x * log(x);
     if (x < 1.0) ent += (1.0 - x) * log1p(-x);
@@ -1336,7 +1340,10 @@ void launch_rr2_assemble(const Launch& L, int part) {
   if (!L.map.total) return;
   k_rr2_assemble<<<L.map.total, 256, 0, L.stream>>>(L.ka, part);
 }
-void launch_occupations(const Launch& L) { k_occupations<<<L.ka.nprob, 32, 0, L.stream>>>(L.ka); }
+template <typename T>
+void launch_occupations(const Launch& L) {
+  k_occupations<T><<<L.ka.nprob, 32, 0, L.stream>>>(L.ka);
+}
 void linalg_set_smem_limits(size_t bytes) {
   (void)bytes;
   // the NN kernel also has 8 KB of static shared memory: request only what it uses
@@ -1353,7 +1360,8 @@ void linalg_set_smem_limits(size_t bytes) {
   template void launch_line_min<T>(const Launch&, int, int, int, int);                          \
   template void launch_random_init<T>(const Launch&, int, unsigned long long);                  \
   template void launch_copy_in<T>(const Launch&, int, const double*, int, bool);                \
-  template void launch_copy_out<T>(const Launch&, int, double*, int);
+  template void launch_copy_out<T>(const Launch&, int, double*, int);                           \
+  template void launch_occupations<T>(const Launch&);
 INST(float)
 INST(double)
 #undef INST

@@ -50,7 +50,7 @@ __host__ __device__ inline int nn_rows_f64(int nb, int npw) {
   return 4 * (256 / cg < cap ? 256 / cg : cap);
 }
 constexpr int BAND_THREADS = 256;
-constexpr int GRID_CHUNK = 4096;       // grid points per CTA of the local forces
+constexpr int GRID_CHUNK = 4096;       // grid points per CTA of the local forces and of the mixed path's grid sums
 constexpr int RR_THREADS = 1024;
 constexpr int RR_CLUSTER = 8;          // CTAs of the cluster Rayleigh-Ritz (large subspaces)
 constexpr int LF_GROUP = 4;            // atoms per local-force CTA
@@ -245,7 +245,7 @@ size_t rr_cluster_smem(int n);
 size_t rr_cluster_smem64(int n);
 template <typename T>
 bool launch_rr_cluster(const Launch& L, int n_max, unsigned char* scratch, size_t stride, int max_sweeps, int blk = 1);
-void launch_occupations(const Launch& L);
+template <typename T> void launch_occupations(const Launch& L);
 void linalg_set_smem_limits(size_t bytes);
 
 // k_grid.cu  (grid sources/destinations: 0 rho_in, 1 rho_out, 2 resid, 3 vion_r)
@@ -266,12 +266,14 @@ template <typename T> void launch_potential_g(const Launch& L);
 void launch_vion_g(const Launch& L);
 void launch_rho0_g(const Launch& L);
 void launch_pulay_mix(const Launch& L, double a, double q0);
-// (part: [problem][maxchunk][8], maxchunk chunks of GRID_EW_POINTS at most)
+// (part: [problem][maxchunk][8], chunks of grid_red_chunk points; T = float on the mixed path)
+int grid_red_chunk(bool fp64);
 template <typename T> void launch_grid_energies(const Launch& L, double* part, int maxchunk);
+template <typename T>
 void launch_finish_iteration(const Launch& L, const double* part, int maxchunk, double tol_e, double tol_rho,
                              int count_iter);
-void launch_pulay_gram(const Launch& L, double* part, int maxchunk, int hist);
-void launch_pulay_solve(const Launch& L, const double* part, int maxchunk, int hist);
+template <typename T> void launch_pulay_gram(const Launch& L, double* part, int maxchunk, int hist);
+template <typename T> void launch_pulay_solve(const Launch& L, const double* part, int maxchunk, int hist);
 template <typename T> void launch_build_projectors(const Launch& Latoms, int deriv);
 void launch_local_forces(const Launch& Latom_chunks, int maxchunk);
 void launch_force_total(const Launch& L, int maxchunk);

@@ -296,7 +296,7 @@ __host__ __device__ constexpr int fold_shift() { return log2i(W) - fold_bits<R>(
 
 // Sums of up to 8 values per thread over a block of 256, in tot[8] (shared, valid after the call);
 // red: 64 doubles of shared memory.  Nine additions per warp instead of 40: FP64 additions are what
-// the reductions of the grid kernels cost.
+// the reductions of the grid kernels cost.  (Every value is added in the order of block_sum.)
 __device__ __forceinline__ void block_sums8(const double (&v)[8], double* red, double* tot) {
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   const double s = fold_sums<double, 8, 32>(v, lane);
@@ -304,9 +304,8 @@ __device__ __forceinline__ void block_sums8(const double (&v)[8], double* red, d
   if ((lane & ((1 << S) - 1)) == 0) red[w * 8 + (lane >> S)] = s;
   __syncthreads();
   if (threadIdx.x < 8) {
-    double t = 0.0;
-    for (int k = 0; k < 8; ++k) t += red[k * 8 + threadIdx.x];
-    tot[threadIdx.x] = t;
+    const double* r = red + threadIdx.x;
+    tot[threadIdx.x] = ((r[0] + r[32]) + (r[16] + r[48])) + ((r[8] + r[40]) + (r[24] + r[56]));
   }
   __syncthreads();
 }

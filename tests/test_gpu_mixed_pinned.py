@@ -73,6 +73,36 @@ def products(sgo, name, bands, tensor_cores):
     return _hash(ctx.subspace_matrix(x, y)) + _hash(ctx.subspace_matrix(x, x)) + _hash(ctx.block_update(x, m, -1.5, 0.5, y)) + _hash(h)
 
 
+def _cluster(n, ecut, seed, xc="lda"):
+    rng = np.random.default_rng(seed)
+    cell = np.eye(3) * 20.0
+    bands = int(np.ceil(1.3 * 5 * n))
+    return workloads.Structure(f"cluster{n}", cell, [dict(workloads.SPECIES_Z10)], np.zeros(n, np.int32),
+                               workloads._random_cluster(rng, n, 3.0, 20.0), ecut, bands,
+                               workloads.fft_grid(cell, ecut), 0.01, xc)
+
+
+STRUCTURES = {
+    "cluster3": lambda: _cluster(3, 11.7, 1), "cluster4": lambda: _cluster(4, 9.7, 2, "pbe"),
+    "cluster5": lambda: _cluster(5, 9.0, 3), "cluster6": lambda: _cluster(6, 10.7, 4),
+    "cluster7": lambda: _cluster(7, 8.1, 5), "cluster8": lambda: _cluster(8, 11.5, 6, "pbe"),
+    "cluster10": lambda: _cluster(10, 9.9, 7), "cluster11": lambda: _cluster(11, 9.0, 8),
+    "cluster13": lambda: _cluster(13, 8.9, 9), "tiny2": lambda: workloads.tiny(nat=2, ecut=3.0),
+    "tiny3": lambda: workloads.tiny(nat=3, ecut=8.8), "diamond8": workloads.diamond8,
+    "de44": lambda: workloads.de_candidate(44), "layer": workloads.honeycomb24,
+    "mesh": lambda: dataclasses.replace(workloads.diamond8(), kT=0.01, kgrid=(1, 2, 2)),
+}
+
+
+def evaluation(sgo, name, nbands=None, **opts):
+    st = STRUCTURES[name]()
+    st = dataclasses.replace(st, nbands=nbands or st.nbands)
+    tol = 3e-6 if name.startswith(("cluster", "layer")) else 1e-5
+    ctx = sgo.Context(st, precision="mixed", scf_tol_e=1e-7 * len(st.pos), scf_tol_rho=tol, max_scf=150, **opts)
+    F, forces = ctx.energy_forces(check=False)
+    return [float(F)] + [float(v) for v in np.asarray(forces).ravel()]
+
+
 # every pinned result: name -> how it is computed
 CASES = {}
 for _g in GRIDS:
@@ -81,6 +111,8 @@ for _g, _n in DENSITIES:
     CASES["density %dx%dx%d, %d bands" % (*_g, _n)] = lambda s, g=_g, n=_n: density(s, g, n)
 for _p in PRODUCTS:
     CASES["products %s, %d bands, gemm_tc=%d" % _p] = lambda s, p=_p: products(s, *p)
+for _n in STRUCTURES:  # (the eigensolve of a cluster of CTAs at every size)
+    CASES["evaluation %s, rr_cluster=1" % _n] = lambda s, n=_n: evaluation(s, n, rr_cluster=1)
 
 
 @pytest.mark.parametrize("name", CASES)
