@@ -127,10 +127,12 @@ typedef struct {
                              requested bands get headroom; occupations, eigenvalues, energies and
                              the eig_tol test cover the requested bands only (-1, default:
                              4 + nbands / 32; 0 = none) */
-  int rr_cluster;         /* subspace diagonalisation kernel: -1 (default) or 0 the tridiagonal one
-                             (one CTA or a small cluster per member) up to 184 bands (FP64: 128),
-                             beyond it the Jacobi one on a cluster of 8 CTAs per member; 1 = always
-                             the latter.  Taken from the first member of a batch. */
+  int rr_cluster;         /* subspace diagonalisation kernel: -1 (default) on the mixed path one CTA per
+                             member while its matrices fit in shared memory, in FP64 the tridiagonal
+                             kernel (one CTA or a small cluster per member) up to 128 bands, else a
+                             thread-block cluster of 8 CTAs per member; 0 = as -1, but one CTA over a
+                             global scratch where -1 takes that cluster; 1 = always the cluster of 8.
+                             Taken from the first member of a batch. */
   int eigensolver;        /* 0 (default): Algorithm 1's all-band CG steps (Sec. II D): per band a
                              preconditioned, conjugated, projected search direction, a line
                              minimisation, then a Rayleigh-Ritz over the n_b bands.  1: block
@@ -261,8 +263,9 @@ SGO_API sgo_status sgo_get_terms(sgo_ctx* ctx, double terms[8]);
 SGO_API sgo_status sgo_get_info(sgo_ctx* ctx, int info[10]);
 
 /* Diagnostics of the last SCF: [0] iterations, [1] Jacobi sweeps summed over its
- * subspace diagonalisations on the cluster (rr_cluster; the one-CTA kernel makes none),
- * [2] final density residual, [3] final |F_k - F_{k-1}|, [4] CG steps taken after the SCF stopping rule held (eig_tol), [5] the largest residual
+ * subspace diagonalisations (0 where the FP64 path's tridiagonal kernel made them all),
+ * [2] final density residual, [3] final |F_k - F_{k-1}|,
+ * [4] CG steps taken after the SCF stopping rule held (eig_tol), [5] the largest residual
  * |H psi - eps psi| over the bands with occupation above 1e-6 at the end, [6] subspace
  * diagonalisations that stopped at their iteration cap, [7] SCF iterations of the
  * last SCF loop that started from a state set by sgo_set_state (0 otherwise). */

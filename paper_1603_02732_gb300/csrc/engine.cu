@@ -1015,17 +1015,26 @@ Engine::Engine(const std::vector<sgo_ctx*>& ctxs, cudaStream_t stream) : ctx_(ct
   }
   const sgo_opts& o0 = ctxs[0]->opts;
   wait_ns_ = o0.watchdog_ms > 0.0 ? (long long)(o0.watchdog_ms * 1e6) : 2000000000LL;
-  // subspace diagonalisation: k_rr_td.cu per member up to rr_td_max bands (184 on the mixed path,
-  // 128 in FP64), beyond (or when asked for) one thread-block cluster per member (k_rr_cluster)
+  // subspace diagonalisation.  FP64 path: k_rr_td.cu up to rr_td_max() bands.  Mixed path: the one-CTA
+  // Jacobi kernels while their matrices fit in shared memory (FP32 deviation form up to nb = 105, FP64
+  // up to nb = 91): slower (24-atom layer 299 us a solve, 256 by divide and conquer with a correction),
+  // but any other rounding moves the mixed path's results (see the grid transforms above), so they
+  // stay.  Beyond, or when asked for, one thread-block cluster per member over a global scratch
+  // (k_rr_cluster), or (rr_cluster = 0) the one-CTA kernels over a global scratch.
   // (the block Davidson steps diagonalise the 2 n_b block [X, W])
   davidson_ = o0.eigensolver == 1;
   cg_adapt_ = o0.cg_adapt;
   gga_ = o0.xc == 1;
   rr_n_ = (davidson_ ? 2 : 1) * max_nb_;
   rr_f32_ = precision_ == 1 && !o0.rr_fp64;
-  const size_t ts = rr_f32_ ? sizeof(float) : sizeof(double);
-  rr_cluster_ = o0.rr_cluster > 0 || rr_n_ > rr_td_max(ts);
-  rr_stride_ = ((rr_cluster_ ? rr_cluster_scratch_bytes(rr_n_, ts) : rr_td_scratch_bytes(rr_n_, ts)) + 255) / 256 * 256;
+  const size_t ts = rr_f32_ ? sizeof(float) : sizeof(double), jn = rr_n_;
+  rr_td_ = precision_ == 0 && o0.rr_cluster <= 0 && rr_n_ <= rr_td_max();
+  const size_t jacobi = rr_f32_ ? 5 * jn * (jn | 1) * ts : 3 * jn * jn * ts;  // matrices of the one-CTA kernels
+  rr_smem_ = precision_ == 1 && jacobi <= (rr_f32_ ? 216 : 200) * 1024 ? jacobi : 0;
+  // (the one-CTA kernels' pair tables hold 256 pairs: beyond 512 bands the cluster is used)
+  rr_cluster_ = !rr_td_ && (o0.rr_cluster > 0 || (o0.rr_cluster < 0 && !rr_smem_) || rr_n_ > 512);
+  rr_stride_ = rr_td_ ? rr_td_scratch_bytes(rr_n_) : rr_cluster_ ? rr_cluster_scratch_bytes(rr_n_, ts) : rr_smem_ ? 0 : jacobi;
+  rr_stride_ = (rr_stride_ + 255) / 256 * 256;
   if (rr_stride_) {
     if (!cuda_ok(dev_malloc(&d_rr_, rr_stride_ * n_), "dev_malloc(rr scratch)")) return;
     allocs_.push_back(d_rr_);
@@ -1318,10 +1327,12 @@ void Engine::rr_solve(int blk) {
     const bool launched = rr_f32_ ? launch_rr_cluster<float>(l, rr_n_, d_rr_, rr_stride_, cap, blk)
                                   : launch_rr_cluster<double>(l, rr_n_, d_rr_, rr_stride_, 30, blk);
     if (!launched) set_error("cluster Rayleigh-Ritz launch refused");
+  } else if (rr_td_) {
+    launch_rr_td(L(m_prob_), blk * max_nb_, d_rr_, rr_stride_, blk);
   } else if (rr_f32_) {
-    launch_rr_td<float>(L(m_prob_), blk * max_nb_, d_rr_, rr_stride_, blk);
+    launch_rr_f32(L(m_prob_), rr_smem_, reinterpret_cast<float*>(d_rr_), rr_stride_ / sizeof(float), cap, blk);
   } else {
-    launch_rr_td<double>(L(m_prob_), blk * max_nb_, d_rr_, rr_stride_, blk);
+    launch_rr(L(m_prob_), rr_smem_ > 0, rr_smem_, reinterpret_cast<double*>(d_rr_), rr_stride_ / sizeof(double), 30, blk);
   }
   tend(TK_RR);
   work_mult_ = 1;

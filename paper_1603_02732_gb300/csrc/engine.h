@@ -208,7 +208,9 @@ class Engine {
   double* d_gpart_ = nullptr;
   int maxchunk_ = 1;
   bool rr_f32_ = false;
-  bool rr_cluster_ = false;          // subspace too large for one CTA: cluster eigensolve
+  bool rr_td_ = false;               // k_rr_td (FP64 path)
+  size_t rr_smem_ = 0;               // shared memory of the one-CTA Jacobi kernels (0: global scratch)
+  bool rr_cluster_ = false;          // cluster eigensolve
   bool davidson_ = false;            // block Davidson steps (2 n_b Rayleigh-Ritz) instead of CG
   bool gga_ = false;                 // PBE exchange-correlation
   double cg_adapt_ = 0.0;            // density residual above which the last CG step is left out

@@ -9,8 +9,8 @@
 //    by the Rayleigh-Ritz eigenvectors, the projection P -= Psi C, the nonlocal apply.
 //  * per-band kernels: residual + preconditioner + conjugate direction, normalisation,
 //    line minimisation.
-//  * rr: the subspace diagonalisation of Algorithm 1 for subspaces beyond k_rr_td.cu, on a
-//    cluster of CTAs.
+//  * rr: the subspace diagonalisation of Algorithm 1 by cyclic Jacobi: the mixed path's, and the
+//    FP64 path's beyond k_rr_td.cu.
 //  * occupations: Fermi-Dirac with the chemical potential by safeguarded Newton.
 #include <cooperative_groups.h>
 
@@ -65,10 +65,14 @@ __device__ __forceinline__ void rr_out_eps(const Prob& P, int rk, double e) {
 // residuals of a random start are nearly collinear): its column of the factor is zero, its
 // row of the inverse factor is zero (so the projected matrix has a zero row and column,
 // which no rotation touches), and its eigenvalue is taken as RR_DROP_DIAG, so that it ranks
-// above every kept Ritz value.  (The same bound fails the Cholesky of an X direction.)
+// above every kept Ritz value.  (In the FP32 and cluster kernels the same bound fails the
+// Cholesky of an X direction.)
 constexpr double RR_DROP = 1e-3;
 constexpr double RR_DROP_DIAG = 1e12;
 constexpr float RR_DROPPED = -2.f;  // pivot deviation recorded for a left-out direction
+// Jacobi sweeps of the FP32 eigensolve with at most this many entries above the threshold run
+// as sparse passes (k_rr_f32)
+constexpr int RR_SPARSE = 256;
 
 // ---------------------------------------------------------------------------
 // C = A^T B, split-K partials.  CTA = (problem, tile block, split).  The outputs are dealt in
@@ -775,10 +779,627 @@ __global__ void k_copy_out(KArgs ka, int role, double* dst, int nvec) {
 }
 
 // ---------------------------------------------------------------------------
+// Rayleigh-Ritz in FP64, one CTA per problem (orthonormalisation + subspace
+// diagonalisation of Algorithm 1).
+//   S = L L^T (Cholesky), C = L^-1 Hs L^-T, C = V diag(eps) V^T (cyclic Jacobi,
+//   round-robin parallel ordering; Golub & Van Loan, Alg. 8.4.3), Tm = L^-T V,
+//   so that X Tm is orthonormal and diagonalises H in the subspace.
+// Matrices: A, L, V in shared memory when 3 nb^2 doubles fit, else in global scratch.
+// ---------------------------------------------------------------------------
+__global__ void __launch_bounds__(RR_THREADS) k_rr(KArgs ka, int use_smem, double* gscratch, size_t gstride,
+                                                   int max_sweeps, int blk) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  __shared__ double red[33];
+  __shared__ double cs_c[256], cs_s[256];
+  __shared__ int pr_p[256], pr_q[256];
+  __shared__ int flag;
+  __shared__ unsigned char drp[512];  // left-out directions (blk = 2)
+  const int p = blockIdx.x;
+  if (!ka.active[p]) return;
+  const Prob& P = ka.probs[p];
+  const int n = blk * P.nb;
+  const double* Sin = rr_in_s(P, blk);
+  const double* Hin = rr_in_h(P, blk);
+  double *A, *L, *V;
+  if (use_smem) {
+    A = reinterpret_cast<double*>(smem_raw);
+  } else {
+    A = gscratch + (size_t)p * gstride;
+  }
+  L = A + n * n;
+  V = L + n * n;
+  const int tid = threadIdx.x, nt = blockDim.x;
+  if (tid == 0) flag = 0;
+  // symmetrised inputs
+  for (int e = tid; e < n * n; e += nt) {
+    int i = e / n, j = e % n;
+    L[e] = 0.5 * (Sin[i * n + j] + Sin[j * n + i]);
+    A[e] = 0.5 * (Hin[i * n + j] + Hin[j * n + i]);
+  }
+  __syncthreads();
+  // Cholesky of L in place (lower triangle); a left-out direction (blk = 2) gets a unit
+  // pivot and a zero column (its row of L^-1 is cleared below)
+  for (int k = 0; k < n; ++k) {
+    if (tid == 0) {
+      double d = L[k * n + k];
+      const bool dr = blk == 2 && k >= P.nb && d <= RR_DROP;
+      if (dr) d = 1.0;
+      if (!(d > 0.0)) { flag = 1; d = 1.0; }
+      L[k * n + k] = sqrt(d);
+      drp[k] = dr ? 1 : 0;
+    }
+    __syncthreads();
+    const bool drop = drp[k] != 0;
+    const double dk = L[k * n + k];
+    for (int i = k + 1 + tid; i < n; i += nt) L[i * n + k] = drop ? 0.0 : L[i * n + k] / dk;
+    __syncthreads();
+    const int m = n - k - 1;
+    for (int e = tid; e < m * m; e += nt) {
+      int i = k + 1 + e / m, j = k + 1 + e % m;
+      if (j <= i) L[i * n + j] -= L[i * n + k] * L[j * n + k];
+    }
+    __syncthreads();
+  }
+  // L := L^-1 (lower), row by row: X[i][j] = -(sum_{k=j}^{i-1} L[i][k] X[k][j]) / L[i][i]
+  // done out of place into V, then copied back.
+  for (int e = tid; e < n * n; e += nt) V[e] = 0.0;
+  __syncthreads();
+  for (int i = 0; i < n; ++i) {
+    const double lii = L[i * n + i];
+    for (int j = tid; j <= i; j += nt) {
+      if (j == i) {
+        V[i * n + i] = 1.0 / lii;
+      } else {
+        double s = 0.0;
+        for (int k = j; k < i; ++k) s += L[i * n + k] * V[k * n + j];
+        V[i * n + j] = -s / lii;
+      }
+    }
+    __syncthreads();
+  }
+  // (rows of L^-1 of left-out directions cleared)
+  for (int e = tid; e < n * n; e += nt) L[e] = drp[e / n] ? 0.0 : V[e];
+  __syncthreads();
+  // V := A L^T ; A := L V   (C = L^-1 Hs L^-T, symmetric)
+  for (int e = tid; e < n * n; e += nt) {
+    int i = e / n, j = e % n;
+    double s = 0.0;
+    for (int k = 0; k <= j; ++k) s += A[i * n + k] * L[j * n + k];
+    V[e] = s;
+  }
+  __syncthreads();
+  for (int e = tid; e < n * n; e += nt) {
+    int i = e / n, j = e % n;
+    double s = 0.0;
+    for (int k = 0; k <= i; ++k) s += L[i * n + k] * V[k * n + j];
+    A[e] = s;
+  }
+  __syncthreads();
+  for (int e = tid; e < n * n; e += nt) {
+    int i = e / n, j = e % n;
+    if (j > i) {
+      double s = 0.5 * (A[i * n + j] + A[j * n + i]);
+      A[i * n + j] = s;
+      A[j * n + i] = s;
+    }
+  }
+  // accumulate the rotations onto L^-T, so that V ends as Tm = L^-T U directly
+  for (int e = tid; e < n * n; e += nt) {
+    int i = e / n, j = e % n;
+    V[e] = L[j * n + i];
+  }
+  __syncthreads();
+  // cyclic Jacobi, round-robin pairing over m = n rounded up to even.  A rotation whose
+  // |a_pq| is below 1e-14 sqrt(|a_pp a_qq|) is skipped; sweeps stop once the
+  // off-diagonal norm is below 1e-11 of the diagonal norm (FP64 rounding floor ~1e-15).
+  const int m = n + (n & 1);
+  const int half = m / 2;
+  int sweeps = 0, capped = 0;
+  for (int sweep = 0;; ++sweep) {
+    double off = 0.0, dia = 0.0;
+    for (int e = tid; e < n * n; e += nt) {
+      int i = e / n, j = e % n;
+      double v = A[e] * A[e];
+      if (i == j) dia += v; else off += v;
+    }
+    off = block_sum(off, red);
+    dia = block_sum(dia, red);
+    if (off <= 1e-22 * dia || off == 0.0) break;
+    if (sweep == max_sweeps) {
+      capped = 1;
+      break;
+    }
+    ++sweeps;
+    for (int r = 0; r < m - 1; ++r) {
+      if (tid < half) {
+        // tournament: position 0 fixed, positions 1..m-1 rotate by r
+        int a = tid, b = m - 1 - tid;
+        int pa = a == 0 ? 0 : 1 + (a - 1 + r) % (m - 1);
+        int pb = b == 0 ? 0 : 1 + (b - 1 + r) % (m - 1);
+        int pp = min(pa, pb), qq = max(pa, pb);
+        double c = 1.0, s = 0.0;
+        if (qq < n) {
+          double apq = A[pp * n + qq];
+          double app = A[pp * n + pp], aqq = A[qq * n + qq];
+          if (fabs(apq) > 1e-14 * sqrt(fabs(app * aqq)) && fabs(apq) > 1e-300) {
+            double tau = (aqq - app) / (2.0 * apq);
+            double t = (tau >= 0.0 ? 1.0 : -1.0) / (fabs(tau) + sqrt(1.0 + tau * tau));
+            c = 1.0 / sqrt(1.0 + t * t);
+            s = t * c;
+          }
+        }
+        cs_c[tid] = c;
+        cs_s[tid] = s;
+        pr_p[tid] = pp;
+        pr_q[tid] = qq;
+      }
+      __syncthreads();
+      // rows: A <- J^T A
+      for (int e = tid; e < half * n; e += nt) {
+        int k = e / n, j = e % n;
+        double s = cs_s[k];
+        if (s == 0.0) continue;
+        int pp = pr_p[k], qq = pr_q[k];
+        double c = cs_c[k];
+        double ap = A[pp * n + j], aq = A[qq * n + j];
+        A[pp * n + j] = c * ap - s * aq;
+        A[qq * n + j] = s * ap + c * aq;
+      }
+      __syncthreads();
+      // columns: A <- A J, V <- V J
+      for (int e = tid; e < half * n; e += nt) {
+        int k = e / n, i = e % n;
+        double s = cs_s[k];
+        if (s == 0.0) continue;
+        int pp = pr_p[k], qq = pr_q[k];
+        double c = cs_c[k];
+        double ap = A[i * n + pp], aq = A[i * n + qq];
+        A[i * n + pp] = c * ap - s * aq;
+        A[i * n + qq] = s * ap + c * aq;
+        double vp = V[i * n + pp], vq = V[i * n + qq];
+        V[i * n + pp] = c * vp - s * vq;
+        V[i * n + qq] = s * vp + c * vq;
+      }
+      __syncthreads();
+    }
+  }
+  // ascending order: rank of each eigenvalue (a left-out direction ranks last)
+  for (int j = tid; j < n; j += nt) {
+    double ej = drp[j] ? RR_DROP_DIAG : A[j * n + j];
+    int rank = 0;
+    for (int k2 = 0; k2 < n; ++k2) {
+      double ek = drp[k2] ? RR_DROP_DIAG : A[k2 * n + k2];
+      rank += (ek < ej) || (ek == ej && k2 < j);
+    }
+    rr_out_eps(P, rank, ej);
+    P.bv[BV_TMP0 * P.nb + j] = (double)rank;  // (blk = 2: rows BV_TMP0 and BV_TMP1)
+  }
+  __syncthreads();
+  // Tm[:, rank(j)] = V[:, j]  (= L^-T U)
+  for (int e = tid; e < n * n; e += nt) {
+    int i = e / n, j = e % n;
+    rr_out_vec(P, i, (int)P.bv[BV_TMP0 * P.nb + j], V[e]);
+  }
+  if (tid == 0) {
+    P.scal[SC_RRSWEEPS] += sweeps;
+    P.scal[SC_RRCAP] += capped;
+  }
+  if (tid == 0 && flag) P.status[0] = 1;
+}
+
+// ---------------------------------------------------------------------------
+// Rayleigh-Ritz for the mixed path, one CTA per problem, in FP32 shared memory.
+// The overlap is factored in deviation form: S = I + E, L = I + D (Cholesky), L^-1 =
+// I + G.  Every stored quantity is then of the size of E and keeps FP32 relative
+// accuracy, so the factors are as accurate as an FP64 factorisation of the same S (whose
+// entries carry the GEMM's FP32 rounding anyway): for column k, with x = E_kk - sum D_kj^2
+// (the running trailing entry), d_k = sqrt(1 + x) - 1 = x / (1 + sqrt(1 + x)), and
+// D_ik = (E_ik - sum_j D_ij D_kj) / (1 + d_k).  G follows from (I + D)(I + G) = I row by
+// row.  Then C = (I + G) H (I + G)^T, its cyclic Jacobi eigensolve accumulated onto
+// V = (I + G)^T, and Tm = V in ascending eigenvalue order.  The eigen-rotation feeds the
+// FP32 block rotation, so accuracy beyond FP32 would be discarded there.
+// Shared memory: D, G, Hf (then V^T), W, A, each n x ns floats with an odd row stride
+// ns = n | 1, so that walks down a column hit distinct banks.
+// ---------------------------------------------------------------------------
+__device__ __forceinline__ float warp_sum_f(float v) {
+  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+  return v;
+}
+
+__global__ void __launch_bounds__(RR_THREADS) k_rr_f32(KArgs ka, float* gscratch, size_t gstride, int max_sweeps,
+                                                       int blk) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  __shared__ float red[32];
+  __shared__ float dkv[512];  // Cholesky pivots d_k (n <= 512: the pair tables below hold 256 pairs)
+  // (the rotations of a round, or, while a sparse pass is being scheduled, the round
+  // masks of every index)
+  __shared__ union {
+    struct {
+      float c[256], s[256];
+    } cs;
+    unsigned used[512];
+  } ru;
+  float* cs_c = ru.cs.c;
+  float* cs_s = ru.cs.s;
+  __shared__ int pr_p[256], pr_q[256];
+  __shared__ int sp_list[RR_SPARSE], sp_sorted[RR_SPARSE], sp_rstart[33];
+  __shared__ unsigned char sp_stamp[512];
+  __shared__ int flag, nbig, sp_rounds, wcnt[32];
+  const int p = blockIdx.x;
+  if (!ka.active[p]) return;
+  const Prob& P = ka.probs[p];
+  const int n = blk * P.nb, ns = n | 1, nn = n * ns;
+  const double* Sin = rr_in_s(P, blk);
+  const double* Hin = rr_in_h(P, blk);
+  // the five matrices live in shared memory, or (large n) in this problem's global scratch
+  float* D = gscratch ? gscratch + (size_t)p * gstride : reinterpret_cast<float*>(smem_raw);
+  float* G = D + nn;
+  float* Hf = G + nn;
+  float* W = Hf + nn;
+  float* A = W + nn;
+  float* Vt = Hf;  // V^T, once Hf is consumed
+  const int tid = threadIdx.x, nt = blockDim.x, tx = tid & 31, ty = tid >> 5, nty = nt >> 5;
+  if (tid == 0) flag = 0;
+  for (int i = ty; i < n; i += nty)
+    for (int j = tx; j < n; j += 32) {
+      D[i * ns + j] = (float)(0.5 * (Sin[i * n + j] + Sin[j * n + i]) - (i == j ? 1.0 : 0.0));
+      Hf[i * ns + j] = (float)(0.5 * (Hin[i * n + j] + Hin[j * n + i]));
+      G[i * ns + j] = 0.f;
+    }
+  __syncthreads();
+  // Cholesky in deviation form, right-looking, one barrier per column: step k reads the
+  // lower column k (final after step k - 1), writes the scaled column L_ik = D_ik / (1 + d_k)
+  // into the upper row k (D_ki, never read in step k) and updates the lower trailing block
+  // with the scaled values formed on the fly; d_k goes to dkv
+  // (a left-out direction of the block [X, W]: zero scaled column, no update, pivot mark
+  // RR_DROPPED in dkv)
+  for (int k = 0; k < n; ++k) {
+    const float x = D[k * ns + k];
+    const bool drop = blk == 2 && k >= P.nb && x <= (float)RR_DROP - 1.f;
+    const float xs = drop ? 0.f : fmaxf(x, -0.999f);
+    const float dk = xs / (1.f + sqrtf(1.f + xs));
+    const float inv = drop ? 0.f : 1.f / (1.f + dk);
+    if (tid == 0) {
+      if (!drop && !(x > -0.999f)) flag = 1;  // S not positive definite (to FP32 resolution)
+      dkv[k] = drop ? RR_DROPPED : dk;
+    }
+    for (int i = k + 1 + tid; i < n; i += nt) D[k * ns + i] = D[i * ns + k] * inv;
+    if (!drop)
+      for (int i = k + 1 + ty; i < n; i += nty) {
+        const float lik = D[i * ns + k] * inv;
+        for (int j = k + 1 + tx; j <= i; j += 32) D[i * ns + j] -= lik * (D[j * ns + k] * inv);
+      }
+    __syncthreads();
+  }
+  // G: G_ii = -d_i / (1 + d_i), G_ij = -(L_ij + sum_{j<=k<i} L_ik G_kj) / (1 + d_i) with
+  // L_ik = D_ki; every column j of G is an independent forward substitution: one warp per
+  // column, lanes splitting the sum, no block barrier until all columns are done
+  // (a left-out direction's row of I + G is zero: G_jj = -1, G_ij = 0)
+  for (int j = ty; j < n; j += nty) {
+    if (tx == 0) G[j * ns + j] = dkv[j] == RR_DROPPED ? -1.f : -dkv[j] / (1.f + dkv[j]);
+    __syncwarp();
+    for (int i = j + 1; i < n; ++i) {
+      float sacc = 0.f;
+      for (int k = j + tx; k < i; k += 32) sacc += D[k * ns + i] * G[k * ns + j];
+      sacc = warp_sum_f(sacc);
+      if (tx == 0) G[i * ns + j] = dkv[i] == RR_DROPPED ? 0.f : -(D[j * ns + i] + sacc) / (1.f + dkv[i]);
+      __syncwarp();
+    }
+  }
+  __syncthreads();
+  // W = (I + G) Hf, A = W (I + G)^T
+  for (int i = ty; i < n; i += nty)
+    for (int j = tx; j < n; j += 32) {
+      float s = 0.f;
+      for (int k = 0; k <= i; ++k) s += G[i * ns + k] * Hf[k * ns + j];
+      W[i * ns + j] = Hf[i * ns + j] + s;
+    }
+  __syncthreads();
+  for (int i = ty; i < n; i += nty)
+    for (int j = tx; j < n; j += 32) {
+      float s = 0.f;
+      for (int k = 0; k <= j; ++k) s += W[i * ns + k] * G[j * ns + k];
+      A[i * ns + j] = W[i * ns + j] + s;
+    }
+  __syncthreads();
+  float amax = 0.f;
+  for (int i = ty; i < n; i += nty)
+    for (int j = tx; j < n; j += 32) {
+      if (j > i) {
+        const float sy = 0.5f * (A[i * ns + j] + A[j * ns + i]);
+        A[i * ns + j] = sy;
+        A[j * ns + i] = sy;
+      }
+      if (i == j) amax = fmaxf(amax, fabsf(A[i * ns + i]));
+      Vt[i * ns + j] = (i == j ? 1.f : 0.f) + G[i * ns + j];  // V = (I + G)^T = L^-T
+    }
+  for (int o = 16; o > 0; o >>= 1) amax = fmaxf(amax, __shfl_xor_sync(0xffffffffu, amax, o));
+  if (tx == 0) red[ty] = amax;
+  __syncthreads();
+  float mm = 0.f;
+  for (int w = 0; w < nty; ++w) mm = fmaxf(mm, red[w]);
+  // rotations below 2e-7 max|a_ii| (about the FP32 resolution of the matrix) are skipped
+  const float thr = 2e-7f * mm;
+  // Threshold Jacobi.  Each sweep starts by listing the off-diagonal entries above thr.
+  // Many of them (more than RR_SPARSE, or more than two per index, where the colouring
+  // below would need about as many rounds as a sweep): a cyclic sweep in round-robin
+  // order, where a round
+  // maps every 2x2 block of pair rows P and pair columns Q as A_PQ <- J_P^T A_PQ J_Q (one
+  // pass) and V_{:,Q} <- V_{:,Q} J_Q.  Few (the sweeps after the first, once the
+  // convergence is quadratic): a sparse pass that rotates only the listed pairs, packed
+  // into rounds of disjoint pairs by a greedy edge colouring (a pair takes the first round
+  // in which neither of its indices is used yet; pairs that find none of the 32 rounds
+  // free wait for the next pass).  Any order that keeps visiting every entry above the
+  // threshold converges (the threshold cyclic Jacobi with a skipped-rotation rule).
+  const int m = n + (n & 1);
+  const int half = m / 2;
+  int sweeps = 0, capped = 0;
+  for (int sweep = 0;; ++sweep) {
+    // the entries above the threshold: counted per warp, then (a sparse pass) listed in a
+    // fixed order, warp after warp, each warp's rows in order, so that the rotation order
+    // and hence the rounding never depend on the scheduling
+    {
+      int cnt = 0;
+      for (int i = ty; i < n; i += nty)
+        for (int j0 = i + 1; j0 < n; j0 += 32) {
+          const int j = j0 + tx;
+          cnt += __popc(__ballot_sync(0xffffffffu, j < n && fabsf(A[i * ns + j]) > thr));
+        }
+      if (tx == 0) wcnt[ty] = cnt;
+    }
+    __syncthreads();
+    if (tid == 0) {
+      int s = 0;
+      for (int w = 0; w < nty; ++w) {
+        const int c = wcnt[w];
+        wcnt[w] = s;
+        s += c;
+      }
+      nbig = s;
+    }
+    __syncthreads();
+    const int nlist = nbig;
+    if (nlist == 0) break;
+    const bool sparse = nlist <= min(RR_SPARSE, 2 * m);
+    if (sparse) {
+      int k = wcnt[ty];
+      for (int i = ty; i < n; i += nty)
+        for (int j0 = i + 1; j0 < n; j0 += 32) {
+          const int j = j0 + tx;
+          const bool big = j < n && fabsf(A[i * ns + j]) > thr;
+          const unsigned bal = __ballot_sync(0xffffffffu, big);
+          if (big) sp_list[k + __popc(bal & ((1u << tx) - 1u))] = i | (j << 10);
+          k += __popc(bal);
+        }
+      __syncthreads();
+    }
+    if (sweep == max_sweeps) {  // still off-diagonal entries above the threshold
+      capped = 1;
+      break;
+    }
+    ++sweeps;
+    if (sparse) {
+      // schedule: round masks and stamps cleared, greedy colouring by one thread, then the
+      // pairs bucketed by round (counts, scan, placement)
+      for (int i = tid; i < n; i += nt) {
+        ru.used[i] = 0u;
+        sp_stamp[i] = 0;
+      }
+      if (tid < 33) sp_rstart[tid] = 0;
+      __syncthreads();
+      if (tid == 0) {
+        int nr = 0;
+        for (int k = 0; k < nlist; ++k) {
+          const int e = sp_list[k];
+          const int a = e & 1023, b = e >> 10;
+          const unsigned fr = ~(ru.used[a] | ru.used[b]);
+          if (fr == 0u) {
+            sp_list[k] = -1;
+            continue;
+          }
+          const int r = __ffs(fr) - 1;
+          ru.used[a] |= 1u << r;
+          ru.used[b] |= 1u << r;
+          sp_list[k] = e | (r << 20);
+          sp_rstart[r + 1] += 1;
+          nr = max(nr, r + 1);
+        }
+        for (int r = 0; r < nr; ++r) sp_rstart[r + 1] += sp_rstart[r];
+        sp_rounds = nr;
+      }
+      __syncthreads();
+      if (tid < 32) {  // placement: one warp, pairs in list order within each round
+        for (int k0 = 0; k0 < nlist; k0 += 32) {
+          const int k = k0 + tid;
+          const int e = k < nlist ? sp_list[k] : -1;
+          const int r = e < 0 ? -1 : e >> 20;
+          for (int rr = 0; rr < sp_rounds; ++rr) {
+            const unsigned bal = __ballot_sync(0xffffffffu, r == rr);
+            if (r == rr) sp_sorted[sp_rstart[rr] + __popc(bal & ((1u << tid) - 1u))] = e & 0xfffff;
+            __syncwarp();
+            if (tid == 0) sp_rstart[rr] += __popc(bal);
+            __syncwarp();
+          }
+        }
+        // (sp_rstart[r] now holds the end of round r; the start is the end of r - 1)
+      }
+      __syncthreads();
+      const int nr = sp_rounds;
+      for (int r = 0; r < nr; ++r) {
+        const int b0 = r == 0 ? 0 : sp_rstart[r - 1], kr = sp_rstart[r] - b0;
+        if (tid < kr) {
+          const int e = sp_sorted[b0 + tid];
+          const int pp = e & 1023, qq = e >> 10;
+          float c = 1.f, s = 0.f;
+          const float apq = A[pp * ns + qq];
+          if (fabsf(apq) > thr) {
+            const float tau = __fdividef(A[qq * ns + qq] - A[pp * ns + pp], 2.f * apq);
+            const float t = copysignf(__fdividef(1.f, fabsf(tau) + sqrtf(fmaf(tau, tau, 1.f))), tau);
+            c = rsqrtf(fmaf(t, t, 1.f));
+            s = t * c;
+          }
+          cs_c[tid] = c;
+          cs_s[tid] = s;
+          pr_p[tid] = pp;
+          pr_q[tid] = qq;
+          sp_stamp[pp] = (unsigned char)(r + 1);
+          sp_stamp[qq] = (unsigned char)(r + 1);
+        }
+        __syncthreads();
+        // 2x2 blocks between the round's pairs; pair rows against the other columns (row
+        // rotation, mirrored into the symmetric column entries); V
+        for (int P2 = ty; P2 < kr; P2 += nty) {
+          const float sp = cs_s[P2], cp = cs_c[P2];
+          const int p0 = pr_p[P2], p1 = pr_q[P2];
+          for (int Q2 = tx; Q2 < kr; Q2 += 32) {
+            const float sq = cs_s[Q2];
+            if (sp == 0.f && sq == 0.f) continue;
+            const float cq = cs_c[Q2];
+            const int q0 = pr_p[Q2], q1 = pr_q[Q2];
+            const float a00 = A[p0 * ns + q0], a01 = A[p0 * ns + q1];
+            const float a10 = A[p1 * ns + q0], a11 = A[p1 * ns + q1];
+            const float b00 = cp * a00 - sp * a10, b01 = cp * a01 - sp * a11;
+            const float b10 = sp * a00 + cp * a10, b11 = sp * a01 + cp * a11;
+            A[p0 * ns + q0] = cq * b00 - sq * b01;
+            A[p0 * ns + q1] = sq * b00 + cq * b01;
+            A[p1 * ns + q0] = cq * b10 - sq * b11;
+            A[p1 * ns + q1] = sq * b10 + cq * b11;
+          }
+          if (sp == 0.f) continue;
+          for (int j = tx; j < n; j += 32) {
+            if (sp_stamp[j] == (unsigned char)(r + 1)) continue;
+            const float a0 = A[p0 * ns + j], a1 = A[p1 * ns + j];
+            const float b0 = cp * a0 - sp * a1, b1 = sp * a0 + cp * a1;
+            A[p0 * ns + j] = b0;
+            A[p1 * ns + j] = b1;
+            A[j * ns + p0] = b0;
+            A[j * ns + p1] = b1;
+          }
+          for (int i = tx; i < n; i += 32) {
+            const float v0 = Vt[p0 * ns + i], v1 = Vt[p1 * ns + i];
+            Vt[p0 * ns + i] = cp * v0 - sp * v1;
+            Vt[p1 * ns + i] = sp * v0 + cp * v1;
+          }
+        }
+        __syncthreads();
+      }
+      continue;
+    }
+    for (int r = 0; r < m - 1; ++r) {
+      if (tid < half) {
+        const int a = tid, b = m - 1 - tid;
+        int ta = a - 1 + r, tb = b - 1 + r;  // (both < 2 (m - 1): one conditional subtraction)
+        if (ta >= m - 1) ta -= m - 1;
+        if (tb >= m - 1) tb -= m - 1;
+        const int pa = a == 0 ? 0 : 1 + ta;
+        const int pb = b == 0 ? 0 : 1 + tb;
+        const int pp = min(pa, pb), qq = max(pa, pb);
+        float c = 1.f, s = 0.f;
+        if (qq < n) {
+          const float apq = A[pp * ns + qq];
+          if (fabsf(apq) > thr) {
+            // (fast reciprocals: any orthogonal rotation near the exact one converges the sweep)
+            const float tau = __fdividef(A[qq * ns + qq] - A[pp * ns + pp], 2.f * apq);
+            const float t = copysignf(__fdividef(1.f, fabsf(tau) + sqrtf(fmaf(tau, tau, 1.f))), tau);
+            c = rsqrtf(fmaf(t, t, 1.f));
+            s = t * c;
+          }
+        }
+        cs_c[tid] = c;
+        cs_s[tid] = s;
+        pr_p[tid] = pp;
+        pr_q[tid] = qq;
+      }
+      __syncthreads();
+      // blocks (P, Q) with P <= Q, each written with its mirror (Q, P): the upper triangle
+      // of the half x half block grid, folded so that block rows P and half - 1 - P share
+      // one row of half + 1 items, dealt to all threads; rows / columns equal to n (the
+      // odd dummy) are absent
+      {
+        const int wrow = half + 1, nitem = ((half + 1) / 2) * wrow;
+        const float inv_wrow = 1.f / (float)wrow;
+        for (int e = tid; e < nitem; e += nt) {
+          int P2 = __float2int_rz(((float)e + 0.5f) * inv_wrow);
+          int Q2 = e - P2 * wrow;  // (offset d in the folded row)
+          if (Q2 < half - P2) {
+            Q2 += P2;
+          } else {
+            const int P3 = half - 1 - P2;
+            if (P3 == P2) continue;  // (odd half: the middle row holds only its own part)
+            Q2 = P3 + Q2 - (half - P2);
+            P2 = P3;
+          }
+          const float sp = cs_s[P2], sq = cs_s[Q2];
+          if (sp == 0.f && sq == 0.f) continue;
+          const float cp = cs_c[P2], cq = cs_c[Q2];
+          const int p0 = pr_p[P2], p1 = pr_q[P2], q0 = pr_p[Q2], q1 = pr_q[Q2];
+          const bool h1 = p1 < n, g1 = q1 < n;
+          const float a00 = A[p0 * ns + q0];
+          const float a01 = g1 ? A[p0 * ns + q1] : 0.f;
+          const float a10 = h1 ? A[p1 * ns + q0] : 0.f;
+          const float a11 = (h1 && g1) ? A[p1 * ns + q1] : 0.f;
+          const float b00 = cp * a00 - sp * a10, b01 = cp * a01 - sp * a11;  // rows: J_P^T
+          const float b10 = sp * a00 + cp * a10, b11 = sp * a01 + cp * a11;
+          const float c00 = cq * b00 - sq * b01, c01 = sq * b00 + cq * b01;  // columns: J_Q
+          const float c10 = cq * b10 - sq * b11, c11 = sq * b10 + cq * b11;
+          A[p0 * ns + q0] = c00;
+          if (g1) A[p0 * ns + q1] = c01;
+          if (h1) A[p1 * ns + q0] = c10;
+          if (h1 && g1) A[p1 * ns + q1] = c11;
+          if (P2 != Q2) {
+            A[q0 * ns + p0] = c00;
+            if (g1) A[q1 * ns + p0] = c01;
+            if (h1) A[q0 * ns + p1] = c10;
+            if (h1 && g1) A[q1 * ns + p1] = c11;
+          }
+        }
+      }
+      // V_{:,Q} <- V_{:,Q} J_Q, (pair, row) items dealt to all threads
+      {
+        const int nitem = half * n;
+        const float inv_n = 1.f / (float)n;
+        for (int e = tid; e < nitem; e += nt) {
+          const int Q2 = __float2int_rz(((float)e + 0.5f) * inv_n);
+          const float sq = cs_s[Q2];
+          if (sq == 0.f) continue;
+          const float cq = cs_c[Q2];
+          const int q0 = pr_p[Q2], q1 = pr_q[Q2], i = e - Q2 * n;
+          const float v0 = Vt[q0 * ns + i], v1 = Vt[q1 * ns + i];
+          Vt[q0 * ns + i] = cq * v0 - sq * v1;
+          Vt[q1 * ns + i] = sq * v0 + cq * v1;
+        }
+      }
+      __syncthreads();
+    }
+  }
+  for (int j = tid; j < n; j += nt) {  // (a left-out direction ranks last)
+    const float ej = dkv[j] == RR_DROPPED ? (float)RR_DROP_DIAG : A[j * ns + j];
+    int rank = 0;
+    for (int k2 = 0; k2 < n; ++k2) {
+      const float ek = dkv[k2] == RR_DROPPED ? (float)RR_DROP_DIAG : A[k2 * ns + k2];
+      rank += (ek < ej) || (ek == ej && k2 < j);
+    }
+    rr_out_eps(P, rank, (double)ej);
+    P.bv[BV_TMP0 * P.nb + j] = (double)rank;  // (blk = 2: rows BV_TMP0 and BV_TMP1)
+  }
+  __syncthreads();
+  for (int j = ty; j < n; j += nty) {
+    const int rj = (int)P.bv[BV_TMP0 * P.nb + j];
+    if (rj >= P.nb) continue;
+    for (int i = tx; i < n; i += 32) rr_out_vec(P, i, rj, (double)Vt[j * ns + i]);
+  }
+  if (tid == 0) {
+    P.scal[SC_RRSWEEPS] += sweeps;
+    P.scal[SC_RRCAP] += capped;
+    if (flag) P.status[0] = 1;
+  }
+}
+
+// ---------------------------------------------------------------------------
 // Rayleigh-Ritz for subspaces too large for one CTA's shared memory (the 330-band cluster):
 // one thread-block cluster of RR_CLUSTER CTAs per problem, its matrices in the problem's
 // global scratch (L2-resident), row i dealt to the CTA of rank i % RR_CLUSTER, hardware
-// cluster barriers between the steps.  The factorisation is that of k_rr_td.cu (deviation form):
+// cluster barriers between the steps.  Same mathematics as k_rr_f32 (deviation form):
 //  1. D = S - I and Hf, symmetrised.
 //  2. Cholesky S = (I + L)(I + L)^T in deviation form: column k's pivot d_k and scaled
 //     entries are formed by every CTA from the column (final after step k - 1), and each
@@ -1312,6 +1933,14 @@ void launch_copy_out(const Launch& L, int role, double* dst, int nvec) {
   if (!L.map.total) return;
   k_copy_out<T><<<L.map.total, 256, 0, L.stream>>>(L.ka, role, dst, nvec);
 }
+void launch_rr_f32(const Launch& L, size_t smem, float* gscratch, size_t gstride, int max_sweeps, int blk) {
+  k_rr_f32<<<L.ka.nprob, RR_THREADS, gscratch ? 0 : smem, L.stream>>>(L.ka, gscratch, gstride, max_sweeps, blk);
+}
+void launch_rr(const Launch& L, int use_smem, size_t smem, double* gscratch, size_t gstride, int max_sweeps,
+               int blk) {
+  k_rr<<<L.ka.nprob, RR_THREADS, use_smem ? smem : 0, L.stream>>>(L.ka, use_smem, gscratch, gstride, max_sweeps,
+                                                                     blk);
+}
 // S2 and H2 of the block [X, W] from n_b x n_b products (block Davidson): part 0 takes
 // S = X^T X, Hs = X^T HX, Tm = X^T W, Cm = X^T HW (the X rows and, by symmetry, the X
 // columns); part 1 takes S = W^T W, Hs = W^T HW (the W W block).  CTA = (problem, 256
@@ -1345,7 +1974,10 @@ void launch_occupations(const Launch& L) {
   k_occupations<T><<<L.ka.nprob, 32, 0, L.stream>>>(L.ka);
 }
 void linalg_set_smem_limits(size_t bytes) {
-  (void)bytes;
+  cudaFuncSetAttribute(k_rr, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+  // (k_rr_f32 keeps its matrices in shared memory up to 216 KB; its static arrays take the
+  // rest of the 227 KB)
+  cudaFuncSetAttribute(k_rr_f32, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)std::min(bytes, (size_t)216 * 1024));
   // the NN kernel also has 8 KB of static shared memory: request only what it uses
   cudaFuncSetAttribute(k_gemm_nn<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, NN_KP * 64 * (int)sizeof(float));
 }

@@ -1,31 +1,25 @@
-// Rayleigh-Ritz of one CTA or one cluster of CTAs per problem (orthonormalisation + subspace diagonalisation of
-// Algorithm 1): S = L L^T, C = L^-1 Hs L^-T, C = V diag(eps) V^T, Tm = L^-T V, so that X Tm is
-// orthonormal and diagonalises H in the subspace.  T = float on the mixed path, double on the
-// plain one.
+// FP64 Rayleigh-Ritz, one CTA or one cluster of CTAs per problem (orthonormalisation + subspace
+// diagonalisation of Algorithm 1): S = L L^T, C = L^-1 Hs L^-T, C = V diag(eps) V^T, Tm = L^-T V, so
+// that X Tm is orthonormal and diagonalises H in the subspace.
 //
-//  1. Cholesky in deviation form: S = I + E, L = I + D, d_k = x / (1 + sqrt(1 + x)) with
-//     x = E_kk, D_ik = E_ik / (1 + d_k).  Every stored quantity has the size of E, so FP32 keeps
-//     its relative accuracy (the entries of S carry the product's FP32 rounding anyway).
+//  1. Cholesky in deviation form: S = I + E, d_k = E_kk, L_ik = E_ik / sqrt(1 + d_k).
 //  2. W = L^-1 Hs and C = W L^-T by forward substitution down columns.
 //  3. Householder tridiagonalisation of C (Golub & Van Loan, section 8.3.1).
-//  4. Divide and conquer on the tridiagonal matrix (Cuppen, Numer. Math. 36, 177 (1981)): small
-//     leaves by QL steps, merged pairwise, a merge being the rank-one problem diag(delta) + rho z z^T.  Roots of its secular equation by the
-//     two-pole rational interpolation of Bunch, Nielsen & Sorensen (Numer. Math. 31, 31 (1978)),
-//     each as an offset from its nearest pole; z is then recomputed from the roots (Gu &
-//     Eisenstat, SIAM J. Matrix Anal. 15, 1266 (1994)), which makes the vectors orthogonal to
-//     rounding however close the roots lie.  Nothing is deflated: poles closer than one unit of
-//     rounding of the matrix are moved that far apart and weights below rounding are raised to
-//     it, both of the size of the rounding errors already there; a negligible rho leaves the two
-//     halves as they are.
-//  5. V = Householder reflectors applied to the eigenvectors; FP32: one correction of V by its
-//     residuals C v_j - lam_j v_j (first-order perturbation theory), one Newton-Schulz step of its
-//     orthonormality; Tm = L^-T V by back substitution.
+//  4. Divide and conquer on the tridiagonal matrix (Cuppen, Numer. Math. 36, 177 (1981)): leaves of
+//     two rows, merged pairwise, a merge being the rank-one problem diag(delta) + rho z z^T.  Roots of
+//     its secular equation by the two-pole rational interpolation of Bunch, Nielsen & Sorensen (Numer.
+//     Math. 31, 31 (1978)), each as an offset from its nearest pole; z is then recomputed from the
+//     roots (Gu & Eisenstat, SIAM J. Matrix Anal. 15, 1266 (1994)), which makes the vectors orthogonal
+//     to rounding however close the roots lie.  Nothing is deflated: poles closer than one unit of
+//     rounding of the matrix are moved that far apart and weights below rounding are raised to it,
+//     both of the size of the rounding errors already there; a negligible rho leaves the two halves as
+//     they are.
+//  5. V = Householder reflectors applied to the eigenvectors; Tm = L^-T V by back substitution.
 //
 // What bounds it, and why this form: one CTA (one SM) works on a chain of dependent steps, so the
-// time is barriers, latencies and, with many warps, the issue of the steps' overhead; on the FP64
-// path it is the two FP64 lanes of the SM (a warp's DFMA holds them 16 cycles).  The cyclic Jacobi
-// eigensolve before it took about 200 rounds of two block barriers and 6 n^2 operations each.
-// Here the matrices stay in the registers of MW matrix warps, row i in warp i / RPW, column j in
+// time is barriers, latencies and the two FP64 lanes of the SM (a warp's DFMA holds them 16 cycles).
+// A cyclic Jacobi eigensolve (k_rr) takes about 200 rounds of two block barriers and 6 n^2 operations
+// each.  Here the matrices stay in the registers of MW matrix warps, row i in warp i / RPW, column j in
 // lane j mod 32 (few warps with 8 to 16 rows each: the overhead of a step is paid per warp); the
 // Cholesky needs one barrier per RPW columns, the tridiagonalisation two per column, the
 // substitutions and the back transformation none (a warp owns whole columns).
@@ -34,10 +28,8 @@
 // columns and vectors of its own rows.  The leaves and the sorting are done by every CTA alike.
 // Results do not depend on the number of CTAs or warps (the sums over lanes have one shape, fused
 // multiply-adds are written out).
-// Measured, mean per launch over an evaluation, Jacobi kernels -> one CTA -> now: FP32 70 bands 299 ->
-// 256 us (one CTA), 91 bands 553 -> 335 us (one CTA), 169 bands (an 8-CTA cluster before) 3565 -> 1403
-// -> 990 us, 10 bands 31 -> 38 us (one CTA); FP64 24 bands 317 -> 288 -> 205 us, 70 bands 2500 ->
-// 1883 -> 762 us, up to 80 bands in six members 3550 -> 2118 -> 818 us.
+// Measured, mean per launch over an evaluation, Jacobi kernel -> here: 24 bands 317 -> 205 us, 70 bands
+// 2500 -> 762 us, up to 80 bands in six members 3550 -> 818 us.
 #include "kernels.h"
 
 namespace sgo {
@@ -51,17 +43,17 @@ namespace {
 // C is set above the spectrum, so that it ranks after every kept Ritz value.
 constexpr double TD_DROP = 1e-3;
 // Lanes per root of a merge of m poles out of n.  A root's own arithmetic is done by all its lanes,
-// so more lanes only pay while they shorten a chain of terms that is long against it, and on the
-// FP64 path only until about four warps keep the FP64 lanes busy.  (Not a function of the block
+// so more lanes only pay while they shorten a chain of terms that is long against it, and only until
+// about four warps keep the FP64 lanes busy.  (Not a function of the block
 // size: the sums must not depend on the batch a member is in.)
-template <typename T>
 __device__ __forceinline__ int td_lanes(int m, int n) {
-  if (sizeof(T) == 8 && n > 32) return m > 32 ? 4 : m > 8 ? 2 : 1;
-  return m > 16 && n <= 64 && sizeof(T) == 4 ? 8 : m > 8 ? 4 : m > 4 ? 2 : 1;  // (64: one pass of 512 threads)
+  if (n > 32) return m > 32 ? 4 : m > 8 ? 2 : 1;
+  return m > 8 ? 4 : m > 4 ? 2 : 1;
 }
 
-template <typename T>
-struct TdNum;
+using T = double;
+template <typename F>
+struct TdNum;  // (float: the starting phase of the roots)
 template <>
 struct TdNum<float> {
   static constexpr float eps = 1.1920929e-7f, ztiny = 1e-7f, floor = 1e-30f, step = 3e-5f;
@@ -86,10 +78,6 @@ __device__ __forceinline__ double td_rcp(double x) {
   r = fma(r, fma(-x, r, 1.0), r);
   return fma(r, fma(-x, r, 1.0), r);
 }
-__device__ __forceinline__ float td_rsqrt(float x) {
-  const float r = rsqrtf(x);
-  return fmaf(0.5f * r, fmaf(-x * r, r, 1.f), r);
-}
 __device__ __forceinline__ double td_rsqrt(double x) {  // two Newton steps on the approximate one
   double r;
   asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(x));
@@ -97,7 +85,6 @@ __device__ __forceinline__ double td_rsqrt(double x) {  // two Newton steps on t
   return fma(0.5 * r, fma(-x * r, r, 1.0), r);
 }
 
-template <typename T>
 __device__ __forceinline__ T wsum(T v) {
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) v = v + __shfl_xor_sync(0xffffffffu, v, o);
@@ -105,8 +92,8 @@ __device__ __forceinline__ T wsum(T v) {
 }
 
 // sum over the g lanes of a root
-template <typename T>
-__device__ __forceinline__ T gsum(T v, int g) {
+template <typename F>
+__device__ __forceinline__ F gsum(F v, int g) {
   for (int o = g >> 1; o > 0; o >>= 1) v = v + __shfl_xor_sync(0xffffffffu, v, o);
   return v;
 }
@@ -114,19 +101,19 @@ __device__ __forceinline__ T gsum(T v, int g) {
 // Root in the pole interval of the two-pole model c + s / (p - mu) + S / (q - mu) = 0; right:
 // offsets from the right pole (p = -w, q = 0), else from the left one (p = 0, q = w).  S = 0: no
 // right pole (the last root; the quadratic would lose the root to its other one at w).
-template <typename T>
-__device__ __forceinline__ T two_pole_root(T c, T s, T S, T w, bool right) {
-  if (S == T(0)) return s * td_rcp(c);
-  const T b = right ? fma(-c, w, s + S) : fma(c, w, s) + S;
-  const T d = right ? -S * w : s * w;
-  const T disc = fma(b, b, -(T(4) * c * d));
-  const T r = sqrt(disc > T(0) ? disc : T(0));
-  const T num = b >= T(0) ? T(2) * d : b - r, den = b >= T(0) ? b + r : T(2) * c;
+template <typename F>
+__device__ __forceinline__ F two_pole_root(F c, F s, F S, F w, bool right) {
+  if (S == F(0)) return s * td_rcp(c);
+  const F b = right ? fma(-c, w, s + S) : fma(c, w, s) + S;
+  const F d = right ? -S * w : s * w;
+  const F disc = fma(b, b, -(F(4) * c * d));
+  const F r = sqrt(disc > F(0) ? disc : F(0));
+  const F num = b >= F(0) ? F(2) * d : b - r, den = b >= F(0) ? b + r : F(2) * c;
   return num * td_rcp(den);
 }
 
 // poles relative to the nearest one, in F
-template <typename F, typename T>
+template <typename F>
 struct Poles {
   const T* d;
   T b;
@@ -184,16 +171,14 @@ __device__ __forceinline__ bool secular(const PO& pole, const F* zw, int lo, int
   return done;
 }
 
-// Largest block the divide and conquer starts from.  FP32: QL steps on 8 rows take 10 us where
-// three merge levels of the smallest blocks take 20; FP64: on 2 rows (one rotation), since the
-// steps are chains of FP64 operations (8 rows 100 us, the levels 40).
-template <typename T>
-__host__ __device__ constexpr int td_leaf_rows() { return sizeof(T) == 4 ? 8 : 2; }
+// Largest block the divide and conquer starts from: 2 rows (one rotation), since longer QL iterations
+// are chains of FP64 operations (8 rows 100 us, three merge levels instead 40).
+constexpr int TD_LEAF = 2;
 
 // Eigenvectors of a symmetric tridiagonal leaf of m0 <= M rows by implicit QL steps with
 // Wilkinson's shift (EISPACK's tql2: Bowdler, Martin, Reinsch & Wilkinson, Numer. Math. 11, 293
 // (1968)): every lane carries the whole of d and e and one row z of the vectors.
-template <typename T, int M>
+template <int M>
 __device__ __forceinline__ void td_leaf(T (&d)[M], T (&e)[M], T (&z)[M], int m0, T norm) {
   const T tiny = T(1e-3) * TdNum<T>::eps * norm;
   for (int l = 0; l + 1 < m0; ++l) {
@@ -273,9 +258,6 @@ struct Team {
       }
     }
   }
-  static __device__ __forceinline__ void st(unsigned a, float v) {
-    asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(a), "f"(v) : "memory");
-  }
   static __device__ __forceinline__ void st(unsigned a, double v) {
     asm volatile("st.shared::cluster.f64 [%0], %1;" ::"r"(a), "d"(v) : "memory");
   }
@@ -306,23 +288,14 @@ struct Team {
   }
 };
 
-// R consecutive shared values (aligned to R values or 16 bytes) as vector loads
-template <typename T, int R>
+// R consecutive shared values (aligned to 16 bytes) as vector loads
+template <int R>
 __device__ __forceinline__ void ldv(const T* p, T (&o)[R]) {
-  constexpr int W = sizeof(T) == 4 && R % 4 == 0 ? 4 : 2;
-  static_assert(R % W == 0, "whole vectors");
+  static_assert(R % 2 == 0, "whole vectors");
 #pragma unroll
-  for (int i = 0; i < R / W; ++i) {
-    if constexpr (W == 4) {
-      const float4 v = reinterpret_cast<const float4*>(p)[i];
-      o[4 * i] = v.x; o[4 * i + 1] = v.y; o[4 * i + 2] = v.z; o[4 * i + 3] = v.w;
-    } else if constexpr (sizeof(T) == 4) {
-      const float2 v = reinterpret_cast<const float2*>(p)[i];
-      o[2 * i] = v.x; o[2 * i + 1] = v.y;
-    } else {
-      const double2 v = reinterpret_cast<const double2*>(p)[i];
-      o[2 * i] = v.x; o[2 * i + 1] = v.y;
-    }
+  for (int i = 0; i < R / 2; ++i) {
+    const double2 v = reinterpret_cast<const double2*>(p)[i];
+    o[2 * i] = v.x; o[2 * i + 1] = v.y;
   }
 }
 
@@ -330,16 +303,15 @@ __host__ __device__ inline int td_zs(int n) { return n > 16 ? ((n + 1) / 2) | 1 
 __host__ __device__ inline int td_us(int n) { return (n + 3) & ~3; }        // row stride of the merge matrix
 constexpr int TD_PAD = 32;  // vectors are read in whole groups of rows past n
 __host__ __device__ inline int td_vn(int n) { return ((n + 3) & ~3) + TD_PAD; }
-__host__ __device__ inline size_t td_vec_bytes(int n, size_t ts) {
-  return ((size_t)(13 * td_vn(n) + 32) * ts + (size_t)(3 * td_vn(n) + 16) * 4 + 15) / 16 * 16;
+__host__ __device__ inline size_t td_vec_bytes(int n) {
+  return ((size_t)(13 * td_vn(n) + 32) * sizeof(T) + (size_t)(3 * td_vn(n) + 16) * 4 + 15) / 16 * 16;
 }
 
 }  // namespace
 
 // all: L, the reflectors, U and Z in shared memory; else L, the reflectors and the transposes go
-// through the member's global scratch (3 n^2 elements) and share U's place in turn.  FP32 keeps C
-// and the factors of the correction's products in the scratch too (rr_td_scratch_bytes).
-template <typename T, int NR, int MW, int NW, int CL>
+// through the member's global scratch (3 n^2 elements) and share U's place in turn.
+template <int NR, int MW, int NW, int CL>
 __global__ void __launch_bounds__(32 * NW, 1)
     k_rr_td(KArgs ka, T* gscratch, size_t gstride, int all, int blk) {
   static_assert(CL == 1 || MW == NW, "in a cluster every warp is a matrix warp");
@@ -375,17 +347,15 @@ __global__ void __launch_bounds__(32 * NW, 1)
   int* perm = reinterpret_cast<int*>(red + 32);
   int* kx = perm + vn;
   int* bk = kx + vn;                       // block of each index: lo | mid << 10 | hi << 20
-  float* fz = reinterpret_cast<float*>(wv);  // (FP64) the weights as floats
+  float* fz = reinterpret_cast<float*>(wv);  // the weights as floats
   int* flags = bk + vn;                      // [0] Cholesky failed, [1] left-out directions, [2] close poles, [3] capped
-  T* Ub = reinterpret_cast<T*>(smem_raw + td_vec_bytes(n, sizeof(T)));  // [n][us]; L or the reflectors [n][ns]
+  T* Ub = reinterpret_cast<T*>(smem_raw + td_vec_bytes(n));  // [n][us]; L or the reflectors [n][ns]
   T* Zb = Ub + (size_t)n * (ns > us ? ns : us);                        // [n][zs]
   T* Lb = all ? Zb + ((size_t)n * zs + 3) / 4 * 4 : Ub;                // L: row k holds column k
   T* Vb = all ? Lb + (size_t)n * ns : Ub;                              // reflectors, row k
   T* gW = gscratch ? gscratch + (size_t)p * gstride : nullptr;         // transposes
   T* gL = gW + (size_t)n * n;
   T* gV = gL + (size_t)n * n;
-  T* gC = all ? gW : gV + (size_t)n * n;                               // (FP32) C
-  T* gS = gW + ((all ? 1 : 4) * (size_t)n * n + 3) / 4 * 4;            // (FP32) [MW][n][RPW], 16-byte aligned
   if (tid < 16) flags[tid] = 0;
   team.barrier();
 
@@ -556,12 +526,6 @@ __global__ void __launch_bounds__(32 * NW, 1)
         for (int c = 0; c < NR; ++c)
           if (i0 + a < n && i0 + a == lane + 32 * c && dk[i0 + a] == T(0)) A[a][c] = T(2) * rs + T(1);
     }
-    if constexpr (sizeof(T) == 4)
-#pragma unroll
-      for (int a = 0; a < RPW; ++a)
-#pragma unroll
-        for (int c = 0; c < NR; ++c)
-          if (i0 + a < n && lane + 32 * c < n) gC[(size_t)(i0 + a) * n + lane + 32 * c] = A[a][c];
     // ---- 3. tridiagonalisation: reflector k from row k (warp k / RPW), v_{k+1} = 1 ----
     for (int k = 0; k + 2 < n; ++k) {
       T* v = vbuf + (k & 1) * vn;
@@ -674,7 +638,6 @@ __global__ void __launch_bounds__(32 * NW, 1)
   team.barrier();
   // ---- 4. divide and conquer (in a cluster, the leaves, sorting and poles in every CTA alike; a CTA
   // takes the roots, weights and vectors of its own rows) ----
-  constexpr int TD_LEAF = td_leaf_rows<T>();
   // blocks: at shift sh, block q holds the indices (q n) >> sh .. ((q + 1) n) >> sh.  The leaves are
   // the blocks of at most TD_LEAF rows, torn apart at their ends (d -= |e| on either side of a
   // tear).
@@ -730,7 +693,7 @@ __global__ void __launch_bounds__(32 * NW, 1)
         A[a][c] = lev == 0 && i0 + a < n && lane + 32 * c < n ? Zb[(size_t)(i0 + a) * zs + lane + 32 * c] : T(0);
   for (int l = 0; l < lev; ++l) {
     const int sh = lev - l - 1;
-    const int g = td_lanes<T>((n + (1 << sh) - 1) >> sh, n);  // lanes per root
+    const int g = td_lanes((n + (1 << sh) - 1) >> sh, n);  // lanes per root
     const int sub = tid & (g - 1), GR = NT / g, root0 = tid / g;
     const int slots = (c1 - c0 + GR - 1) / GR;
     team.barrier();
@@ -792,10 +755,8 @@ __global__ void __launch_bounds__(32 * NW, 1)
       }
       __syncthreads();
     }
-    if constexpr (sizeof(T) == 8) {
-      for (int i = tid; i < n; i += NT) fz[i] = (float)zw[i];
-      __syncthreads();
-    }
+    for (int i = tid; i < n; i += NT) fz[i] = (float)zw[i];
+    __syncthreads();
     // roots
     for (int sl = 0; sl < slots; ++sl) {
       const int i = c0 + sl * GR + root0;
@@ -812,12 +773,10 @@ __global__ void __launch_bounds__(32 * NW, 1)
       tot = gsum(tot, g);
       const T w = last ? tot : ds[nx] - ds[ii];
       // the sign at the middle tells the nearer pole; the root of the two-pole model there starts
-      // the iteration.  FP64: both in floats, then two or three FP64 steps.
+      // the iteration.  Both in floats, then two or three FP64 steps.
       const F wf = (F)w, hf = 0.5f * wf;
-      const F* zf = nullptr;
-      if constexpr (sizeof(T) == 8) zf = fz;
-      else zf = zw;
-      auto fpole = [&](int K) { return Poles<F, T>{ds, ds[K]}; };
+      const F* zf = fz;
+      auto fpole = [&](int K) { return Poles<F>{ds, ds[K]}; };
       F fm = 0.f;
       if (solve) {
         const auto po = fpole(ii);
@@ -829,14 +788,11 @@ __global__ void __launch_bounds__(32 * NW, 1)
       F xf = two_pole_root(fma(2.f * (zf[ii] - (last ? 0.f : zf[nx])), td_rcp(wf), fm), zf[ii], last ? 0.f : zf[nx], wf, right);
       const F af = right ? -wf : 0.f, bf = right ? 0.f : wf;
       if (!(xf > af && xf < bf)) xf = right ? -0.5f * hf : 0.5f * hf;
-      bool done = secular(fpole(K), zf, lo, hi, ii, sub, g, wf, right, last, af, bf, !solve,
-                          sizeof(T) == 8 ? 12 : TD_ITERS, &xf);
+      secular(fpole(K), zf, lo, hi, ii, sub, g, wf, right, last, af, bf, !solve, 12, &xf);
       T x = (T)xf;
-      if constexpr (sizeof(T) == 8) {
-        const T a = right ? -w : T(0), b = right ? T(0) : w;
-        if (!(x > a && x < b)) x = right ? -0.25 * w : 0.25 * w;
-        done = secular(Poles<T, T>{ds, ds[K]}, zw, lo, hi, ii, sub, g, w, right, last, a, b, !solve, TD_ITERS, &x);
-      }
+      const T a = right ? -w : T(0), b = right ? T(0) : w;
+      if (!(x > a && x < b)) x = right ? -0.25 * w : 0.25 * w;
+      const bool done = secular(Poles<T>{ds, ds[K]}, zw, lo, hi, ii, sub, g, w, right, last, a, b, !solve, TD_ITERS, &x);
       if (live && sub == 0) {
         team.put(&kx[i], solve ? K : -1);  // -1: the halves stay as they are
         team.put(&mu[i], solve ? x : T(0));
@@ -969,126 +925,6 @@ __global__ void __launch_bounds__(32 * NW, 1)
 #pragma unroll
           for (int a = 0; a < RPW; ++a) A[a][c] = fma(-q[a], v[c], A[a][c]);
     }
-  if constexpr (sizeof(T) == 4) {
-    // Correction in FP32.  The steps so far leave |V^T C V - diag| and |V^T V - I| near 2e-6, a few
-    // times what the rotations of a Jacobi left; in the SCF that is noise in rho and F.  With
-    // r_j = C v_j - lam_j v_j: V += V E, E_ij = v_i.r_j / (lam_j - lam_i) for pairs far enough apart,
-    // lam_j += v_j.r_j; then V += V (I - V^T V) / 2.  Five small products bring both to 5e-7, below
-    // the Jacobi's (fewer SCF iterations at tight density rules), for a tenth of the time.
-    // V^T in Ub; V by rows in Vb where there is room (after C, which takes that room first), else
-    // by columns of V^T
-    const T* Xv = all ? Vb : Ub;
-    const int xk = all ? ns : 1, xr = all ? 1 : us;
-    const T* Xc = all ? Vb : gC;
-    const int cs = all ? ns : n;
-    T* const mine = gS + (size_t)warp * n * RPW;  // the warp's own factor, [k][RPW]
-    auto vt = [&](int a, int c) -> T {            // component lane + 32 c of vector i0 + a
-      return i0 + a < n && lane + 32 * c < n ? Ub[(lane + 32 * c) * us + i0 + a] : T(0);
-    };
-    auto stage = [&]() {
-      __syncwarp();
-#pragma unroll
-      for (int a = 0; a < RPW; ++a)
-#pragma unroll
-        for (int c = 0; c < NR; ++c)
-          if (lane + 32 * c < n) mine[(lane + 32 * c) * RPW + a] = A[a][c];
-      __syncwarp();
-    };
-    // A[a][c] = sum_k f[k][a] X(k, lane + 32 c), f = the staged factor or the columns of V^T
-    auto product = [&](const T* f, int fs, const T* X, int sk, int sr) {
-#pragma unroll
-      for (int a = 0; a < RPW; ++a)
-#pragma unroll
-        for (int c = 0; c < NR; ++c) A[a][c] = T(0);
-#pragma unroll 4
-      for (int k = 0; k < n; ++k) {
-        T u[RPW];
-        ldv(f + k * fs, u);
-#pragma unroll
-        for (int c = 0; c < NR; ++c) {
-          const int r = lane + 32 * c;
-          const T x = X[k * sk + r * sr];  // (lanes r >= n read on into what follows; their sums are not used)
-#pragma unroll
-          for (int a = 0; a < RPW; ++a) A[a][c] = fma(u[a], x, A[a][c]);
-        }
-      }
-    };
-    auto put_vt = [&]() {
-#pragma unroll
-      for (int a = 0; a < RPW; ++a)
-#pragma unroll
-        for (int c = 0; c < NR; ++c)
-          if (i0 + a < n && lane + 32 * c < n) team.put(&Ub[(lane + 32 * c) * us + i0 + a], A[a][c]);
-    };
-    team.matrix_barrier(MT);  // (the reflectors are done with)
-    put_vt();
-    if (all)
-      for (int e = tid; e < n * n; e += MT) Vb[(size_t)(e / n) * ns + e % n] = gC[e];
-    team.matrix_barrier(MT);
-    if (i0 < n) {
-      product(Ub + i0, us, Xc, cs, 1);  // C v_j
-#pragma unroll
-      for (int a = 0; a < RPW; ++a)
-#pragma unroll
-        for (int c = 0; c < NR; ++c) A[a][c] = fma(-dg[min(i0 + a, n - 1)], vt(a, c), A[a][c]);
-      stage();
-    }
-    if (all) {
-      team.matrix_barrier(MT);
-#pragma unroll
-      for (int a = 0; a < RPW; ++a)
-#pragma unroll
-        for (int c = 0; c < NR; ++c)
-          if (i0 + a < n && lane + 32 * c < n) team.put(&Vb[(i0 + a) * ns + lane + 32 * c], vt(a, c));
-    }
-    if (i0 < n) {
-      product(mine, RPW, Ub, us, 1);  // v_i.r_j
-#pragma unroll
-      for (int a = 0; a < RPW; ++a)
-#pragma unroll
-        for (int c = 0; c < NR; ++c) {
-          const int i = lane + 32 * c, j = i0 + a;
-          const T y = A[a][c], lj = dg[min(j, n - 1)], dl = lj - dg[min(i, n - 1)];
-          if (i == j && i < n) team.put(&nd[i], lj + y);
-          // (closer pairs stay as they are: their quotients are rounding)
-          A[a][c] = i < n && fabs(dl) > T(5e-4) * norm && fabs(y) <= T(2e-3) * fabs(dl) ? y * td_rcp(dl) : T(0);
-        }
-      stage();
-    }
-    if (all) team.matrix_barrier(MT);
-    if (i0 < n) {
-      product(mine, RPW, Xv, xk, xr);
-#pragma unroll
-      for (int a = 0; a < RPW; ++a)
-#pragma unroll
-        for (int c = 0; c < NR; ++c) A[a][c] += vt(a, c);
-    }
-    team.matrix_barrier(MT);
-    put_vt();
-    if (all)
-#pragma unroll
-      for (int a = 0; a < RPW; ++a)
-#pragma unroll
-        for (int c = 0; c < NR; ++c)
-          if (i0 + a < n && lane + 32 * c < n) team.put(&Vb[(i0 + a) * ns + lane + 32 * c], A[a][c]);
-    team.matrix_barrier(MT);
-    if (i0 < n) {
-      product(Ub + i0, us, Ub, us, 1);  // v_i.v_j
-#pragma unroll
-      for (int a = 0; a < RPW; ++a)
-#pragma unroll
-        for (int c = 0; c < NR; ++c)
-          A[a][c] = T(0.5) * ((lane + 32 * c == i0 + a ? T(1) : T(0)) - A[a][c]);
-      stage();
-      product(mine, RPW, Xv, xk, xr);
-#pragma unroll
-      for (int a = 0; a < RPW; ++a)
-#pragma unroll
-        for (int c = 0; c < NR; ++c) A[a][c] += vt(a, c);
-    }
-    for (int i = tid; i < n; i += MT) dg[i] = nd[i];
-    team.matrix_barrier(MT);
-  }
   if (!all) {
     team.matrix_barrier(MT);
     for (int e = tid; e < n * n; e += MT) Ub[(size_t)(e / n) * ns + e % n] = gL[e];
@@ -1119,34 +955,19 @@ __global__ void __launch_bounds__(32 * NW, 1)
             for (int a = 0; a < RPW; ++a) A[a][c] = fma(-lr[c], x[a], A[a][c]);
       }
     }
-    // ascending: the corrected eigenvalues of close pairs may have changed places
-    int rank[RPW];
-#pragma unroll
-    for (int a = 0; a < RPW; ++a) {
-      rank[a] = i0 + a;
-      if constexpr (sizeof(T) == 4) {
-        const T d = dg[min(i0 + a, n - 1)];
-        rank[a] = 0;
-#pragma unroll
-        for (int c = 0; c < NR; ++c) {
-          const int k = lane + 32 * c;
-          rank[a] += __popc(__ballot_sync(0xffffffffu, k < n && (dg[min(k, n - 1)] < d || (dg[min(k, n - 1)] == d && k < i0 + a))));
-        }
-      }
-    }
     // the lowest n_b Ritz pairs: rows r < n_b are the coefficients on X, the others those on W
 #pragma unroll
     for (int a = 0; a < RPW; ++a) {
-      const int i = rank[a];
-      if (i0 + a >= n || i >= P.nb) continue;
+      const int i = i0 + a;
+      if (i >= n || i >= P.nb) continue;
 #pragma unroll
       for (int c = 0; c < NR; ++c) {
         const int r = lane + 32 * c;
         if (r >= n) continue;
-        if (r < P.nb) P.Tm[(size_t)r * P.nb + i] = (double)A[a][c];
-        else P.Cm[(size_t)(r - P.nb) * P.nb + i] = (double)A[a][c];
+        if (r < P.nb) P.Tm[(size_t)r * P.nb + i] = A[a][c];
+        else P.Cm[(size_t)(r - P.nb) * P.nb + i] = A[a][c];
       }
-      if (lane == 0) P.eps[i] = (double)dg[i0 + a];
+      if (lane == 0) P.eps[i] = dg[i];
     }
   }
   if (warp == 0 && lane == 0) {
@@ -1156,28 +977,24 @@ __global__ void __launch_bounds__(32 * NW, 1)
 }
 
 namespace {
-size_t td_smem(int n, size_t ts, bool all) {
+size_t td_smem(int n, bool all) {
   const size_t ns = n | 1, us = td_us(n), u = (size_t)n * (ns > us ? ns : us), z = ((size_t)n * td_zs(n) + 3) / 4 * 4;
-  return td_vec_bytes(n, ts) + (u + z + (all ? 2 * (size_t)n * ns + 32 : 0)) * ts;  // (32: rows are read on past n)
+  return td_vec_bytes(n) + (u + z + (all ? 2 * (size_t)n * ns + 32 : 0)) * sizeof(T);  // (32: rows are read on past n)
 }
 constexpr size_t TD_SMEM_MAX = 227 * 1024;
 }  // namespace
 
-// Subspaces the kernel takes: FP32 up to 184 (the merge matrix and the vectors fill the shared
-// memory), FP64 up to 128 (an 8 x 4 tile of the matrix per thread).
-int rr_td_max(size_t tsize) { return tsize == 4 ? 184 : 128; }
+// Subspaces the kernel takes: an 8 x 4 tile of the matrix per thread.
+int rr_td_max() { return 128; }
 
 // bytes of global scratch per problem (0: everything fits in shared memory)
-size_t rr_td_scratch_bytes(int n, size_t tsize) {
-  const size_t nn = (size_t)n * n, big = td_smem(n, tsize, true) <= TD_SMEM_MAX ? 0 : 3 * nn;
-  return (big + (tsize == 4 ? nn + 8 + (size_t)n * (n + 16) : 0)) * tsize;
-}
+size_t rr_td_scratch_bytes(int n) { return td_smem(n, true) <= TD_SMEM_MAX ? 0 : 3 * (size_t)n * n * sizeof(T); }
 
-template <typename T, int NR, int MW, int NW, int CL>
+template <int NR, int MW, int NW, int CL>
 static void td_launch(const Launch& L, int n, unsigned char* scratch, size_t stride, int blk) {
-  const bool all = td_smem(n, sizeof(T), true) <= TD_SMEM_MAX;
-  const size_t smem = td_smem(n, sizeof(T), all);
-  auto* fn = k_rr_td<T, NR, MW, NW, CL>;
+  const bool all = td_smem(n, true) <= TD_SMEM_MAX;
+  const size_t smem = td_smem(n, all);
+  auto* fn = k_rr_td<NR, MW, NW, CL>;
   cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = L.ka.nprob * CL;
@@ -1195,42 +1012,30 @@ static void td_launch(const Launch& L, int n, unsigned char* scratch, size_t str
 }
 
 // n: the largest subspace of the launch (n_b, or 2 n_b for blk = 2).  CTAs per problem: more of them
-// shorten the column-owning steps and, on the FP64 path, share the FP64 lanes' work; each barrier
-// costs 0.4 us more.  So a cluster wherever it is faster, while the launch leaves half the SMs to the
-// sub-batches that run beside it.  Measured, one problem, 1 / 4 / 8 CTAs: FP64 24 bands 269 / 219 / 191 us, 52 bands 851 / 550 /
-// 472, 70 bands 1825 / 925 / 724, 119 bands 5074 / 1953 / 1438; FP32 52 bands 141 / 185 / 195, 70
-// bands 237 / 279 / 297, 119 bands 525 / 502 / 526, 169 bands 1345 / 934 / 918.
-template <typename T>
+// shorten the column-owning steps and share the FP64 lanes' work; each barrier costs 0.4 us more.  So
+// a cluster wherever the launch leaves half the SMs to the sub-batches that run beside it.  Measured,
+// one problem, 1 / 4 / 8 CTAs: 24 bands 269 / 219 / 191 us, 52 bands 851 / 550 / 472, 70 bands 1825 /
+// 925 / 724, 119 bands 5074 / 1953 / 1438.  (In one CTA: 8 to 16 rows in as few warps as the registers
+// allow, since every warp's own sums use the FP64 lanes too.)
 void launch_rr_td(const Launch& L, int n, unsigned char* scratch, size_t stride, int blk) {
   constexpr int SMS = 152 / 2;
   const int np = L.ka.nprob;
-  // (FP32: 4 to 12 rows per warp, bound by issue and latency; FP64 in one CTA: 8 to 16 rows in as few
-  // warps as the registers allow, bound by the FP64 lanes, which every warp's own sums use too)
-  if constexpr (sizeof(T) == 4) {
-    if (n <= 32) td_launch<T, 1, 8, 8, 1>(L, n, scratch, stride, blk);
-    else if (n <= 64) td_launch<T, 2, 16, 16, 1>(L, n, scratch, stride, blk);
-    else if (n <= 96) td_launch<T, 3, 16, 16, 1>(L, n, scratch, stride, blk);
-    else if (n <= 128) td_launch<T, 4, 16, 16, 1>(L, n, scratch, stride, blk);
-    else if (np * 4 <= SMS) td_launch<T, 6, 8, 8, 4>(L, n, scratch, stride, blk);
-    else td_launch<T, 6, 16, 16, 1>(L, n, scratch, stride, blk);
-  } else if (np * 8 <= SMS) {
-    if (n <= 32) td_launch<T, 1, 2, 2, 8>(L, n, scratch, stride, blk);
-    else if (n <= 64) td_launch<T, 2, 4, 4, 8>(L, n, scratch, stride, blk);
-    else if (n <= 96) td_launch<T, 3, 6, 6, 8>(L, n, scratch, stride, blk);
-    else td_launch<T, 4, 8, 8, 8>(L, n, scratch, stride, blk);
+  if (np * 8 <= SMS) {
+    if (n <= 32) td_launch<1, 2, 2, 8>(L, n, scratch, stride, blk);
+    else if (n <= 64) td_launch<2, 4, 4, 8>(L, n, scratch, stride, blk);
+    else if (n <= 96) td_launch<3, 6, 6, 8>(L, n, scratch, stride, blk);
+    else td_launch<4, 8, 8, 8>(L, n, scratch, stride, blk);
   } else if (np * 4 <= SMS) {
-    if (n <= 32) td_launch<T, 1, 2, 2, 4>(L, n, scratch, stride, blk);
-    else if (n <= 64) td_launch<T, 2, 4, 4, 4>(L, n, scratch, stride, blk);
-    else if (n <= 96) td_launch<T, 3, 6, 6, 4>(L, n, scratch, stride, blk);
-    else td_launch<T, 4, 8, 8, 4>(L, n, scratch, stride, blk);
+    if (n <= 32) td_launch<1, 2, 2, 4>(L, n, scratch, stride, blk);
+    else if (n <= 64) td_launch<2, 4, 4, 4>(L, n, scratch, stride, blk);
+    else if (n <= 96) td_launch<3, 6, 6, 4>(L, n, scratch, stride, blk);
+    else td_launch<4, 8, 8, 4>(L, n, scratch, stride, blk);
   } else {
-    if (n <= 32) td_launch<T, 1, 4, 8, 1>(L, n, scratch, stride, blk);
-    else if (n <= 64) td_launch<T, 2, 8, 8, 1>(L, n, scratch, stride, blk);
-    else if (n <= 96) td_launch<T, 3, 8, 8, 1>(L, n, scratch, stride, blk);
-    else td_launch<T, 4, 8, 8, 1>(L, n, scratch, stride, blk);
+    if (n <= 32) td_launch<1, 4, 8, 1>(L, n, scratch, stride, blk);
+    else if (n <= 64) td_launch<2, 8, 8, 1>(L, n, scratch, stride, blk);
+    else if (n <= 96) td_launch<3, 8, 8, 1>(L, n, scratch, stride, blk);
+    else td_launch<4, 8, 8, 1>(L, n, scratch, stride, blk);
   }
 }
-template void launch_rr_td<float>(const Launch&, int, unsigned char*, size_t, int);
-template void launch_rr_td<double>(const Launch&, int, unsigned char*, size_t, int);
 
 }  // namespace sgo

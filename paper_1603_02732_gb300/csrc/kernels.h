@@ -227,19 +227,24 @@ template <typename T> void launch_random_init(const Launch& L, int xrole, unsign
 // rows >= nvec: zero, or (keep_tail) left as they are
 template <typename T> void launch_copy_in(const Launch& L, int role, const double* src, int nvec, bool keep_tail = false);
 template <typename T> void launch_copy_out(const Launch& L, int role, double* dst, int nvec);
-// subspace diagonalisation, one CTA or cluster per problem (k_rr_td.cu): T = float or double; n the largest
-// subspace of the launch, at most rr_td_max(sizeof(T)); scratch of rr_td_scratch_bytes(n) bytes
-// per problem (none when it is 0)
-// blk = 1: the n_b x n_b subspace (S, Hs -> Tm); blk = 2: the 2 n_b block [X, W] of the block
-// Davidson step (S2, H2 -> the lowest n_b Ritz vectors, X coefficients in Tm, W in Cm)
-int rr_td_max(size_t tsize);
-size_t rr_td_scratch_bytes(int n, size_t tsize);
-template <typename T> void launch_rr_td(const Launch& L, int n, unsigned char* scratch, size_t stride, int blk);
+// subspace diagonalisation.  blk = 1: the n_b x n_b subspace (S, Hs -> Tm); blk = 2: the 2 n_b block
+// [X, W] of the block Davidson step (S2, H2 -> the lowest n_b Ritz vectors, X coefficients in Tm, W in
+// Cm).
+// FP64 path: one CTA or cluster per problem (k_rr_td.cu); n the largest subspace of the launch, at most
+// rr_td_max(); scratch of rr_td_scratch_bytes(n) bytes per problem (none when it is 0)
+int rr_td_max();
+size_t rr_td_scratch_bytes(int n);
+void launch_rr_td(const Launch& L, int n, unsigned char* scratch, size_t stride, int blk);
+// one-CTA Jacobi (mixed path); max_sweeps caps the sweeps (a stop at the cap is counted in SC_RRCAP)
+void launch_rr(const Launch& L, int use_smem, size_t smem, double* gscratch, size_t gstride, int max_sweeps = 30,
+               int blk = 1);
+void launch_rr_f32(const Launch& L, size_t smem, float* gscratch = nullptr, size_t gstride = 0, int max_sweeps = 10,
+                   int blk = 1);
 void launch_rr2_assemble(const Launch& L, int part);
 // Rayleigh-Ritz of large subspaces: one thread-block cluster per problem, matrices in a
-// per-problem global scratch of rr_cluster_scratch_bytes(n, sizeof(T)) bytes; max_sweeps caps the
-// Jacobi sweeps (a stop at the cap is counted in SC_RRCAP).  False if the launch was refused (its
-// shared memory would not fit).
+// per-problem global scratch of rr_cluster_scratch_bytes(n, sizeof(T)) bytes (T = float:
+// deviation-form FP32 as k_rr_f32; T = double: the same in FP64).  False if the launch
+// was refused (its shared memory would not fit).
 size_t rr_cluster_scratch_bytes(int n, size_t tsize);
 size_t rr_cluster_smem(int n);
 size_t rr_cluster_smem64(int n);

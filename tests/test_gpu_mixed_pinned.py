@@ -103,6 +103,14 @@ def evaluation(sgo, name, nbands=None, **opts):
     return [float(F)] + [float(v) for v in np.asarray(forces).ravel()]
 
 
+def population(sgo, sub_batches):
+    sts = [workloads.de_candidate(i) for i in (1, 8, 26, 44)] + [workloads.tiny(nat=2, ecut=9.0)]
+    ctxs = [sgo.Context(st, precision="mixed", scf_tol_e=1e-7 * len(st.pos), scf_tol_rho=1e-5, max_scf=150, autotune=0,
+                        sub_batches=sub_batches) for st in sts]
+    F, forces, _ = sgo.Batch(ctxs).energy_forces()
+    return [float(v) for v in F] + [float(v) for f in forces for v in np.asarray(f).ravel()]
+
+
 # every pinned result: name -> how it is computed
 CASES = {}
 for _g in GRIDS:
@@ -113,6 +121,16 @@ for _p in PRODUCTS:
     CASES["products %s, %d bands, gemm_tc=%d" % _p] = lambda s, p=_p: products(s, *p)
 for _n in STRUCTURES:  # (the eigensolve of a cluster of CTAs at every size)
     CASES["evaluation %s, rr_cluster=1" % _n] = lambda s, n=_n: evaluation(s, n, rr_cluster=1)
+for _n in STRUCTURES:
+    CASES["evaluation %s" % _n] = lambda s, n=_n: evaluation(s, n)
+CASES["evaluation diamond8, 130 bands, rr_cluster=0"] = lambda s: evaluation(s, "diamond8", 130, rr_cluster=0)
+for _n in ("cluster5", "de44"):
+    CASES["evaluation %s, rr_fp64=1" % _n] = lambda s, n=_n: evaluation(s, n, rr_fp64=1)
+CASES["evaluation de44, gemm_tc=0"] = lambda s: evaluation(s, "de44", gemm_tc=0)
+CASES["evaluation tiny3, davidson"] = lambda s: evaluation(s, "tiny3", eigensolver="davidson")
+CASES["evaluation cluster5, davidson"] = lambda s: evaluation(s, "cluster5", eigensolver="davidson")
+for _k in (1, 2):
+    CASES["population, sub_batches=%d" % _k] = lambda s, k=_k: population(s, k)
 
 
 @pytest.mark.parametrize("name", CASES)
