@@ -2,7 +2,7 @@
 // diagonalisation of Algorithm 1): S = L L^T, C = L^-1 Hs L^-T, C = V diag(eps) V^T, Tm = L^-T V, so
 // that X Tm is orthonormal and diagonalises H in the subspace.
 //
-//  1. Cholesky in deviation form: S = I + E, d_k = E_kk, L_ik = E_ik / sqrt(1 + d_k).
+//  1. Cholesky of S.
 //  2. W = L^-1 Hs and C = W L^-T by forward substitution down columns.
 //  3. Householder tridiagonalisation of C (Golub & Van Loan, section 8.3.1).
 //  4. Divide and conquer on the tridiagonal matrix (Cuppen, Numer. Math. 36, 177 (1981)): leaves of
@@ -330,7 +330,7 @@ __global__ void __launch_bounds__(32 * NW, 1)
   const int tid = threadIdx.x, lane = tid & 31, lwarp = tid >> 5;
   const int warp = team.rank * MW + lwarp;  // (a matrix warp's number)
   // vectors
-  T* dk = reinterpret_cast<T*>(smem_raw);  // 1 / (1 + d_k); 0 marks a left-out direction
+  T* dk = reinterpret_cast<T*>(smem_raw);  // 1 / L_kk; 0 marks a left-out direction
   T* vbuf = dk + vn;                       // [2][vn] Householder vectors in turn
   T* pv = vbuf + 2 * vn;                   // C v
   T* wv = pv + vn;                         // the rank-two update's w
@@ -372,9 +372,7 @@ __global__ void __launch_bounds__(32 * NW, 1)
         const int i = i0 + a, j = lane + 32 * c;
         A[a][c] = T(0);
         if (i < n && j < n) {
-          double s = Sin[(size_t)i * n + j];
-          if (i == j) s -= 1.0;
-          A[a][c] = (T)s;
+          A[a][c] = Sin[(size_t)i * n + j];
         }
       }
     // (only entries j >= i of the trailing rows are kept up to date)
@@ -395,9 +393,9 @@ __global__ void __launch_bounds__(32 * NW, 1)
           for (int c = 0; c < NR; ++c)
             if (c == (k >> 5)) x = row[c];
           x = __shfl_sync(0xffffffffu, x, k & 31);
-          const bool drop = blk == 2 && k >= P.nb && x <= T(TD_DROP) - T(1);
-          const bool bad = !drop && !(x > T(-0.999));
-          const T inv = drop ? T(0) : td_rsqrt(T(1) + (bad ? T(-0.999) : x));
+          const bool drop = blk == 2 && k >= P.nb && x <= TD_DROP;
+          const bool bad = !drop && !(x > T(0));  // (S not positive definite; the bands need no norm of 1)
+          const T inv = drop ? T(0) : td_rsqrt(bad ? T(1) : x);
           if (lane == 0) {
             team.put(&dk[k], inv);
             if (bad) team.put(&flags[0], 1);
@@ -436,7 +434,7 @@ __global__ void __launch_bounds__(32 * NW, 1)
       }
     }
     // ---- 2. W = L^-1 Hs, C = W L^-T (a warp owns columns i0 .. i0 + RPW - 1; no barriers) ----
-    // forward substitution: x_k = h_k / (1 + d_k), h_r -= D_rk x_k for r > k
+    // forward substitution: x_k = h_k / L_kk, h_r -= L_rk x_k for r > k
     auto forward = [&](T(&X)[RPW][NR]) {
 #pragma unroll
       for (int ck = 0; ck < NR; ++ck) {

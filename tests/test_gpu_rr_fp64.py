@@ -1,0 +1,60 @@
+"""The FP64 path's subspace diagonalisation (Cholesky of the overlap, tridiagonalisation, divide and
+conquer): the blocks of wavefunctions it has to take, and each form of its launch."""
+import dataclasses
+
+import numpy as np
+import pytest
+
+import workloads
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def sgo():
+    from paper_1603_02732_gb300 import build
+    build.build()
+    import paper_1603_02732_gb300 as pkg
+    pkg.load_library()
+    return pkg
+
+
+OPTS = dict(precision="fp64", scf_tol_e=1e-10, scf_tol_rho=1e-8, max_scf=100)
+
+
+# a start of small norm, and two bands that nearly agree (squared distance 8e-4, 2e-6), in every size class
+@pytest.mark.parametrize("bands", [5, 40, 80, 120])
+@pytest.mark.parametrize("change", ["scaled 0.03", "scaled 1e-5", "overlap 0.9996", "overlap 0.999999"])
+def test_states_need_not_be_orthonormal(sgo, bands, change):
+    """sgo_set_state takes wavefunctions that are not orthonormal: the evaluation from them converges to
+    the same F (second order in the density error of 1e-8 per electron: below 1e-9)."""
+    st = dataclasses.replace(workloads.tiny(nat=2 if bands > 5 else 1, ecut=9.0, kT=0.01), nbands=bands)
+    ref = sgo.Context(st, **OPTS)
+    F = ref.energy_forces()[0]
+    rho, psi = ref.get_state()
+    what, by = change.split()
+    psi = psi.copy()
+    if what == "scaled":
+        psi *= float(by)
+    else:
+        psi[1] = float(by) * psi[0] + np.sqrt(1.0 - float(by) ** 2) * psi[1]
+    ctx = sgo.Context(st, **OPTS)
+    ctx.set_state(rho, psi)
+    got = ctx.energy_forces()[0]  # (raises unless SGO_OK)
+    assert abs(got - F) < 1e-9
+    psi = ctx.get_state()[1]
+    assert np.abs(psi @ psi.T - np.eye(bands)).max() < 1e-12
+
+
+@pytest.mark.parametrize("missing", [0, 1, 3])
+def test_nearly_as_many_bands_as_plane_waves(sgo, missing):
+    """The random start is not normalised, and with (nearly) as many bands as plane waves its last
+    directions are nearly dependent."""
+    st = dataclasses.replace(workloads.tiny(nat=1, ecut=2.0, kT=0.01), nbands=3)
+    npw = sgo.Context(st, extra_bands=0, precision="fp64").npw
+    assert npw <= 128
+    st = dataclasses.replace(st, nbands=npw - missing)
+    ctx = sgo.Context(st, extra_bands=0, **OPTS)
+    ctx.energy_forces()
+    psi = ctx.get_state()[1]
+    assert np.abs(psi @ psi.T - np.eye(npw - missing)).max() < 1e-11
