@@ -1780,7 +1780,6 @@ bool launch_rr_cluster(const Launch& L, int n_max, unsigned char* scratch, size_
   const bool rows_smem = rr_cluster_rows_fit(n_max, sizeof(T));
   const size_t smem = rr_cluster_smem_t(n_max, sizeof(T), rows_smem);
   if (smem > 227 * 1024) return false;
-  cudaFuncSetAttribute(k_rr_cluster<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(L.ka.nprob * RR_CLUSTER);
   cfg.blockDim = dim3(RR_THREADS);
@@ -1978,6 +1977,14 @@ void linalg_set_smem_limits(size_t bytes) {
   // (k_rr_f32 keeps its matrices in shared memory up to 216 KB; its static arrays take the
   // rest of the 227 KB)
   cudaFuncSetAttribute(k_rr_f32, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)std::min(bytes, (size_t)216 * 1024));
+  // (all that the static arrays leave; set here and not at the launch, where another thread's smaller
+  // structure could lower it again)
+  cudaFuncAttributes at;
+  if (cudaFuncGetAttributes(&at, k_rr_cluster<float>) == cudaSuccess)
+    cudaFuncSetAttribute(k_rr_cluster<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024 - (int)at.sharedSizeBytes);
+  if (cudaFuncGetAttributes(&at, k_rr_cluster<double>) == cudaSuccess)
+    cudaFuncSetAttribute(k_rr_cluster<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024 - (int)at.sharedSizeBytes);
+  rr_td_set_smem_limits();
   // the NN kernel also has 8 KB of static shared memory: request only what it uses
   cudaFuncSetAttribute(k_gemm_nn<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, NN_KP * 64 * (int)sizeof(float));
 }

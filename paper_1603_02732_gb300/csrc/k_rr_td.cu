@@ -993,7 +993,6 @@ static void td_launch(const Launch& L, int n, unsigned char* scratch, size_t str
   const bool all = td_smem(n, true) <= TD_SMEM_MAX;
   const size_t smem = td_smem(n, all);
   auto* fn = k_rr_td<NR, MW, NW, CL>;
-  cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = L.ka.nprob * CL;
   cfg.blockDim = 32 * NW;
@@ -1006,7 +1005,8 @@ static void td_launch(const Launch& L, int n, unsigned char* scratch, size_t str
   at[0].val.clusterDim.z = 1;
   cfg.attrs = at;
   cfg.numAttrs = CL > 1 ? 1 : 0;
-  cudaLaunchKernelEx(&cfg, fn, L.ka, reinterpret_cast<T*>(scratch), stride / sizeof(T), all ? 1 : 0, blk);
+  cuda_ok(cudaLaunchKernelEx(&cfg, fn, L.ka, reinterpret_cast<T*>(scratch), stride / sizeof(T), all ? 1 : 0, blk),
+          "subspace eigensolve launch");
 }
 
 // n: the largest subspace of the launch (n_b, or 2 n_b for blk = 2).  CTAs per problem: more of them
@@ -1034,6 +1034,18 @@ void launch_rr_td(const Launch& L, int n, unsigned char* scratch, size_t stride,
     else if (n <= 96) td_launch<3, 8, 8, 1>(L, n, scratch, stride, blk);
     else td_launch<4, 8, 8, 1>(L, n, scratch, stride, blk);
   }
+}
+
+// (Every size's limit, once per engine: the limit belongs to the process, so that one set before each
+// launch could be lowered by another thread's smaller structure in between.)
+template <int NR, int MW, int NW, int CL>
+static void td_limit() {
+  cudaFuncSetAttribute(k_rr_td<NR, MW, NW, CL>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)TD_SMEM_MAX);
+}
+void rr_td_set_smem_limits() {
+  td_limit<1, 2, 2, 8>(), td_limit<2, 4, 4, 8>(), td_limit<3, 6, 6, 8>(), td_limit<4, 8, 8, 8>();
+  td_limit<1, 2, 2, 4>(), td_limit<2, 4, 4, 4>(), td_limit<3, 6, 6, 4>(), td_limit<4, 8, 8, 4>();
+  td_limit<1, 4, 8, 1>(), td_limit<2, 8, 8, 1>(), td_limit<3, 8, 8, 1>(), td_limit<4, 8, 8, 1>();
 }
 
 }  // namespace sgo

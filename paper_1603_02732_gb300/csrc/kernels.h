@@ -234,6 +234,7 @@ template <typename T> void launch_copy_out(const Launch& L, int role, double* ds
 // rr_td_max(); scratch of rr_td_scratch_bytes(n) bytes per problem (none when it is 0)
 int rr_td_max();
 size_t rr_td_scratch_bytes(int n);
+void rr_td_set_smem_limits();
 void launch_rr_td(const Launch& L, int n, unsigned char* scratch, size_t stride, int blk);
 // one-CTA Jacobi (mixed path); max_sweeps caps the sweeps (a stop at the cap is counted in SC_RRCAP)
 void launch_rr(const Launch& L, int use_smem, size_t smem, double* gscratch, size_t gstride, int max_sweeps = 30,

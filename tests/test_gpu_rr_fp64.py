@@ -1,6 +1,7 @@
 """The FP64 path's subspace diagonalisation (Cholesky of the overlap, tridiagonalisation, divide and
 conquer): the blocks of wavefunctions it has to take, and each form of its launch."""
 import dataclasses
+import threading
 
 import numpy as np
 import pytest
@@ -58,3 +59,35 @@ def test_nearly_as_many_bands_as_plane_waves(sgo, missing):
     ctx.energy_forces()
     psi = ctx.get_state()[1]
     assert np.abs(psi @ psi.T - np.eye(npw - missing)).max() < 1e-11
+
+
+# two sizes of one launch form, in FP64 and on the cluster of 8 CTAs
+@pytest.mark.parametrize("opts,bands", [(dict(OPTS, max_scf=3), (66, 96)), (dict(OPTS, max_scf=3, rr_cluster=1), (20, 100)),
+                                        (dict(precision="mixed", max_scf=3, rr_cluster=1), (20, 120))])
+def test_contexts_on_two_threads(sgo, opts, bands):
+    """Different contexts may be used from different threads (include/sgo.h): a small and a large
+    structure evaluated side by side give what each gives alone."""
+    import torch
+    made = []
+    for n in bands:
+        st = dataclasses.replace(workloads.tiny(nat=2, ecut=9.0, kT=0.01), nbands=n)
+        stream = torch.cuda.Stream()
+        ctx = sgo.Context(st, stream=stream.cuda_stream, extra_bands=0, **opts)
+        made.append((stream, ctx, ctx.energy_forces(check=False)[0]))
+    wrong = []
+
+    def work(ctx, want):
+        for _ in range(100):
+            try:
+                got = ctx.energy_forces(check=False)[0]
+            except Exception as e:  # noqa: BLE001
+                got = str(e)
+            if got != want:
+                wrong.append((got, want))
+
+    threads = [threading.Thread(target=work, args=(c, w)) for _, c, w in made]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    assert not wrong, (len(wrong), wrong[0])
