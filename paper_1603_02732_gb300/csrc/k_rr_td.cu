@@ -301,10 +301,11 @@ __device__ __forceinline__ void ldv(const T* p, T (&o)[R]) {
 
 __host__ __device__ inline int td_zs(int n) { return n > 16 ? ((n + 1) / 2) | 1 : 9; }  // row stride of the vectors
 __host__ __device__ inline int td_us(int n) { return (n + 3) & ~3; }        // row stride of the merge matrix
+constexpr int TD_RED = 64;  // one value for each matrix warp of a cluster
 constexpr int TD_PAD = 32;  // vectors are read in whole groups of rows past n
 __host__ __device__ inline int td_vn(int n) { return ((n + 3) & ~3) + TD_PAD; }
 __host__ __device__ inline size_t td_vec_bytes(int n) {
-  return ((size_t)(13 * td_vn(n) + 32) * sizeof(T) + (size_t)(3 * td_vn(n) + 16) * 4 + 15) / 16 * 16;
+  return ((size_t)(13 * td_vn(n) + TD_RED) * sizeof(T) + (size_t)(3 * td_vn(n) + 16) * 4 + 15) / 16 * 16;
 }
 
 }  // namespace
@@ -317,6 +318,7 @@ __global__ void __launch_bounds__(32 * NW, 1)
   static_assert(CL == 1 || MW == NW, "in a cluster every warp is a matrix warp");
   constexpr int RPW = 32 * NR / (MW * CL), NT = 32 * NW, MT = 32 * MW;
   static_assert(RPW * MW * CL == 32 * NR && RPW % 2 == 0, "whole vectors of rows");
+  static_assert(MW * CL <= TD_RED && NW <= TD_RED, "a value of red for every warp");
   using N = TdNum<T>;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const int p = blockIdx.x / CL;
@@ -342,9 +344,9 @@ __global__ void __launch_bounds__(32 * NW, 1)
   T* zw = ds + vn;                         // rho z^2, sorted
   T* zh = zw + vn;                         // z, sorted
   T* mu = zh + vn;                         // root i = ds[kx[i]] + mu[i]
-  T* red = mu + vn;                        // [32]
+  T* red = mu + vn;                        // [TD_RED]
   T* nd = vbuf;                            // new eigenvalues (the reflectors are done with by then)
-  int* perm = reinterpret_cast<int*>(red + 32);
+  int* perm = reinterpret_cast<int*>(red + TD_RED);
   int* kx = perm + vn;
   int* bk = kx + vn;                       // block of each index: lo | mid << 10 | hi << 20
   float* fz = reinterpret_cast<float*>(wv);  // the weights as floats
