@@ -101,3 +101,23 @@ def test_davidson_blocks(sgo, bands):
     st = dataclasses.replace(workloads.tiny(nat=2 if bands > 5 else 1, ecut=9.0, kT=0.01), nbands=bands)
     F = [sgo.Context(st, extra_bands=0, eigensolver=e, **OPTS).energy_forces()[0] for e in ("cg", "davidson")]
     assert abs(F[0] - F[1]) < 1e-9
+
+
+# 8, 4 and 1 CTAs per problem (9, 10 and 20 members a launch) above 64 bands, with the matrices in shared
+# memory and (from about 90 bands) the factors and reflectors in global scratch
+@pytest.mark.parametrize("members", [9, 10, 20])
+@pytest.mark.parametrize("bands", [80, 96, 120, 128])
+def test_launch_forms(sgo, members, bands):
+    """A member's F and spectrum after a few iterations are bitwise those of a batch of two: the CTAs of a
+    problem share its work without changing a sum."""
+    st = dataclasses.replace(workloads.tiny(nat=2, ecut=9.0, kT=0.01), nbands=bands)
+
+    def run(n):
+        ctxs = [sgo.Context(st, precision="fp64", max_scf=3, autotune=0, sub_batches=1, extra_bands=0) for _ in range(n)]
+        F = sgo.Batch(ctxs).energy_forces()[0]
+        return F, [c.eigen()[0] for c in ctxs]
+
+    F, eps = run(members)
+    F2, eps2 = run(2)
+    assert np.all(F == F2[0])
+    assert all(np.array_equal(e, eps2[0]) for e in eps)
