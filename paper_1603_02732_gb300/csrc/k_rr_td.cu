@@ -66,24 +66,9 @@ struct TdNum<double> {
 // square being below rounding)
 constexpr int TD_ITERS = 60;  // cap of the root iteration (typically 4)
 
-// 1 / x by the approximate reciprocal and Newton steps r += r (1 - x r): one in FP32, two in FP64
-// (4 FP64 operations)
-__device__ __forceinline__ float td_rcp(float x) {
-  const float r = __fdividef(1.f, x);
-  return fmaf(r, fmaf(-x, r, 1.f), r);
-}
-__device__ __forceinline__ double td_rcp(double x) {
-  double r;
-  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(x));
-  r = fma(r, fma(-x, r, 1.0), r);
-  return fma(r, fma(-x, r, 1.0), r);
-}
-__device__ __forceinline__ double td_rsqrt(double x) {  // two Newton steps on the approximate one
-  double r;
-  asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(x));
-  r = fma(0.5 * r, fma(-x * r, r, 1.0), r);
-  return fma(0.5 * r, fma(-x * r, r, 1.0), r);
-}
+// (correctly rounded over the whole range, subnormal numbers among it)
+__device__ __forceinline__ float td_rcp(float x) { return __frcp_rn(x); }
+__device__ __forceinline__ double td_rcp(double x) { return __drcp_rn(x); }
 
 __device__ __forceinline__ T wsum(T v) {
 #pragma unroll
@@ -207,7 +192,7 @@ __device__ __forceinline__ void td_leaf(T (&d)[M], T (&e)[M], T (&z)[M], int m0,
       for (int i = M - 2; i >= 0; --i)
         if (i < m && i >= l && !cut) {
           const T f = s * e[i], b = c * e[i], h = fma(f, f, g * g);
-          const T ir = td_rsqrt(h);
+          const T ir = rsqrt(h);
           if (h > TdNum<T>::floor) {
             e[i + 1] = h * ir;
             s = f * ir;
@@ -397,7 +382,7 @@ __global__ void __launch_bounds__(32 * NW, 1)
           x = __shfl_sync(0xffffffffu, x, k & 31);
           const bool drop = blk == 2 && k >= P.nb && x <= TD_DROP;
           const bool bad = !drop && !(x > T(0));  // (S not positive definite; the bands need no norm of 1)
-          const T inv = drop ? T(0) : td_rsqrt(bad ? T(1) : x);
+          const T inv = drop ? T(0) : rsqrt(bad ? T(1) : x);
           if (lane == 0) {
             team.put(&dk[k], inv);
             if (bad) team.put(&flags[0], 1);
@@ -553,7 +538,7 @@ __global__ void __launch_bounds__(32 * NW, 1)
         sg = wsum(sg);
         T beta = x1, f = T(0), tk = T(0);
         if (sg > T(0)) {
-          const T s2 = fma(x1, x1, sg), r = td_rsqrt(s2), m = s2 * r;  // |x| = m
+          const T s2 = fma(x1, x1, sg), r = rsqrt(s2), m = s2 * r;  // |x| = m
           beta = x1 > T(0) ? -m : m;
           f = td_rcp(x1 - beta);
           tk = fma(fabs(x1), r, T(1));
@@ -839,7 +824,7 @@ __global__ void __launch_bounds__(32 * NW, 1)
       }
       s = gsum(s, g);
       if (K >= 0) {
-        const T f = td_rsqrt(s);
+        const T f = rsqrt(s);
         for (int j = lo + sub; j < hi; j += g) Ub[(size_t)perm[j] * us + i] *= f;
       } else if (live && sub == 0) {
         Ub[(size_t)perm[i] * us + i] = T(1);

@@ -121,3 +121,16 @@ def test_launch_forms(sgo, members, bands):
     F2, eps2 = run(2)
     assert np.all(F == F2[0])
     assert all(np.array_equal(e, eps2[0]) for e in eps)
+
+
+@pytest.mark.parametrize("bands", [5, 40])
+def test_state_of_subnormal_overlaps(sgo, bands):
+    """The reciprocals and square roots of the Cholesky cover the subnormal numbers: from wavefunctions
+    scaled by 1e-156 (overlaps near 1e-312, 11 digits) the evaluation converges to the same F."""
+    st = dataclasses.replace(workloads.tiny(nat=2 if bands > 5 else 1, ecut=9.0, kT=0.01), nbands=bands)
+    ref = sgo.Context(st, **OPTS)
+    F = ref.energy_forces()[0]
+    rho, psi = ref.get_state()
+    ctx = sgo.Context(st, **OPTS, extra_bands=0)
+    ctx.set_state(rho, 1e-156 * psi)
+    assert abs(ctx.energy_forces()[0] - F) < 1e-9
