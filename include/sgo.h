@@ -215,8 +215,9 @@ SGO_API sgo_status sgo_batch_create(int n, sgo_ctx* const* ctxs, sgo_batch** out
 
 /* The GEMM tile knobs the batch's autotuner picked when the batch was created (mixed path;
  * the defaults otherwise): knobs[0] = K chunk of the tensor-core TN GEMM (of 256, 512, 1024,
- * 2048), knobs[1] = 128-wave tiles per tensor-core NN CTA (of 2, 4, 8, 16), knobs[2] = K
- * chunk of the CUDA-core TN GEMM (of 128, 256, 512).  Each candidate is timed on the batch's
+ * 2048), knobs[1] = 128-wave tiles per tensor-core NN CTA, at most (of 2, 4, 8, 16; a
+ * launch with less than a CTA per SM takes fewer; the default where that makes all of them one),
+ * knobs[2] = K chunk of the CUDA-core TN GEMM (of 128, 256, 512).  Each candidate is timed on the batch's
  * own buffers; the fastest is kept.  A batch split into sub-batches tunes each on its own;
  * knobs are those of the first sub-batch (the one given the costliest member). */
 SGO_API sgo_status sgo_batch_tuning(const sgo_batch* batch, int* knobs);

@@ -776,12 +776,14 @@ void Engine::autotune() {
     if (cudaEventElapsedTime(&ms, a, b) != cudaSuccess) ms = 1e30f;
     return ms;
   };
-  auto pick = [&](int* knob, std::initializer_list<int> cands, auto&& fn) {
+  // same(v): whether candidate v makes the launches of one already timed
+  auto pick = [&](int* knob, std::initializer_list<int> cands, auto&& fn, auto&& same) {
     int best = *knob;
     float tbest = 1e30f;
     for (int v : cands) {
       *knob = v;
       build_gemm_maps();
+      if (same()) continue;
       const float t = time_of(fn);
       if (t < tbest) {
         tbest = t;
@@ -791,9 +793,29 @@ void Engine::autotune() {
     *knob = best;
     build_gemm_maps();
   };
-  if (tc_ok_[OPK_WB]) pick(&tc_kc_, {256, 512, 1024, 2048}, [&] { tn<float>(OPK_WB, WB_X, OPK_WB, WB_HX, DD_HS); });
-  pick(&tn_kc_, {128, 256, 512}, [&] { tn<float>(OPK_WB, WB_X, OPK_WB, WB_X, DD_S, false); });
-  if (nn_tc_ok_[OPK_WB]) pick(&nn_tpc_, {2, 4, 8, 16}, [&] { nn<float>(OPK_WB, WB_X, DD_TM, WB_W, 1.0, 0.0); });
+  auto never = [] { return false; };
+  if (tc_ok_[OPK_WB])
+    pick(&tc_kc_, {256, 512, 1024, 2048}, [&] { tn<float>(OPK_WB, WB_X, OPK_WB, WB_HX, DD_HS); }, never);
+  pick(&tn_kc_, {128, 256, 512}, [&] { tn<float>(OPK_WB, WB_X, OPK_WB, WB_X, DD_S, false); }, never);
+  // the rotation of four blocks, the SCF's largest; few tiles cap the knob (build_gemm_maps), so that
+  // candidates beyond the cap are one launch: the smallest such counts, and the default stays where
+  // there is only one
+  if (nn_tc_ok_[OPK_WB]) {
+    const RolePairs four{4, {WB_X, WB_HX, WB_PP, WB_W2}, {WB_P, WB_HP, WB_W, WB_RP}};
+    std::vector<std::pair<int, int>> seen;
+    const int keep = nn_tpc_;
+    pick(&nn_tpc_, {2, 4, 8, 16}, [&] { nn_pairs<float>(OPK_WB, four, DD_TM, 1.0, 0.0, false); },
+         [&] {
+           const std::pair<int, int> v(nn_tiles_[0], nn_tiles_[1]);
+           if (std::find(seen.begin(), seen.end(), v) != seen.end()) return true;
+           seen.push_back(v);
+           return false;
+         });
+    if (seen.size() == 1) {
+      nn_tpc_ = keep;
+      build_gemm_maps();
+    }
+  }
   cudaGetLastError();
   cudaEventDestroy(a);
   cudaEventDestroy(b);

@@ -178,3 +178,12 @@ def test_occupations(sgo, nbands, kT):
     part = occ * (2.0 - occ) > 1e-6
     mu = (eps - kT * np.log(2.0 / occ.clip(1e-300) - 1.0))[part] if part.any() else np.zeros(1)
     assert np.ptp(mu) < 1e-9 * max(1.0, kT) + 1e-12
+
+
+def test_autotuner_of_few_tiles(sgo):
+    """Two small members have less than a CTA per SM for any number of tiles per rotation CTA: the
+    candidates are one launch, and the tuned batch keeps the default on every creation."""
+    st = workloads.tiny(nat=2, ecut=6.0)
+    for _ in range(8):
+        b = sgo.Batch([sgo.Context(st, precision="mixed") for _ in range(2)])
+        assert b.tuning()["nn_tc_tiles_per_cta"] == 4
