@@ -152,14 +152,17 @@ __global__ void __launch_bounds__(256) k_gemm_tn(KArgs ka, int akind, int arole,
   const int ld = P.ld;
   const int ti0 = 4 * bi * pa, tj0 = 4 * bj * pb;
   const int ca = min(pa, ga - bi * pa), cb = min(pb, gb - bj * pb);  // tiles of this block
-  const int nt = tri ? ca * (ca + 1) / 2 : ca * cb;
-  const int ks = sizeof(T) == 8 ? 256 / nt : 1;
   const int k0 = split * kc, k1 = min(P.npw, k0 + kc);
   const int t = threadIdx.x;
-  const int tile = t % nt, slice = t / nt;
-  const bool work = slice < ks;
-  int ti, tj;
-  tn_tile(tile, ca, cb, tri, &ti, &tj);
+  int ti = t & 15, tj = t >> 4, nt = 256, ks = 1, slice = 0;
+  bool work = ti < ca && tj < cb && (!tri || ti <= tj);
+  if constexpr (sizeof(T) == 8) {
+    nt = tri ? ca * (ca + 1) / 2 : ca * cb;
+    ks = 256 / nt;
+    slice = t / nt;
+    work = slice < ks;
+    tn_tile(t % nt, ca, cb, tri, &ti, &tj);
+  }
   T acc[4][4];
 #pragma unroll
   for (int a = 0; a < 4; ++a)
@@ -198,25 +201,31 @@ __global__ void __launch_bounds__(256) k_gemm_tn(KArgs ka, int akind, int arole,
     }
     __syncthreads();
     if (kb + TN_K < k1) fetch(kb + TN_K);
-    const int kn = min(TN_K, k1 - kb);
-    if (work) {
-      int kk = kk0;
+    auto step = [&](int kk) {
+      T a[4], b[4];
+      lds4(&As[kk][4 * ti], a);
+      lds4(&Bs[kk][4 * tj], b);
+#pragma unroll
+      for (int i = 0; i < 4; ++i)
+#pragma unroll
+        for (int j2 = 0; j2 < 4; ++j2) acc[i][j2] += a[i] * b[j2];
+    };
+    if constexpr (sizeof(T) == 8) {
+      const int kn = min(TN_K, k1 - kb);
+      if (work) {
+        int kk = kk0;
 #pragma unroll 4
-      for (; kk < kn; kk += ks) {
-        T a[4], b[4];
-        lds4(&As[kk][4 * ti], a);
-        lds4(&Bs[kk][4 * tj], b);
-#pragma unroll
-        for (int i = 0; i < 4; ++i)
-#pragma unroll
-          for (int j2 = 0; j2 < 4; ++j2) acc[i][j2] += a[i] * b[j2];
+        for (; kk < kn; kk += ks) step(kk);
+        kk0 = kk - TN_K;
       }
-      kk0 = kk - TN_K;
+    } else if (work) {  // (one slice: whole chunks, the rows beyond the split's end are zero)
+#pragma unroll 8
+      for (int kk = 0; kk < TN_K; ++kk) step(kk);
     }
     __syncthreads();
   }
   double* part = part_base + (size_t)p * part_stride + (size_t)split * na * nbv;
-  if (ks > 1) {  // add the slices of each tile in order
+  if (sizeof(T) == 8 && ks > 1) {  // add the slices of each tile in order
     T* red = reinterpret_cast<T*>(stage);  // [16][256]
     if (work)
 #pragma unroll
