@@ -25,7 +25,8 @@ struct sgo_batch {
 namespace {
 
 sgo::Engine* solo_engine(sgo_ctx* c) {
-  // A context's own engine (batch of one); rebuilt on every call (cheap: a few small maps).
+  // A context's own engine (batch of one), rebuilt on every call: about thirty small maps, each an
+  // allocation and a blocking copy (most of the host's 1.7 ms of an H psi call of the 24-atom layer).
   return new sgo::Engine(std::vector<sgo_ctx*>{c}, c->stream);
 }
 

@@ -248,7 +248,8 @@ __global__ void __launch_bounds__(PLANE_THREADS, sizeof(T) == 4 ? PLANE_MIN_BLOC
 // (24-atom layer 1020 -> 673 us, 8 atoms 215 -> 74 us, six members 1917 -> 1386 us).
 // ---------------------------------------------------------------------------
 template <typename T>
-__global__ void __launch_bounds__(PLANE_THREADS, sizeof(T) == 4 ? PLANE_MIN_BLOCKS : 2) k_plane_density(KArgs ka, const double* occ_override) {
+__global__ void __launch_bounds__(PLANE_THREADS, sizeof(T) == 4 ? PLANE_MIN_BLOCKS : 2)
+    k_plane_density(KArgs ka, const double* occ_override) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const int p = locate(ka.start, ka.nprob, blockIdx.x);
   if (!ka.active[p]) return;  // (a cluster belongs to one problem)

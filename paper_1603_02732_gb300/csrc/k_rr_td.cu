@@ -714,16 +714,12 @@ __global__ void __launch_bounds__(32 * NW, 1)
     for (int i = tid; i < n; i += NT)
       if (i > (bk[i] & 1023) && !(ds[i] - ds[i - 1] >= gap)) flags[2] = 1;
     if constexpr (CL == 1) {
-      for (int e = tid; e < n * us / (16 / (int)sizeof(T)); e += NT) reinterpret_cast<float4*>(Ub)[e] = make_float4(0.f, 0.f, 0.f, 0.f);
+      for (int e = tid; e < n * us / 2; e += NT) reinterpret_cast<double2*>(Ub)[e] = make_double2(0.0, 0.0);
     } else {  // the CTA's own columns
-      constexpr int V = RPW % (16 / (int)sizeof(T)) ? 1 : 16 / (int)sizeof(T), CW = MW * RPW / V;
+      constexpr int CW = MW * RPW / 2;
       for (int e = tid; e < n * CW; e += NT) {
-        const int j = c0 + e % CW * V;
-        if (j < us) {
-          T* const q = &Ub[(size_t)(e / CW) * us + j];
-          if constexpr (V > 1) *reinterpret_cast<float4*>(q) = make_float4(0.f, 0.f, 0.f, 0.f);
-          else *q = T(0);
-        }
+        const int j = c0 + e % CW * 2;
+        if (j < us) *reinterpret_cast<double2*>(&Ub[(size_t)(e / CW) * us + j]) = make_double2(0.0, 0.0);
       }
     }
     __syncthreads();
