@@ -28,8 +28,8 @@
 // columns and vectors of its own rows.  The leaves and the sorting are done by every CTA alike.
 // Results do not depend on the number of CTAs or warps (the sums over lanes have one shape, fused
 // multiply-adds are written out).
-// Measured, mean per launch over an evaluation, Jacobi kernel -> here: 24 bands 317 -> 205 us, 70 bands
-// 2500 -> 762 us, up to 80 bands in six members 3550 -> 818 us.
+// Measured, mean per launch over an evaluation, Jacobi kernel -> here: 24 bands 317 -> 207 us, 70 bands
+// 2500 -> 772 us, up to 80 bands in six members 3550 -> 829 us.
 #include "kernels.h"
 
 namespace sgo {
